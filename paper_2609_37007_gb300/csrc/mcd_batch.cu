@@ -1146,16 +1146,11 @@ static cudaError_t enqueue_frame(const FrameParams& p, const BatchState* bs, cud
     for (int l = 0; l < L && bs->use_tc; ++l) {
       const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
       const int Rtc = b.Rtc, qd = p.NH * p.D;
-      const dim3 pblk(tc::kPThreads);
       // RMSNorm -> QKV (hi + lo operand; after layer 0 written by the previous layer's last
       // residual pass)
       if (l == 0)
         tc_norm_operand_kernel<<<256, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi, b.xn_lo);
-      {
-        const tc::GemmArgs g{wl + bs->tw.off.qkv, nullptr, b.xn_hi, b.xn_lo, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns};
-        tc_qkv_kernel<<<tc_grid(tc_tiles(Rtc, kTcBN, p.qkv_dim, 1), p.n_cta), pblk, tc::PLayout<kTcBN, false, true>::kSmemBytes, s>>>(
-            g, b.qkv, p.qkv_dim, &b.info->M);
-      }
+      tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
       batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
       // Wo (k-split partials) -> residual, ss, the gate/up operand
       tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, s);

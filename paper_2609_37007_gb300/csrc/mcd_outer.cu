@@ -599,7 +599,7 @@ using namespace mcd;
 // last row then runs through outer_kernel, which reads that cache and samples c0.
 struct OuterTc {
   bool on = false;
-  int Rtc = 0;                     // prompt rows, rounded up to the tile width
+  int Rtc = 0;                     // capacity in operand rows
   uint8_t* w = nullptr;            // per layer: SW128 copies of the weights
   TcLayerOffsets off;
   float* X = nullptr;              // [Rtc][H] residual stream
@@ -1279,8 +1279,10 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
   const OuterTc& t = o->tc;
   const OuterStep& st = o->st;
   cudaStream_t s = o->stream;
-  const int H = p.H, L = p.L, Rtc = t.Rtc, qd = p.NH * p.D, kvl = p.NKV * st.cap * p.D;
-  const dim3 pblk(tc::kPThreads);
+  // operand rows of this prompt, not of the capacity: the tiles are shared out over the SMs by
+  // the rows there are (255 rows of 640: 144 CTAs instead of 64 to 96 per product)
+  const int H = p.H, L = p.L, qd = p.NH * p.D, kvl = p.NKV * st.cap * p.D;
+  const int Rtc = tc_operand_rows(n, p.qkv_dim, p.n_cta);
   pf_set_rows_kernel<<<1, 1, 0, s>>>(t.rows, n);
   pf_embed_kernel<<<n, 128, 0, s>>>(text_ids, t.rows, st.text_table, st.text_vocab, H, t.X, t.ss, p.err);
   tc_norm_operand_kernel<<<256, 256, 0, s>>>(t.X, p.attn_norm, t.ss, H, p.eps, t.rows, Rtc, t.xn_hi, t.xn_lo);
@@ -1288,11 +1290,7 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
     const uint8_t* wl = t.w + (size_t)l * t.off.layer;
     uint16_t* kc = reinterpret_cast<uint16_t*>(st.kcache) + (size_t)l * kvl;
     uint16_t* vc = reinterpret_cast<uint16_t*>(st.vcache) + (size_t)l * kvl;
-    {
-      const tc::GemmArgs g{wl + t.off.qkv, nullptr, t.xn_hi, t.xn_lo, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns};
-      tc_qkv_kernel<<<tc_grid(tc_tiles(Rtc, kTcBN, p.qkv_dim, 1), p.n_cta), pblk, tc::PLayout<kTcBN, false, true>::kSmemBytes, s>>>(
-          g, t.qkv, p.qkv_dim, t.rows);
-    }
+    tc_launch_qkv(wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, s);
     const int vecs = p.NH + 2 * p.NKV;
     pf_rope_kv_kernel<<<(n * vecs + 7) / 8, 256, 0, s>>>(t.qkv, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
                                                          p.q_norm + (size_t)l * p.D, p.k_norm + (size_t)l * p.D, p.eps,

@@ -71,6 +71,16 @@ __global__ void __launch_bounds__(tc::kPThreads, 1) tc_qkv_kernel(const tc::Gemm
   });
 }
 
+// The same product, one 128 x pitch tile per CTA.
+constexpr int kQkvThreads = 256;
+__global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::GemmArgs g, float* out, int ld,
+                                                                      const int* nrows) {
+  const int M = *nrows;
+  tc::gemm_tile<kTcBN, false, true>(g, [&](int m, int n, float v, float) {
+    if (n < M) out[(size_t)n * ld + m] = v;
+  });
+}
+
 // gate/up -> SwiGLU, one 128 x pitch tile per CTA (gemm_tile_run).  A is the interleaved
 // gate/up matrix of 2F rows written by tc_tile_layer: rows 0..63 of tile b are the gate rows
 // of features 64b..64b+63, rows 64..127 the up rows of the same features.  The accumulator is
@@ -254,6 +264,9 @@ inline cudaError_t tc_block_set_smem() {
   cudaError_t e = cudaFuncSetAttribute(tc_qkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        tc::PLayout<kTcBN, false, true>::kSmemBytes);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tc_qkv_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc::Layout<kTcBN, false, true>::kSmemBytes);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tc_gu_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<128>::kSmemBytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tc_gu_kernel<176>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<176>::kSmemBytes);
@@ -274,6 +287,34 @@ inline cudaError_t tc_block_set_smem() {
 // Persistent launch shape: one CTA per SM at most, one per tile at least.
 inline dim3 tc_grid(int n_tiles, int n_sm) { return dim3(n_tiles < n_sm ? n_tiles : n_sm); }
 inline int tc_tiles(int N, int BN, int M, int splits) { return (N / BN) * (M / tc::kBM) * splits; }
+
+// The QKV product's form at n packed rows: the persistent one when its 128-column tiles give at
+// least four fifths of the SMs a tile, else one tile per CTA with the columns shared out over
+// all SMs (QKV of 4096 x 1024 on 152 SMs: from 385 rows on).  Measured both ways: 512 rows
+// (128 streams) 343.9 us per call persistent, 346.2 one tile per CTA; 128 rows (32 streams)
+// 267.2 and 265.7; a prompt of 255 rows is 64 tiles of 128 columns against 128 of 64.
+inline bool tc_qkv_persistent(int n, int qkv_dim, int n_sm) {
+  return tc_tiles((n + kTcBN - 1) / kTcBN * kTcBN, kTcBN, qkv_dim, 1) * 5 >= n_sm * 4;
+}
+// Operand rows for n packed rows: what the QKV form needs, else the next multiple of 16.
+inline int tc_operand_rows(int n, int qkv_dim, int n_sm) {
+  const int unit = tc_qkv_persistent(n, qkv_dim, n_sm) ? kTcBN : 16;
+  return (n + unit - 1) / unit * unit;
+}
+// q, k, v of Rtc operand rows.  Below tc_qkv_persistent's line the pitch is at most kTcBN: nt
+// tiles of 128 columns over n_mt weight tiles with nt n_mt < 0.8 n_sm leave n_sm / n_mt >= nt.
+inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t* xn_lo, float* out, int qkv_dim, int Rtc,
+                          int H, const int* nrows, int* err, unsigned long long wait_ns, int n_sm, cudaStream_t s) {
+  tc::GemmArgs g{w, nullptr, xn_hi, xn_lo, qkv_dim, Rtc, H, nrows, err, wait_ns, 0};
+  if (tc_qkv_persistent(Rtc, qkv_dim, n_sm)) {
+    tc_qkv_kernel<<<tc_grid(tc_tiles(Rtc, kTcBN, qkv_dim, 1), n_sm), tc::kPThreads,
+                    tc::PLayout<kTcBN, false, true>::kSmemBytes, s>>>(g, out, qkv_dim, nrows);
+  } else {
+    g.bn = tc::tile_pitch(qkv_dim, Rtc, n_sm);
+    tc_qkv_tile_kernel<<<dim3((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM), kQkvThreads,
+                         tc::Layout<kTcBN, false, true>::kSmemBytes, s>>>(g, out, qkv_dim, nrows);
+  }
+}
 
 // gate/up -> SwiGLU into the down product's operand.  gu: the interleaved gate/up matrix
 // (2F rows); xn: the normalised operand of Rtc rows.  The tile pitch over the packed rows fills

@@ -8,9 +8,13 @@
 //   pack -> embed -> 5 x [QKV GEMM -> attention -> Wo GEMM (+residual) -> gate/up GEMM
 //   (SwiGLU) -> down GEMM (+residual)] -> LM-head GEMM (grouped by head) -> top-k -> accept
 //
-// captured once per context as a CUDA graph holding n_pos call bodies (a call never emits
-// fewer than one code, so n_pos calls always finish a frame; bodies after the last active
-// call find no rows and return at once).  RMSNorm never gets its own pass.  With bf16
+// captured once per context as a CUDA graph: a while node whose body is one call, repeated
+// until every stream's frame is complete (a call never emits fewer than one code, so n_pos
+// calls always finish a frame).  Where the caller itself captures a graph, which cannot embed
+// one that holds a conditional node, the n_pos bodies are enqueued one after another; bodies
+// after the last active call find no rows and return at once.  Measured with frames of 5 calls of
+// 15: 1792 us per frame of 8 streams and 2486 of 128 with the bodies enqueued, 1327 and 1955
+// with the while node.  RMSNorm never gets its own pass.  With bf16
 // weights whose widths are multiples of 128 (the MultiCodeDecoder's) every product runs on
 // the tcgen05 GEMM (mcd_tcgemm.cuh, block kernels in mcd_tcops.cuh): weights and operand
 // rows as 128-byte swizzled tiles, TMEM accumulators, the residual products split over k
@@ -62,6 +66,14 @@ struct BatchInfo {
   int n_pairs;            // (row, j) distributions of the call
   int head_rows[16];      // rows reading LM head P (entries in head_list)
   int head_off[16];
+  int call, next_call;    // index of the current call of the frame, and of the next one
+  unsigned arrived;       // acceptance CTAs done (low half) and streams not complete (high half)
+};
+
+// The while node of the frame graph (valid = 0: the calls are enqueued one by one).
+struct BatchLoop {
+  cudaGraphConditionalHandle handle;
+  int valid;
 };
 
 // Per-frame arguments, copied to the device before each graph launch.
@@ -237,6 +249,9 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
     }
     b.info->M = s_cnt[8 + 7];
     b.info->n_pairs = s_pc[8 + 7];
+    const int call = b.info->next_call;
+    b.info->call = call;
+    b.info->next_call = call + 1;
   }
   __syncthreads();
   if (tid < S && nr > 0) {
@@ -819,23 +834,38 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
 // ------------------------------------------------------------------------------------
 // top-k of every (row, j) distribution of the call; then the acceptance per stream
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParams p, BatchBufs b, int call) {
+__global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParams p, BatchBufs b) {
   __shared__ __align__(16) uint8_t smem_raw[sizeof(TopkScratch)];
   TopkScratch& ts = *reinterpret_cast<TopkScratch*>(smem_raw);
   if ((int)blockIdx.x >= b.info->n_pairs) return;
   const int e = b.pairs[blockIdx.x], r = e >> 3, j = e & 7;
   const int greedy = (j > 0 && p.draft_mode == MCD_DRAFT_GREEDY) ? 1 : 0;
-  TopkRec* recs = b.recs + (size_t)(call & 1) * b.R * kRecSlots;
+  TopkRec* recs = b.recs + (size_t)(b.info->call & 1) * b.R * kRecSlots;
   block_topk(b.logits + ((size_t)r * kRecSlots + j) * p.V, p.V, p.top_k, p.T, greedy, ts,
              recs + (size_t)r * kRecSlots + j);
 }
 
-__global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FrameParams p, BatchBufs b, int call) {
-  const int s = blockIdx.x;
+// End of a stream's acceptance (thread 0 of its CTA; `more`: its frame is not complete): the CTA
+// that arrives last decides whether the while node runs another call.  The counter is back at
+// zero for the next call.
+__device__ __forceinline__ void batch_call_end(const FrameParams& p, const BatchBufs& b, const BatchLoop& loop, int call,
+                                               bool more) {
+  if (!loop.valid) return;
+  const unsigned mine = 1u + (more ? 0x10000u : 0u);
+  const unsigned all = atomicAdd(&b.info->arrived, mine) + mine;
+  if ((all & 0xFFFFu) != gridDim.x) return;
+  b.info->arrived = 0u;
+  cudaGraphSetConditional(loop.handle, (all >> 16) != 0u && call + 1 < p.P ? 1u : 0u);
+}
+
+__global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
+  const int s = blockIdx.x, call = b.info->call;
   const BatchFrame* fa = b.frame;
-  if (s >= fa->S) return;
-  const int base = b.sbase[s];
-  if (base < 0) return;
+  const int base = s < fa->S ? b.sbase[s] : -1;
+  if (base < 0) {                       // no such stream, or its frame is complete
+    if (threadIdx.x == 0) batch_call_end(p, b, loop, call, false);
+    return;
+  }
   DevState* st = p.st + s;
   __shared__ AcceptResult s_res;
   __shared__ int s_next[kMaxDraft], s_old[kMaxDraft + 1];
@@ -979,11 +1009,16 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FramePar
             __ldcg(b.logits + ((size_t)(base + m) * kRecSlots + n + 1) * p.V + v);
     }
   }
+  if (threadIdx.x == 0) batch_call_end(p, b, loop, call, a_new < p.P);
 }
 
 __global__ void batch_begin_kernel(FrameParams p, BatchBufs b) {
   const BatchFrame* fa = b.frame;
   for (int s = threadIdx.x; s < fa->S; s += blockDim.x) init_stream_state(p.st + s, p.C0V > 0 ? fa->c0[s] : -1);
+  if (threadIdx.x == 0) {
+    b.info->next_call = 0;
+    b.info->arrived = 0u;
+  }
 }
 
 }  // namespace mcd
@@ -1134,130 +1169,161 @@ static int split_k(dim3 grid, int K, int n_sm) {
   return z;
 }
 
-// Every kernel of one frame, in stream order on `s` (captured into the graph).
-static cudaError_t enqueue_frame(const FrameParams& p, const BatchState* bs, cudaStream_t s) {
+// Every kernel of one call, in stream order on `s`.
+static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, const BatchLoop& loop, cudaStream_t s) {
   const BatchBufs& b = bs->b;
   const int R = b.R, L = p.L, H = p.H;
   const dim3 blk(256);
-  batch_begin_kernel<<<1, 256, 0, s>>>(p, b);
-  for (int call = 0; call < p.P; ++call) {
-    batch_pack_kernel<<<1, 256, 0, s>>>(p, b);
-    batch_embed_kernel<<<R, 256, 0, s>>>(p, b);
-    for (int l = 0; l < L && bs->use_tc; ++l) {
-      const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
-      const int Rtc = b.Rtc, qd = p.NH * p.D;
-      // RMSNorm -> QKV (hi + lo operand; after layer 0 written by the previous layer's last
-      // residual pass)
-      if (l == 0)
-        tc_norm_operand_kernel<<<256, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi, b.xn_lo);
-      tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
-      batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
-      // Wo (k-split partials) -> residual, ss, the gate/up operand
-      tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
-      tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
-                                             p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, nullptr);
-      // gate/up -> SwiGLU (into the down product's operand)
-      tc_launch_gu(wl + bs->tw.off.gu, b.xn_hi, b.act_t, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, s);
-      // down (k-split partials) -> residual, ss, the next layer's QKV operand
-      tc_launch_resid(wl + bs->tw.off.d, b.act_t, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
-      const bool last = l + 1 == L;
-      tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
-                                             last ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);
-    }
-    for (int l = 0; l < L && !bs->use_tc; ++l) {
-      {   // RMSNorm -> QKV
-        GemmArgs a = gemm_args(p, b);
-        a.W = p.w_qkv + (size_t)l * p.g[MAT_QKV].stride;
-        a.g = p.g[MAT_QKV];
-        a.X = b.X;
-        a.ldx = H;
-        a.gain = p.attn_norm + (size_t)l * H;
-        a.ss = b.ss + (size_t)(2 * l) * R;
-        a.out = b.qkv;
-        a.ld = p.qkv_dim;
-        batch_gemm_kernel<BSRC_NORM_HILO, EPI_QKV>
-            <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN), blk, kGemmSmemHilo, s>>>(a);
-      }
-      batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);
-      {   // Wo + residual
-        GemmArgs a = gemm_args(p, b);
-        a.W = p.w_wo + (size_t)l * p.g[MAT_WO].stride;
-        a.g = p.g[MAT_WO];
-        a.Xb = b.att;
-        a.ldx = p.NH * p.D;
-        a.out = b.X;
-        a.ld = H;
-        const dim3 grid(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN);
-        batch_gemm_kernel<BSRC_BF16, EPI_RESID><<<dim3(grid.x, grid.y, split_k(grid, a.g.K, p.n_cta)), blk, kGemmSmem, s>>>(a);
-        batch_rowss_kernel<<<R / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * l + 1) * R, b.info);
-      }
-      {   // RMSNorm -> gate/up -> SwiGLU
-        GemmArgs a = gemm_args(p, b);
-        a.W = p.w_gu + (size_t)l * p.g[MAT_GU].stride;
-        a.g = p.g[MAT_GU];
-        a.X = b.X;
-        a.ldx = H;
-        a.gain = p.ffn_norm + (size_t)l * H;
-        a.ss = b.ss + (size_t)(2 * l + 1) * R;
-        a.act = b.act;
-        a.ld = p.F;
-        batch_gemm_kernel<BSRC_NORM, EPI_SWIGLU><<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN), blk, kGemmSmem, s>>>(a);
-      }
-      {   // down + residual
-        GemmArgs a = gemm_args(p, b);
-        a.W = p.w_wd + (size_t)l * p.g[MAT_WD].stride;
-        a.g = p.g[MAT_WD];
-        a.Xb = b.act;
-        a.ldx = p.F;
-        a.out = b.X;
-        a.ld = H;
-        const dim3 grid(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN);
-        batch_gemm_kernel<BSRC_BF16, EPI_RESID><<<dim3(grid.x, grid.y, split_k(grid, a.g.K, p.n_cta)), blk, kGemmSmem, s>>>(a);
-        batch_rowss_kernel<<<R / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * l + 2) * R, b.info);
-      }
-    }
-    if (bs->tw.heads) {   // final RMSNorm -> LM heads on the tensor cores, tiles grouped by head
-      tc_heads_operand_kernel<<<512, blk, 0, s>>>(b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
-                                                 b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
-      const tc::GemmArgs g{nullptr, nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns};
-      tc_heads_kernel<<<dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
-                        tc::Layout<kHeadTileMax, false, true>::kSmemBytes, s>>>(g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
-                                                                        p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
-    } else {   // final RMSNorm -> LM heads, one grid slice per head
+  batch_pack_kernel<<<1, 256, 0, s>>>(p, b);
+  batch_embed_kernel<<<R, 256, 0, s>>>(p, b);
+  for (int l = 0; l < L && bs->use_tc; ++l) {
+    const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
+    const int Rtc = b.Rtc, qd = p.NH * p.D;
+    // RMSNorm -> QKV (hi + lo operand; after layer 0 written by the previous layer's last
+    // residual pass)
+    if (l == 0)
+      tc_norm_operand_kernel<<<256, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi, b.xn_lo);
+    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
+    batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
+    // Wo (k-split partials) -> residual, ss, the gate/up operand
+    tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
+    tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
+                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, nullptr);
+    // gate/up -> SwiGLU (into the down product's operand)
+    tc_launch_gu(wl + bs->tw.off.gu, b.xn_hi, b.act_t, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, s);
+    // down (k-split partials) -> residual, ss, the next layer's QKV operand
+    tc_launch_resid(wl + bs->tw.off.d, b.act_t, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
+    const bool last = l + 1 == L;
+    tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
+                                           last ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);
+  }
+  for (int l = 0; l < L && !bs->use_tc; ++l) {
+    {   // RMSNorm -> QKV
       GemmArgs a = gemm_args(p, b);
-      a.W = p.w_head;
-      a.g = p.g[MAT_HEAD];
+      a.W = p.w_qkv + (size_t)l * p.g[MAT_QKV].stride;
+      a.g = p.g[MAT_QKV];
       a.X = b.X;
       a.ldx = H;
-      a.gain = p.final_norm;
-      a.ss = b.ss + (size_t)(2 * L) * R;
-      a.logits = b.logits;
-      a.head_bias = p.head_bias;
-      batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>
-          <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN, p.P), blk, kGemmSmemHilo, s>>>(a);
+      a.gain = p.attn_norm + (size_t)l * H;
+      a.ss = b.ss + (size_t)(2 * l) * R;
+      a.out = b.qkv;
+      a.ld = p.qkv_dim;
+      batch_gemm_kernel<BSRC_NORM_HILO, EPI_QKV>
+          <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN), blk, kGemmSmemHilo, s>>>(a);
     }
-    batch_topk_kernel<<<R * (p.K + 1), kConsumerThreads, 0, s>>>(p, b, call);
-    batch_accept_kernel<<<bs->max_streams, kConsumerThreads, 0, s>>>(p, b, call);
+    batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);
+    {   // Wo + residual
+      GemmArgs a = gemm_args(p, b);
+      a.W = p.w_wo + (size_t)l * p.g[MAT_WO].stride;
+      a.g = p.g[MAT_WO];
+      a.Xb = b.att;
+      a.ldx = p.NH * p.D;
+      a.out = b.X;
+      a.ld = H;
+      const dim3 grid(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN);
+      batch_gemm_kernel<BSRC_BF16, EPI_RESID><<<dim3(grid.x, grid.y, split_k(grid, a.g.K, p.n_cta)), blk, kGemmSmem, s>>>(a);
+      batch_rowss_kernel<<<R / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * l + 1) * R, b.info);
+    }
+    {   // RMSNorm -> gate/up -> SwiGLU
+      GemmArgs a = gemm_args(p, b);
+      a.W = p.w_gu + (size_t)l * p.g[MAT_GU].stride;
+      a.g = p.g[MAT_GU];
+      a.X = b.X;
+      a.ldx = H;
+      a.gain = p.ffn_norm + (size_t)l * H;
+      a.ss = b.ss + (size_t)(2 * l + 1) * R;
+      a.act = b.act;
+      a.ld = p.F;
+      batch_gemm_kernel<BSRC_NORM, EPI_SWIGLU><<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN), blk, kGemmSmem, s>>>(a);
+    }
+    {   // down + residual
+      GemmArgs a = gemm_args(p, b);
+      a.W = p.w_wd + (size_t)l * p.g[MAT_WD].stride;
+      a.g = p.g[MAT_WD];
+      a.Xb = b.act;
+      a.ldx = p.F;
+      a.out = b.X;
+      a.ld = H;
+      const dim3 grid(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN);
+      batch_gemm_kernel<BSRC_BF16, EPI_RESID><<<dim3(grid.x, grid.y, split_k(grid, a.g.K, p.n_cta)), blk, kGemmSmem, s>>>(a);
+      batch_rowss_kernel<<<R / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * l + 2) * R, b.info);
+    }
   }
+  if (bs->tw.heads) {   // final RMSNorm -> LM heads on the tensor cores, tiles grouped by head
+    tc_heads_operand_kernel<<<512, blk, 0, s>>>(b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
+                                               b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
+    const tc::GemmArgs g{nullptr, nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns};
+    tc_heads_kernel<<<dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
+                      tc::Layout<kHeadTileMax, false, true>::kSmemBytes, s>>>(g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
+                                                                      p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
+  } else {   // final RMSNorm -> LM heads, one grid slice per head
+    GemmArgs a = gemm_args(p, b);
+    a.W = p.w_head;
+    a.g = p.g[MAT_HEAD];
+    a.X = b.X;
+    a.ldx = H;
+    a.gain = p.final_norm;
+    a.ss = b.ss + (size_t)(2 * L) * R;
+    a.logits = b.logits;
+    a.head_bias = p.head_bias;
+    batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>
+        <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN, p.P), blk, kGemmSmemHilo, s>>>(a);
+  }
+  batch_topk_kernel<<<R * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);
+  batch_accept_kernel<<<bs->max_streams, kConsumerThreads, 0, s>>>(p, b, loop);
   return cudaGetLastError();
+}
+
+// The frame's graph: the state reset, then the while node over the calls.
+static cudaError_t build_graph(const FrameParams& p, BatchState* bs) {
+  cudaStream_t s = bs->cap;
+  cudaError_t e = cudaGraphCreate(&bs->graph, 0);
+  if (e != cudaSuccess) return e;
+  auto capture = [&](cudaGraph_t g, auto enqueue) {
+    cudaError_t c = cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (c != cudaSuccess) return c;
+    const cudaError_t q = enqueue();
+    cudaGraph_t out = nullptr;
+    c = cudaStreamEndCapture(s, &out);
+    return q != cudaSuccess ? q : c;
+  };
+  e = capture(bs->graph, [&] {
+    batch_begin_kernel<<<1, 256, 0, s>>>(p, bs->b);
+    return cudaGetLastError();
+  });
+  if (e != cudaSuccess) return e;
+  cudaGraphNode_t begin = nullptr, loop_node = nullptr;
+  size_t n_nodes = 1;
+  if ((e = cudaGraphGetNodes(bs->graph, &begin, &n_nodes)) != cudaSuccess) return e;
+  BatchLoop loop{0, 1};
+  e = cudaGraphConditionalHandleCreate(&loop.handle, bs->graph, 1, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) return e;
+  cudaGraphNodeParams np = {};
+  np.type = cudaGraphNodeTypeConditional;
+  np.conditional.handle = loop.handle;
+  np.conditional.type = cudaGraphCondTypeWhile;
+  np.conditional.size = 1;
+  if ((e = cudaGraphAddNode(&loop_node, bs->graph, &begin, nullptr, 1, &np)) != cudaSuccess) return e;
+  e = capture(np.conditional.phGraph_out[0], [&] { return enqueue_call(p, bs, loop, s); });
+  if (e != cudaSuccess) return e;
+  return cudaGraphInstantiate(&bs->exec, bs->graph, 0);
 }
 
 mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t stream, int n, const uint32_t* stream_ids,
                         const uint32_t* frame_ids, const float* cond, const int32_t* c0, const float* c0_emb,
                         int32_t* codes_out, mcd_frame_stats* stats, uint8_t* trace) {
   if (n < 1 || n > bs->max_streams) return MCD_ERR_INVALID_ARG;
-  if (!bs->exec) {
-    cudaStream_t s = bs->cap;
-    MCD_CHECK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_frame(p, bs, s);
-    cudaGraph_t g = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(s, &g);
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      return cuda_status(e != cudaSuccess ? e : e2);
+  // a graph with a conditional node cannot become part of a graph that the caller captures
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  MCD_CHECK(cudaStreamIsCapturing(stream, &capturing));
+  const bool unrolled = capturing == cudaStreamCaptureStatusActive;
+  if (!unrolled && !bs->exec) {
+    const cudaError_t e = build_graph(p, bs);
+    if (e != cudaSuccess) {
+      if (bs->graph) cudaGraphDestroy(bs->graph);
+      bs->graph = nullptr;
+      return cuda_status(e);
     }
-    bs->graph = g;
-    MCD_CHECK(cudaGraphInstantiate(&bs->exec, g, 0));
   }
   BatchFrame& f = bs->host_frame;
   memset(&f, 0, sizeof(f));
@@ -1273,7 +1339,13 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
   f.stats = stats;
   f.trace = trace;
   MCD_CHECK(cudaMemcpyAsync(bs->b.frame, &f, sizeof(f), cudaMemcpyHostToDevice, stream));
-  MCD_CHECK(cudaGraphLaunch(bs->exec, stream));
+  if (!unrolled) {
+    MCD_CHECK(cudaGraphLaunch(bs->exec, stream));
+    return MCD_OK;
+  }
+  batch_begin_kernel<<<1, 256, 0, stream>>>(p, bs->b);
+  MCD_CHECK(cudaGetLastError());
+  for (int call = 0; call < p.P; ++call) MCD_CHECK(enqueue_call(p, bs, BatchLoop{0, 0}, stream));
   return MCD_OK;
 }
 

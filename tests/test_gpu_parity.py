@@ -387,6 +387,30 @@ def test_gemm_path_full_size(n_streams, checked):
     env.dec.close()
 
 
+def test_gemm_path_inside_a_captured_graph():
+    """A frame captured into the caller's own graph (there the calls are enqueued one after
+    another; the context's own graph loops over them) gives the codes of a direct call."""
+    cfg = TINY_BF16.replace(max_streams=16)
+    stream = torch.cuda.Stream()
+    dec = mcd.Decoder(cfg, make_weights(cfg), stream=stream)
+    frames = [make_frame(cfg, f) for f in range(16)]
+    cond, emb = t(np.stack([f.cond for f in frames])), t(np.stack([f.c0_emb for f in frames]))
+    ids = list(range(16))
+    codes = [torch.full((16, cfg.n_pos), -1, dtype=torch.int32, device=DEV) for _ in range(2)]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        mcd.mcd_decode_frames(dec.ctx, ids, ids, cond, None, emb, codes[0])
+    with torch.cuda.stream(stream):
+        graph.replay()
+    mcd.mcd_sync(dec.ctx)
+    mcd.mcd_decode_frames(dec.ctx, ids, ids, cond, None, emb, codes[1])
+    mcd.mcd_sync(dec.ctx)
+    assert (codes[0] >= 0).all() and torch.equal(codes[0], codes[1])
+    graph.reset()
+    dec.close()
+
+
 # ------------------------------------------------- sparse tree verification (Fig. 2) ---
 def _trees():
     from oracle.tree import Tree, grow_tree

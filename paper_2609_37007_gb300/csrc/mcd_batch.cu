@@ -1000,14 +1000,11 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FramePar
     }
     float* vlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls);
     float* dlog = vlog + (size_t)kMaxCalls * kMaxRows * p.V;
-    for (int idx = threadIdx.x; idx < kMaxRows * p.V; idx += blockDim.x) {
-      const int n = idx / p.V, v = idx - n * p.V;
-      if (n >= fr && n < n_rows)
-        vlog[((size_t)call * kMaxRows + n) * p.V + v] = __ldcg(b.logits + ((size_t)(base + n) * kRecSlots) * p.V + v);
-      if (n < n_next)
-        dlog[((size_t)call * kMaxRows + n) * p.V + v] =
-            __ldcg(b.logits + ((size_t)(base + m) * kRecSlots + n + 1) * p.V + v);
-    }
+    for (int n = fr; n < n_rows; ++n)
+      copy_logits(vlog + ((size_t)call * kMaxRows + n) * p.V, b.logits + (size_t)(base + n) * kRecSlots * p.V, p.V);
+    for (int n = 0; n < n_next; ++n)
+      copy_logits(dlog + ((size_t)call * kMaxRows + n) * p.V,
+                  b.logits + ((size_t)(base + m) * kRecSlots + n + 1) * p.V, p.V);
   }
   if (threadIdx.x == 0) batch_call_end(p, b, loop, call, a_new < p.P);
 }

@@ -678,6 +678,29 @@ __device__ __noinline__ void attention_tree_task(const FrameParams& p, int layer
   consumer_sync();
 }
 
+// Trace of a verify call: the verify logits of each packed row, every row by another CTA (those
+// after the CTAs that built the call's distributions).  Runs once the CTA has signalled its
+// distributions; the logits stay until the next call's LM heads, which wait for every CTA.  (One
+// CTA copying every row before it released the next call cost 14 us per call at one row, 20 us
+// at four and 127 us at 33.)
+__device__ __noinline__ void trace_verify_rows(const FrameParams& p) {
+  const CallInfo* ci = smem_layout(mcd_dyn_smem).ci;
+  const bool tree = p.draft_mode == MCD_DRAFT_TREE, noisy = p.draft_mode == MCD_DRAFT_NOISY_TARGET;
+  int at = 0;                                   // distributions of the call
+  for (int r = 0; r < ci->M; ++r)
+    if (ci->r_pos[r] >= 1) at += 1 + (noisy ? 0 : min(p.K, p.P - ci->r_pos[r]));
+  for (int r = 0; r < ci->M; ++r) {
+    if (ci->r_pos[r] < 1 || (at + r) % p.n_cta != (int)blockIdx.x) continue;
+    const int s = ci->r_s[r], round = ci->st[s].round;
+    if (round >= kMaxCalls) continue;
+    uint8_t* tb = p.trace + (size_t)s * p.trace_stride + sizeof(mcd_call_trace) * kMaxCalls;
+    const size_t chain = (size_t)2 * kMaxCalls * kMaxRows * p.V * 4 + sizeof(mcd_tree_trace) * kMaxCalls;
+    float* dst = tree ? reinterpret_cast<float*>(tb + chain) + ((size_t)round * kMaxTreeRows + ci->row0 + r) * p.V
+                      : reinterpret_cast<float*>(tb) + ((size_t)round * kMaxRows + ci->r_n[r]) * p.V;
+    copy_logits(dst, p.logits + (size_t)(ci->row0 + r) * (kMaxDraft + 1) * p.V, p.V);
+  }
+}
+
 // ------------------------------------------------------------------------------------
 // One call
 // ------------------------------------------------------------------------------------
@@ -1170,24 +1193,15 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
       for (int j = 0; j < kMaxRows; ++j) tr->next_drafts[j] = (j < s_nnext && !noisy) ? s_next[j] : -1;
       tr->draft_row = m;
     }
-    float* vlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls);
-    float* dlog = vlog + (size_t)kMaxCalls * kMaxRows * p.V;
-    for (int idx = threadIdx.x; idx < kMaxRows * p.V; idx += kConsumerThreads) {
-      const int n = idx / p.V, v = idx - n * p.V;
-      if (n >= fr && n < n_rows)
-        vlog[((size_t)round * kMaxRows + n) * p.V + v] =
-            __ldcg(p.logits + ((size_t)(base + n) * (kMaxDraft + 1)) * p.V + v);
-      if (n < s_nnext && !noisy)
-        dlog[((size_t)round * kMaxRows + n) * p.V + v] =
-            __ldcg(p.logits + ((size_t)(base + m) * (kMaxDraft + 1) + n + 1) * p.V + v);
-    }
+    // the draft rows of row m (the verify rows were copied by the top-k stage)
+    float* dlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls) + (size_t)kMaxCalls * kMaxRows * p.V;
+    for (int n = 0; n < s_nnext && !noisy; ++n)
+      copy_logits(dlog + ((size_t)round * kMaxRows + n) * p.V, p.logits + ((size_t)(base + m) * (kMaxDraft + 1) + n + 1) * p.V,
+                  p.V);
   }
-  if (p.single_call && p.logits_out) {
-    for (int idx = threadIdx.x; idx < (n_rows - fr) * p.V; idx += kConsumerThreads) {
-      const int n = fr + idx / p.V, v = idx % p.V;
-      p.logits_out[idx] = __ldcg(p.logits + ((size_t)(base + n) * (kMaxDraft + 1)) * p.V + v);
-    }
-  }
+  if (p.single_call && p.logits_out)
+    for (int n = fr; n < n_rows; ++n)
+      copy_logits(p.logits_out + (size_t)(n - fr) * p.V, p.logits + (size_t)(base + n) * (kMaxDraft + 1) * p.V, p.V);
   consumer_sync();
   if (s == 0) timeline_p(p, sm.ci, 7, true);
   if (threadIdx.x == 0) {
@@ -1380,8 +1394,8 @@ __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
     p.tree_cand[i] = (d < n_next && r < p.tree_m[d]) ? t_next[d][r] : -1;
   }
   consumer_sync();
-  // optional trace: the chain record, the draft row's logits, the tree record and every row's
-  // verify logits
+  // optional trace: the chain record, the draft row's logits and the tree record (every row's
+  // verify logits were copied by the top-k stage)
   if (p.trace && round < kMaxCalls) {
     uint8_t* tb = p.trace;
     mcd_call_trace* tr = reinterpret_cast<mcd_call_trace*>(tb) + round;
@@ -1389,7 +1403,6 @@ __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
                   (size_t)kMaxCalls * kMaxRows * p.V;
     const size_t chain_bytes = sizeof(mcd_call_trace) * kMaxCalls + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4;
     mcd_tree_trace* tt = reinterpret_cast<mcd_tree_trace*>(tb + chain_bytes) + round;
-    float* vall = reinterpret_cast<float*>(tb + chain_bytes + sizeof(mcd_tree_trace) * kMaxCalls);
     if (threadIdx.x == 0) {
       tr->a = a;
       tr->n_rows = n_rows;
@@ -1425,15 +1438,8 @@ __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
         for (int r = 0; r < kMaxTreeRank; ++r)
           tt->next_cand[d][r] = (d < n_next && d < kMaxDraft && r < p.tree_m[d]) ? t_next[d][r] : -1;
     }
-    for (int idx = threadIdx.x; idx < kMaxTreeRows * p.V; idx += kConsumerThreads) {
-      const int n = idx / p.V, v = idx - n * p.V;
-      if (n < n_rows && (pos0 > 0 || n > 0))                  // the conditioning row reads no head
-        vall[((size_t)round * kMaxTreeRows + n) * p.V + v] =
-            __ldcg(p.logits + ((size_t)n * (kMaxDraft + 1)) * p.V + v);
-      if (n < n_next)
-        dlog[((size_t)round * kMaxRows + n) * p.V + v] =
-            __ldcg(p.logits + ((size_t)drow * (kMaxDraft + 1) + n + 1) * p.V + v);
-    }
+    for (int n = 0; n < n_next; ++n)
+      copy_logits(dlog + ((size_t)round * kMaxRows + n) * p.V, p.logits + ((size_t)drow * (kMaxDraft + 1) + n + 1) * p.V, p.V);
   }
   consumer_sync();
   if (threadIdx.x == 0) red_release_add(p.ctr + (size_t)(call + 1) * p.ctr_stride + ctr_ready(p.L), 1u);
@@ -1677,6 +1683,7 @@ __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constan
         else
           accept_step(p, call, sm.flags[4]);
       }
+      if (p.trace && !sm.ci->emu) trace_verify_rows(p);
     }
     if (tid == 0) sm.flags[0] = 1;  // stop the producer
   }

@@ -56,6 +56,27 @@ __device__ __forceinline__ float exp32_cw(float d) {
 
 __device__ __forceinline__ uint32_t weight24(float e) { return __float2uint_rd(__fmul_rn(e, 16777216.0f)); }
 
+// Copy of a logits row (src 16-byte aligned, V a multiple of 16) by threads 0..nt-1 of the CTA:
+// 16-byte pieces, four in flight per thread, where the destination is aligned, else words.
+__device__ inline __noinline__ void copy_logits(float* dst, const float* src, int V, int nt = kConsumerThreads) {
+  if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+    float4* d = reinterpret_cast<float4*>(dst);
+    const float4* q = reinterpret_cast<const float4*>(src);
+    const int n = V >> 2;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * nt) {
+      float4 v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (i0 + e * nt < n) v[e] = __ldcg(q + i0 + e * nt);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (i0 + e * nt < n) d[i0 + e * nt] = v[e];
+    }
+  } else {
+    for (int i = threadIdx.x; i < V; i += nt) dst[i] = __ldcg(src + i);
+  }
+}
+
 // ---- exact 128-bit helpers -------------------------------------------------------------
 struct U128 {
   unsigned long long lo, hi;

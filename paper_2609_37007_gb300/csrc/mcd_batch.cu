@@ -270,6 +270,8 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
 
 // embed: X[r] = the row's input vector; ss[0][r] = sum of squares.
 __global__ void __launch_bounds__(256) batch_embed_kernel(FrameParams p, BatchBufs b) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= b.info->M) return;
   const BatchRow row = b.rows[r];
@@ -562,6 +564,8 @@ __global__ void __launch_bounds__(256) tc_heads_operand_kernel(const float* __re
                                                                const BatchInfo* info, const int* __restrict__ head_list,
                                                                int n_pos, int Qcap, uint8_t* hi, uint8_t* lo) {
   __shared__ int s_off[16], s_rows[16], s_q[16];
+  tc::pdl_wait();
+  tc::pdl_trigger();
   if (threadIdx.x < 16) {
     const int P = threadIdx.x;
     s_off[P] = info->head_off[P];
@@ -602,6 +606,8 @@ __global__ void __launch_bounds__(kHeadsThreads, 1) tc_heads_kernel(const tc::Ge
                                                                     size_t head_bytes, float* logits,
                                                                     const float* head_bias, const BatchInfo* info,
                                                                     const int* head_list, int n_pos, int K, int V) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   int P = 0, qoff = 0, c0 = 0, nw = 0, rows = 0;
   for (int i = 1, o = 0, t = blockIdx.x; i <= n_pos; ++i) {
     const int r = info->head_rows[i], nt = tc_head_tiles(r);
@@ -631,9 +637,9 @@ __global__ void __launch_bounds__(kHeadsThreads, 1) tc_heads_kernel(const tc::Ge
   ga.a = w_heads + (size_t)(P - 1) * head_bytes;
   ga.n_active = nullptr;
   const int q0 = qoff + c0;
-  tc::gemm_tile<kHeadTileMax, false, true>(
+  tc::gemm_tile<kHeadTileMax, true>(
       ga,
-      [&](int m, int n, float v, float) {
+      [&](int m, int n, float v) {
         const int e = s_entry[n - q0];
         if (e >= 0) {
           const int r = e >> 3, j = e & 7;
@@ -678,6 +684,8 @@ __global__ void __launch_bounds__(256) batch_rowss_kernel(const float* X, int H,
 // lane summed over the keys.  Row and head of a query vector come from a table, not a
 // division.
 __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, BatchBufs b, int layer) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int s = blockIdx.x, g = blockIdx.y;
   if (s >= b.frame->S) return;
   const int base = b.sbase[s];
@@ -837,6 +845,8 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
 __global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParams p, BatchBufs b) {
   __shared__ __align__(16) uint8_t smem_raw[sizeof(TopkScratch)];
   TopkScratch& ts = *reinterpret_cast<TopkScratch*>(smem_raw);
+  tc::pdl_wait();
+  tc::pdl_trigger();
   if ((int)blockIdx.x >= b.info->n_pairs) return;
   const int e = b.pairs[blockIdx.x], r = e >> 3, j = e & 7;
   const int greedy = (j > 0 && p.draft_mode == MCD_DRAFT_GREEDY) ? 1 : 0;
@@ -859,6 +869,8 @@ __device__ __forceinline__ void batch_call_end(const FrameParams& p, const Batch
 }
 
 __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int s = blockIdx.x, call = b.info->call;
   const BatchFrame* fa = b.frame;
   const int base = s < fa->S ? b.sbase[s] : -1;
@@ -1126,7 +1138,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
   if (bs->use_tc &&
       (tc_block_set_smem() != cudaSuccess ||
        cudaFuncSetAttribute(tc_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            tc::Layout<kHeadTileMax, false, true>::kSmemBytes) != cudaSuccess))
+                            tc::Layout<kHeadTileMax, true>::kSmemBytes) != cudaSuccess))
     return fail(MCD_ERR_CUDA);
   *out = bs;
   return MCD_OK;
@@ -1171,28 +1183,35 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
   const BatchBufs& b = bs->b;
   const int R = b.R, L = p.L, H = p.H;
   const dim3 blk(256);
+  // The products are dependent launches (their weights stream in while the kernel before them
+  // runs); the small kernels between them start the ordinary way.  Frames of 5 calls, 8 / 128
+  // streams: 1235 / 1868 us with ordinary launches, 1169 / 1805 with dependent products, 1208 /
+  // 1810 with every kernel dependent, 1275 / 1901 with only the small ones.  Outside the while
+  // node the last bodies of a frame are empty: no prefetch there.
+  const bool pdl = loop.valid != 0;
   batch_pack_kernel<<<1, 256, 0, s>>>(p, b);
-  batch_embed_kernel<<<R, 256, 0, s>>>(p, b);
+  tc::launch(false, batch_embed_kernel, dim3(R), blk, 0, s, p, b);
   for (int l = 0; l < L && bs->use_tc; ++l) {
     const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
     const int Rtc = b.Rtc, qd = p.NH * p.D;
     // RMSNorm -> QKV (hi + lo operand; after layer 0 written by the previous layer's last
     // residual pass)
     if (l == 0)
-      tc_norm_operand_kernel<<<256, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi, b.xn_lo);
-    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
-    batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
+      tc::launch(false, tc_norm_operand_kernel, dim3(256), blk, 0, s, b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi,
+                     b.xn_lo);
+    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc::launch(false, batch_attn_kernel, dim3(bs->max_streams, p.NKV), blk, 0, s, p, b, l);      // -> att_t
     // Wo (k-split partials) -> residual, ss, the gate/up operand
-    tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
-    tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
-                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, nullptr);
+    tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
+                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, (uint8_t*)nullptr);
     // gate/up -> SwiGLU (into the down product's operand)
-    tc_launch_gu(wl + bs->tw.off.gu, b.xn_hi, b.act_t, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, s);
+    tc_launch_gu(wl + bs->tw.off.gu, b.xn_hi, b.act_t, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     // down (k-split partials) -> residual, ss, the next layer's QKV operand
-    tc_launch_resid(wl + bs->tw.off.d, b.act_t, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, s);
+    tc_launch_resid(wl + bs->tw.off.d, b.act_t, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
     const bool last = l + 1 == L;
-    tc_resid_norm_kernel<<<R, 128, 0, s>>>(b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
-                                           last ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);
+    tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
+                                           last ? (const float*)nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);
   }
   for (int l = 0; l < L && !bs->use_tc; ++l) {
     {   // RMSNorm -> QKV
@@ -1247,11 +1266,11 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     }
   }
   if (bs->tw.heads) {   // final RMSNorm -> LM heads on the tensor cores, tiles grouped by head
-    tc_heads_operand_kernel<<<512, blk, 0, s>>>(b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
+    tc::launch(false, tc_heads_operand_kernel, dim3(512), blk, 0, s, b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
                                                b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
-    const tc::GemmArgs g{nullptr, nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns};
-    tc_heads_kernel<<<dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
-                      tc::Layout<kHeadTileMax, false, true>::kSmemBytes, s>>>(g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
+    const tc::GemmArgs g{nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns, false, 0};
+    tc::launch(false, tc_heads_kernel, dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
+                   tc::Layout<kHeadTileMax, true>::kSmemBytes, s, g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
                                                                       p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
   } else {   // final RMSNorm -> LM heads, one grid slice per head
     GemmArgs a = gemm_args(p, b);
@@ -1266,8 +1285,8 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>
         <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN, p.P), blk, kGemmSmemHilo, s>>>(a);
   }
-  batch_topk_kernel<<<R * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);
-  batch_accept_kernel<<<bs->max_streams, kConsumerThreads, 0, s>>>(p, b, loop);
+  tc::launch(false, batch_topk_kernel, dim3(R * (p.K + 1)), dim3(kConsumerThreads), 0, s, p, b);
+  tc::launch(false, batch_accept_kernel, dim3(bs->max_streams), dim3(kConsumerThreads), 0, s, p, b, loop);
   return cudaGetLastError();
 }
 

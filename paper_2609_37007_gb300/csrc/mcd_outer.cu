@@ -618,6 +618,8 @@ __global__ void pf_set_rows_kernel(int* rows, int n) { *rows = n; }
 __global__ void __launch_bounds__(128) pf_embed_kernel(const int* __restrict__ ids, const int* nrows,
                                                        const uint8_t* __restrict__ table, int vocab, int H, float* X,
                                                        float* ss, int* err) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= *nrows) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -652,6 +654,8 @@ __global__ void __launch_bounds__(256) pf_rope_kv_kernel(const float* __restrict
                                                          int NH, int NKV, int D, int qk_norm, const float* qn,
                                                          const float* kn, float eps, const float2* __restrict__ rope,
                                                          uint16_t* kc, uint16_t* vc, int cap, float* q) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int vecs = NH + 2 * NKV, w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int r = w / vecs, vi = w - r * vecs;
   if (r >= *nrows) return;
@@ -758,6 +762,8 @@ __global__ void __launch_bounds__(kPfWarps * 32) pf_attn_kernel(const float* __r
                                                                 uint8_t* att_t) {
   using S = PfAttn<D>;
   extern __shared__ __align__(16) uint8_t pf_smem[];
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int M = *nrows, r0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * kPfRows, h = blockIdx.y, g = h / (NH / NKV);
   if (r0 >= M) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, t = lane & 3;
@@ -937,10 +943,11 @@ static cudaError_t pf_attn_set_smem() {
 static void launch_pf_attn(const float* q, const int* nrows, int n, int NH, int NKV, int D, const uint16_t* kc,
                            const uint16_t* vc, int cap, int Rtc, uint8_t* att_t, cudaStream_t s) {
   const dim3 grid((n + kPfRows - 1) / kPfRows, NH);
-  if (D == 128)
-    pf_attn_kernel<128><<<grid, kPfWarps * 32, PfAttn<128>::kSmemBytes, s>>>(q, nrows, NH, NKV, kc, vc, cap, Rtc, att_t);
-  else
-    pf_attn_kernel<64><<<grid, kPfWarps * 32, PfAttn<64>::kSmemBytes, s>>>(q, nrows, NH, NKV, kc, vc, cap, Rtc, att_t);
+  auto go = [&](auto kernel, int smem) {
+    tc::launch(true, kernel, grid, dim3(kPfWarps * 32), smem, s, q, nrows, NH, NKV, kc, vc, cap, Rtc, att_t);
+  };
+  if (D == 128) go(pf_attn_kernel<128>, PfAttn<128>::kSmemBytes);
+  else go(pf_attn_kernel<64>, PfAttn<64>::kSmemBytes);
 }
 
 struct mcd_outer {
@@ -1283,26 +1290,28 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
   // the rows there are (255 rows of 640: 144 CTAs instead of 64 to 96 per product)
   const int H = p.H, L = p.L, qd = p.NH * p.D, kvl = p.NKV * st.cap * p.D;
   const int Rtc = tc_operand_rows(n, p.qkv_dim, p.n_cta);
+  // every kernel a dependent launch: 2333 us for a 256-token prompt, 2444 with the products alone
+  const bool pdl = true;
   pf_set_rows_kernel<<<1, 1, 0, s>>>(t.rows, n);
-  pf_embed_kernel<<<n, 128, 0, s>>>(text_ids, t.rows, st.text_table, st.text_vocab, H, t.X, t.ss, p.err);
-  tc_norm_operand_kernel<<<256, 256, 0, s>>>(t.X, p.attn_norm, t.ss, H, p.eps, t.rows, Rtc, t.xn_hi, t.xn_lo);
+  tc::launch(pdl, pf_embed_kernel, dim3(n), dim3(128), 0, s, text_ids, t.rows, st.text_table, st.text_vocab, H, t.X, t.ss, p.err);
+  tc::launch(pdl, tc_norm_operand_kernel, dim3(256), dim3(256), 0, s, t.X, p.attn_norm, t.ss, H, p.eps, t.rows, Rtc, t.xn_hi, t.xn_lo);
   for (int l = 0; l < L; ++l) {
     const uint8_t* wl = t.w + (size_t)l * t.off.layer;
     uint16_t* kc = reinterpret_cast<uint16_t*>(st.kcache) + (size_t)l * kvl;
     uint16_t* vc = reinterpret_cast<uint16_t*>(st.vcache) + (size_t)l * kvl;
-    tc_launch_qkv(wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, s);
+    tc_launch_qkv(wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
     const int vecs = p.NH + 2 * p.NKV;
-    pf_rope_kv_kernel<<<(n * vecs + 7) / 8, 256, 0, s>>>(t.qkv, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
+    tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
                                                          p.q_norm + (size_t)l * p.D, p.k_norm + (size_t)l * p.D, p.eps,
                                                          st.rope, kc, vc, st.cap, t.q);
     launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, s);
-    tc_launch_resid(wl + t.off.o, t.att_t, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, s);
-    tc_resid_norm_kernel<<<n, 128, 0, s>>>(t.X, t.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
-                                           p.eps, t.xn_hi, nullptr);
-    tc_launch_gu(wl + t.off.gu, t.xn_hi, t.act_t, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, s);
-    tc_launch_resid(wl + t.off.d, t.act_t, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, s);
-    tc_resid_norm_kernel<<<n, 128, 0, s>>>(t.X, t.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss,
-                                           l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : nullptr, p.eps, t.xn_hi,
+    tc_launch_resid(wl + t.off.o, t.att_t, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
+                                           p.eps, t.xn_hi, (uint8_t*)nullptr);
+    tc_launch_gu(wl + t.off.gu, t.xn_hi, t.act_t, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid(wl + t.off.d, t.act_t, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss,
+                                           l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : (const float*)nullptr, p.eps, t.xn_hi,
                                            t.xn_lo);
   }
   MCD_CHECK(cudaGetLastError());

@@ -31,7 +31,7 @@ template <int BN>
 __global__ void __launch_bounds__(kStoreThreads, 1) gemm_store_kernel(const GemmArgs g, float* __restrict__ Y) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  gemm_tile<BN, false, false>(g, [&](int m, int n, float v, float) { Y[(size_t)n * g.M + m] = v; });
+  gemm_tile<BN, false>(g, [&](int m, int n, float v) { Y[(size_t)n * g.M + m] = v; });
 }
 
 template <int BN>
@@ -101,7 +101,7 @@ extern "C" mcd_status mcd_tc_gemm(int32_t M, int32_t N, int32_t K, int32_t bn, c
   }
   int herr = 0;
   if (e == cudaSuccess) {
-    tc::GemmArgs g{ta, nullptr, tb, nullptr, M, N, K, nullptr, err, 2000000000ull, bn ? 0 : tc::auto_pitch(M, N)};
+    tc::GemmArgs g{ta, tb, nullptr, M, N, K, nullptr, err, 2000000000ull, false, bn ? 0 : tc::auto_pitch(M, N)};
     e = bn == 128 ? tc::launch_store<128>(g, Y, st) : bn == 256 ? tc::launch_store<256>(g, Y, st)
                                                              : tc::launch_store_pitch(g, Y, st);
   }
@@ -130,8 +130,8 @@ extern "C" mcd_status mcd_tc_gemm_tiled(int32_t M, int32_t N, int32_t K, int32_t
   if (M % tc::kBM || K % tc::kBK || (bn != 0 && bn != 128 && bn != 256) || N % (bn ? bn : 16))
     return MCD_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(A_tiled) | reinterpret_cast<uintptr_t>(B_tiled)) & 1023u) return MCD_ERR_UNSUPPORTED;
-  tc::GemmArgs g{static_cast<const uint8_t*>(A_tiled), nullptr, static_cast<const uint8_t*>(B_tiled), nullptr,
-                 M, N, K, nullptr, err, 2000000000ull, bn ? 0 : tc::auto_pitch(M, N)};
+  tc::GemmArgs g{static_cast<const uint8_t*>(A_tiled), static_cast<const uint8_t*>(B_tiled), nullptr,
+                 M, N, K, nullptr, err, 2000000000ull, false, bn ? 0 : tc::auto_pitch(M, N)};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return cuda_status(bn == 128   ? tc::launch_store<128>(g, Y, st)
                      : bn == 256 ? tc::launch_store<256>(g, Y, st)

@@ -35,9 +35,8 @@ __host__ __device__ __forceinline__ size_t sw128_offset(int R, int row, int kt, 
   return (size_t)kt * R * 128 + (size_t)(row >> 3) * 1024 + (size_t)(row & 7) * 128 + (size_t)((c ^ (row & 7)) << 4);
 }
 
-// kDualA: a second A matrix (same shape) multiplies the same B into a second accumulator
-// (gate and up projections side by side); kDualB: a second B operand (the low bf16 half of
-// a hi + lo split) accumulates into the same accumulator.
+// kDualB: a second B operand (the low bf16 half of a hi + lo split) accumulates into the same
+// accumulator.  kBudget: shared memory for the ring.
 // TMEM allocations are powers of two of at least 32 columns.
 __host__ __device__ constexpr int tmem_cols_for(int cols) {
   int c = 32;
@@ -45,21 +44,30 @@ __host__ __device__ constexpr int tmem_cols_for(int cols) {
   return c;
 }
 
-template <int BN, bool kDualA = false, bool kDualB = false>
+template <int BN, bool kDualB = false, int kBudget = kStageBudget>
 struct Layout {
   static_assert(BN % 16 == 0 && BN >= 32 && BN <= 256, "UMMA N");
   static constexpr int kABytes = kBM * 128;
   static constexpr int kBBytes = BN * 128;
-  static constexpr int kStageBytes = (kDualA ? 2 : 1) * kABytes + (kDualB ? 2 : 1) * kBBytes;
-  static constexpr int kTmemCols = tmem_cols_for((kDualA ? 2 : 1) * BN);
-  static constexpr int kStages = kStageBudget / kStageBytes > 8 ? 8 : kStageBudget / kStageBytes;
+  static constexpr int kStageBytes = kABytes + (kDualB ? 2 : 1) * kBBytes;
+  static constexpr int kTmemCols = tmem_cols_for(BN);
+  static constexpr int kStages = kBudget / kStageBytes > 8 ? 8 : kBudget / kStageBytes;
   static constexpr int kBarOff = kStages * kStageBytes;                 // full[s], empty[s], accum
   static constexpr int kTmemSlotOff = kBarOff + (2 * kStages + 1) * 8;
   static constexpr int kFlagOff = kTmemSlotOff + 4;
   static constexpr int kSmemBytes = kFlagOff + 4 + 1024;               // + alignment slack
   static_assert(kSmemBytes <= 227 * 1024, "tensor-core GEMM stages exceed shared memory");
-  static_assert(kTmemCols <= 512, "TMEM columns");
+  static_assert(kStages >= 2 && kTmemCols <= 512, "ring stages, TMEM columns");
 };
+
+// Programmatic dependent launch.  pdl_wait: every earlier kernel of the stream has completed and
+// its writes are visible (returns at once in a kernel launched without the attribute); it comes
+// before a kernel's first access to anything an earlier kernel writes or still reads, in every
+// thread that makes one and in at least one thread of every CTA, so that a grid never completes
+// before the grids in front of it.  pdl_trigger: the next kernel's CTAs may start where there is
+// room for them; always after pdl_wait, so at most two kernels of a stream overlap.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t smem_addr) {
@@ -147,13 +155,13 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* err
 
 struct GemmArgs {
   const uint8_t* a;      // A in SW128 tiles, M rows
-  const uint8_t* a2;     // kDualA: the second A (same layout)
   const uint8_t* b;      // B in SW128 tiles, N rows
   const uint8_t* b2;     // kDualB: the second B (same layout)
   int M, N, K;           // M % 128 == 0, N % BN == 0, K % 64 == 0
   const int* n_active;   // optional (device): columns n >= *n_active are not computed
   int* err;
   unsigned long long wait_ns;
+  bool ahead;            // kPdl: fetch weights before pdl_wait
   int bn;                // gemm_tile: 0 = tiles of BN columns; else tile x covers columns
                          // x * bn .. min(N, (x + 1) * bn) - 1 (bn a multiple of 16, <= BN)
 };
@@ -177,14 +185,29 @@ struct TileRun {
   bool ok;         // every MMA completed (false after a timeout)
 };
 
+// Every thread of the CTA, after the last TMEM load: the accumulator's columns are freed.
+template <int BN>
+__device__ __forceinline__ void gemm_tile_free(const TileRun& t) {
+  tc_fence_before();
+  __syncthreads();
+  if ((threadIdx.x >> 5) == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(t.tmem), "r"((uint32_t)tmem_cols_for(BN))
+                 : "memory");
+}
+
 // Set-up, operand stream and MMAs of the tile of this CTA: columns n0 .. n0 + nw - 1 (by
 // default x * pitch .. for x = blockIdx.x; else as given, n0 and nw multiples of 16, nw <= BN).
 // false: the tile is empty (its first column at or past *n_active, or no k-slices in its
 // split) and nothing is held; else every thread returns after the accumulator is complete
 // (t.ok) or the tile gave up, and the CTA must call gemm_tile_free.
-template <int BN, bool kDualA, bool kDualB>
+// kPdl: the kernel is a dependent launch and has not yet called pdl_wait; this does, in every
+// thread, after the set-up.  The weights are no earlier kernel's output, so the CTAs of the
+// first column tile (live whenever any is) fill their ring with them before the wait: the
+// stream of weights runs on through the kernel boundary.
+template <int BN, bool kDualB, int kBudget = kStageBudget, bool kPdl = false>
 __device__ __forceinline__ bool gemm_tile_run(const GemmArgs& g, TileRun& t, int n0 = -1, int nw = 0) {
-  using L = Layout<BN, kDualA, kDualB>;
+  using L = Layout<BN, kDualB, kBudget>;
+  constexpr int S = L::kStages;
   extern __shared__ uint8_t tc_smem_raw[];
   const int m0 = blockIdx.y * kBM;
   if (n0 < 0) {
@@ -192,26 +215,55 @@ __device__ __forceinline__ bool gemm_tile_run(const GemmArgs& g, TileRun& t, int
     n0 = blockIdx.x * pitch;
     nw = min(pitch, g.N - n0);                                    // this tile's columns
   }
-  if (g.n_active && n0 >= __ldg(g.n_active)) return false;    // uniform over the CTA
   const int nk_all = g.K / kBK, per = (nk_all + gridDim.z - 1) / gridDim.z;
   const int kt0 = blockIdx.z * per, kt1 = min(nk_all, kt0 + per), nk = kt1 - kt0;
-  if (nk <= 0) return false;
+  if constexpr (!kPdl) {
+    if (g.n_active && n0 >= __ldg(g.n_active)) return false;  // uniform over the CTA
+    if (nk <= 0) return false;
+  } else if (nk <= 0 || !g.ahead) {
+    pdl_wait();
+    pdl_trigger();
+    if (nk <= 0 || (g.n_active && n0 >= __ldcg(g.n_active))) return false;
+  }
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
-  uint64_t* empty = full + L::kStages;
-  uint64_t* accum = empty + L::kStages;
+  uint64_t* empty = full + S;
+  uint64_t* accum = empty + S;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kTmemSlotOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kFlagOff);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool producer = warp == 0 && lane == 0;
+  // a stage is full after two arrivals, the A copy's and the B copies', and their bytes
+  auto issue_a = [&](int i, uint64_t pol) {
+    const int s = i % S;
+    mbar_arrive_expect_tx(&full[s], L::kABytes);
+    bulk_g2s(smem + s * L::kStageBytes, g.a + (size_t)(kt0 + i) * g.M * 128 + (size_t)m0 * 128, L::kABytes, &full[s], pol);
+  };
+  auto issue_b = [&](int i, uint64_t pol) {
+    const int s = i % S;
+    const size_t bo = (size_t)(kt0 + i) * g.N * 128 + (size_t)n0 * 128;
+    const uint32_t b_bytes = (uint32_t)nw * 128u;
+    uint8_t* sb = smem + s * L::kStageBytes + L::kABytes;
+    mbar_arrive_expect_tx(&full[s], (kDualB ? 2 : 1) * b_bytes);
+    bulk_g2s(sb, g.b + bo, b_bytes, &full[s], pol);
+    if (kDualB) bulk_g2s(sb + L::kBBytes, g.b2 + bo, b_bytes, &full[s], pol);
+  };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < L::kStages; ++s) {
-      mbar_init(&full[s], 1);
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 2);
       mbar_init(&empty[s], 1);
     }
     mbar_init(accum, 1);
     *abort_flag = 0;
     fence_barrier_init();
+    fence_proxy_async();
+  }
+  const uint64_t pol_a = policy_evict_first(), pol_b = policy_evict_last();
+  int a_issued = 0;                        // (producer) stages whose A copy is under way
+  if constexpr (kPdl) {
+    if (g.ahead && producer && blockIdx.x == 0)   // the thread that initialised the barriers
+      for (; a_issued < min(nk, S); ++a_issued) issue_a(a_issued, pol_a);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -223,118 +275,88 @@ __device__ __forceinline__ bool gemm_tile_run(const GemmArgs& g, TileRun& t, int
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  bool live = true;
+  if constexpr (kPdl) {
+    pdl_wait();
+    pdl_trigger();
+    live = !(g.n_active && n0 >= __ldcg(g.n_active));             // uniform over the CTA
+  }
 
-  if (warp == 0 && lane == 0) {
-    // producer: k-slice kt of the A tile(s) (rows m0..) and the B tile(s) (rows n0..)
-    const uint64_t pol_a = policy_evict_first(), pol_b = policy_evict_last();
+  if (producer) {
+    // k-slice i of the A tile (rows m0..) and the B tile(s) (rows n0..)
     int issued = 0;
-    for (int i = 0; i < nk; ++i) {
-      const int s = i % L::kStages, kt = kt0 + i;
-      if (i >= L::kStages && !tc_wait(&empty[s], ((i / L::kStages) - 1) & 1, g.err, g.wait_ns)) {
+    for (int i = 0; live && i < nk; ++i) {
+      const int s = i % S;
+      if (i >= S && !tc_wait(&empty[s], ((i / S) - 1) & 1, g.err, g.wait_ns)) {
         *abort_flag = 1;
         break;
       }
       if (*abort_flag) break;
-      uint8_t* st = smem + s * L::kStageBytes;
-      const size_t ao = (size_t)kt * g.M * 128 + (size_t)m0 * 128, bo = (size_t)kt * g.N * 128 + (size_t)n0 * 128;
-      const uint32_t b_bytes = (uint32_t)nw * 128u;
-      mbar_arrive_expect_tx(&full[s], (kDualA ? 2 : 1) * L::kABytes + (kDualB ? 2 : 1) * b_bytes);
-      bulk_g2s(st, g.a + ao, L::kABytes, &full[s], pol_a);
-      if (kDualA) bulk_g2s(st + L::kABytes, g.a2 + ao, L::kABytes, &full[s], pol_a);
-      uint8_t* sb = st + (kDualA ? 2 : 1) * L::kABytes;
-      bulk_g2s(sb, g.b + bo, b_bytes, &full[s], pol_b);
-      if (kDualB) bulk_g2s(sb + L::kBBytes, g.b2 + bo, b_bytes, &full[s], pol_b);
+      if (i >= a_issued) issue_a(i, pol_a);
+      issue_b(i, pol_b);
       ++issued;
     }
-    // every issued copy lands before the CTA may exit
-    for (int i = (issued > L::kStages ? issued - L::kStages : 0); i < issued; ++i)
-      tc_wait(&full[i % L::kStages], (i / L::kStages) & 1, g.err, g.wait_ns);
-  } else if (warp == 1 && lane == 0) {
+    // every issued copy lands before the CTA may exit (a stage that got its weights only is
+    // completed without operand bytes)
+    for (; issued < a_issued; ++issued) mbar_arrive(&full[issued % S]);
+    for (int i = (issued > S ? issued - S : 0); i < issued; ++i) tc_wait(&full[i % S], (i / S) & 1, g.err, g.wait_ns);
+  } else if (live && warp == 1 && lane == 0) {
     // MMA issuer
     const uint32_t idesc = idesc_bf16_n(nw);
     for (int i = 0; i < nk; ++i) {
-      const int s = i % L::kStages;
-      if (!tc_wait(&full[s], (i / L::kStages) & 1, g.err, g.wait_ns)) {
+      const int s = i % S;
+      if (!tc_wait(&full[s], (i / S) & 1, g.err, g.wait_ns)) {
         *abort_flag = 1;
         break;
       }
       if (*abort_flag) break;
       tc_fence_after();
       const uint32_t sa = smem_u32(smem + s * L::kStageBytes);
-      const uint32_t sb = sa + (kDualA ? 2 : 1) * L::kABytes;
+      const uint32_t sb = sa + L::kABytes;
 #pragma unroll
       for (int j = 0; j < kBK / 16; ++j) {
         const bool acc = (i | j) != 0;
         umma_bf16(tmem, sw128_desc(sa + 32 * j), sw128_desc(sb + 32 * j), idesc, acc);
         if (kDualB) umma_bf16(tmem, sw128_desc(sa + 32 * j), sw128_desc(sb + L::kBBytes + 32 * j), idesc, true);
-        if (kDualA)
-          umma_bf16(tmem + BN, sw128_desc(sa + L::kABytes + 32 * j), sw128_desc(sb + 32 * j), idesc, acc);
       }
       umma_commit(&empty[s]);         // the stage is free once these MMAs have read it
     }
     umma_commit(accum);               // every MMA issued so far has completed
   }
-  t.ok = tc_wait(accum, 0, g.err, g.wait_ns) && !*abort_flag;
-  __syncwarp();                       // the .sync.aligned TMEM loads need whole warps
-  tc_fence_after();
   t.smem = smem;
   t.tmem = tmem;
   t.m0 = m0;
   t.n0 = n0;
   t.nw = nw;
+  if (!live) {
+    t.ok = false;
+    gemm_tile_free<BN>(t);
+    return false;
+  }
+  t.ok = tc_wait(accum, 0, g.err, g.wait_ns) && !*abort_flag;
+  __syncwarp();                       // the .sync.aligned TMEM loads need whole warps
+  tc_fence_after();
   return true;
 }
 
-// Every thread of the CTA, after the last TMEM load: the accumulator's columns are freed.
-template <int BN, bool kDualA, bool kDualB>
-__device__ __forceinline__ void gemm_tile_free(const TileRun& t) {
-  using L = Layout<BN, kDualA, kDualB>;
-  tc_fence_before();
-  __syncthreads();
-  if ((threadIdx.x >> 5) == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(t.tmem), "r"((uint32_t)L::kTmemCols)
-                 : "memory");
-}
-
-// The GEMM body for the tile of rows m0 = blockIdx.y * 128 of A and n0 = blockIdx.x * BN of B
-// over the k-slices of split blockIdx.z of gridDim.z (the CTAs that share an A tile are
-// adjacent in launch order, so the weights stream from HBM about once while the activation
-// tiles stay in L2); epi(m, n, v, v2) for every m and n of the tile (each thread: one m, BN
-// values of n in order; v2 = the second accumulator with kDualA, else 0).  A tile whose
-// first column is at or past *n_active returns at once.  n0 >= 0: the tile's columns are
-// n0 .. n0 + nw - 1 instead (see gemm_tile_run).
-template <int BN, bool kDualA, bool kDualB, class Epi>
-__device__ __forceinline__ void gemm_tile(const GemmArgs& g, Epi epi, int n0 = -1, int nw = 0) {
-  TileRun t;
-  if (!gemm_tile_run<BN, kDualA, kDualB>(g, t, n0, nw)) return;
+// epi(m, n, v) for every m and n of the finished tile (each thread: one m, values of n in
+// order), then the accumulator is freed.
+template <int BN, class Epi>
+__device__ __forceinline__ void gemm_tile_drain(const TileRun& t, Epi epi) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = t.m0;
-  n0 = t.n0;
-  nw = t.nw;
-  const uint32_t tmem = t.tmem;
-  // epilogue: every warp, after the accumulator is complete
   if (t.ok) {
     // warp w reads TMEM lanes 32 (w % 4) ..; with more than four warps the 16-column chunks
     // are shared out (chunk c to the warps w / 4 == c mod (warps / 4))
     const int quarter = warp & 3, part = warp >> 2, n_parts = (int)(blockDim.x >> 7);
-    const int m = m0 + quarter * 32 + lane, n_ch = nw >> 4;
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (kDualA) {
-#pragma unroll 1
-      for (int ch = part; ch < n_ch; ch += n_parts) {
-        float v[16], v2[16];
-        tmem_ld16(lane_base + (uint32_t)(16 * ch), v);
-        tmem_ld16(lane_base + (uint32_t)(BN + 16 * ch), v2);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) epi(m, n0 + 16 * ch + j, v[j], v2[j]);
-      }
-    } else if (part < n_ch) {
+    const int m = t.m0 + quarter * 32 + lane, n_ch = t.nw >> 4;
+    const uint32_t lane_base = t.tmem + ((uint32_t)(quarter * 32) << 16);
+    if (part < n_ch) {
       // the next chunk's TMEM load is in flight while this chunk's values are stored (two
       // register sets, alternating)
       uint32_t ra[16], rb[16];
       auto store = [&](const uint32_t (&r)[16], int ch) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) epi(m, n0 + 16 * ch + j, __uint_as_float(r[j]), 0.f);
+        for (int j = 0; j < 16; ++j) epi(m, t.n0 + 16 * ch + j, __uint_as_float(r[j]));
       };
       int ch = part;
       tmem_ld16_async(lane_base + (uint32_t)(16 * ch), ra);
@@ -356,7 +378,18 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, Epi epi, int n0 = -
       }
     }
   }
-  gemm_tile_free<BN, kDualA, kDualB>(t);
+  gemm_tile_free<BN>(t);
+}
+
+// The GEMM body for the tile of rows m0 = blockIdx.y * 128 of A and n0 = blockIdx.x * BN of B
+// over the k-slices of split blockIdx.z of gridDim.z (the CTAs that share an A tile are
+// adjacent in launch order, so the weights stream from HBM about once while the activation
+// tiles stay in L2).  A tile whose first column is at or past *n_active returns at once.
+// n0 >= 0: the tile's columns are n0 .. n0 + nw - 1 instead (see gemm_tile_run).
+template <int BN, bool kDualB, class Epi>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, Epi epi, int n0 = -1, int nw = 0) {
+  TileRun t;
+  if (gemm_tile_run<BN, kDualB>(g, t, n0, nw)) gemm_tile_drain<BN>(t, epi);
 }
 
 // ---- persistent form ----------------------------------------------------------------------
@@ -365,13 +398,13 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, Epi epi, int n0 = -
 // through the shared-memory ring across tile boundaries, warp 1 issues the MMAs into one of
 // two TMEM accumulator buffers (tile i uses buffer i % 2), warps 2..5 read a finished buffer
 // back (warp w: TMEM lanes 32 (w % 4) ..) while the MMAs of the next tile already run, then
-// release it.  epi(m, n, split, v, v2).  Tiles whose first column is at or past *n_active are
+// release it.  epi(m, n, split, v) for the live columns n < *n_active.  Tiles whose first column is at or past *n_active are
 // skipped by every role alike.
 constexpr int kPThreads = 192;
-template <int BN, bool kDualA, bool kDualB>
+template <int BN, bool kDualB>
 struct PLayout {
-  using L = Layout<BN, kDualA, kDualB>;
-  static constexpr int kAccCols = (kDualA ? 2 : 1) * BN;     // one accumulator buffer
+  using L = Layout<BN, kDualB>;
+  static constexpr int kAccCols = BN;     // one accumulator buffer
   static constexpr int kTmemCols = tmem_cols_for(2 * kAccCols);
   static_assert(kTmemCols <= 512, "TMEM columns");
   static constexpr int kBarOff = L::kStages * L::kStageBytes;  // full[S], empty[S], acc_full[2], acc_empty[2], drain
@@ -381,10 +414,10 @@ struct PLayout {
   static_assert(kSmemBytes <= 227 * 1024, "tensor-core GEMM stages exceed shared memory");
 };
 
-template <int BN, bool kDualA, bool kDualB, class Epi>
+template <int BN, bool kDualB, class Epi>
 __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, Epi epi) {
-  using L = Layout<BN, kDualA, kDualB>;
-  using PL = PLayout<BN, kDualA, kDualB>;
+  using L = Layout<BN, kDualB>;
+  using PL = PLayout<BN, kDualB>;
   constexpr int S = L::kStages;
   extern __shared__ uint8_t tc_smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -398,7 +431,7 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_nt = g.N / BN, n_mt = g.M / kBM, n_tiles = n_nt * n_mt * splits;
   const int nk_all = g.K / kBK, per = (nk_all + splits - 1) / splits;
-  const int n_live = g.n_active ? *g.n_active : g.N;
+  int n_live = g.N;
   // tile t -> (n0, m0, split, k-slice range); false for a skipped tile
   auto tile_of = [&](int t, int& n0, int& m0, int& z, int& kt0, int& nk) {
     const int nt = t % n_nt, rest = t / n_nt;
@@ -433,6 +466,9 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
+  if (g.n_active) n_live = __ldcg(g.n_active);
 
   if (warp == 0) {
     if (lane == 0) {                          // producer
@@ -453,8 +489,7 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
           const size_t ao = (size_t)kt * g.M * 128 + (size_t)m0 * 128, bo = (size_t)kt * g.N * 128 + (size_t)n0 * 128;
           mbar_arrive_expect_tx(&full[s], L::kStageBytes);
           bulk_g2s(st, g.a + ao, L::kABytes, &full[s], pol_a);
-          if (kDualA) bulk_g2s(st + L::kABytes, g.a2 + ao, L::kABytes, &full[s], pol_a);
-          uint8_t* sb = st + (kDualA ? 2 : 1) * L::kABytes;
+          uint8_t* sb = st + L::kABytes;
           bulk_g2s(sb, g.b + bo, L::kBBytes, &full[s], pol_b);
           if (kDualB) bulk_g2s(sb + L::kBBytes, g.b2 + bo, L::kBBytes, &full[s], pol_b);
         }
@@ -485,14 +520,12 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + s * L::kStageBytes);
-          const uint32_t sb = sa + (kDualA ? 2 : 1) * L::kABytes;
+          const uint32_t sb = sa + L::kABytes;
 #pragma unroll
           for (int j = 0; j < kBK / 16; ++j) {
             const bool ac = (i | j) != 0;
             umma_bf16(acc, sw128_desc(sa + 32 * j), sw128_desc(sb + 32 * j), idesc, ac);
             if (kDualB) umma_bf16(acc, sw128_desc(sa + 32 * j), sw128_desc(sb + L::kBBytes + 32 * j), idesc, true);
-            if (kDualA)
-              umma_bf16(acc + BN, sw128_desc(sa + L::kABytes + 32 * j), sw128_desc(sb + 32 * j), idesc, ac);
           }
           umma_commit(&empty[s]);
         }
@@ -519,11 +552,11 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * PL::kAccCols);
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 16) {
-        float vv[16], v2[16];
+        float vv[16];
         tmem_ld16(base + (uint32_t)c0, vv);
-        if (kDualA) tmem_ld16(base + (uint32_t)(BN + c0), v2);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) epi(m, n0 + c0 + j, z, vv[j], kDualA ? v2[j] : 0.f);
+        for (int j = 0; j < 16; ++j)
+          if (n0 + c0 + j < n_live) epi(m, n0 + c0 + j, z, vv[j]);
       }
       tc_fence_before();
       __syncwarp();
@@ -543,6 +576,23 @@ __device__ __forceinline__ void gemm_persistent(const GemmArgs& g, int splits, E
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)PL::kTmemCols)
                  : "memory");
   }
+}
+
+// Launch, with pdl as a programmatic dependent of the kernel before it in the stream (see
+// pdl_wait).
+template <class... P, class... A>
+inline cudaError_t launch(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 }  // namespace tc

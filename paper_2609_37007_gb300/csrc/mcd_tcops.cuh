@@ -20,6 +20,8 @@ namespace {
 __global__ void __launch_bounds__(256) tc_norm_operand_kernel(const float* __restrict__ X, const float* __restrict__ gain,
                                                               const float* __restrict__ ss, int H, float eps,
                                                               const int* nrows, int Rtc, uint8_t* hi, uint8_t* lo) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int M = *nrows, cpr = H / 8;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M * cpr; i += gridDim.x * blockDim.x) {
     const int r = i / cpr, ch = i - r * cpr, k = ch * 8;
@@ -62,21 +64,24 @@ constexpr int kTcSplit = 6;       // k-splits of the residual products (at most)
 // (3 x 8 x 6 = 144 CTAs at 128 rows, where 128-column tiles would leave 32 CTAs).
 inline int tc_resid_split(int Rtc) { return Rtc >= 512 ? 4 : kTcSplit; }
 
-// q, k, v = W (x . g / rms) with the hi + lo operand.
-__global__ void __launch_bounds__(tc::kPThreads, 1) tc_qkv_kernel(const tc::GemmArgs g, float* out, int ld,
-                                                                   const int* nrows) {
-  const int M = *nrows;
-  tc::gemm_persistent<kTcBN, false, true>(g, 1, [&](int m, int n, int, float v, float) {
-    if (n < M) out[(size_t)n * ld + m] = v;
-  });
-}
+// Shared memory for the ring of a tile of up to 128 columns: two CTAs of consecutive kernels fit
+// an SM together, so the next product's weights stream in while this one finishes.
+constexpr int kTcCompact = 100 * 1024;
+constexpr int kTcCompactRows = 384;
 
+// q, k, v = W (x . g / rms) with the hi + lo operand.
+__global__ void __launch_bounds__(tc::kPThreads, 1) tc_qkv_kernel(const tc::GemmArgs g, float* out, int ld) {
+  tc::gemm_persistent<kTcBN, true>(g, 1, [&](int m, int n, int, float v) { out[(size_t)n * ld + m] = v; });
+}
 // The same product, one 128 x pitch tile per CTA.
 constexpr int kQkvThreads = 256;
+template <int BN, int kBudget>
 __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::GemmArgs g, float* out, int ld,
                                                                       const int* nrows) {
+  tc::TileRun t;
+  if (!tc::gemm_tile_run<BN, true, kBudget, true>(g, t)) return;
   const int M = *nrows;
-  tc::gemm_tile<kTcBN, false, true>(g, [&](int m, int n, float v, float) {
+  tc::gemm_tile_drain<BN>(t, [&](int m, int n, float v) {
     if (n < M) out[(size_t)n * ld + m] = v;
   });
 }
@@ -89,14 +94,14 @@ __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::G
 // silu(gate) * up as one 16-byte bf16 chunk of the down product's SW128 operand (k-slice b,
 // element (row n, feature m)).  Packed rows at or past *nrows are not written.
 constexpr int kGuThreads = 256;
-template <int BN>
+template <int BN, int kBudget>
 __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs g, uint8_t* act_t, int Rtc,
                                                                const int* nrows) {
-  using L = tc::Layout<BN>;
+  using L = tc::Layout<BN, false, kBudget>;
   constexpr int kSP = tc::kBM + 4;                  // staged column stride (floats)
   static_assert((size_t)BN * kSP * 4 <= (size_t)L::kStages * L::kStageBytes, "gate/up staging exceeds the ring");
   tc::TileRun t;
-  if (!tc::gemm_tile_run<BN, false, false>(g, t)) return;
+  if (!tc::gemm_tile_run<BN, false, kBudget, true>(g, t)) return;
   float* S = reinterpret_cast<float*>(t.smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quarter = warp & 3, part = warp >> 2, n_parts = (int)(blockDim.x >> 7);
@@ -131,19 +136,21 @@ __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs
                      pack_bf16x2(v[6], v[7]));
     }
   }
-  tc::gemm_tile_free<BN, false, false>(t);
+  tc::gemm_tile_free<BN>(t);
 }
 
 // Residual products (Wo, down): one 128 x pitch tile per CTA over the k-slices of split
 // blockIdx.z of kTcSplit; split z writes its partial sums part[z][n][m] (plain stores);
 // tc_resid_norm_kernel adds them into the residual stream.
 constexpr int kResidThreads = 256;
-template <int BN>
+template <int BN, int kBudget>
 __global__ void __launch_bounds__(kResidThreads, 1) tc_resid_kernel(const tc::GemmArgs g, float* part, int ld, int Rtc,
                                                                      const int* nrows) {
+  tc::TileRun t;
+  if (!tc::gemm_tile_run<BN, false, kBudget, true>(g, t)) return;
   const int M = *nrows;
   const size_t zoff = (size_t)blockIdx.z * Rtc;
-  tc::gemm_tile<BN, false, false>(g, [&](int m, int n, float v, float) {
+  tc::gemm_tile_drain<BN>(t, [&](int m, int n, float v) {
     if (n < M) part[(zoff + n) * ld + m] = v;
   });
 }
@@ -155,6 +162,8 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
                                                             int H, const int* nrows, float* ss_out,
                                                             const float* __restrict__ gain, float eps, uint8_t* hi,
                                                             uint8_t* lo) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= *nrows) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -261,26 +270,23 @@ inline void tc_tile_layer(const FrameParams& p, cudaStream_t st, const uint8_t* 
 }
 // Dynamic shared memory of the block kernels (once per translation unit).
 inline cudaError_t tc_block_set_smem() {
-  cudaError_t e = cudaFuncSetAttribute(tc_qkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       tc::PLayout<kTcBN, false, true>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_qkv_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Layout<kTcBN, false, true>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_gu_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<128>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_gu_kernel<176>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<176>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_gu_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<256>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_resid_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Layout<128>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_resid_kernel<176>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Layout<176>::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_resid_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Layout<256>::kSmemBytes);
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto fn, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  set(tc_qkv_kernel, tc::PLayout<kTcBN, true>::kSmemBytes);
+  set(tc_qkv_tile_kernel<64, kTcCompact>, tc::Layout<64, true, kTcCompact>::kSmemBytes);
+  set(tc_qkv_tile_kernel<128, tc::kStageBudget>, tc::Layout<128, true>::kSmemBytes);
+  set(tc_gu_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
+  set(tc_gu_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
+  set(tc_gu_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
+  set(tc_gu_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
+  set(tc_gu_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
+  set(tc_resid_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
+  set(tc_resid_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
+  set(tc_resid_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
+  set(tc_resid_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
+  set(tc_resid_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
   return e;
 }
 
@@ -304,32 +310,37 @@ inline int tc_operand_rows(int n, int qkv_dim, int n_sm) {
 // q, k, v of Rtc operand rows.  Below tc_qkv_persistent's line the pitch is at most kTcBN: nt
 // tiles of 128 columns over n_mt weight tiles with nt n_mt < 0.8 n_sm leave n_sm / n_mt >= nt.
 inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t* xn_lo, float* out, int qkv_dim, int Rtc,
-                          int H, const int* nrows, int* err, unsigned long long wait_ns, int n_sm, cudaStream_t s) {
-  tc::GemmArgs g{w, nullptr, xn_hi, xn_lo, qkv_dim, Rtc, H, nrows, err, wait_ns, 0};
+                          int H, const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
+  tc::GemmArgs g{w, xn_hi, xn_lo, qkv_dim, Rtc, H, nrows, err, wait_ns, pdl, 0};
   if (tc_qkv_persistent(Rtc, qkv_dim, n_sm)) {
-    tc_qkv_kernel<<<tc_grid(tc_tiles(Rtc, kTcBN, qkv_dim, 1), n_sm), tc::kPThreads,
-                    tc::PLayout<kTcBN, false, true>::kSmemBytes, s>>>(g, out, qkv_dim, nrows);
-  } else {
-    g.bn = tc::tile_pitch(qkv_dim, Rtc, n_sm);
-    tc_qkv_tile_kernel<<<dim3((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM), kQkvThreads,
-                         tc::Layout<kTcBN, false, true>::kSmemBytes, s>>>(g, out, qkv_dim, nrows);
+    tc::launch(pdl, tc_qkv_kernel, tc_grid(tc_tiles(Rtc, kTcBN, qkv_dim, 1), n_sm), dim3(tc::kPThreads),
+                   tc::PLayout<kTcBN, true>::kSmemBytes, s, g, out, qkv_dim);
+    return;
   }
+  g.bn = tc::tile_pitch(qkv_dim, Rtc, n_sm);
+  const dim3 grid((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM);
+  if (g.bn <= 64)
+    tc::launch(pdl, tc_qkv_tile_kernel<64, kTcCompact>, grid, dim3(kQkvThreads), tc::Layout<64, true, kTcCompact>::kSmemBytes,
+                   s, g, out, qkv_dim, nrows);
+  else
+    tc::launch(pdl, tc_qkv_tile_kernel<128, tc::kStageBudget>, grid, dim3(kQkvThreads), tc::Layout<128, true>::kSmemBytes, s,
+                   g, out, qkv_dim, nrows);
 }
 
 // gate/up -> SwiGLU into the down product's operand.  gu: the interleaved gate/up matrix
 // (2F rows); xn: the normalised operand of Rtc rows.  The tile pitch over the packed rows fills
 // the SMs with one tile per CTA (three tiles of 176 / 176 / 160 rows at 512 rows, F = 3072).
 inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, uint8_t* act_t, int Rtc, const int* nrows, int F,
-                         int H, int* err, unsigned long long wait_ns, int n_sm, cudaStream_t s) {
+                         int H, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
   const int pitch = tc::tile_pitch(2 * F, Rtc, n_sm);
-  const tc::GemmArgs g{gu, nullptr, xn, nullptr, 2 * F, Rtc, H, nrows, err, wait_ns, pitch};
+  const tc::GemmArgs g{gu, xn, nullptr, 2 * F, Rtc, H, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, 2 * F / tc::kBM);
-  if (pitch <= 128)
-    tc_gu_kernel<128><<<grid, kGuThreads, tc::Layout<128>::kSmemBytes, s>>>(g, act_t, Rtc, nrows);
-  else if (pitch <= 176)
-    tc_gu_kernel<176><<<grid, kGuThreads, tc::Layout<176>::kSmemBytes, s>>>(g, act_t, Rtc, nrows);
-  else
-    tc_gu_kernel<256><<<grid, kGuThreads, tc::Layout<256>::kSmemBytes, s>>>(g, act_t, Rtc, nrows);
+  auto go = [&](auto kernel, int smem) { tc::launch(pdl, kernel, grid, dim3(kGuThreads), smem, s, g, act_t, Rtc, nrows); };
+  if (pitch <= 64) go(tc_gu_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
+  else if (pitch <= 128 && Rtc <= kTcCompactRows) go(tc_gu_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
+  else if (pitch <= 128) go(tc_gu_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
+  else if (pitch <= 176) go(tc_gu_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
+  else go(tc_gu_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
 }
 
 // Wo or down (A = w: H rows of K, B = act: Rtc rows) -> tc_resid_split(Rtc) partial sums.
@@ -337,21 +348,21 @@ inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, uint8_t* act_t, i
 // (H = 1024: T = 4 of 128 packed rows at 512 rows, 128 CTAs; T = 3 of 48 / 48 / 32 at 128
 // rows, 144 CTAs).
 inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, float* part, int H, int Rtc, int K, const int* nrows,
-                            int* err, unsigned long long wait_ns, int n_sm, cudaStream_t s) {
+                            int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
   const int n_mt = H / tc::kBM, units = Rtc / 16, z = tc_resid_split(Rtc);
   int T = n_sm / (n_mt * z);
   if (T < 1) T = 1;
   if (T < (Rtc + 255) / 256) T = (Rtc + 255) / 256;
   if (T > units) T = units;
   const int pitch = (units + T - 1) / T * 16;
-  const tc::GemmArgs g{w, nullptr, act, nullptr, H, Rtc, K, nrows, err, wait_ns, pitch};
+  const tc::GemmArgs g{w, act, nullptr, H, Rtc, K, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, n_mt, z);
-  if (pitch <= 128)
-    tc_resid_kernel<128><<<grid, kResidThreads, tc::Layout<128>::kSmemBytes, s>>>(g, part, H, Rtc, nrows);
-  else if (pitch <= 176)
-    tc_resid_kernel<176><<<grid, kResidThreads, tc::Layout<176>::kSmemBytes, s>>>(g, part, H, Rtc, nrows);
-  else
-    tc_resid_kernel<256><<<grid, kResidThreads, tc::Layout<256>::kSmemBytes, s>>>(g, part, H, Rtc, nrows);
+  auto go = [&](auto kernel, int smem) { tc::launch(pdl, kernel, grid, dim3(kResidThreads), smem, s, g, part, H, Rtc, nrows); };
+  if (pitch <= 64) go(tc_resid_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
+  else if (pitch <= 128 && Rtc <= kTcCompactRows) go(tc_resid_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
+  else if (pitch <= 128) go(tc_resid_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
+  else if (pitch <= 176) go(tc_resid_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
+  else go(tc_resid_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
 }
 
 }  // namespace

@@ -290,17 +290,13 @@ bool mcd::make_geom(int M, int K, int Mu, int tile_bytes, int max_cols, MatGeom&
 }
 
 bool mcd::backbone_geom(FrameParams& p, int head_rows) {
-  // bytes per 16 x 16 tile; one-byte W8A16 tiles go two m-tiles per unit to keep units at 32 KB
-  const int tb = p.wdtype == MCD_WEIGHT_BF16 ? 512 : p.wdtype == MCD_WEIGHT_INT8 ? 256 : 1024;
-  const int mu = p.wdtype == MCD_WEIGHT_INT8 ? 2 : 1;
-  auto mu_for = [&](int rows) { return rows % (mu * 16) == 0 ? mu : 1; };
-  bool ok = make_geom(p.qkv_dim, p.H, mu_for(p.qkv_dim), tb, 1024, p.g[MAT_QKV]) && p.g[MAT_QKV].n_kc == 1;
+  const int tb = p.wdtype == MCD_WEIGHT_BF16 ? 512 : p.wdtype == MCD_WEIGHT_INT8 ? 256 : 1024;   // bytes per 16 x 16 tile
+  bool ok = make_geom(p.qkv_dim, p.H, 1, tb, 1024, p.g[MAT_QKV]) && p.g[MAT_QKV].n_kc == 1;
   int mu_o = 8;
   while (mu_o > 1 && (mu_o * (p.D / 16) * tb > kSlotBytes || p.H % (mu_o * 16))) mu_o >>= 1;
   ok = ok && make_geom(p.H, p.NH * p.D, mu_o, tb, p.D, p.g[MAT_WO]) && p.g[MAT_WO].Ku * 16 == p.D;
-  ok = ok && make_geom(2 * p.F, p.H, mu_for(2 * p.F), tb, 1024, p.g[MAT_GU]) && p.g[MAT_GU].n_kc == 1;
-  ok = ok && make_geom(p.H, p.F, mu_for(p.H), tb, 1024, p.g[MAT_WD]);
-  // (heads keep one m-tile per unit: the draft-offset bias tiles are staged per 16 rows)
+  ok = ok && make_geom(2 * p.F, p.H, 1, tb, 1024, p.g[MAT_GU]) && p.g[MAT_GU].n_kc == 1;
+  ok = ok && make_geom(p.H, p.F, 1, tb, 1024, p.g[MAT_WD]);
   ok = ok && make_geom(head_rows, p.H, 1, tb, 1024, p.g[MAT_HEAD]) && p.g[MAT_HEAD].n_kc == 1;
   return ok;
 }

@@ -292,76 +292,87 @@ __device__ __noinline__ void attention_stream(const FrameParams& p, int layer, i
 
 
 // Attention of query head h for the nr rows of stream s (packed rows base..base+nr-1), the
-// single-stream form; same outputs and cache writes as attention_stream (o[base + n][D] in
-// act).  (A) all threads stage the stream's cached K / V rows, the new rows' raw q / k / v,
-// their RoPE rows and the QK-norm gains in shared memory (independent 16-byte loads, all in
-// flight together); (B) one warp per new q / k vector applies QK-norm and RoPE in registers
-// (lane l holds dims l + 32 i, so each rotate-half pair sits in one lane) and the KV writer
-// stores the new keys and values; (C) the warp of query row n scores its keys with two lanes
-// per key (interleaved 16-byte chunks, one shuffle), takes the softmax across its lanes and
-// sums P.V with four dims per lane.  Three barriers in all; keys: positions 0..15 (c15 is
-// never fed).
+// form of the single-stream stages; same outputs and cache writes as attention_stream (o[base + n][D] in
+// act).  What the call's own QKV product does not write -- the stream's cached K / V rows, the
+// RoPE rows and the QK-norm gains -- is staged in shared memory by attention_ahead, which a CTA
+// runs while it waits for that product.  Then (A) one warp per new vector loads q, or k and v,
+// straight into registers (lane l holds dims l + 32 i, so each rotate-half pair sits in one
+// lane), applies QK-norm and RoPE and writes the row to shared memory, the KV writer also to
+// the cache; (B) the warp of query row n scores its keys with two lanes per key (interleaved
+// 16-byte chunks, one shuffle), takes the softmax across its lanes and sums P.V with four dims
+// per lane.  Two barriers; keys: positions 0..15 (c15 is never fed).  Staged whole after the
+// wait, through shared memory and a third barrier, it took 3.6 to 4.9 us per layer.
 constexpr int kAttnKeys = 16;
-__device__ __noinline__ void attention_rows(const FrameParams& p, int layer, int h, bool write_kv, int nr, int pos0, int base,
-                                           int s) {
-  Smem sm = smem_layout(mcd_dyn_smem);
-  const int D = p.D, half = D >> 1, g = h / (p.NH / p.NKV);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cs_shift = D == 128 ? 5 : 4, cpr = 1 << cs_shift;   // 16-byte chunks per row
-  constexpr int KS = 136;                                       // padded q / k row stride
-  float* o = sm.act;                                          // [kMaxCols][D]
-  float* ks = o + kMaxCols * 128;                               // [kAttnKeys][KS]
-  float* vs = ks + kAttnKeys * KS;                              // [kAttnKeys][128]
-  float* qs = vs + kAttnKeys * 128;                             // [kMaxRows][KS]
-  float2* cs = reinterpret_cast<float2*>(qs + kMaxRows * KS);   // [kMaxRows][D/2]
-  float* gq = reinterpret_cast<float*>(cs + kMaxRows * 64);     // [D]
-  float* gk = gq + 128;                                         // [D]
+struct AttnSmem {
+  static constexpr int kLd = 136;                               // padded q / k row stride
+  float *o, *ks, *vs, *qs, *gq, *gk;                            // o [kMaxCols][D], rows of up to 128
+  float2* cs;                                                   // [kMaxRows][64] RoPE rows
+  __device__ __forceinline__ explicit AttnSmem(const Smem& sm) {
+    o = sm.act;
+    ks = o + kMaxCols * 128;
+    vs = ks + kAttnKeys * kLd;
+    qs = vs + kAttnKeys * 128;
+    cs = reinterpret_cast<float2*>(qs + kMaxRows * kLd);
+    gq = reinterpret_cast<float*>(cs + kMaxRows * 64);
+    gk = gq + 128;
+  }
+};
+// 16-byte cp.async chunks, waited for by the issuing thread; a barrier must follow.
+template <bool STD>
+__device__ __noinline__ void attention_ahead(const FrameParams& p, int layer, int h, int nr, int pos0, int s) {
+  const AttnSmem a(smem_layout(mcd_dyn_smem));
+  const int D = STD ? 128 : p.D, g = h / (p.NH / p.NKV), cs_shift = D == 128 ? 5 : 4, cpr = 1 << cs_shift;
   const size_t cache_off = (size_t)s * p.kv_stride + ((size_t)layer * p.NKV + g) * p.kv_slots * D;
-  const float* qkv = p.qkv;
+  const int n_old = min(pos0, kAttnKeys);
+  const int n_rows = 2 * n_old + nr + (p.qk_norm ? 2 : 0);
+  for (int i = threadIdx.x; i < (n_rows << cs_shift); i += kConsumerThreads) {
+    int r = i >> cs_shift;
+    const int ch = i & (cpr - 1);
+    const float* src;
+    float* dst;
+    if (r < 2 * n_old) {
+      const bool isv = r >= n_old;
+      const int j = isv ? r - n_old : r;
+      src = (isv ? p.vcache : p.kcache) + cache_off + (size_t)j * D;
+      dst = isv ? a.vs + j * 128 : a.ks + j * AttnSmem::kLd;
+    } else if ((r -= 2 * n_old) < nr) {
+      src = reinterpret_cast<const float*>(p.rope + (size_t)(pos0 + r) * (D >> 1));
+      dst = reinterpret_cast<float*>(a.cs + r * 64);
+    } else {
+      r -= nr;
+      src = (r == 0 ? p.q_norm : p.k_norm) + (size_t)layer * D;
+      dst = r == 0 ? a.gq : a.gk;
+    }
+    cpa16(dst + 4 * ch, src + 4 * ch);
+  }
+  cpa_wait_all();
+}
+
+template <bool STD>
+__device__ __noinline__ void attention_rows(const FrameParams& p, int layer, int h, int g, bool write_kv, int nr, int pos0,
+                                           int base, int s) {
+  const AttnSmem a(smem_layout(mcd_dyn_smem));
+  const int D = STD ? 128 : p.D;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int KS = AttnSmem::kLd;
+  const size_t cache_off = (size_t)s * p.kv_stride + ((size_t)layer * p.NKV + g) * p.kv_slots * D;
   const int qoff = h * D, koff = p.NH * D + g * D, voff = p.NH * D + p.NKV * D + g * D;
   if (pos0 + nr > kAttnKeys) {                // positions beyond c14's row are never fed
-    if (tid == 0) atomicCAS(p.err, 0, (int)MCD_ERR_STATE);
+    if (threadIdx.x == 0) atomicCAS(p.err, 0, (int)MCD_ERR_STATE);
     nr = max(0, kAttnKeys - pos0);
   }
-  // ---- (A) staging: rows [cached K | cached V | q | k | v | RoPE | gains], 16-byte chunks --
-  {
-    const int n_rows = 2 * pos0 + 4 * nr + (p.qk_norm ? 2 : 0);
-    for (int i = tid; i < (n_rows << cs_shift); i += kConsumerThreads) {
-      int r = i >> cs_shift;
-      const int ch = i & (cpr - 1);
-      const float* src;
-      float* dst;
-      if (r < 2 * pos0) {
-        const bool isv = r >= pos0;
-        const int j = isv ? r - pos0 : r;
-        src = (isv ? p.vcache : p.kcache) + cache_off + (size_t)j * D;
-        dst = isv ? vs + j * 128 : ks + j * KS;
-      } else if ((r -= 2 * pos0) < 3 * nr) {
-        const int seg = r >= 2 * nr ? 2 : r >= nr ? 1 : 0, m = r - seg * nr;
-        src = qkv + (size_t)(base + m) * p.qkv_dim + (seg == 0 ? qoff : seg == 1 ? koff : voff);
-        dst = seg == 0 ? qs + m * KS : seg == 1 ? ks + (pos0 + m) * KS : vs + (pos0 + m) * 128;
-      } else if ((r -= 3 * nr) < nr) {
-        src = reinterpret_cast<const float*>(p.rope + (size_t)(pos0 + r) * half);
-        dst = reinterpret_cast<float*>(cs + r * 64);
-      } else {
-        r -= nr;
-        src = (r == 0 ? p.q_norm : p.k_norm) + (size_t)layer * D;
-        dst = r == 0 ? gq : gk;
-      }
-      cpa16(dst + 4 * ch, src + 4 * ch);
-    }
-    cpa_wait_all();
-  }
-  consumer_sync();
-  // ---- (B) QK-norm + RoPE of the new q / k rows; the KV writer stores k / v -------------
+  // ---- (A) the new rows: QK-norm + RoPE in registers; the KV writer stores k / v ----------
   const int nd = D >> 5;   // dims per lane: 4 (D = 128) or 2 (D = 64)
   for (int vi = warp; vi < 2 * nr; vi += kConsumerWarps) {
     const bool isq = vi < nr;
     const int n = isq ? vi : vi - nr;
-    float* row = isq ? qs + n * KS : ks + (pos0 + n) * KS;
-    float x[4];
+    const float* row_g = p.qkv + (size_t)(base + n) * p.qkv_dim;
+    float x[4], v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = i < nd ? row[lane + 32 * i] : 0.f;
+    for (int i = 0; i < 4; ++i) {
+      x[i] = i < nd ? __ldcg(row_g + (isq ? qoff : koff) + lane + 32 * i) : 0.f;
+      v[i] = !isq && i < nd ? __ldcg(row_g + voff + lane + 32 * i) : 0.f;
+    }
     if (p.qk_norm) {
       float ss = 0.f;
 #pragma unroll
@@ -369,7 +380,7 @@ __device__ __noinline__ void attention_rows(const FrameParams& p, int layer, int
 #pragma unroll
       for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
       const float sc = rsqrtf(ss / (float)D + p.eps);
-      const float* gg = isq ? gq : gk;
+      const float* gg = isq ? a.gq : a.gk;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (i < nd) x[i] = x[i] * sc * gg[lane + 32 * i];
@@ -377,39 +388,39 @@ __device__ __noinline__ void attention_rows(const FrameParams& p, int layer, int
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       if (i < nd / 2) {
-        const float2 r = cs[n * 64 + lane + 32 * i];
-        const float a = x[i], b = x[i + nd / 2];
-        x[i] = a * r.x - b * r.y;
-        x[i + nd / 2] = b * r.x + a * r.y;
+        const float2 r = a.cs[n * 64 + lane + 32 * i];
+        const float e = x[i], f = x[i + nd / 2];
+        x[i] = e * r.x - f * r.y;
+        x[i + nd / 2] = f * r.x + e * r.y;
       }
     }
+    float* row = isq ? a.qs + n * KS : a.ks + (pos0 + n) * KS;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (i < nd) row[lane + 32 * i] = x[i];
-    if (write_kv && !isq) {
-      float* kdst = p.kcache + cache_off + (size_t)(pos0 + n) * D;
-      float* vdst = p.vcache + cache_off + (size_t)(pos0 + n) * D;
-      const float* vrow = vs + (pos0 + n) * 128;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (i < nd) {
-          kdst[lane + 32 * i] = x[i];
-          vdst[lane + 32 * i] = vrow[lane + 32 * i];
+    for (int i = 0; i < 4; ++i) {
+      if (i < nd) {
+        row[lane + 32 * i] = x[i];
+        if (!isq) {
+          a.vs[(pos0 + n) * 128 + lane + 32 * i] = v[i];
+          if (write_kv) {
+            p.kcache[cache_off + (size_t)(pos0 + n) * D + lane + 32 * i] = x[i];
+            p.vcache[cache_off + (size_t)(pos0 + n) * D + lane + 32 * i] = v[i];
+          }
         }
+      }
     }
   }
   consumer_sync();
-  // ---- (C) warp n: scores (lanes 2j, 2j+1 for key j), softmax, P.V -----------------------
+  // ---- (B) warp n: scores (lanes 2j, 2j+1 for key j), softmax, P.V -----------------------
   if (warp < nr) {
     const int n = warp, npos = pos0 + n + 1;
     const int j = lane >> 1, hf = lane & 1;
     const bool live = j < npos;                      // causal: keys 0..pos0+n
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
     if (live) {
-      const float4* q4 = reinterpret_cast<const float4*>(qs + n * KS) + hf;
-      const float4* k4 = reinterpret_cast<const float4*>(ks + j * KS) + hf;
-#pragma unroll 4
-      for (int ch = 0; ch < (cpr >> 1); ++ch) {
+      const float4* q4 = reinterpret_cast<const float4*>(a.qs + n * KS) + hf;
+      const float4* k4 = reinterpret_cast<const float4*>(a.ks + j * KS) + hf;
+#pragma unroll 8
+      for (int ch = 0; ch < (D >> 3); ++ch) {
         const float4 q = q4[2 * ch], k = k4[2 * ch];
         a0 += q.x * k.x;
         a1 += q.y * k.y;
@@ -430,29 +441,41 @@ __device__ __noinline__ void attention_rows(const FrameParams& p, int layer, int
     const float pj = e / sum;
     const int d0 = 4 * lane;                         // four dims per lane
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int jj = 0; jj < npos; ++jj) {
-      const float w = __shfl_sync(0xFFFFFFFFu, pj, 2 * jj);
-      if (d0 < D) {
-        const float4 v = *reinterpret_cast<const float4*>(vs + jj * 128 + d0);
-        acc.x += w * v.x;
-        acc.y += w * v.y;
-        acc.z += w * v.z;
-        acc.w += w * v.w;
+#pragma unroll
+    for (int jb = 0; jb < kAttnKeys; jb += 8) {      // keys past npos have weight 0
+      if (jb < npos) {
+        float4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          v[q] = jb + q < npos && d0 < D ? *reinterpret_cast<const float4*>(a.vs + (jb + q) * 128 + d0)
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float w = __shfl_sync(0xFFFFFFFFu, pj, 2 * (jb + q));
+          acc.x += w * v[q].x;
+          acc.y += w * v[q].y;
+          acc.z += w * v[q].z;
+          acc.w += w * v[q].w;
+        }
       }
     }
-    if (d0 < D) *reinterpret_cast<float4*>(o + (base + n) * D + d0) = acc;
+    if (d0 < D) *reinterpret_cast<float4*>(a.o + (base + n) * D + d0) = acc;
   }
   consumer_sync();
 }
 
 // Attention of query head h for every stream with rows in the call (outputs at the
-// streams' packed rows).
-__device__ void attention_head(Cons& c, int layer, int h, bool write_kv) {
+// streams' packed rows).  `ahead`: attention_ahead has run for the call's only stream.
+template <bool STD>
+__device__ __forceinline__ void attention_head(Cons& c, int layer, int h, int g, bool write_kv, bool ahead) {
   const CallInfo* ci = c.sm.ci;
   for (int i = 0; i < ci->n_act; ++i) {
-    const int s = ci->act[i];
-    attention_rows(c.p, layer, h, write_kv, ci->st[s].n_rows, ci->st[s].pos0, ci->base[s], s);
+    const int s = ci->act[i], nr = ci->st[s].n_rows, pos0 = ci->st[s].pos0;
+    if (!ahead) {
+      attention_ahead<STD>(c.p, layer, h, nr, pos0, s);
+      consumer_sync();
+    }
+    attention_rows<STD>(c.p, layer, h, g, write_kv, nr, pos0, ci->base[s], s);
   }
 }
 
@@ -704,49 +727,55 @@ __device__ __noinline__ void trace_verify_rows(const FrameParams& p) {
 // ------------------------------------------------------------------------------------
 // One call
 // ------------------------------------------------------------------------------------
-template <int WT, bool WIDE>
+// STD: the standard geometry's single-stream instantiation (mcd_stage.cuh).
+template <int WT, bool WIDE, bool STD>
 __device__ __forceinline__ void run_call(Cons& c, int call) {
   const FrameParams& p = c.p;
   Smem& sm = c.sm;
   const CallInfo* ci = sm.ci;
-  const int L = p.L, H = p.H, D = p.D, F = p.F;
+  const int L = p.L, H = STD ? 1024 : p.H, D = STD ? 128 : p.D, F = p.F;
   unsigned* ctr = p.ctr + (size_t)call * p.ctr_stride;
   const int n_rows = ci->M;                 // packed rows of every stream in the call
   const unsigned N = (unsigned)p.n_cta;
   const float* x = p.x;
   auto from_x = [&](int n, int k, auto w) { return ld_global_v<decltype(w)::value>(x + (size_t)n * H + k); };
 
+  // a unit's m-block and k-chunk (the standard shapes' m-block counts are powers of two)
+  constexpr int lg_wo = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WO>::Mu)), lg_wd = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WD>::Mu));
+  auto wo_key = [&](int u) { return STD ? u >> lg_wo : u / p.g[MAT_WO].n_mb; };
+  auto wd_key = [&](int u) { return STD ? u >> lg_wd : u / p.g[MAT_WD].n_mb; };
+  auto wo_mb = [&](int u) { return STD ? u & ((1 << lg_wo) - 1) : u % p.g[MAT_WO].n_mb; };
+  auto wd_mb = [&](int u) { return STD ? u & ((1 << lg_wd) - 1) : u % p.g[MAT_WD].n_mb; };
+  auto units_of = [&](int kind) { return p.g[kind].n_units; };
   auto no_key = [](int) { return 0; };
   auto no_prep = [](int, int, int) {};
   for (int l = 0; l < L; ++l) {
     // ---- S1: RMSNorm -> QKV  (q, k, v = W (x . g) / rms) -------------------------------
-    g2s_vec(sm.vec, p.attn_norm + (size_t)l * H, H);      // independent of the wait below
-    const StagePlan sp_qkv = plan_stage<WT, WIDE>(c, 4 * l + 0, p.g[MAT_QKV].n_units, n_rows, no_key);
+    NarrowGain gain;
+    fetch_gain<STD>(c, gain, p.attn_norm + (size_t)l * H, H);      // independent of the wait below
+    const auto sp_qkv = plan_of<WT, WIDE, STD, MAT_QKV>(c, 4 * l + 0, units_of(MAT_QKV), n_rows, no_key);
+    const bool seeds = STD ? first_unit(sp_qkv) == 0 : blockIdx.x == 0;
+    auto qkv_epi = [&](int u, int mi, int rr, int n, float v, float, float inv) {
+      const int row = (u * (STD ? StdUnit<WT, MAT_QKV>::Mu : p.g[MAT_QKV].Mu) + mi) * 16 + rr;   // one k-chunk
+      p.qkv[(size_t)n * p.qkv_dim + row] = v * inv * wscale<WT>(p.s_qkv, (size_t)l * p.qkv_dim + row);
+    };
     if (l == 0) {
-      // layer-0 rows straight from their sources (cond / c0 vector / embedding rows); CTA 0
-      // also seeds the residual stream x
-      consumer_sync();                     // the gain is in shared memory
-      prep_operand<WT, WIDE>(
-          c, n_rows, H, 0, H, sm.vec, true,
+      // layer-0 rows straight from their sources (cond / c0 vector / embedding rows); one CTA
+      // (register operands: that of unit 0) also seeds the residual stream x
+      if (!STD) consumer_sync();           // the gain is in shared memory
+      norm_product<WT, WIDE, STD, MAT_QKV>(
+          c, call, 4 * l, sp_qkv, n_rows, H, gain,
           [&](int n, int k, auto w) {
             constexpr int W = decltype(w)::value;
             const uint8_t* src = ci->r_src[n];
             return ci->r_f32[n] ? ldg_f32_v<W>(src, k) : ldg_bf16_v<W>(src, k);
           },
-          blockIdx.x == 0 ? p.x : nullptr);
+          seeds ? p.x : nullptr, no_prep, qkv_epi);
     } else {
       if (!cons_wait(c, ctr + ctr_stage(l - 1, 3), N)) return;
-      prep_operand<WT, WIDE>(c, n_rows, H, 0, H, sm.vec, true, from_x);
+      norm_product<WT, WIDE, STD, MAT_QKV>(c, call, 4 * l, sp_qkv, n_rows, H, gain, from_x, nullptr, no_prep, qkv_epi);
     }
-    {
-      const MatGeom& g = p.g[MAT_QKV];
-      run_stage<WT, WIDE>(c, call, sp_qkv, H, no_key, no_prep,
-                    [&](int u, int mi, int rr, int n, float v, float) {
-                      const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr;
-                      p.qkv[(size_t)n * p.qkv_dim + row] = v * sm.inv_rms[n] * wscale<WT>(p.s_qkv, (size_t)l * p.qkv_dim + row);
-                    });
-      if (c.abort_) return;
-    }
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 0), call, 10 + 4 * (4 * l + 0));
 
     // ---- S2: attention (per query head) -> Wo + residual --------------------------------
@@ -755,9 +784,27 @@ __device__ __forceinline__ void run_call(Cons& c, int call) {
     // units compute that attention themselves.  Several streams: first one task per
     // (stream, query head) spread over the CTAs writes the outputs to global memory, then
     // Wo reads them.
-    auto wo_key = [&](int u) { return u / p.g[MAT_WO].n_mb; };
-    const StagePlan sp_wo = plan_stage<WT, WIDE>(c, 4 * l + 1, p.g[MAT_WO].n_units, n_rows, wo_key);
-    if (!WIDE && threadIdx.x == 0) sm.flags[3] = -1;     // ordered by the wait's barrier
+    const auto sp_wo = plan_of<WT, WIDE, STD, MAT_WO>(c, 4 * l + 1, units_of(MAT_WO), n_rows, wo_key);
+    const int u_wo = first_unit(sp_wo);
+    const bool ahead = !WIDE && ci->n_act == 1 && has_units(sp_wo);
+    // KV head of a unit's query head, and whether this CTA writes the head's K / V: the CTA that
+    // holds m-block 0 of a group's first head
+    auto kv_head = [&](int u, int& writer) {
+      const int h = wo_key(u), group = p.NH / p.NKV, g = h / group;
+      writer = 0;
+      if (g * group == h) for_units(sp_wo, [&](int v) { writer |= wo_key(v) == h && wo_mb(v) == 0; });
+      return g;
+    };
+    int writer0 = 0, g0 = 0;
+    if (!WIDE) {
+      g0 = kv_head(u_wo, writer0);
+      pin(writer0);
+      pin(g0);
+    }
+    if (ahead) {
+      const int s0 = ci->act[0];
+      attention_ahead<STD>(p, l, wo_key(u_wo), ci->st[s0].n_rows, ci->st[s0].pos0, s0);
+    }
     if (!cons_wait(c, ctr + ctr_stage(l, 0), N)) return;
     if (WIDE) {
       if (p.draft_mode == MCD_DRAFT_TREE && ci->st[0].pos0 > 0) {
@@ -782,107 +829,63 @@ __device__ __forceinline__ void run_call(Cons& c, int call) {
       }
       cons_signal(c, ctr + ctr_att(L, l), call, kTimelineSlots);
       if (!cons_wait(c, ctr + ctr_att(L, l), N)) return;
-      const MatGeom& g = p.g[MAT_WO];
-      if (threadIdx.x == 0) sm.flags[3] = -1;
-      consumer_sync();
-      run_stage<WT, WIDE, true>(
-          c, call, sp_wo, D, wo_key,
-          [&](int u, int, int) {
-            const int h = u / g.n_mb;
-            if (sm.flags[3] != h) {
-              const float* src = p.attn + h * D;
-              prep_operand<WT, WIDE>(c, n_rows, D, 0, D, nullptr, false,
-                                     [&](int n, int k, auto w) { return ld_global_v<decltype(w)::value>(src + (size_t)n * p.NH * D + k); });
-              if (threadIdx.x == 0) sm.flags[3] = h;
-            }
-          },
-          [&](int u, int mi, int rr0, int n, float4 v) {
-            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr0;
-            const size_t si = (size_t)l * H + row;
-            red_add_f32x4(p.x + (size_t)n * H + row,
-                          make_float4(v.x * wscale<WT>(p.s_wo, si), v.y * wscale<WT>(p.s_wo, si + 1),
-                                      v.z * wscale<WT>(p.s_wo, si + 2), v.w * wscale<WT>(p.s_wo, si + 3)));
-          });
-      if (c.abort_) return;
-    } else {
-      const MatGeom& g = p.g[MAT_WO];
-      const int group = p.NH / p.NKV;
-      run_stage<WT, WIDE, true>(
-          c, call, sp_wo, D, wo_key,
-          [&](int u, int cnt, int step) {
-            const int h = u / g.n_mb;
-            bool writer = false;      // the CTA holding m-block 0 of a group's first head writes K / V
-            for (int r = 0; r < cnt; ++r) writer |= (h % group) == 0 && (u + r * step) % g.n_mb == 0;
-            if (sm.flags[3] != h || writer) {
-              attention_head(c, l, h, writer);
-              c.op = reinterpret_cast<uint8_t*>(sm.act) + kWoOperandOff;
-              prep_operand<WT, WIDE>(c, n_rows, D, 0, D, nullptr, false,
-                               [&](int n, int k, auto w) { return ld_shared_v<decltype(w)::value>(sm.act + n * D + k); });
-              if (threadIdx.x == 0) sm.flags[3] = h;
-            }
-          },
-          [&](int u, int mi, int rr0, int n, float4 v) {
-            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr0;
-            const size_t si = (size_t)l * H + row;
-            red_add_f32x4(p.x + (size_t)n * H + row,
-                          make_float4(v.x * wscale<WT>(p.s_wo, si), v.y * wscale<WT>(p.s_wo, si + 1),
-                                      v.z * wscale<WT>(p.s_wo, si + 2), v.w * wscale<WT>(p.s_wo, si + 3)));
-          });
-      if (c.abort_) return;
     }
-    c.op = reinterpret_cast<uint8_t*>(sm.act);
+    auto resid_epi = [&](const float* scale, int row, int n, float4 v) {
+      const size_t si = (size_t)l * H + row;
+      red_add_f32x4(p.x + (size_t)n * H + row, make_float4(v.x * wscale<WT>(scale, si), v.y * wscale<WT>(scale, si + 1),
+                                                           v.z * wscale<WT>(scale, si + 2), v.w * wscale<WT>(scale, si + 3)));
+    };
+    keyed_product<WT, WIDE, STD, MAT_WO, true>(
+        c, call, 4 * l + 1, sp_wo, n_rows, D, wo_key,
+        [&](int u0) {
+          if (WIDE) return;
+          int writer = writer0, g = g0;
+          if (u0 != u_wo) g = kv_head(u0, writer);
+          attention_head<STD>(c, l, wo_key(u0), g, writer != 0, ahead && u0 == u_wo);
+        },
+        [&](int u0, int n, int k, auto w) {
+          constexpr int W = decltype(w)::value;
+          if constexpr (WIDE) return ld_global_v<W>(p.attn + (size_t)n * p.NH * D + wo_key(u0) * D + k);
+          else return ld_shared_v<W>(sm.act + n * D + k);
+        },
+        reinterpret_cast<uint8_t*>(sm.act) + (WIDE ? 0 : kWoOperandOff),
+        [&](int u, int mi, int rr0, int n, float4 v) {
+          resid_epi(p.s_wo, (wo_mb(u) * (STD ? StdUnit<WT, MAT_WO>::Mu : p.g[MAT_WO].Mu) + mi) * 16 + rr0, n, v);
+        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 1), call, 10 + 4 * (4 * l + 1));
 
     // ---- S3: RMSNorm -> gate/up -> SwiGLU --------------------------------------------------
-    g2s_vec(sm.vec, p.ffn_norm + (size_t)l * H, H);
-    const StagePlan sp_gu = plan_stage<WT, WIDE>(c, 4 * l + 2, p.g[MAT_GU].n_units, n_rows, no_key, true);
+    fetch_gain<STD>(c, gain, p.ffn_norm + (size_t)l * H, H);
+    const auto sp_gu = plan_of<WT, WIDE, STD, MAT_GU>(c, 4 * l + 2, units_of(MAT_GU), n_rows, no_key);
     if (!cons_wait(c, ctr + ctr_stage(l, 1), N)) return;
-    prep_operand<WT, WIDE>(c, n_rows, H, 0, H, sm.vec, true, from_x);
-    {
-      const MatGeom& g = p.g[MAT_GU];
-      // tile rows 0..7 are gate rows j0..j0+7, rows 8..15 the matching up rows
-      run_stage<WT, WIDE>(
-          c, call, sp_gu, H, no_key, no_prep,
-          [&](int u, int mi, int rr, int n, float gate, float up) {
-            const float s = sm.inv_rms[n];
-            const int t16 = ((u % g.n_mb) * g.Mu + mi) * 16 + rr;      // tiled row of the gate
-            const float gt = gate * s * wscale<WT>(p.s_gu, (size_t)l * 2 * F + t16);
-            const float ut = up * s * wscale<WT>(p.s_gu, (size_t)l * 2 * F + t16 + 8);
-            const int j = ((u % g.n_mb) * g.Mu + mi) * 8 + rr;
-            p.mbuf[(size_t)n * F + j] = gt / (1.0f + __expf(-gt)) * ut;
-          });
-      if (c.abort_) return;
-    }
+    // tile rows 0..7 are gate rows j0..j0+7, rows 8..15 the matching up rows
+    norm_product<WT, WIDE, STD, MAT_GU>(
+        c, call, 4 * l + 2, sp_gu, n_rows, H, gain, from_x, nullptr, no_prep,
+        [&](int u, int mi, int rr, int n, float gate, float up, float inv) {
+          const int mt = u * (STD ? StdUnit<WT, MAT_GU>::Mu : p.g[MAT_GU].Mu) + mi;      // one k-chunk
+          const int t16 = mt * 16 + rr;                                                  // tiled row of the gate
+          const float gt = gate * inv * wscale<WT>(p.s_gu, (size_t)l * 2 * F + t16);
+          const float ut = up * inv * wscale<WT>(p.s_gu, (size_t)l * 2 * F + t16 + 8);
+          p.mbuf[(size_t)n * F + mt * 8 + rr] = gt / (1.0f + __expf(-gt)) * ut;
+        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 2), call, 10 + 4 * (4 * l + 2));
 
     // ---- S4: down + residual (k-chunks of F) ---------------------------------------------
-    auto wd_key = [&](int u) { return u / p.g[MAT_WD].n_mb; };
-    const StagePlan sp_wd = plan_stage<WT, WIDE>(c, 4 * l + 3, p.g[MAT_WD].n_units, n_rows, wd_key);
-    if (threadIdx.x == 0) sm.flags[3] = -1;     // ordered by the wait's barrier
+    const auto sp_wd = plan_of<WT, WIDE, STD, MAT_WD>(c, 4 * l + 3, units_of(MAT_WD), n_rows, wd_key);
     if (!cons_wait(c, ctr + ctr_stage(l, 2), N)) return;
-    {
-      const MatGeom& g = p.g[MAT_WD];
-      const int Kc = g.Ku * 16;
-      run_stage<WT, WIDE, true>(
-          c, call, sp_wd, Kc, wd_key,
-          [&](int u, int, int) {
-            const int kc = u / g.n_mb;
-            if (sm.flags[3] != kc) {
-              const float* m = p.mbuf + (size_t)kc * Kc;
-              prep_operand<WT, WIDE>(c, n_rows, Kc, 0, Kc, nullptr, false,
-                               [&](int n, int k, auto w) { return ld_global_v<decltype(w)::value>(m + (size_t)n * F + k); });
-              if (threadIdx.x == 0) sm.flags[3] = kc;
-            }
-          },
-          [&](int u, int mi, int rr0, int n, float4 v) {
-            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr0;
-            const size_t si = (size_t)l * H + row;
-            red_add_f32x4(p.x + (size_t)n * H + row,
-                          make_float4(v.x * wscale<WT>(p.s_wd, si), v.y * wscale<WT>(p.s_wd, si + 1),
-                                      v.z * wscale<WT>(p.s_wd, si + 2), v.w * wscale<WT>(p.s_wd, si + 3)));
-          });
-      if (c.abort_) return;
-    }
+    const int Kc = STD ? 1024 : p.g[MAT_WD].Ku * 16;
+    keyed_product<WT, WIDE, STD, MAT_WD, true>(
+        c, call, 4 * l + 3, sp_wd, n_rows, Kc, wd_key, [](int) {},
+        [&](int u0, int n, int k, auto w) {
+          return ld_global_v<decltype(w)::value>(p.mbuf + (size_t)wd_key(u0) * Kc + (size_t)n * F + k);
+        },
+        reinterpret_cast<uint8_t*>(sm.act),
+        [&](int u, int mi, int rr0, int n, float4 v) {
+          resid_epi(p.s_wd, (wd_mb(u) * (STD ? StdUnit<WT, MAT_WD>::Mu : p.g[MAT_WD].Mu) + mi) * 16 + rr0, n, v);
+        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 3), call, 10 + 4 * (4 * l + 3));
   }
 
@@ -894,47 +897,64 @@ __device__ __forceinline__ void run_call(Cons& c, int call) {
   // heads and row positions: a single stream with at most kPreUnits head units in this CTA
   // loads its tiles before waiting for the last layer (upper half of `vec`, the gain stays
   // in the lower half); otherwise each chunk stages them once the operand is built.
-  g2s_vec(sm.vec, p.final_norm, H);
-  const StagePlan sp_head = plan_stage<WT, WIDE>(c, 4 * L, ci->n_heads * p.g[MAT_HEAD].n_units, n_rows, no_key);
+  NarrowGain gain;
+  fetch_gain<STD>(c, gain, p.final_norm, H);
+  const auto sp_head = plan_of<WT, WIDE, STD, MAT_HEAD>(c, 4 * L, ci->n_heads * units_of(MAT_HEAD), n_rows, no_key);
   constexpr int kPreUnits = kVecFloats / 2 / (16 * 8);
-  const int n_head_units = sp_head.ur.end - sp_head.ur.first;         // contiguous range, step 1
+  const int u_head = first_unit(sp_head), n_head_units = unit_count(sp_head);       // contiguous range
+  const int head_units = units_of(MAT_HEAD);
   const bool pre_bias = !WIDE && n_rows <= 8 && H <= kVecFloats / 2 && n_head_units <= kPreUnits;
   float* bias_pre = sm.vec + kVecFloats / 2;                          // [unit][16 rows][8 columns]
+  // LM head and unit within it of unit u: counted on from the CTA's first unit (no division)
+  int hi0 = u_head / head_units, uu0 = u_head - hi0 * head_units;
+  pin(hi0);
+  pin(uu0);
+  auto head_of = [&](int u, int& uu) {
+    int hi = hi0;
+    uu = uu0 + (u - u_head);
+    while (uu >= head_units) {
+      uu -= head_units;
+      ++hi;
+    }
+    return ci->heads[hi];
+  };
   auto head_bias_at = [&](int u, int rr, int n) -> float {
-    const MatGeom& g = p.g[MAT_HEAD];
-    const int P = ci->heads[u / g.n_units];
+    int uu;
+    const int P = head_of(u, uu);
     if (n >= n_rows) return 0.f;
     const int j = P - ci->r_pos[n];
     if (j < 1 || j > p.K || ci->r_pos[n] < 1) return 0.f;
-    return __ldg(p.head_bias + ((size_t)(P - 1) * p.K + (j - 1)) * p.V + (u % g.n_units) * 16 + rr);
+    return __ldg(p.head_bias + ((size_t)(P - 1) * p.K + (j - 1)) * p.V + uu * 16 + rr);
   };
   if (pre_bias)
     for (int o = threadIdx.x; o < n_head_units * 128; o += kConsumerThreads)
-      bias_pre[o] = head_bias_at(sp_head.ur.first + (o >> 7), (o >> 3) & 15, o & 7);
+      bias_pre[o] = head_bias_at(u_head + (o >> 7), (o >> 3) & 15, o & 7);
   if (!cons_wait(c, ctr + ctr_stage(L - 1, 3), N)) return;
-  prep_operand<WT, WIDE>(c, n_rows, H, 0, H, sm.vec, true, from_x);
   {
-    const MatGeom& g = p.g[MAT_HEAD];
-    float* bias_s = sm.vec;   // [kChunk][16 rows][kMaxCols columns]
+    // a chunk's bias tiles, [kChunk][16 rows][bcols columns]; register operands leave the gain in
+    // place while other warps still read it
+    constexpr int bcols = WIDE ? kMaxCols : 8;
+    float* bias_s = STD ? bias_pre : sm.vec;
     int chunk_u0 = 0;
-    run_stage<WT, WIDE>(
-        c, call, sp_head, H, no_key,
+    norm_product<WT, WIDE, STD, MAT_HEAD>(
+        c, call, 4 * L, sp_head, n_rows, H, gain, from_x, nullptr,
         [&](int u0, int cnt, int step) {
           chunk_u0 = u0;
           if (pre_bias) return;
-          for (int o = threadIdx.x; o < cnt * 16 * kMaxCols; o += kConsumerThreads) {
-            const int r = o / (16 * kMaxCols), rr = (o / kMaxCols) & 15, n = o % kMaxCols;
+          for (int o = threadIdx.x; o < cnt * 16 * bcols; o += kConsumerThreads) {
+            const int r = o / (16 * bcols), rr = (o / bcols) & 15, n = o % bcols;
             bias_s[o] = head_bias_at(u0 + r * step, rr, n);
           }
         },
-        [&](int u, int mi, int rr, int n, float v, float) {
-          const int P = ci->heads[u / g.n_units], pos = ci->r_pos[n], j = P - pos;
+        [&](int u, int, int rr, int n, float v, float, float inv) {      // one m-tile per unit
+          int uu;
+          const int P = head_of(u, uu), pos = ci->r_pos[n], j = P - pos;
           if (pos >= 1 && j >= 0 && j <= p.K) {
-            const int id = (u % g.n_units) * g.Mu * 16 + mi * 16 + rr;
-            const float b = pre_bias ? bias_pre[((u - sp_head.ur.first) * 16 + rr) * 8 + n]
-                                     : bias_s[((u - chunk_u0) * 16 + rr) * kMaxCols + n];
+            const int id = uu * 16 + rr;
+            const float b = pre_bias ? bias_pre[((u - u_head) * 16 + rr) * 8 + n]
+                                     : bias_s[((u - chunk_u0) * 16 + rr) * bcols + n];
             p.logits[((size_t)(ci->row0 + n) * (kMaxDraft + 1) + j) * p.V + id] =
-                v * sm.inv_rms[n] * wscale<WT>(p.s_head, (size_t)(P - 1) * p.V + id) + b;
+                v * inv * wscale<WT>(p.s_head, (size_t)(P - 1) * p.V + id) + b;
           }
         });
     if (c.abort_) return;
@@ -1645,7 +1665,7 @@ __device__ __forceinline__ bool read_call_state(Cons& c, int call, bool first) {
   return true;
 }
 
-template <int WT, bool WIDE>
+template <int WT, bool WIDE, bool STD>
 __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constant__ FrameParams p) {
   Smem sm = smem_layout(mcd_dyn_smem);
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -1657,7 +1677,6 @@ __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constan
     sm.flags[0] = 0;
     sm.flags[1] = 0;
     sm.flags[2] = 0;
-    sm.flags[3] = -1;
     fence_barrier_init();
   }
   __syncthreads();
@@ -1671,7 +1690,7 @@ __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constan
       if (sm.ci->all_done) break;
       // a stepwise launch runs one verify call and the noisy-target passes that follow it
       if (p.single_call && call != call0 && !sm.ci->emu) break;
-      run_call<WT, WIDE>(c, call);
+      run_call<WT, WIDE, STD>(c, call);
       if (c.abort_) break;
       if (sm.flags[2]) {
         if (sm.ci->emu)
@@ -1694,34 +1713,38 @@ __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constan
 
 // host-side launcher ------------------------------------------------------------------
 // WIDE: the call may pack more than 8 rows (several streams), so the operand has up to 4
-// n-tiles; the narrow instantiation serves single-stream decoding.
-template <int WT, bool WIDE>
+// n-tiles; the narrow instantiations serve single-stream decoding, STD those of the standard
+// geometry.
+template <int WT, bool WIDE, bool STD>
 static void* frame_entry() {
-  return (void*)frame_kernel<WT, WIDE>;
+  return (void*)frame_kernel<WT, WIDE, STD>;
 }
 
-static void* frame_fn(int wdtype, bool wide) {
+static void* frame_fn(int wdtype, bool wide, bool std_geom) {
+  if (!wide && std_geom)
+    return wdtype == MCD_WEIGHT_BF16 ? frame_entry<MCD_WEIGHT_BF16, false, true>() : frame_entry<MCD_WEIGHT_INT8, false, true>();
   switch (wdtype) {
-    case MCD_WEIGHT_BF16: return wide ? frame_entry<MCD_WEIGHT_BF16, true>() : frame_entry<MCD_WEIGHT_BF16, false>();
-    case MCD_WEIGHT_INT8: return wide ? frame_entry<MCD_WEIGHT_INT8, true>() : frame_entry<MCD_WEIGHT_INT8, false>();
-    default: return wide ? frame_entry<MCD_WEIGHT_F32, true>() : frame_entry<MCD_WEIGHT_F32, false>();
+    case MCD_WEIGHT_BF16: return wide ? frame_entry<MCD_WEIGHT_BF16, true, false>() : frame_entry<MCD_WEIGHT_BF16, false, false>();
+    case MCD_WEIGHT_INT8: return wide ? frame_entry<MCD_WEIGHT_INT8, true, false>() : frame_entry<MCD_WEIGHT_INT8, false, false>();
+    default: return wide ? frame_entry<MCD_WEIGHT_F32, true, false>() : frame_entry<MCD_WEIGHT_F32, false, false>();
   }
 }
 
 cudaError_t launch_frame_kernel(const FrameParams& p, cudaStream_t stream) {
   void* args[] = {const_cast<FrameParams*>(&p)};
   const bool wide = p.S * max(p.K + 1, 2) > kMaxRows || p.draft_mode == MCD_DRAFT_TREE;
-  return cudaLaunchCooperativeKernel(frame_fn(p.wdtype, wide), dim3(p.n_cta), dim3(kThreads), args, (size_t)kSmemBytes,
-                                     stream);
+  return cudaLaunchCooperativeKernel(frame_fn(p.wdtype, wide, std_geometry(p)), dim3(p.n_cta), dim3(kThreads), args,
+                                     (size_t)kSmemBytes, stream);
 }
 
 cudaError_t prepare_frame_kernel(int* max_ctas_per_sm) {
   for (int wd : {MCD_WEIGHT_F32, MCD_WEIGHT_BF16, MCD_WEIGHT_INT8})
-    for (bool wide : {false, true}) {
-      cudaError_t e = cudaFuncSetAttribute(frame_fn(wd, wide), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    for (int form = 0; form < (wd == MCD_WEIGHT_F32 ? 2 : 3); ++form) {       // narrow, wide, narrow standard
+      cudaError_t e = cudaFuncSetAttribute(frame_fn(wd, form == 1, form == 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           kSmemBytes);
       if (e != cudaSuccess) return e;
     }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(max_ctas_per_sm, frame_fn(MCD_WEIGHT_BF16, false), kThreads,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(max_ctas_per_sm, frame_fn(MCD_WEIGHT_BF16, false, true), kThreads,
                                                        kSmemBytes);
 }
 

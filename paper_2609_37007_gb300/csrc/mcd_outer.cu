@@ -351,10 +351,23 @@ __device__ void outer_sample(Cons& c, const OuterStep& o) {
     *o.c0_out = c0;
     if (o.c0_out2) *o.c0_out2 = c0;
   }
-  const float inv = sm.inv_rms[0];
+  // 1/rms of the row (this CTA need not have had a unit of the head, so it sums the row itself)
   const float* xl = p.x + (size_t)(o.nr - 1) * p.H;
+  float ss = 0.f;
   for (int k = threadIdx.x; k < p.H; k += kConsumerThreads) {
-    const float h = __ldcg(xl + k) * inv * sm.vec[k];
+    const float v = __ldcg(xl + k);
+    ss += v * v;
+  }
+#pragma unroll
+  for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
+  if ((threadIdx.x & 31) == 0) sm.part[threadIdx.x >> 5] = ss;
+  consumer_sync();
+  ss = 0.f;
+#pragma unroll
+  for (int w = 0; w < kConsumerWarps; ++w) ss += sm.part[w];
+  const float inv = rsqrtf(__fmul_rn(ss, __frcp_rn((float)p.H)) + p.eps);
+  for (int k = threadIdx.x; k < p.H; k += kConsumerThreads) {
+    const float h = __ldcg(xl + k) * inv * __ldg(p.final_norm + k);
     const float e = WT == MCD_WEIGHT_BF16
                         ? bf16_bits_to_f32(reinterpret_cast<const uint16_t*>(o.c0_table)[(size_t)c0 * p.H + k])
                         : reinterpret_cast<const float*>(o.c0_table)[(size_t)c0 * p.H + k];
@@ -372,11 +385,11 @@ __device__ void outer_sample(Cons& c, const OuterStep& o) {
 // ------------------------------------------------------------------------------------
 // One launch: prefill rows or one frame row
 // ------------------------------------------------------------------------------------
-template <int WT, bool WIDE>
+template <int WT, bool WIDE, bool STD>
 __device__ void run_outer(Cons& c, const OuterStep& o) {
   const FrameParams& p = c.p;
   Smem& sm = c.sm;
-  const int L = p.L, H = p.H, D = p.D, F = p.F, nr = o.nr;
+  const int L = p.L, H = STD ? 1024 : p.H, D = STD ? 128 : p.D, F = p.F, nr = o.nr;
   unsigned* ctr = p.ctr;
   const unsigned N = (unsigned)p.n_cta;
   const size_t rb = (size_t)H * (WT == MCD_WEIGHT_BF16 ? 2 : 4);   // bytes per table row
@@ -422,118 +435,90 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
   auto no_prep = [](int, int, int) {};
   const int n_blocks = (o.pos0 + nr + kKeyBlock - 1) / kKeyBlock;
 
+  // a unit's m-block and k-chunk (the standard shapes' m-block counts are powers of two)
+  constexpr int lg_wo = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WO>::Mu)), lg_wd = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WD>::Mu));
+  auto wo_key = [&](int u) { return STD ? u >> lg_wo : u / p.g[MAT_WO].n_mb; };
+  auto wd_key = [&](int u) { return STD ? u >> lg_wd : u / p.g[MAT_WD].n_mb; };
+  auto wo_mb = [&](int u) { return STD ? u & ((1 << lg_wo) - 1) : u % p.g[MAT_WO].n_mb; };
+  auto wd_mb = [&](int u) { return STD ? u & ((1 << lg_wd) - 1) : u % p.g[MAT_WD].n_mb; };
+  auto resid_epi = [&](int row, int n, float v) { atomicAdd(p.x + (size_t)n * H + row, v); };
   for (int l = 0; l < L; ++l) {
     // ---- RMSNorm -> QKV -----------------------------------------------------------------
-    g2s_vec(sm.vec, p.attn_norm + (size_t)l * H, H);
+    NarrowGain gain;
+    fetch_gain<STD>(c, gain, p.attn_norm + (size_t)l * H, H);
+    const auto sp_qkv = plan_of<WT, WIDE, STD, MAT_QKV>(c, 4 * l, p.g[MAT_QKV].n_units, nr, no_key);
+    const bool seeds = STD ? first_unit(sp_qkv) == 0 : blockIdx.x == 0;      // the CTA that seeds x
+    auto qkv_epi = [&](int u, int mi, int rr, int n, float v, float, float inv) {
+      p.qkv[(size_t)n * p.qkv_dim + (u * (STD ? StdUnit<WT, MAT_QKV>::Mu : p.g[MAT_QKV].Mu) + mi) * 16 + rr] = v * inv;
+    };
     if (l == 0) {
       consumer_sync();                       // gain and ids in shared memory
-      prep_operand<WT, WIDE>(c, nr, H, 0, H, sm.vec, true, ld0, blockIdx.x == 0 ? p.x : nullptr);
+      norm_product<WT, WIDE, STD, MAT_QKV>(c, 0, 0, sp_qkv, nr, H, gain, ld0, seeds ? p.x : nullptr, no_prep, qkv_epi);
     } else {
       if (!cons_wait(c, ctr + ctr_stage(l - 1, 3), N)) return;
-      prep_operand<WT, WIDE>(c, nr, H, 0, H, sm.vec, true, from_x);
+      norm_product<WT, WIDE, STD, MAT_QKV>(c, 0, 4 * l, sp_qkv, nr, H, gain, from_x, nullptr, no_prep, qkv_epi);
     }
-    {
-      const MatGeom& g = p.g[MAT_QKV];
-      run_stage<WT, WIDE>(c, 0, 4 * l + 0, g.n_units, H, nr, no_key, no_prep,
-                          [&](int u, int mi, int rr, int n, float v, float) {
-                            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr;
-                            p.qkv[(size_t)n * p.qkv_dim + row] = v * sm.inv_rms[n];
-                          });
-      if (c.abort_) return;
-    }
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 0), 0, 0);
 
     // ---- attention: (KV head, key block) tasks, then one grid barrier -------------------------
     if (!cons_wait(c, ctr + ctr_stage(l, 0), N)) return;
     for (int t = blockIdx.x; t < p.NKV * n_blocks; t += p.n_cta) outer_attention<WT>(c, o, l, t % p.NKV, t / p.NKV);
     cons_signal(c, ctr + ctr_att(L, l), 0, 0);
-    if (!cons_wait(c, ctr + ctr_att(L, l), N)) return;
 
-    // ---- Wo + residual: unit u multiplies the merged output of head u / n_mb ----------------
-    {
-      const MatGeom& g = p.g[MAT_WO];
-      float* ao = reinterpret_cast<float*>(sm.bfrag);
-      if (threadIdx.x == 0) sm.flags[3] = -1;
-      consumer_sync();
-      run_stage<WT, WIDE>(
-          c, 0, 4 * l + 1, g.n_units, D, nr, [&](int u) { return u / g.n_mb; },
-          [&](int u, int, int) {
-            const int h = u / g.n_mb;
-            if (sm.flags[3] != h) {
-              outer_merge(c, o, h, ao);
-              prep_operand<WT, WIDE>(c, nr, D, 0, D, nullptr, false,
-                                     [&](int n, int k, auto w) { return ld_shared_v<decltype(w)::value>(ao + n * D + k); });
-              if (threadIdx.x == 0) sm.flags[3] = h;
-            }
-          },
-          [&](int u, int mi, int rr, int n, float v, float) {
-            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr;
-            atomicAdd(p.x + (size_t)n * H + row, v);
-          });
-      if (c.abort_) return;
-    }
+    // ---- Wo + residual: unit u multiplies the merged output of head wo_key(u) ----------------
+    const auto sp_wo = plan_of<WT, WIDE, STD, MAT_WO>(c, 4 * l + 1, p.g[MAT_WO].n_units, nr, wo_key);
+    if (!cons_wait(c, ctr + ctr_att(L, l), N)) return;
+    float* ao = reinterpret_cast<float*>(sm.bfrag);
+    keyed_product<WT, WIDE, STD, MAT_WO, false>(
+        c, 0, 4 * l + 1, sp_wo, nr, D, wo_key, [&](int u0) { outer_merge(c, o, wo_key(u0), ao); },
+        [&](int, int n, int k, auto w) { return ld_shared_v<decltype(w)::value>(ao + n * D + k); },
+        reinterpret_cast<uint8_t*>(sm.act), [&](int u, int mi, int rr, int n, float v) {
+          resid_epi((wo_mb(u) * (STD ? StdUnit<WT, MAT_WO>::Mu : p.g[MAT_WO].Mu) + mi) * 16 + rr, n, v);
+        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 1), 0, 0);
 
     // ---- RMSNorm -> gate/up -> SwiGLU ---------------------------------------------------------
-    g2s_vec(sm.vec, p.ffn_norm + (size_t)l * H, H);
+    fetch_gain<STD>(c, gain, p.ffn_norm + (size_t)l * H, H);
+    const auto sp_gu = plan_of<WT, WIDE, STD, MAT_GU>(c, 4 * l + 2, p.g[MAT_GU].n_units, nr, no_key);
     if (!cons_wait(c, ctr + ctr_stage(l, 1), N)) return;
-    prep_operand<WT, WIDE>(c, nr, H, 0, H, sm.vec, true, from_x);
-    {
-      const MatGeom& g = p.g[MAT_GU];
-      run_stage<WT, WIDE>(
-          c, 0, 4 * l + 2, g.n_units, H, nr, no_key, no_prep,
-          [&](int u, int mi, int rr, int n, float gate, float up) {
-            const float s = sm.inv_rms[n];
-            const float gt = gate * s;
-            const int j = ((u % g.n_mb) * g.Mu + mi) * 8 + rr;
-            p.mbuf[(size_t)n * F + j] = gt / (1.0f + __expf(-gt)) * (up * s);
-          },
-          true);
-      if (c.abort_) return;
-    }
+    norm_product<WT, WIDE, STD, MAT_GU>(c, 0, 4 * l + 2, sp_gu, nr, H, gain, from_x, nullptr, no_prep,
+                                        [&](int u, int mi, int rr, int n, float gate, float up, float inv) {
+                                          const int mt = u * (STD ? StdUnit<WT, MAT_GU>::Mu : p.g[MAT_GU].Mu) + mi;
+                                          const float gt = gate * inv;
+                                          p.mbuf[(size_t)n * F + mt * 8 + rr] = gt / (1.0f + __expf(-gt)) * (up * inv);
+                                        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 2), 0, 0);
 
     // ---- down + residual ------------------------------------------------------------------------
+    const auto sp_wd = plan_of<WT, WIDE, STD, MAT_WD>(c, 4 * l + 3, p.g[MAT_WD].n_units, nr, wd_key);
     if (!cons_wait(c, ctr + ctr_stage(l, 2), N)) return;
-    {
-      const MatGeom& g = p.g[MAT_WD];
-      const int Kc = g.Ku * 16;
-      if (threadIdx.x == 0) sm.flags[3] = -1;
-      consumer_sync();
-      run_stage<WT, WIDE>(
-          c, 0, 4 * l + 3, g.n_units, Kc, nr, [&](int u) { return u / g.n_mb; },
-          [&](int u, int, int) {
-            const int kc = u / g.n_mb;
-            if (sm.flags[3] != kc) {
-              const float* m = p.mbuf + (size_t)kc * Kc;
-              prep_operand<WT, WIDE>(c, nr, Kc, 0, Kc, nullptr, false,
-                                     [&](int n, int k, auto w) { return ld_global_v<decltype(w)::value>(m + (size_t)n * F + k); });
-              if (threadIdx.x == 0) sm.flags[3] = kc;
-            }
-          },
-          [&](int u, int mi, int rr, int n, float v, float) {
-            const int row = (u % g.n_mb) * g.Mu * 16 + mi * 16 + rr;
-            atomicAdd(p.x + (size_t)n * H + row, v);
-          });
-      if (c.abort_) return;
-    }
+    const int Kc = STD ? 1024 : p.g[MAT_WD].Ku * 16;
+    keyed_product<WT, WIDE, STD, MAT_WD, false>(
+        c, 0, 4 * l + 3, sp_wd, nr, Kc, wd_key, [](int) {},
+        [&](int u0, int n, int k, auto w) {
+          return ld_global_v<decltype(w)::value>(p.mbuf + (size_t)wd_key(u0) * Kc + (size_t)n * F + k);
+        },
+        reinterpret_cast<uint8_t*>(sm.act), [&](int u, int mi, int rr, int n, float v) {
+          resid_epi((wd_mb(u) * (STD ? StdUnit<WT, MAT_WD>::Mu : p.g[MAT_WD].Mu) + mi) * 16 + rr, n, v);
+        });
+    if (c.abort_) return;
     cons_signal(c, ctr + ctr_stage(l, 3), 0, 0);
   }
   if (!o.head) return;
 
   // ---- final RMSNorm of the last row -> c0 head -------------------------------------------
-  g2s_vec(sm.vec, p.final_norm, H);
+  NarrowGain gain;
+  fetch_gain<STD>(c, gain, p.final_norm, H);
+  const auto sp_head = plan_of<WT, WIDE, STD, MAT_HEAD>(c, 4 * L, p.g[MAT_HEAD].n_units, 1, no_key);
   if (!cons_wait(c, ctr + ctr_stage(L - 1, 3), N)) return;
   const float* xl = p.x + (size_t)(nr - 1) * H;
-  prep_operand<WT, WIDE>(c, 1, H, 0, H, sm.vec, true, [&](int, int k, auto w) { return ld_global_v<decltype(w)::value>(xl + k); });
-  {
-    const MatGeom& g = p.g[MAT_HEAD];
-    run_stage<WT, WIDE>(c, 0, 4 * L, g.n_units, H, 1, no_key, no_prep,
-                        [&](int u, int mi, int rr, int, float v, float) {
-                          p.logits[(u % g.n_units) * g.Mu * 16 + mi * 16 + rr] = v * sm.inv_rms[0];
-                        });
-    if (c.abort_) return;
-  }
+  norm_product<WT, WIDE, STD, MAT_HEAD>(
+      c, 0, 4 * L, sp_head, 1, H, gain, [&](int, int k, auto w) { return ld_global_v<decltype(w)::value>(xl + k); }, nullptr,
+      no_prep, [&](int u, int, int rr, int, float v, float, float inv) { p.logits[u * 16 + rr] = v * inv; });
+  if (c.abort_) return;
   consumer_sync();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -545,7 +530,7 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
   if (sm.flags[2]) outer_sample<WT>(c, o);
 }
 
-template <int WT, bool WIDE>
+template <int WT, bool WIDE, bool STD>
 __global__ void __launch_bounds__(kThreads, 1)
     outer_kernel(const __grid_constant__ FrameParams p, const __grid_constant__ OuterStep o) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -559,7 +544,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     sm.flags[0] = 0;
     sm.flags[1] = 0;
     sm.flags[2] = 0;
-    sm.flags[3] = -1;
     fence_barrier_init();
   }
   __syncthreads();
@@ -567,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if ((tid & 31) == 0) outer_producer(p, o, sm);
   } else {
     Cons c(p, sm);
-    run_outer<WT, WIDE>(c, o);
+    run_outer<WT, WIDE, STD>(c, o);
     if (tid == 0) sm.flags[0] = 1;   // stop the producer
   }
   __syncthreads();
@@ -577,14 +561,16 @@ __global__ void outer_begin_kernel(unsigned* ctr, int n) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) ctr[i] = 0u;
 }
 
-template <int WT, bool WIDE>
+template <int WT, bool WIDE, bool STD>
 static void* outer_entry() {
-  return (void*)outer_kernel<WT, WIDE>;
+  return (void*)outer_kernel<WT, WIDE, STD>;
 }
 
-static void* outer_fn(int wdtype, bool wide) {
-  return wdtype == MCD_WEIGHT_BF16 ? (wide ? outer_entry<MCD_WEIGHT_BF16, true>() : outer_entry<MCD_WEIGHT_BF16, false>())
-                                   : (wide ? outer_entry<MCD_WEIGHT_F32, true>() : outer_entry<MCD_WEIGHT_F32, false>());
+static void* outer_fn(int wdtype, bool wide, bool std_geom) {
+  if (!wide && std_geom) return outer_entry<MCD_WEIGHT_BF16, false, true>();
+  return wdtype == MCD_WEIGHT_BF16
+             ? (wide ? outer_entry<MCD_WEIGHT_BF16, true, false>() : outer_entry<MCD_WEIGHT_BF16, false, false>())
+             : (wide ? outer_entry<MCD_WEIGHT_F32, true, false>() : outer_entry<MCD_WEIGHT_F32, false, false>());
 }
 
 }  // namespace mcd
@@ -1009,7 +995,7 @@ static mcd_status outer_launch(mcd_outer* o, const OuterStep& s) {
   outer_begin_kernel<<<1, 256, 0, o->stream>>>(p.ctr, p.ctr_stride);
   MCD_CHECK(cudaGetLastError());
   void* args[] = {&p, const_cast<OuterStep*>(&s)};
-  MCD_CHECK(cudaLaunchCooperativeKernel(outer_fn(p.wdtype, s.nr > kMaxRows), dim3(p.n_cta), dim3(kThreads), args,
+  MCD_CHECK(cudaLaunchCooperativeKernel(outer_fn(p.wdtype, s.nr > kMaxRows, std_geometry(p)), dim3(p.n_cta), dim3(kThreads), args,
                                         (size_t)kSmemBytes, o->stream));
   return MCD_OK;
 }
@@ -1058,8 +1044,9 @@ mcd_status mcd_outer_create(const mcd_outer_config* cfg, mcd_ctx* inner, mcd_out
     mcd_outer_destroy(o);
     return s;
   };
-  for (void* fn : {outer_fn(MCD_WEIGHT_BF16, false), outer_fn(MCD_WEIGHT_BF16, true), outer_fn(MCD_WEIGHT_F32, false),
-                   outer_fn(MCD_WEIGHT_F32, true)})
+  for (void* fn : {outer_fn(MCD_WEIGHT_BF16, false, true), outer_fn(MCD_WEIGHT_BF16, false, false),
+                   outer_fn(MCD_WEIGHT_BF16, true, false), outer_fn(MCD_WEIGHT_F32, false, false),
+                   outer_fn(MCD_WEIGHT_F32, true, false)})
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
       return fail(MCD_ERR_CUDA);
   const mcd_outer_config& k = *cfg;

@@ -62,7 +62,7 @@ struct Smem {
   float* part;     // [kConsumerWarps][kMaxCols] partial sums of squares
   uint64_t* full;
   uint64_t* empty;
-  int* flags;      // [0] stop, [1] abort, [2] last-arriver, [3] current head / chunk
+  int* flags;      // [0] stop, [1] abort, [2] last-arriver, [4] stream whose acceptance this CTA runs
   float* inv_rms;  // [kMaxCols]
   CallInfo* ci;    // snapshot of the call's state
 };
@@ -458,6 +458,7 @@ struct WarpRole {
 // (Mu, NT and the warp-group counts are powers of two and Gk divides Ku: shifts instead of
 // divisions.)
 __device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
+__host__ __device__ constexpr int ilog2_c(int v) { return v <= 1 ? 0 : 1 + ilog2_c(v >> 1); }
 __device__ __forceinline__ WarpRole warp_role(const MatGeom& g, int NT, int warp, bool split_n) {
   WarpRole w;
   const int lmu = ilog2(g.Mu), lnt = ilog2(NT);
@@ -686,19 +687,358 @@ __device__ __forceinline__ void run_stage(Cons& c, int call, const StagePlan& sp
   c.rot = rot;
 }
 
-// Plan and run in one step (stages whose plan cannot precede a wait).
-template <int WT, bool WIDE, class Key, class Prep, class Epi>
-__device__ __forceinline__ void run_stage(Cons& c, int call, int si, int n_units, int Kdim, int ncols, Key opkey,
-                                          Prep prep, Epi epi, bool pairs_rows = false) {
-  const StagePlan sp = plan_stage<WT, WIDE>(c, si, n_units, ncols, opkey, pairs_rows);
-  run_stage<WT, WIDE>(c, call, sp, Kdim, opkey, prep, epi);
-}
-
 // Read-only vector (weights) into shared memory; no barrier (a later barrier orders it).
 __device__ __forceinline__ void g2s_vec(float* dst, const float* src, int n) {
   const int n4 = n >> 2;
   for (int i = threadIdx.x; i < n4; i += kConsumerThreads)
     reinterpret_cast<float4*>(dst)[i] = __ldg(reinterpret_cast<const float4*>(src) + i);
+}
+
+// ------------------------------------------------------------------------------------
+// Narrow stages (up to 8 columns) of the standard geometry: operand in registers
+// ------------------------------------------------------------------------------------
+// The kernels are bound by the latency of each stage's short instruction chains, so the
+// single-stream instantiations fix what a stage's code depends on -- the unit shape of each
+// matrix kind, hence warp roles and loop counts -- at compile time, for the shapes of the
+// MultiCodeDecoder and the CodeDecoder (hidden 1024, heads of 128, F a multiple of 1024; 16- or
+// 8-bit weights).  A warp multiplies the same k-tiles of every unit of a chunk, so its B
+// fragments (hi and lo halves) fit its registers: each lane loads the inputs of its fragment
+// entries straight from their source, all loads in flight, with no pass through shared memory.
+// Other shapes keep the operand in shared memory (run_stage).  Frames of the MultiCodeDecoder,
+// operand in shared memory and roles computed at run time against this form: K = 3 633 -> 577 us,
+// autoregressive 1734 -> 1527, W8A16 with K = 5 685 -> 583 (register operands with run-time
+// roles: 645, 1760 and 984; what the plans and the unrolled predicates cost was the point).
+template <int WT, int KIND>
+struct StdUnit {
+  static constexpr int Mu = KIND == MAT_WO ? 8 : 1;      // m-tiles per unit
+  static constexpr int Ku = KIND == MAT_WO ? 8 : 64;     // k-tiles per unit
+  static constexpr int Gk = kConsumerWarps / Mu;         // warps along k
+  static constexpr int kts = Ku / Gk;                    // k-tiles per warp
+  static_assert(kts == 8, "a warp's operand: eight k-tiles in registers");
+};
+// Every matrix of p has the unit shape the standard instantiations are compiled for.
+inline bool std_geometry(const FrameParams& p) {
+  if (p.wdtype == MCD_WEIGHT_F32 || p.H != 1024 || p.D != 128) return false;
+  for (int k = 0; k < MAT_COUNT; ++k) {
+    const int Mu = k == MAT_WO ? 8 : 1, Ku = k == MAT_WO ? 8 : 64;
+    if (p.g[k].Mu != Mu || p.g[k].Ku != Ku) return false;
+  }
+  return p.g[MAT_QKV].n_kc == 1 && p.g[MAT_GU].n_kc == 1 && p.g[MAT_HEAD].n_kc == 1;
+}
+
+// A standard stage's share of this CTA: n units first, first + step, ...; `rot` is the rotation
+// of the next stage.  Everything is computed before the wait for the stage's inputs (pin).
+struct NarrowPlan {
+  int first, step, n, rot;
+};
+__device__ __forceinline__ void pin(int& v) { asm volatile("" : "+r"(v)); }
+template <int KIND>
+__device__ __forceinline__ NarrowPlan plan_narrow(const Cons& c, int n_units) {
+  const int n_cta = c.p.n_cta, cta = blockIdx.x;
+  NarrowPlan s;
+  if (KIND == MAT_HEAD || KIND == MAT_WD) {
+    s.first = (int)(((unsigned)cta * (unsigned)n_units) / (unsigned)n_cta);
+    s.n = (int)(((unsigned)(cta + 1) * (unsigned)n_units) / (unsigned)n_cta) - s.first;
+    s.step = 1;
+  } else {
+    const int f = cta - c.rot;
+    s.first = f < 0 ? f + n_cta : f;
+    s.n = s.first < n_units ? (int)((unsigned)(n_units - 1 - s.first) / (unsigned)n_cta) + 1 : 0;
+    s.step = n_cta;
+  }
+  s.rot = (int)((unsigned)(c.rot + n_units) % (unsigned)n_cta);
+  pin(s.first);
+  pin(s.n);
+  pin(s.rot);
+  return s;
+}
+
+struct NarrowOp {
+  uint32_t hi[8][2], lo[8][2];        // B fragments of the warp's k-tiles
+};
+
+// Packed pairs of fp32 values (one instruction for two IEEE operations).
+__device__ __forceinline__ uint64_t f2_pack(float2 v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(uint64_t r) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
+  return v;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+  return f2_unpack(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)), "l"(f2_pack(c)));
+  return f2_unpack(r);
+}
+
+// The norm gain of this lane's inputs, read before the wait for the stage's rows (the volatile
+// loads are not moved behind it).
+struct NarrowGain {
+  float2 a[8], b[8];
+};
+__device__ __forceinline__ float2 ldg_now(const float* p) {
+  float2 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void load_gain(NarrowGain& g, const float* gain) {
+  const float* q = gain + (threadIdx.x >> 5) * 128 + 2 * (threadIdx.x & 3);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    g.a[e] = ldg_now(q + 16 * e);
+    g.b[e] = ldg_now(q + 16 * e + 8);
+  }
+}
+
+// This warp's B fragments: ld(n, k, Vec2{}) returns elements k, k + 1 of column n (k from the
+// start of the units' k-chunk); a gain multiplies them per input, and the columns' sums of
+// squares then go to `part`, one row of 8 per k-group; store_raw (may be null) receives the raw
+// values as fp32 rows of ldk.
+template <int KIND, class Ld>
+__device__ __forceinline__ void load_narrow(Cons& c, int ncols, const NarrowGain* gain, Ld ld, float* store_raw, int ldk,
+                                            NarrowOp& op) {
+  using U = StdUnit<MCD_WEIGHT_BF16, KIND>;
+  const int lane = threadIdx.x & 31, n = lane >> 2, kg = (threadIdx.x >> 5) / U::Mu;
+  const bool live = n < ncols;
+  const int k_base = kg * 128 + 2 * (lane & 3);
+  float2 va[8], vb[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    va[e] = make_float2(0.f, 0.f);
+    vb[e] = make_float2(0.f, 0.f);
+    if (live) {
+      va[e] = ld(n, k_base + 16 * e, Vec2{});
+      vb[e] = ld(n, k_base + 16 * e + 8, Vec2{});
+    }
+  }
+  if (store_raw && live) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      *reinterpret_cast<float2*>(store_raw + (size_t)n * ldk + k_base + 16 * e) = va[e];
+      *reinterpret_cast<float2*>(store_raw + (size_t)n * ldk + k_base + 16 * e + 8) = vb[e];
+    }
+  }
+  float2 ss = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    float2 x01 = va[e], x89 = vb[e];
+    if (gain) {
+      ss = fma2(x01, x01, ss);
+      ss = fma2(x89, x89, ss);
+      x01 = mul2(x01, gain->a[e]);
+      x89 = mul2(x89, gain->b[e]);
+    }
+    const uint32_t h01 = pack_bf16x2(x01.x, x01.y), h89 = pack_bf16x2(x89.x, x89.y);
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 r01 = fma2(make_float2(bf16_lo_f32(h01), bf16_hi_f32(h01)), m1, x01);      // exact remainders
+    const float2 r89 = fma2(make_float2(bf16_lo_f32(h89), bf16_hi_f32(h89)), m1, x89);
+    op.hi[e][0] = h01;
+    op.hi[e][1] = h89;
+    op.lo[e][0] = pack_bf16x2(r01.x, r01.y);
+    op.lo[e][1] = pack_bf16x2(r89.x, r89.y);
+  }
+  if (gain) {
+    float s = ss.x + ss.y;
+    s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+    s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+    if ((lane & 3) == 0) c.sm.part[kg * 8 + n] = s;
+  }
+}
+
+// A chunk's partial tiles, summed over the k-group warps: row rr of m-tile mi, column n of unit r.
+template <int KIND>
+__device__ __forceinline__ float narrow_sum(const Cons& c, int r, int mi, int rr, int n) {
+  using U = StdUnit<MCD_WEIGHT_BF16, KIND>;
+  const float* red = c.sm.red + ((r * kConsumerWarps + mi) * 32 + (rr & 7) * 4 + (n >> 1)) * 4 + (rr >> 3) * 2 + (n & 1);
+  float v[U::Gk];
+#pragma unroll
+  for (int kg = 0; kg < U::Gk; ++kg) v[kg] = red[kg * U::Mu * 128];
+#pragma unroll
+  for (int h = U::Gk / 2; h; h >>= 1)
+#pragma unroll
+    for (int kg = 0; kg < h; ++kg) v[kg] += v[kg + h];
+  return v[0];
+}
+
+// The planned stage's units with register operands, in chunks of up to kChunk units of one key
+// (contiguous from a unit on): load(u0, op) fills the operand of the units that share u0's
+// key; prep(u0, cnt, step) runs before each chunk's products; epi as in run_stage, its last
+// argument the column's 1/rms (1 without kNorm).
+template <int WT, int KIND, bool kNorm, bool QUAD, class Key, class Load, class Prep, class Epi>
+__device__ __forceinline__ void run_narrow(Cons& c, int call, int si, const NarrowPlan& sp, int ncols, Key opkey, Load load,
+                                           Prep prep, Epi epi) {
+  using U = StdUnit<WT, KIND>;
+  constexpr bool kPairs = KIND == MAT_GU;
+  const FrameParams& p = c.p;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lgn = col_log2(ncols);
+  timeline(c, call, 8 + 4 * si);
+  int done = 0;
+  while (done < sp.n) {               // runs of units with one key, each with its operand
+    const int key = opkey(sp.first + done * sp.step);
+    NarrowOp op;
+    load(sp.first + done * sp.step, op);
+    do {
+      const int u0 = sp.first + done * sp.step;
+      int cnt = 1;
+      while (cnt < kChunk && done + cnt < sp.n && opkey(u0 + cnt * sp.step) == key) ++cnt;
+      prep(u0, cnt, sp.step);
+#pragma unroll 1
+      for (int r = 0; r < cnt; ++r) {
+        const uint32_t slot = (c.seq + r) % kNumSlots;
+        if (!wait_mbar(&c.sm.full[slot], ((c.seq + r) / kNumSlots) & 1u, p.err, p.wait_ns, nullptr))
+          c.sm.flags[1] = 1;
+        if (done == 0 && r == 0) timeline(c, call, 9 + 4 * si);
+        // the warp's m-tile mi and k-tiles kg * kts ..; hi and lo halves, even and odd k-tiles in
+        // accumulators of their own (short dependence chains)
+        const uint8_t* A = c.sm.ring + slot * kSlotBytes;
+        const int a0i = ((warp % U::Mu) * U::Ku + (warp / U::Mu) * U::kts) * 32 + lane;
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+#pragma unroll
+        for (int t = 0; t < U::kts; ++t) {
+          const uint4 a = WT == MCD_WEIGHT_BF16 ? reinterpret_cast<const uint4*>(A)[a0i + t * 32]
+                                                : widen_i8x8(reinterpret_cast<const uint2*>(A)[a0i + t * 32]);
+          mma_bf16_16816(acc[t & 1], a, op.hi[t][0], op.hi[t][1]);
+          mma_bf16_16816(acc[2 + (t & 1)], a, op.lo[t][0], op.lo[t][1]);
+        }
+        reinterpret_cast<float4*>(c.sm.red)[(r * kConsumerWarps + warp) * 32 + lane] =
+            make_float4((acc[0][0] + acc[1][0]) + (acc[2][0] + acc[3][0]), (acc[0][1] + acc[1][1]) + (acc[2][1] + acc[3][1]),
+                        (acc[0][2] + acc[1][2]) + (acc[2][2] + acc[3][2]), (acc[0][3] + acc[1][3]) + (acc[2][3] + acc[3][3]));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c.sm.empty[slot]);
+      }
+      c.seq += cnt;
+      consumer_sync();
+      if (*(volatile int*)&c.sm.flags[1]) {
+        c.abort_ = true;
+        return;
+      }
+      // partials are stored with kg slowest: warp = kg * Mu + mi
+      constexpr int lg_rows = ilog2_c(U::Mu) + (kPairs ? 3 : 4) - (QUAD ? 2 : 0);
+      const int lg_out = lg_rows + lgn;
+#pragma unroll 1
+      for (int o = threadIdx.x; o < (cnt << lg_out); o += kConsumerThreads) {
+        const int r = o >> lg_out, q = o & ((1 << lg_out) - 1), row = q >> lgn, n = q & ((1 << lgn) - 1);
+        if (n >= ncols) continue;
+        const int u = u0 + r * sp.step;
+        if constexpr (QUAD) {
+          const int mi = row >> 2, rr0 = (row & 3) << 2;
+          epi(u, mi, rr0, n,
+              make_float4(narrow_sum<KIND>(c, r, mi, rr0, n), narrow_sum<KIND>(c, r, mi, rr0 + 1, n),
+                          narrow_sum<KIND>(c, r, mi, rr0 + 2, n), narrow_sum<KIND>(c, r, mi, rr0 + 3, n)),
+              1.f);
+        } else {
+          const int mi = row >> (kPairs ? 3 : 4), rr = row & (kPairs ? 7 : 15);
+          float inv = 1.f;
+          if (kNorm) {                // 1/rms of column n from the k-groups' sums (fixed order)
+            const float* q = c.sm.part + n;
+            const float s = ((q[0] + q[8]) + (q[16] + q[24])) + ((q[32] + q[40]) + (q[48] + q[56]));
+            inv = rsqrtf(s * (1.0f / 1024.0f) + p.eps);
+          }
+          const float v = narrow_sum<KIND>(c, r, mi, rr, n);
+          const float v8 = kPairs ? narrow_sum<KIND>(c, r, mi, rr + 8, n) : 0.f;
+          epi(u, mi, rr, n, v, v8, inv);
+        }
+      }
+      done += cnt;
+      if (done < sp.n) consumer_sync();
+    } while (done < sp.n && opkey(sp.first + done * sp.step) == key);
+  }
+  c.rot = sp.rot;
+}
+
+// A stage's plan: the standard geometry's, or the general one.
+template <int WT, bool WIDE, bool STD, int KIND, class Key>
+__device__ __forceinline__ auto plan_of(const Cons& c, int si, int n_units, int ncols, Key opkey) {
+  if constexpr (STD) return plan_narrow<KIND>(c, n_units);
+  else return plan_stage<WT, WIDE>(c, si, n_units, ncols, opkey, KIND == MAT_GU);
+}
+
+__device__ __forceinline__ int first_unit(const NarrowPlan& s) { return s.first; }
+__device__ __forceinline__ int first_unit(const StagePlan& s) { return s.ur.first; }
+__device__ __forceinline__ int unit_count(const NarrowPlan& s) { return s.n; }
+__device__ __forceinline__ int unit_count(const StagePlan& s) {          // contiguous ranges
+  return s.ur.end - s.ur.first;
+}
+__device__ __forceinline__ bool has_units(const NarrowPlan& s) { return s.n > 0; }
+__device__ __forceinline__ bool has_units(const StagePlan& s) { return s.ur.first < s.ur.end; }
+template <class F>
+__device__ __forceinline__ void for_units(const NarrowPlan& s, F f) {
+  for (int i = 0; i < s.n; ++i) f(s.first + i * s.step);
+}
+template <class F>
+__device__ __forceinline__ void for_units(const StagePlan& s, F f) {
+  for (int u = s.ur.first; u < s.ur.end; u += s.ur.step) f(u);
+}
+
+// A normalised product's gain [n], fetched before the wait for its rows: into registers, or
+// (general stages) shared memory.
+template <bool STD>
+__device__ __forceinline__ void fetch_gain(Cons& c, NarrowGain& g, const float* gain, int n) {
+  if constexpr (STD) load_gain(g, gain);
+  else g2s_vec(c.sm.vec, gain, n);
+}
+// A normalised product, W (x . g) / rms: every unit multiplies the same rows x (ld, see
+// prep_operand), the gain from fetch_gain, prep before each chunk, epi(u, mi, rr, n, v, v8, inv).
+template <int WT, bool WIDE, bool STD, int KIND, class Plan, class Ld, class Prep, class Epi>
+__device__ __forceinline__ void norm_product(Cons& c, int call, int si, const Plan& sp, int ncols, int Kdim,
+                                             const NarrowGain& gain, Ld ld, float* store_raw, Prep prep, Epi epi) {
+  auto no_key = [](int) { return 0; };
+  if constexpr (STD) {
+    run_narrow<WT, KIND, true, false>(
+        c, call, si, sp, ncols, no_key,
+        [&](int, NarrowOp& op) { load_narrow<KIND>(c, ncols, &gain, ld, store_raw, Kdim, op); }, prep, epi);
+  } else {
+    prep_operand<WT, WIDE>(c, ncols, Kdim, 0, Kdim, c.sm.vec, true, ld, store_raw);
+    run_stage<WT, WIDE>(c, call, sp, Kdim, no_key, prep, [&](int u, int mi, int rr, int n, float v, float v8) {
+      epi(u, mi, rr, n, v, v8, c.sm.inv_rms[n]);
+    });
+  }
+}
+
+// A residual product, its units' operand given by their key: before(u0) makes the columns of u0's
+// key readable, col(u0, n, k, vec) reads them; epi(u, mi, rr0, n, float4) takes four rows at
+// once (QUAD), or epi(u, mi, rr, n, v) one.
+template <int WT, bool WIDE, bool STD, int KIND, bool QUAD, class Plan, class Key, class Before, class Col, class Epi>
+__device__ __forceinline__ void keyed_product(Cons& c, int call, int si, const Plan& sp, int ncols, int Kdim, Key opkey,
+                                              Before before, Col col, uint8_t* op_smem, Epi epi) {
+  auto each = [&](int u, int mi, int rr, int n, auto v, auto...) { epi(u, mi, rr, n, v); };
+  if constexpr (STD) {
+    run_narrow<WT, KIND, false, QUAD>(
+        c, call, si, sp, ncols, opkey,
+        [&](int u0, NarrowOp& op) {
+          before(u0);
+          load_narrow<KIND>(c, ncols, nullptr, [&](int n, int k, auto w) { return col(u0, n, k, w); }, nullptr, Kdim, op);
+        },
+        [](int, int, int) {}, each);
+  } else {
+    int cur = -1;
+    run_stage<WT, WIDE, QUAD>(
+        c, call, sp, Kdim, opkey,
+        [&](int u0, int, int) {
+          if (opkey(u0) != cur) {
+            before(u0);
+            c.op = op_smem;
+            prep_operand<WT, WIDE>(c, ncols, Kdim, 0, Kdim, nullptr, false,
+                                   [&](int n, int k, auto w) { return col(u0, n, k, w); });
+            cur = opkey(u0);
+          }
+        },
+        each);
+    c.op = reinterpret_cast<uint8_t*>(c.sm.act);
+  }
 }
 
 template <int W> __device__ __forceinline__ vecf<W> ld_global_v(const float* q) {

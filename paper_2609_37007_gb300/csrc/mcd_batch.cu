@@ -1136,7 +1136,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemHilo) != cudaSuccess)
       return fail(MCD_ERR_CUDA);
   if (bs->use_tc &&
-      (tc_block_set_smem() != cudaSuccess ||
+      (tc_block_set_smem<false>() != cudaSuccess ||
        cudaFuncSetAttribute(tc_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             tc::Layout<kHeadTileMax, true>::kSmemBytes) != cudaSuccess))
     return fail(MCD_ERR_CUDA);
@@ -1202,13 +1202,13 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc::launch(false, batch_attn_kernel, dim3(bs->max_streams, p.NKV), blk, 0, s, p, b, l);      // -> att_t
     // Wo (k-split partials) -> residual, ss, the gate/up operand
-    tc_launch_resid(wl + bs->tw.off.o, b.att_t, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid<false>(wl + bs->tw.off.o, b.att_t, nullptr, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
                                            p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, (uint8_t*)nullptr);
     // gate/up -> SwiGLU (into the down product's operand)
-    tc_launch_gu(wl + bs->tw.off.gu, b.xn_hi, b.act_t, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_gu<false>(wl + bs->tw.off.gu, b.xn_hi, nullptr, b.act_t, nullptr, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     // down (k-split partials) -> residual, ss, the next layer's QKV operand
-    tc_launch_resid(wl + bs->tw.off.d, b.act_t, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid<false>(wl + bs->tw.off.d, b.act_t, nullptr, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
     const bool last = l + 1 == L;
     tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
                                            last ? (const float*)nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);

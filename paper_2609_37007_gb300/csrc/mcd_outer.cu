@@ -6,9 +6,9 @@
 // the c0 embedding start the MultiCodeDecoder's frame, which emits c1..c15.  The next
 // frame's CodeDecoder input is the sum of the text row (if any) and the embeddings of the 16
 // codes just emitted.  Before frame 0 the text prompt is prefilled: with the shapes the
-// tcgen05 block kernels take, all rows but the last as one batch on the tensor cores
-// (outer_tc_prefill), else up to 16 rows per outer_kernel launch; the last row always runs
-// through outer_kernel, which samples frame 0's c0.
+// tcgen05 block kernels take, every row as one batch on the tensor cores (outer_tc_prefill, hi + lo
+// operands like outer_kernel's), else up to 16 rows per outer_kernel launch; outer_kernel
+// then runs the c0 head of the last row and samples frame 0's c0.
 //
 // outer_kernel is one cooperative launch of one CTA per SM, built on the same weight ring
 // and unit GEMMs as the frame kernel (mcd_stage.cuh): per layer QKV -> attention -> Wo ->
@@ -46,6 +46,7 @@ struct OuterStep {
   int cap;
   const float2* rope;              // [cap][D/2] (cos, sin)
   int pos0, nr, head;              // first new position, new rows, 1 = c0 head + sampling
+  int l0;                          // first layer to run (L: the c0 head alone, on the row in p.x)
   const int* text_ids;             // prefill: ids of the rows (device), else null
   const int* prev_codes;           // frame step: c0..c_P of the previous frame (device)
   int text_id;                     // frame step: text row added to the sum, -1 = none
@@ -77,7 +78,7 @@ __device__ void outer_producer(const FrameParams& p, const OuterStep& o, Smem& s
   uint32_t issued = 0;
   int rot = 0;
   bool halt = false;
-  for (int si = 0; si < ns && !halt; ++si) {
+  for (int si = 4 * o.l0; si < ns && !halt; ++si) {
     const int n = stage_units(p, si, 1);
     const uint32_t bytes = (uint32_t)p.g[stage_kind(si, p.L)].unit_bytes;
     const UnitRange ur = unit_range(si, p.L, n, blockIdx.x, rot, p.n_cta);
@@ -442,7 +443,7 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
   auto wo_mb = [&](int u) { return STD ? u & ((1 << lg_wo) - 1) : u % p.g[MAT_WO].n_mb; };
   auto wd_mb = [&](int u) { return STD ? u & ((1 << lg_wd) - 1) : u % p.g[MAT_WD].n_mb; };
   auto resid_epi = [&](int row, int n, float v) { atomicAdd(p.x + (size_t)n * H + row, v); };
-  for (int l = 0; l < L; ++l) {
+  for (int l = o.l0; l < L; ++l) {
     // ---- RMSNorm -> QKV -----------------------------------------------------------------
     NarrowGain gain;
     fetch_gain<STD>(c, gain, p.attn_norm + (size_t)l * H, H);
@@ -513,7 +514,11 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
   NarrowGain gain;
   fetch_gain<STD>(c, gain, p.final_norm, H);
   const auto sp_head = plan_of<WT, WIDE, STD, MAT_HEAD>(c, 4 * L, p.g[MAT_HEAD].n_units, 1, no_key);
-  if (!cons_wait(c, ctr + ctr_stage(L - 1, 3), N)) return;
+  if (o.l0 < L) {
+    if (!cons_wait(c, ctr + ctr_stage(L - 1, 3), N)) return;
+  } else {
+    consumer_sync();                         // the gain, where it is in shared memory
+  }
   const float* xl = p.x + (size_t)(nr - 1) * H;
   norm_product<WT, WIDE, STD, MAT_HEAD>(
       c, 0, 4 * L, sp_head, 1, H, gain, [&](int, int k, auto w) { return ld_global_v<decltype(w)::value>(xl + k); }, nullptr,
@@ -580,9 +585,12 @@ using namespace mcd;
 // ------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------
-// Prompt prefill on the tensor cores: rows 0..T-2 of a T-token prompt go through the 28
-// layers as one batch (tcgen05 products, causal attention, K / V written to the cache); the
-// last row then runs through outer_kernel, which reads that cache and samples c0.
+// Prompt prefill on the tensor cores: the rows of a prompt of two or more tokens go through the
+// layers as one batch (tcgen05 products with hi + lo operands, causal attention, K / V written
+// to the cache); outer_kernel then runs the c0 head on the last row's residual and samples c0.
+// With single bf16 operands outside QKV the last row had to run through outer_kernel's layers
+// again: 2.30 ms for 256 tokens, 0.61 of them in that row, against 1.66 ms; and the prompt's
+// outputs were 8.6e-5 off a 64-bit evaluation against 2.1e-5.
 struct OuterTc {
   bool on = false;
   int Rtc = 0;                     // capacity in operand rows
@@ -593,7 +601,7 @@ struct OuterTc {
   float* qkv = nullptr;            // [Rtc][qkv_dim]
   float* q = nullptr;              // [Rtc][NH * D] normalised, rotated queries
   float* part = nullptr;           // [kTcSplit][Rtc][H] partial sums of the residual products
-  uint8_t *xn_hi = nullptr, *xn_lo = nullptr, *att_t = nullptr, *act_t = nullptr;   // operands
+  uint8_t *xn_hi = nullptr, *xn_lo = nullptr, *att_t = nullptr, *att_lo = nullptr, *act_t = nullptr, *act_lo = nullptr;   // operands
   int* rows = nullptr;             // device: live rows
 };
 
@@ -745,7 +753,7 @@ template <int D>
 __global__ void __launch_bounds__(kPfWarps * 32) pf_attn_kernel(const float* __restrict__ q, const int* nrows, int NH,
                                                                 int NKV, const uint16_t* __restrict__ kc,
                                                                 const uint16_t* __restrict__ vc, int cap, int Rtc,
-                                                                uint8_t* att_t) {
+                                                                uint8_t* att_t, uint8_t* att_lo) {
   using S = PfAttn<D>;
   extern __shared__ __align__(16) uint8_t pf_smem[];
   tc::pdl_wait();
@@ -915,9 +923,16 @@ __global__ void __launch_bounds__(kPfWarps * 32) pf_attn_kernel(const float* __r
       v[4] += wt[w] * b.x; v[5] += wt[w] * b.y; v[6] += wt[w] * b.z; v[7] += wt[w] * b.w;
     }
     const int f = h * D + d;
-    *reinterpret_cast<uint4*>(att_t + tc::sw128_offset(Rtc, r, f >> 6, (f & 63) >> 3)) =
-        make_uint4(pack_bf16x2(v[0] * inv, v[1] * inv), pack_bf16x2(v[2] * inv, v[3] * inv),
-                   pack_bf16x2(v[4] * inv, v[5] * inv), pack_bf16x2(v[6] * inv, v[7] * inv));
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float a = v[2 * e] * inv, b = v[2 * e + 1] * inv;
+      hi[e] = pack_bf16x2(a, b);
+      lo[e] = pack_bf16x2(a - bf16_lo_f32(hi[e]), b - bf16_hi_f32(hi[e]));
+    }
+    const size_t off = tc::sw128_offset(Rtc, r, f >> 6, (f & 63) >> 3);
+    *reinterpret_cast<uint4*>(att_t + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(att_lo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
 }
 static cudaError_t pf_attn_set_smem() {
@@ -927,10 +942,10 @@ static cudaError_t pf_attn_set_smem() {
   return e;
 }
 static void launch_pf_attn(const float* q, const int* nrows, int n, int NH, int NKV, int D, const uint16_t* kc,
-                           const uint16_t* vc, int cap, int Rtc, uint8_t* att_t, cudaStream_t s) {
+                           const uint16_t* vc, int cap, int Rtc, uint8_t* att_t, uint8_t* att_lo, cudaStream_t s) {
   const dim3 grid((n + kPfRows - 1) / kPfRows, NH);
   auto go = [&](auto kernel, int smem) {
-    tc::launch(true, kernel, grid, dim3(kPfWarps * 32), smem, s, q, nrows, NH, NKV, kc, vc, cap, Rtc, att_t);
+    tc::launch(true, kernel, grid, dim3(kPfWarps * 32), smem, s, q, nrows, NH, NKV, kc, vc, cap, Rtc, att_t, att_lo);
   };
   if (D == 128) go(pf_attn_kernel<128>, PfAttn<128>::kSmemBytes);
   else go(pf_attn_kernel<64>, PfAttn<64>::kSmemBytes);
@@ -990,8 +1005,10 @@ static int prefill_rows(const mcd_outer* o) {
   return std::min(kMaxPrefillRows, kMaxQVec / (o->fp.NH / o->fp.NKV));
 }
 
-static mcd_status outer_launch(mcd_outer* o, const OuterStep& s) {
-  FrameParams& p = o->fp;
+// x: the residual row of a launch that runs the c0 head alone (null: the context's rows).
+static mcd_status outer_launch(mcd_outer* o, const OuterStep& s, float* x = nullptr) {
+  FrameParams p = o->fp;
+  if (x) p.x = x;
   outer_begin_kernel<<<1, 256, 0, o->stream>>>(p.ctr, p.ctr_stride);
   MCD_CHECK(cudaGetLastError());
   void* args[] = {&p, const_cast<OuterStep*>(&s)};
@@ -1147,9 +1164,11 @@ mcd_status mcd_outer_create(const mcd_outer_config* cfg, mcd_ctx* inner, mcd_out
     OUTER_ALLOC(t.xn_hi, (size_t)Rtc * p.H * 2);
     OUTER_ALLOC(t.xn_lo, (size_t)Rtc * p.H * 2);
     OUTER_ALLOC(t.att_t, (size_t)Rtc * p.NH * p.D * 2);
+    OUTER_ALLOC(t.att_lo, (size_t)Rtc * p.NH * p.D * 2);
     OUTER_ALLOC(t.act_t, (size_t)Rtc * p.F * 2);
+    OUTER_ALLOC(t.act_lo, (size_t)Rtc * p.F * 2);
     OUTER_ALLOC(t.rows, sizeof(int));
-    if (tc_block_set_smem() != cudaSuccess || pf_attn_set_smem() != cudaSuccess) return fail(MCD_ERR_CUDA);
+    if (tc_block_set_smem<true>() != cudaSuccess || pf_attn_set_smem() != cudaSuccess) return fail(MCD_ERR_CUDA);
   }
 #undef OUTER_ALLOC
   s.c0_out = o->c0_buf;
@@ -1291,12 +1310,12 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
     tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
                                                          p.q_norm + (size_t)l * p.D, p.k_norm + (size_t)l * p.D, p.eps,
                                                          st.rope, kc, vc, st.cap, t.q);
-    launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, s);
-    tc_launch_resid(wl + t.off.o, t.att_t, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
+    launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, t.att_lo, s);
+    tc_launch_resid<true>(wl + t.off.o, t.att_t, t.att_lo, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
-                                           p.eps, t.xn_hi, (uint8_t*)nullptr);
-    tc_launch_gu(wl + t.off.gu, t.xn_hi, t.act_t, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid(wl + t.off.d, t.act_t, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
+                                           p.eps, t.xn_hi, t.xn_lo);
+    tc_launch_gu<true>(wl + t.off.gu, t.xn_hi, t.xn_lo, t.act_t, t.act_lo, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid<true>(wl + t.off.d, t.act_t, t.act_lo, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss,
                                            l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : (const float*)nullptr, p.eps, t.xn_hi,
                                            t.xn_lo);
@@ -1313,16 +1332,16 @@ mcd_status mcd_outer_prefill(mcd_outer* o, uint32_t stream_id, int32_t n_tokens,
   const int R = prefill_rows(o);
   o->stream_id = stream_id;
   o->st.stream_id = stream_id;
-  // all but the last row on the tensor cores (when the shapes allow), the last through
-  // outer_kernel (c0 head and sampling)
-  int first = 0;
-  if (o->tc.on && n_tokens >= 2) {
-    mcd_status r = outer_tc_prefill(o, text_ids, n_tokens - 1);
+  // every layer on the tensor cores (when the shapes allow), then outer_kernel for the c0 head
+  // and the draw of the last row
+  const bool batch = o->tc.on && n_tokens >= 2;
+  if (batch) {
+    mcd_status r = outer_tc_prefill(o, text_ids, n_tokens);
     if (r != MCD_OK) return r;
-    first = n_tokens - 1;
   }
-  for (int s0 = first; s0 < n_tokens; s0 += R) {
+  for (int s0 = batch ? n_tokens - 1 : 0; s0 < n_tokens; s0 += R) {
     OuterStep s = o->st;
+    s.l0 = batch ? o->fp.L : 0;
     s.pos0 = s0;
     s.nr = std::min(R, n_tokens - s0);
     s.head = s0 + s.nr == n_tokens ? 1 : 0;
@@ -1332,7 +1351,7 @@ mcd_status mcd_outer_prefill(mcd_outer* o, uint32_t stream_id, int32_t n_tokens,
     s.c0_out2 = s.head ? c0_out : nullptr;
     s.frame_id = 0;
     s.trace = (o->trace && o->trace_frames > 0) ? o->trace : nullptr;
-    mcd_status r = outer_launch(o, s);
+    mcd_status r = outer_launch(o, s, batch ? o->tc.X + (size_t)(n_tokens - 1) * o->fp.H : nullptr);
     if (r != MCD_OK) return r;
   }
   o->n_tok = n_tokens;

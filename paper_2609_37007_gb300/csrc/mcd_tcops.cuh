@@ -8,6 +8,8 @@
 // Every kernel reads its live row count from device memory (*nrows, rows beyond it are
 // neither computed nor written).  Internal linkage: each translation unit has its copy.
 #pragma once
+#include <type_traits>
+
 #include "mcd_internal.cuh"
 #include "mcd_tcgemm.cuh"
 
@@ -93,15 +95,16 @@ __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::G
 // the gate and up values of eight consecutive features of one packed row; it writes
 // silu(gate) * up as one 16-byte bf16 chunk of the down product's SW128 operand (k-slice b,
 // element (row n, feature m)).  Packed rows at or past *nrows are not written.
+// kHilo (the prompt): the operand and the result are hi + lo pairs of bf16 (about 16 mantissa bits).
 constexpr int kGuThreads = 256;
-template <int BN, int kBudget>
-__global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs g, uint8_t* act_t, int Rtc,
+template <int BN, bool kHilo, int kBudget>
+__global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs g, uint8_t* act_t, uint8_t* act_lo, int Rtc,
                                                                const int* nrows) {
-  using L = tc::Layout<BN, false, kBudget>;
+  using L = tc::Layout<BN, kHilo, kBudget>;
   constexpr int kSP = tc::kBM + 4;                  // staged column stride (floats)
   static_assert((size_t)BN * kSP * 4 <= (size_t)L::kStages * L::kStageBytes, "gate/up staging exceeds the ring");
   tc::TileRun t;
-  if (!tc::gemm_tile_run<BN, false, kBudget, true>(g, t)) return;
+  if (!tc::gemm_tile_run<BN, kHilo, kBudget, true>(g, t)) return;
   float* S = reinterpret_cast<float*>(t.smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quarter = warp & 3, part = warp >> 2, n_parts = (int)(blockDim.x >> 7);
@@ -131,9 +134,15 @@ __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs
       float v[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) v[e] = gt[e] / (1.0f + __expf(-gt[e])) * up[e];
-      *reinterpret_cast<uint4*>(act_t + tc::sw128_offset(Rtc, n, kt, c)) =
-          make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                     pack_bf16x2(v[6], v[7]));
+      const size_t off = tc::sw128_offset(Rtc, n, kt, c);
+      uint32_t h[4], lo[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+        lo[q] = pack_bf16x2(v[2 * q] - bf16_lo_f32(h[q]), v[2 * q + 1] - bf16_hi_f32(h[q]));
+      }
+      *reinterpret_cast<uint4*>(act_t + off) = make_uint4(h[0], h[1], h[2], h[3]);
+      if (kHilo) *reinterpret_cast<uint4*>(act_lo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
   }
   tc::gemm_tile_free<BN>(t);
@@ -143,11 +152,11 @@ __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs
 // blockIdx.z of kTcSplit; split z writes its partial sums part[z][n][m] (plain stores);
 // tc_resid_norm_kernel adds them into the residual stream.
 constexpr int kResidThreads = 256;
-template <int BN, int kBudget>
+template <int BN, bool kHilo, int kBudget>
 __global__ void __launch_bounds__(kResidThreads, 1) tc_resid_kernel(const tc::GemmArgs g, float* part, int ld, int Rtc,
                                                                      const int* nrows) {
   tc::TileRun t;
-  if (!tc::gemm_tile_run<BN, false, kBudget, true>(g, t)) return;
+  if (!tc::gemm_tile_run<BN, kHilo, kBudget, true>(g, t)) return;
   const int M = *nrows;
   const size_t zoff = (size_t)blockIdx.z * Rtc;
   tc::gemm_tile_drain<BN>(t, [&](int m, int n, float v) {
@@ -268,7 +277,19 @@ inline void tc_tile_layer(const FrameParams& p, cudaStream_t st, const uint8_t* 
   tile(wo, H, qd, H, 0, H, 0, t.o);
   tile(wd, H, F, H, 0, F, 0, t.d);
 }
+// The instantiation of a gate/up or residual product for a tile pitch, as go(std::integral_constant
+// BN, budget); a compact ring where two CTAs of consecutive kernels shall share an SM.
+template <bool kHilo, class Go>
+inline void tc_pick(int pitch, int Rtc, Go go) {
+  if (pitch <= 64) go(std::integral_constant<int, 64>{}, std::integral_constant<int, kTcCompact>{});
+  else if (!kHilo && pitch <= 128 && Rtc <= kTcCompactRows)
+    go(std::integral_constant<int, 128>{}, std::integral_constant<int, kTcCompact>{});
+  else if (pitch <= 128) go(std::integral_constant<int, 128>{}, std::integral_constant<int, tc::kStageBudget>{});
+  else if (pitch <= 176) go(std::integral_constant<int, 176>{}, std::integral_constant<int, tc::kStageBudget>{});
+  else go(std::integral_constant<int, 256>{}, std::integral_constant<int, tc::kStageBudget>{});
+}
 // Dynamic shared memory of the block kernels (once per translation unit).
+template <bool kHilo>
 inline cudaError_t tc_block_set_smem() {
   cudaError_t e = cudaSuccess;
   auto set = [&](auto fn, int bytes) {
@@ -277,16 +298,13 @@ inline cudaError_t tc_block_set_smem() {
   set(tc_qkv_kernel, tc::PLayout<kTcBN, true>::kSmemBytes);
   set(tc_qkv_tile_kernel<64, kTcCompact>, tc::Layout<64, true, kTcCompact>::kSmemBytes);
   set(tc_qkv_tile_kernel<128, tc::kStageBudget>, tc::Layout<128, true>::kSmemBytes);
-  set(tc_gu_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
-  set(tc_gu_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
-  set(tc_gu_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
-  set(tc_gu_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
-  set(tc_gu_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
-  set(tc_resid_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
-  set(tc_resid_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
-  set(tc_resid_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
-  set(tc_resid_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
-  set(tc_resid_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
+  auto both = [&](auto bn, auto budget) {
+    constexpr int BN = decltype(bn)::value, B = decltype(budget)::value;
+    set(tc_gu_kernel<BN, kHilo, B>, tc::Layout<BN, kHilo, B>::kSmemBytes);
+    set(tc_resid_kernel<BN, kHilo, B>, tc::Layout<BN, kHilo, B>::kSmemBytes);
+  };
+  for (int pitch : {64, 128, 176, 256})
+    for (int rows : {16, kTcCompactRows + 16}) tc_pick<kHilo>(pitch, rows, both);
   return e;
 }
 
@@ -330,39 +348,40 @@ inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t*
 // gate/up -> SwiGLU into the down product's operand.  gu: the interleaved gate/up matrix
 // (2F rows); xn: the normalised operand of Rtc rows.  The tile pitch over the packed rows fills
 // the SMs with one tile per CTA (three tiles of 176 / 176 / 160 rows at 512 rows, F = 3072).
-inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, uint8_t* act_t, int Rtc, const int* nrows, int F,
-                         int H, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
+template <bool kHilo>
+inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, const uint8_t* xn_lo, uint8_t* act_t, uint8_t* act_lo, int Rtc,
+                         const int* nrows, int F, int H, int* err, unsigned long long wait_ns, int n_sm, bool pdl,
+                         cudaStream_t s) {
   const int pitch = tc::tile_pitch(2 * F, Rtc, n_sm);
-  const tc::GemmArgs g{gu, xn, nullptr, 2 * F, Rtc, H, nrows, err, wait_ns, pdl, pitch};
+  const tc::GemmArgs g{gu, xn, xn_lo, 2 * F, Rtc, H, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, 2 * F / tc::kBM);
-  auto go = [&](auto kernel, int smem) { tc::launch(pdl, kernel, grid, dim3(kGuThreads), smem, s, g, act_t, Rtc, nrows); };
-  if (pitch <= 64) go(tc_gu_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
-  else if (pitch <= 128 && Rtc <= kTcCompactRows) go(tc_gu_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
-  else if (pitch <= 128) go(tc_gu_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
-  else if (pitch <= 176) go(tc_gu_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
-  else go(tc_gu_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
+  tc_pick<kHilo>(pitch, Rtc, [&](auto bn, auto budget) {
+    constexpr int BN = decltype(bn)::value, B = decltype(budget)::value;
+    tc::launch(pdl, tc_gu_kernel<BN, kHilo, B>, grid, dim3(kGuThreads), tc::Layout<BN, kHilo, B>::kSmemBytes, s, g, act_t,
+               act_lo, Rtc, nrows);
+  });
 }
 
 // Wo or down (A = w: H rows of K, B = act: Rtc rows) -> tc_resid_split(Rtc) partial sums.
 // T column tiles x (H / 128) weight tiles x z splits fill the SMs with one tile per CTA
 // (H = 1024: T = 4 of 128 packed rows at 512 rows, 128 CTAs; T = 3 of 48 / 48 / 32 at 128
 // rows, 144 CTAs).
-inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, float* part, int H, int Rtc, int K, const int* nrows,
-                            int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
+template <bool kHilo>
+inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, const uint8_t* act_lo, float* part, int H, int Rtc, int K,
+                            const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
   const int n_mt = H / tc::kBM, units = Rtc / 16, z = tc_resid_split(Rtc);
   int T = n_sm / (n_mt * z);
   if (T < 1) T = 1;
   if (T < (Rtc + 255) / 256) T = (Rtc + 255) / 256;
   if (T > units) T = units;
   const int pitch = (units + T - 1) / T * 16;
-  const tc::GemmArgs g{w, act, nullptr, H, Rtc, K, nrows, err, wait_ns, pdl, pitch};
+  const tc::GemmArgs g{w, act, act_lo, H, Rtc, K, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, n_mt, z);
-  auto go = [&](auto kernel, int smem) { tc::launch(pdl, kernel, grid, dim3(kResidThreads), smem, s, g, part, H, Rtc, nrows); };
-  if (pitch <= 64) go(tc_resid_kernel<64, kTcCompact>, tc::Layout<64, false, kTcCompact>::kSmemBytes);
-  else if (pitch <= 128 && Rtc <= kTcCompactRows) go(tc_resid_kernel<128, kTcCompact>, tc::Layout<128, false, kTcCompact>::kSmemBytes);
-  else if (pitch <= 128) go(tc_resid_kernel<128, tc::kStageBudget>, tc::Layout<128>::kSmemBytes);
-  else if (pitch <= 176) go(tc_resid_kernel<176, tc::kStageBudget>, tc::Layout<176>::kSmemBytes);
-  else go(tc_resid_kernel<256, tc::kStageBudget>, tc::Layout<256>::kSmemBytes);
+  tc_pick<kHilo>(pitch, Rtc, [&](auto bn, auto budget) {
+    constexpr int BN = decltype(bn)::value, B = decltype(budget)::value;
+    tc::launch(pdl, tc_resid_kernel<BN, kHilo, B>, grid, dim3(kResidThreads), tc::Layout<BN, kHilo, B>::kSmemBytes, s, g,
+               part, H, Rtc, nrows);
+  });
 }
 
 }  // namespace

@@ -541,14 +541,14 @@ mcd_status mcd_create(const mcd_config* cfg, void* cuda_stream, mcd_ctx** out) {
   if ((e = ctx_alloc(c, &p.tree_cand, sizeof(int) * kMaxDraft * kMaxTreeRank)) != cudaSuccess)
     return fail(cuda_status(e));
   if (k.draft_mode == MCD_DRAFT_TREE) {       // until mcd_set_tree: the chain of K rank-0 nodes
-    p.tree_n = k.draft_len;
-    p.tree_maxd = k.draft_len;
+    p.tree.n = k.draft_len;
+    p.tree.maxd = k.draft_len;
     for (int i = 0; i < k.draft_len; ++i) {
-      p.tree_parent[i] = (signed char)(i - 1);
-      p.tree_rank[i] = 0;
-      p.tree_depth[i] = (signed char)(i + 1);
-      p.tree_m[i] = 1;
-      p.tree_anc[i] = (2ull << i) - 1ull;
+      p.tree.parent[i] = (signed char)(i - 1);
+      p.tree.rank[i] = 0;
+      p.tree.depth[i] = (signed char)(i + 1);
+      p.tree.m[i] = 1;
+      p.tree.anc[i] = (2ull << i) - 1ull;
     }
   }
   if (cudaMemsetAsync(p.err, 0, sizeof(int), c->stream) != cudaSuccess) return fail(MCD_ERR_CUDA);
@@ -561,6 +561,13 @@ mcd_status mcd_create(const mcd_config* cfg, void* cuda_stream, mcd_ctx** out) {
   if (k.max_streams > kMaxStreams || batch_rows(p, k.max_streams) > kMaxCols || batch_prefers(p, k.max_streams)) {
     mcd_status bs = batch_create(p, k.max_streams, &c->batch);
     if (bs != MCD_OK) return fail(bs);
+  } else if (batch_tree_supported(p)) {
+    // larger trees run on the batched kernels; without memory for their buffers the frame
+    // kernel takes every tree
+    if (batch_create(p, 1, &c->batch) != MCD_OK) {
+      c->batch = nullptr;
+      (void)cudaGetLastError();
+    }
   }
   *out = c;
   return MCD_OK;
@@ -728,8 +735,11 @@ mcd_status mcd_decode_frames(mcd_ctx* c, int32_t n_streams, const uint32_t* stre
                              mcd_frame_stats* stats) {
   if (!c || !codes_out) return MCD_ERR_INVALID_ARG;
   if (!c->weights_loaded) return MCD_ERR_STATE;
+  // (a tree call's stage stamps come from the frame kernel)
+  const bool tree_batch = c->batch && n_streams == 1 && batch_tree_supported(c->fp) && batch_tree_prefers(c->fp.tree.n) &&
+                          !c->fp.timeline;
   if (n_streams > kMaxStreams || batch_rows(c->fp, n_streams) > kMaxCols ||
-      (c->batch && batch_prefers(c->fp, n_streams))) {
+      (c->batch && batch_prefers(c->fp, n_streams)) || tree_batch) {
     // many streams: the batched GEMM path (one CUDA graph launch per frame)
     const FrameParams& p = c->fp;
     if (!c->batch || n_streams > c->cfg.max_streams) return MCD_ERR_INVALID_ARG;
@@ -737,6 +747,14 @@ mcd_status mcd_decode_frames(mcd_ctx* c, int32_t n_streams, const uint32_t* stre
     if (p.C0V > 0 && !c0) return MCD_ERR_INVALID_ARG;
     if (p.C0V == 0 && !c0_emb) return MCD_ERR_INVALID_ARG;
     c->frame_begun = false;
+    if (tree_batch) {            // as begin_frame leaves a context: 16-byte rows, the frame's counters
+      if ((reinterpret_cast<uintptr_t>(cond) & 15u) || (reinterpret_cast<uintptr_t>(c0_emb) & 15u))
+        return MCD_ERR_INVALID_ARG;
+      c->fp.stream_ids[0] = stream_ids[0];
+      c->fp.frame_ids[0] = frame_idx[0];
+      c->fp.S = 1;
+      c->frame_begun = true;
+    }
     return batch_decode(c->batch, p, c->stream, n_streams, stream_ids, frame_idx, cond, c0, c0_emb, codes_out, stats,
                         p.trace);
   }
@@ -817,15 +835,15 @@ mcd_status mcd_set_tree(mcd_ctx* c, int32_t n_nodes, const int32_t* parent, cons
     m[depth[i] - 1] = std::max(m[depth[i] - 1], rank[i] + 1);
     maxd = std::max(maxd, depth[i]);
   }
-  p.tree_n = n_nodes;
-  p.tree_maxd = maxd;
+  p.tree.n = n_nodes;
+  p.tree.maxd = maxd;
   for (int i = 0; i < n_nodes; ++i) {
-    p.tree_parent[i] = (signed char)parent[i];
-    p.tree_rank[i] = (signed char)rank[i];
-    p.tree_depth[i] = (signed char)depth[i];
-    p.tree_anc[i] = (parent[i] < 0 ? 0ull : p.tree_anc[parent[i]]) | (1ull << i);
+    p.tree.parent[i] = (signed char)parent[i];
+    p.tree.rank[i] = (signed char)rank[i];
+    p.tree.depth[i] = (signed char)depth[i];
+    p.tree.anc[i] = (parent[i] < 0 ? 0ull : p.tree.anc[parent[i]]) | (1ull << i);
   }
-  for (int d = 0; d < kMaxDraft; ++d) p.tree_m[d] = m[d];
+  for (int d = 0; d < kMaxDraft; ++d) p.tree.m[d] = m[d];
   return MCD_OK;
 }
 

@@ -1,5 +1,5 @@
 // Batched decoding of many independent streams (up to 128 streams, 512 packed rows per
-// call): the per-frame draft-and-verify loop of arXiv 2609.37007 (Sec. 2.2, Fig. 3) for
+// call), and of one stream's larger sparse trees: the per-frame draft-and-verify loop of arXiv 2609.37007 (Sec. 2.2, Fig. 3) for
 // every stream at once, with the rows of all unfinished streams re-packed every call.
 //
 // With hundreds of rows per call the weight matrices are multiplied as real GEMMs, so this
@@ -32,6 +32,7 @@
 #include "mcd_sampler.cuh"
 #include "mcd_tcgemm.cuh"
 #include "mcd_tcops.cuh"
+#include "mcd_tree.cuh"
 
 namespace mcd {
 
@@ -87,6 +88,7 @@ struct BatchFrame {
   int* codes_out;
   mcd_frame_stats* stats;
   uint8_t* trace;
+  TreeDef tree;           // TREE mode (one stream)
 };
 
 struct BatchBufs {
@@ -110,6 +112,8 @@ struct BatchBufs {
   uint8_t* xn_lo;
   uint8_t* att_t;         // attention outputs
   uint8_t* act_t;         // SwiGLU outputs
+  uint8_t *att_lo, *act_lo;   // TREE mode: their low halves
+  float* tree_q;          // TREE mode: [R][NH * D] normalised, rotated queries
   float* part;            // [kTcSplit][Rtc][H] k-split partial sums of the residual products
   int Qcap;               // LM-head operand rows: every (row, j) pair, groups padded per head
   uint8_t* hq_hi;         // LM-head operand (normalised rows of the pairs, grouped by head)
@@ -850,7 +854,14 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParam
   if ((int)blockIdx.x >= b.info->n_pairs) return;
   const int e = b.pairs[blockIdx.x], r = e >> 3, j = e & 7;
   const int greedy = (j > 0 && p.draft_mode == MCD_DRAFT_GREEDY) ? 1 : 0;
-  TopkRec* recs = b.recs + (size_t)(b.info->call & 1) * b.R * kRecSlots;
+  const int call = b.info->call;
+  TopkRec* recs = b.recs + (size_t)(call & 1) * b.R * kRecSlots;
+  if (p.draft_mode == MCD_DRAFT_TREE && j == 0 && b.frame->trace && call < kMaxCalls) {
+    // a tree call's verify logits, one row per CTA (the chain's are copied by its acceptance)
+    uint8_t* tb = b.frame->trace + sizeof(mcd_call_trace) * kMaxCalls + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4 +
+                  sizeof(mcd_tree_trace) * kMaxCalls;
+    copy_logits(reinterpret_cast<float*>(tb) + ((size_t)call * kMaxTreeRows + r) * p.V, b.logits + (size_t)r * kRecSlots * p.V, p.V);
+  }
   block_topk(b.logits + ((size_t)r * kRecSlots + j) * p.V, p.V, p.top_k, p.T, greedy, ts,
              recs + (size_t)r * kRecSlots + j);
 }
@@ -1021,6 +1032,237 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FramePar
   if (threadIdx.x == 0) batch_call_end(p, b, loop, call, a_new < p.P);
 }
 
+// ------------------------------------------------------------------------------------
+// tree calls: one stream, every row of the call (up to 65) in one pass
+// ------------------------------------------------------------------------------------
+// Row m >= 1 of a tree call is node m - 1 (the nodes whose candidates exist, a prefix of the
+// breadth-first list), row 0 the last emitted code; the first call feeds [cond, c0].  K / V of
+// the call's rows go to cache slots kMaxPos + m (row 0: its position) until the acceptance
+// step moves the kept ones.  Every product takes hi + lo operands.
+__device__ __forceinline__ int tree_row_slot(const DevState* st, int r) {
+  return st->pos0 == 0 ? r : (r == 0 ? st->pos0 : kMaxPos + r);
+}
+
+// pack: one thread per row.
+__global__ void __launch_bounds__(128) batch_tree_pack_kernel(FrameParams p, BatchBufs b) {
+  __shared__ int s_head[16], s_hcur[16], s_rows, s_pairs;
+  const BatchFrame* fa = b.frame;
+  const TreeDef& tree = fa->tree;
+  const DevState* st = p.st;
+  const int r = threadIdx.x;
+  if (r < 16) s_head[r] = 0;
+  if (r == 0) s_rows = s_pairs = 0;
+  __syncthreads();
+  const int a = st->a, pos0 = st->pos0;
+  int pos = -1, id = -1;
+  if (!st->done) {
+    if (pos0 == 0) {
+      if (r < 2) {
+        pos = r;
+        id = r == 0 ? -1 : st->codes[0];
+      }
+    } else if (r == 0) {
+      pos = pos0;
+      id = st->codes[a];
+    } else if (r <= tree.n && tree.depth[r - 1] <= st->n_d && a + tree.depth[r - 1] < p.P) {
+      const int d = tree.depth[r - 1];
+      pos = pos0 + d;
+      id = p.tree_cand[(d - 1) * kMaxTreeRank + tree.rank[r - 1]];
+    }
+  }
+  const int kn = pos >= 1 ? min(p.K, p.P - pos) : -1;         // draft heads of the row (-1: none at all)
+  if (pos >= 0) {
+    atomicAdd(&s_rows, 1);
+    BatchRow row;
+    row.s = 0;
+    row.n = r;
+    row.pos = pos;
+    if (pos == 0 || (pos == 1 && p.C0V == 0)) {
+      row.src = reinterpret_cast<const uint8_t*>(pos == 0 ? fa->cond : fa->c0emb);
+      row.f32 = 1;
+    } else {
+      const int table = pos - 1;
+      if (id < 0 || id >= (table == 0 ? p.C0V : p.V)) {
+        atomicCAS(p.err, 0, (int)MCD_ERR_INVALID_ARG);
+        id = 0;
+      }
+      row.src = p.embed + (long long)table * p.embed_stride + (long long)id * p.H * 2;
+      row.f32 = 0;
+    }
+    row.id = id;
+    b.rows[r] = row;
+    for (int j = 0; j <= kn; ++j) atomicAdd(&s_head[pos + j], 1);
+  }
+  __syncthreads();
+  if (r == 0) {
+    int off = 0;
+    for (int P = 0; P < 16; ++P) {
+      b.info->head_rows[P] = s_head[P];
+      b.info->head_off[P] = off;
+      s_hcur[P] = off;
+      off += s_head[P];
+    }
+    b.info->M = s_rows;
+    b.info->n_pairs = off;
+    const int call = b.info->next_call;
+    b.info->call = call;
+    b.info->next_call = call + 1;
+  }
+  __syncthreads();
+  for (int j = 0; j <= kn; ++j) {
+    b.pairs[atomicAdd(&s_pairs, 1)] = (r << 3) | j;
+    b.head_list[atomicAdd(&s_hcur[pos + j], 1)] = (r << 3) | j;
+  }
+}
+
+// QK-norm + RoPE of every row's query and key heads; K and V to the row's cache slot, the
+// queries to tree_q.  One warp per (row, vector), lane holding dims lane + 32 i.
+__global__ void __launch_bounds__(256) batch_tree_rope_kernel(FrameParams p, BatchBufs b, int layer) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
+  const int vecs = p.NH + 2 * p.NKV, w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int r = w / vecs, vi = w - r * vecs;
+  if (r >= b.info->M) return;
+  const int NH = p.NH, D = p.D, nd = D >> 5;
+  const int kind = vi < NH ? 0 : (vi < NH + p.NKV ? 1 : 2), h = kind == 0 ? vi : (kind == 1 ? vi - NH : vi - NH - p.NKV);
+  const float* src = b.qkv + (size_t)r * p.qkv_dim + vi * D;
+  float x[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = i < nd ? __ldcg(src + lane + 32 * i) : 0.f;
+  if (kind < 2) {
+    if (p.qk_norm) {
+      float ss = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ss += x[i] * x[i];
+#pragma unroll
+      for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
+      const float scl = rsqrtf(ss / (float)D + p.eps);
+      const float* gg = (kind == 0 ? p.q_norm : p.k_norm) + (size_t)layer * D;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < nd) x[i] = x[i] * scl * __ldg(gg + lane + 32 * i);
+    }
+    const float2* rope = p.rope + (size_t)b.rows[r].pos * (D >> 1);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (i < nd / 2) {
+        const float2 cs = __ldg(rope + lane + 32 * i);
+        const float e = x[i], f = x[i + nd / 2];
+        x[i] = e * cs.x - f * cs.y;
+        x[i + nd / 2] = f * cs.x + e * cs.y;
+      }
+    }
+  }
+  float* dst = kind == 0 ? b.tree_q + ((size_t)r * NH + h) * D
+                         : (kind == 1 ? p.kcache : p.vcache) +
+                               (((size_t)layer * p.NKV + h) * p.kv_slots + tree_row_slot(p.st, r)) * D;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (i < nd) dst[lane + 32 * i] = x[i];
+}
+
+// Attention of one (row, query head) per warp over the cache: the committed positions, row 0, the
+// row's ancestors and itself (the sparse tree mask of Fig. 2); the first call is causal.  At
+// most 15 + 1 + 7 keys: lane j holds key j's slot and score, four dims per lane of every K and V
+// row, eight rows in flight.  Outputs as hi + lo halves to the Wo product's operand.
+__global__ void __launch_bounds__(256) batch_tree_attn_kernel(FrameParams p, BatchBufs b, int layer) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int NH = p.NH, D = p.D, r = w / NH, h = w - r * NH, g = h / (NH / p.NKV);
+  if (r >= b.info->M) return;
+  const DevState* st = p.st;
+  const int pos0 = st->pos0;
+  const unsigned long long anc = pos0 > 0 && r > 0 ? b.frame->tree.anc[r - 1] : 0ull;
+  const int nk = pos0 == 0 ? r + 1 : pos0 + 1 + __popcll(anc);
+  int slot = lane;                                   // committed positions, row 0's, the first call's rows
+  if (pos0 > 0 && lane > pos0 && lane < nk) {        // ancestor number lane - pos0 - 1, in tree order
+    unsigned long long m = anc;
+    for (int i = pos0 + 1; i < lane; ++i) m &= m - 1ull;
+    slot = kMaxPos + __ffsll((long long)m);          // node i is row i + 1
+  }
+  const size_t head_off = ((size_t)layer * p.NKV + g) * p.kv_slots * D;
+  const int d0 = 4 * lane;
+  const bool own = d0 < D;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 q = own ? __ldcg(reinterpret_cast<const float4*>(b.tree_q + ((size_t)r * NH + h) * D + d0)) : z;
+  float score = -INFINITY;
+  for (int jb = 0; jb < nk; jb += 8) {
+    float4 kv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int sl = __shfl_sync(0xFFFFFFFFu, slot, (jb + i) & 31);
+      kv[i] = jb + i < nk && own ? __ldcg(reinterpret_cast<const float4*>(p.kcache + head_off + (size_t)sl * D + d0)) : z;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float s = (q.x * kv[i].x + q.y * kv[i].y) + (q.z * kv[i].z + q.w * kv[i].w);
+#pragma unroll
+      for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      if (lane == jb + i && jb + i < nk) score = s * rsqrtf((float)D);
+    }
+  }
+  float mx = score;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
+  const float e = lane < nk ? __expf(score - mx) : 0.f;
+  float sum = e;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+  const float pj = e / sum;
+  float4 acc = z;
+  for (int jb = 0; jb < nk; jb += 8) {
+    float4 kv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int sl = __shfl_sync(0xFFFFFFFFu, slot, (jb + i) & 31);
+      kv[i] = jb + i < nk && own ? __ldcg(reinterpret_cast<const float4*>(p.vcache + head_off + (size_t)sl * D + d0)) : z;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float wgt = __shfl_sync(0xFFFFFFFFu, pj, (jb + i) & 31);
+      if (jb + i < nk) {
+        acc.x += wgt * kv[i].x;
+        acc.y += wgt * kv[i].y;
+        acc.z += wgt * kv[i].z;
+        acc.w += wgt * kv[i].w;
+      }
+    }
+  }
+  if (own) {
+    const int f = h * D + d0;
+    const size_t off = tc::sw128_offset(b.Rtc, r, f >> 6, (f & 63) >> 3) + (f & 7) * 2;
+    const uint2 hi = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
+    *reinterpret_cast<uint2*>(b.att_t + off) = hi;
+    *reinterpret_cast<uint2*>(b.att_lo + off) = make_uint2(
+        pack_bf16x2(acc.x - bf16_lo_f32(hi.x), acc.y - bf16_hi_f32(hi.x)),
+        pack_bf16x2(acc.z - bf16_lo_f32(hi.y), acc.w - bf16_hi_f32(hi.y)));
+  }
+}
+
+// Acceptance of a tree call (mcd_tree.cuh) and the while node's condition.  heads_read counts a
+// call of more than 32 rows as the passes of 32 rows the frame kernel runs it in.
+__global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
+  tc::pdl_wait();
+  tc::pdl_trigger();
+  __shared__ DevState st;
+  __shared__ int cand[kMaxDraft][kMaxTreeRank];
+  const int call = b.info->call;
+  for (int i = threadIdx.x; i < (int)(sizeof(DevState) / 4); i += kConsumerThreads)
+    reinterpret_cast<int*>(&st)[i] = __ldcg(reinterpret_cast<const int*>(p.st) + i);
+  for (int i = threadIdx.x; i < kMaxDraft * kMaxTreeRank; i += kConsumerThreads)
+    cand[i / kMaxTreeRank][i % kMaxTreeRank] = __ldcg(p.tree_cand + i);
+  __syncthreads();
+  if (!st.done) {
+    const BatchFrame* fa = b.frame;
+    const int heads = (min(p.P, st.top_pos + p.K) - st.a) * ((st.n_rows + kMaxCols - 1) / kMaxCols);
+    const TreeCall t{&fa->tree, &st, cand, b.recs + (size_t)(call & 1) * b.R * kRecSlots, b.logits, heads,
+                     fa->stream_ids[0], fa->frame_ids[0], fa->codes_out, fa->stats, fa->trace};
+    accept_tree_call(p, t);
+  }
+  if (threadIdx.x == 0) batch_call_end(p, b, loop, call, !__ldcg(&p.st->done));
+}
+
 __global__ void batch_begin_kernel(FrameParams p, BatchBufs b) {
   const BatchFrame* fa = b.frame;
   for (int s = threadIdx.x; s < fa->S; s += blockDim.x) init_stream_state(p.st + s, p.C0V > 0 ? fa->c0[s] : -1);
@@ -1042,6 +1284,7 @@ struct BatchState {
   BatchFrame host_frame;
   int max_streams = 0;
   bool use_tc = false;        // QKV, Wo, gate/up and down on the tcgen05 GEMM
+  bool tree = false;          // TREE mode: one stream's tree calls
   TcWeights tw;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -1079,16 +1322,29 @@ bool batch_prefers(const FrameParams& p, int n_streams) {
          p.draft_mode != MCD_DRAFT_TREE;
 }
 
+// A tree call of 1 + nodes rows is one pass here; the persistent frame kernel pays for every row and
+// starts a new pass every 32.  Measured per call, frame kernel / batched (us): 12 nodes 231 / 269,
+// 16 nodes 270 / 271, 20 nodes 298 / 277, 31 nodes 330 / 281, 32 nodes 459 / 281, 64 nodes 737 / 293.
+// Every operand is hi + lo here, at any row count (the frame kernel's are single bf16 values above
+// 16 rows: 1.7e-3 off a 64-bit evaluation at 32 nodes against 3.6e-6).
+bool batch_tree_supported(const FrameParams& p) {
+  return p.draft_mode == MCD_DRAFT_TREE && tc_block_supported(p) && p.V % tc::kBM == 0;
+}
+bool batch_tree_prefers(int nodes) { return nodes >= kBatchMinTreeNodes; }
+
 mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out) {
   *out = nullptr;
   BatchState* bs = new BatchState();
   bs->max_streams = max_streams;
+  bs->tree = p.draft_mode == MCD_DRAFT_TREE;
   auto fail = [&](mcd_status s) {
     batch_destroy(bs);
     return s;
   };
   BatchBufs& b = bs->b;
-  const int R = (batch_rows(p, max_streams) + kGN - 1) / kGN * kGN;
+  memset(&b, 0, sizeof(b));
+  const int rows = bs->tree ? kMaxTreeRows : batch_rows(p, max_streams);
+  const int R = (rows + kGN - 1) / kGN * kGN;
   b.R = R;
   cudaError_t e;
 #define BATCH_ALLOC(ptr, bytes)                                                        \
@@ -1110,8 +1366,13 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
   BATCH_ALLOC(b.recs, sizeof(TopkRec) * 2 * R * kRecSlots);
   bs->use_tc = tc_block_supported(p);
   if (bs->use_tc) {
-    const int Rtc = (R + 127) / 128 * 128;
+    const int Rtc = bs->tree ? tc_operand_rows(rows, p.qkv_dim, p.n_cta) : (R + 127) / 128 * 128;
     b.Rtc = Rtc;
+    if (bs->tree) {
+      BATCH_ALLOC(b.att_lo, (size_t)Rtc * p.NH * p.D * 2);
+      BATCH_ALLOC(b.act_lo, (size_t)Rtc * p.F * 2);
+      BATCH_ALLOC(b.tree_q, sizeof(float) * (size_t)R * p.NH * p.D);
+    }
     BATCH_ALLOC(b.xn_hi, (size_t)Rtc * p.H * 2);
     BATCH_ALLOC(b.xn_lo, (size_t)Rtc * p.H * 2);
     BATCH_ALLOC(b.att_t, (size_t)Rtc * p.NH * p.D * 2);
@@ -1136,7 +1397,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemHilo) != cudaSuccess)
       return fail(MCD_ERR_CUDA);
   if (bs->use_tc &&
-      (tc_block_set_smem<false>() != cudaSuccess ||
+      ((bs->tree ? tc_block_set_smem<true>() : tc_block_set_smem<false>()) != cudaSuccess ||
        cudaFuncSetAttribute(tc_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             tc::Layout<kHeadTileMax, true>::kSmemBytes) != cudaSuccess))
     return fail(MCD_ERR_CUDA);
@@ -1176,6 +1437,19 @@ static int split_k(dim3 grid, int K, int n_sm) {
   int z = 1;
   while (ctas * z < 2 * n_sm && chunks / (2 * z) >= 4) z *= 2;
   return z;
+}
+
+// Final RMSNorm -> LM heads on the tensor cores, tiles grouped by head.
+static void enqueue_heads(const FrameParams& p, const BatchState* bs, cudaStream_t s) {
+  const BatchBufs& b = bs->b;
+  const int R = b.R, L = p.L, H = p.H;
+  const dim3 blk(256);
+  tc::launch(false, tc_heads_operand_kernel, dim3(512), blk, 0, s, b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
+                                             b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
+  const tc::GemmArgs g{nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns, false, 0};
+  tc::launch(false, tc_heads_kernel, dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
+                 tc::Layout<kHeadTileMax, true>::kSmemBytes, s, g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
+                                                                    p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
 }
 
 // Every kernel of one call, in stream order on `s`.
@@ -1265,13 +1539,8 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
       batch_rowss_kernel<<<R / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * l + 2) * R, b.info);
     }
   }
-  if (bs->tw.heads) {   // final RMSNorm -> LM heads on the tensor cores, tiles grouped by head
-    tc::launch(false, tc_heads_operand_kernel, dim3(512), blk, 0, s, b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
-                                               b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
-    const tc::GemmArgs g{nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns, false, 0};
-    tc::launch(false, tc_heads_kernel, dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
-                   tc::Layout<kHeadTileMax, true>::kSmemBytes, s, g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
-                                                                      p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
+  if (bs->tw.heads) {
+    enqueue_heads(p, bs, s);
   } else {   // final RMSNorm -> LM heads, one grid slice per head
     GemmArgs a = gemm_args(p, b);
     a.W = p.w_head;
@@ -1287,6 +1556,36 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
   }
   tc::launch(false, batch_topk_kernel, dim3(R * (p.K + 1)), dim3(kConsumerThreads), 0, s, p, b);
   tc::launch(false, batch_accept_kernel, dim3(bs->max_streams), dim3(kConsumerThreads), 0, s, p, b, loop);
+  return cudaGetLastError();
+}
+
+// Every kernel of one tree call.
+static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs, const BatchLoop& loop, cudaStream_t s) {
+  const BatchBufs& b = bs->b;
+  const int R = b.R, L = p.L, H = p.H, Rtc = b.Rtc, qd = p.NH * p.D, z = tc_resid_split(Rtc);
+  const dim3 blk(256);
+  const bool pdl = loop.valid != 0;
+  const int* M = &b.info->M;
+  batch_tree_pack_kernel<<<1, 128, 0, s>>>(p, b);
+  batch_embed_kernel<<<kMaxTreeRows, blk, 0, s>>>(p, b);
+  tc_norm_operand_kernel<<<64, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, M, Rtc, b.xn_hi, b.xn_lo);
+  for (int l = 0; l < L; ++l) {
+    const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
+    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    batch_tree_rope_kernel<<<(kMaxTreeRows * (p.NH + 2 * p.NKV) + 7) / 8, blk, 0, s>>>(p, b, l);
+    batch_tree_attn_kernel<<<(kMaxTreeRows * p.NH + 7) / 8, blk, 0, s>>>(p, b, l);
+    tc_launch_resid<true>(wl + bs->tw.off.o, b.att_t, b.att_lo, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_resid_norm_kernel<<<kMaxTreeRows, 128, 0, s>>>(b.X, b.part, tc_splits(qd, z), Rtc, H, M, b.ss + (size_t)(2 * l + 1) * R,
+                                                      p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, b.xn_lo);
+    tc_launch_gu<true>(wl + bs->tw.off.gu, b.xn_hi, b.xn_lo, b.act_t, b.act_lo, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid<true>(wl + bs->tw.off.d, b.act_t, b.act_lo, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_resid_norm_kernel<<<kMaxTreeRows, 128, 0, s>>>(b.X, b.part, tc_splits(p.F, z), Rtc, H, M, b.ss + (size_t)(2 * l + 2) * R,
+                                                      l + 1 == L ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi,
+                                                      b.xn_lo);
+  }
+  enqueue_heads(p, bs, s);
+  batch_topk_kernel<<<kMaxTreeRows * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);
+  batch_tree_accept_kernel<<<1, kConsumerThreads, 0, s>>>(p, b, loop);
   return cudaGetLastError();
 }
 
@@ -1320,7 +1619,7 @@ static cudaError_t build_graph(const FrameParams& p, BatchState* bs) {
   np.conditional.type = cudaGraphCondTypeWhile;
   np.conditional.size = 1;
   if ((e = cudaGraphAddNode(&loop_node, bs->graph, &begin, nullptr, 1, &np)) != cudaSuccess) return e;
-  e = capture(np.conditional.phGraph_out[0], [&] { return enqueue_call(p, bs, loop, s); });
+  e = capture(np.conditional.phGraph_out[0], [&] { return (bs->tree ? enqueue_tree_call : enqueue_call)(p, bs, loop, s); });
   if (e != cudaSuccess) return e;
   return cudaGraphInstantiate(&bs->exec, bs->graph, 0);
 }
@@ -1354,6 +1653,7 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
   f.codes_out = codes_out;
   f.stats = stats;
   f.trace = trace;
+  f.tree = p.tree;
   MCD_CHECK(cudaMemcpyAsync(bs->b.frame, &f, sizeof(f), cudaMemcpyHostToDevice, stream));
   if (!unrolled) {
     MCD_CHECK(cudaGraphLaunch(bs->exec, stream));
@@ -1361,7 +1661,7 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
   }
   batch_begin_kernel<<<1, 256, 0, stream>>>(p, bs->b);
   MCD_CHECK(cudaGetLastError());
-  for (int call = 0; call < p.P; ++call) MCD_CHECK(enqueue_call(p, bs, BatchLoop{0, 0}, stream));
+  for (int call = 0; call < p.P; ++call) MCD_CHECK((bs->tree ? enqueue_tree_call : enqueue_call)(p, bs, BatchLoop{0, 0}, stream));
   return MCD_OK;
 }
 

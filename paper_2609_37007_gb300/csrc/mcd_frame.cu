@@ -20,6 +20,7 @@
 #include "mcd_internal.cuh"
 #include "mcd_sampler.cuh"
 #include "mcd_stage.cuh"
+#include "mcd_tree.cuh"
 
 namespace mcd {
 
@@ -513,13 +514,13 @@ __device__ __noinline__ void attention_tree_task(const FrameParams& p, int layer
   const size_t cache_off = ((size_t)layer * p.NKV + g) * p.kv_slots * D;
   const float* qkv = p.qkv;
   const int qoff = h * D, koff = p.NH * D + g * D, voff = p.NH * D + p.NKV * D + g * D;
-  const int nq = hi - lo, dm = min(p.tree_maxd, kMaxPos - 1 - pos0);   // RoPE rows pos0 .. pos0 + dm
+  const int nq = hi - lo, dm = min(p.tree.maxd, kMaxPos - 1 - pos0);   // RoPE rows pos0 .. pos0 + dm
   // ---- key list: row 0 and the union of the queries' ancestor-or-self sets -----------------
   if (tid == 0) {
     unsigned long long U = 0ull;
     for (int n = lo; n < hi; ++n) {
       const int m = row0 + n;
-      const unsigned long long am = m > 0 ? p.tree_anc[m - 1] : 0ull;
+      const unsigned long long am = m > 0 ? p.tree.anc[m - 1] : 0ull;
       qanc[n - lo] = am;
       U |= am;
     }
@@ -548,7 +549,7 @@ __device__ __noinline__ void attention_tree_task(const FrameParams& p, int layer
     const int m = krow[j - pos0];
     return m == 0 ? pos0 : kMaxPos + m;
   };
-  auto row_depth = [&](int m) { return m == 0 ? 0 : (int)p.tree_depth[m - 1]; };
+  auto row_depth = [&](int m) { return m == 0 ? 0 : (int)p.tree.depth[m - 1]; };
   // ---- (A) loads, 16-byte chunks, batches of 8 per thread in flight --------------------------
   {
     const int e_q = nq << cs_shift, e_k = e_q + (nk << cs_shift), e_v = e_k + (nk << cs_shift);
@@ -1233,235 +1234,15 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
   }
 }
 
-// Acceptance step of a tree call (one stream; run by the CTA that finished top-k last).
-// One warp walks the tree from the first row: the children of the current node are tested
-// in rank order, test i keeping its candidate x iff U * S' < 2^53 * W_x, S' being the
-// node's weight sum without the candidates rejected so far (one-hot draft distributions);
-// a kept child continues the walk, otherwise a code is drawn from the remainder (purpose 0)
-// and the call ends.  Then: the next call's candidates (the top-m ids by logit of each
-// draft distribution of the last visited row), the kept nodes' K / V moved to their
-// positions, the state update, the trace and the release of the next call.
+// Acceptance step of a tree call (mcd_tree.cuh) by the CTA that finished top-k last, then the
+// release of the next call.
 __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
   Smem sm = smem_layout(mcd_dyn_smem);
   const CallInfo* ci = sm.ci;
-  const DevState& st0 = ci->st[0];
-  const int a = st0.a, pos0 = st0.pos0, n_rows = st0.n_rows, round = st0.round;
-  const unsigned sid = p.stream_ids[0], fid = p.frame_ids[0];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TopkRec* cur = p.topk;                       // every row's records, buffer 0
-  __shared__ int t_emit[kMaxDraft + 1], t_path[kMaxDraft + 1], t_path_row[kMaxDraft + 1], t_res[4];
-  __shared__ int t_next[kMaxDraft][kMaxTreeRank];
-  if (warp == 0) {
-    int node = -1, row = st0.first_head_row, n_emit = 0, plen = 0, tests = 0;
-    while (true) {
-      const int s = a + 1 + plen;                     // code position of the node's children
-      const TopkRec* pr = cur + (size_t)row * (kMaxDraft + 1);
-      unsigned long long S_rem = pr->S;
-      int rej[kMaxTreeRank];
-      int n_rej = 0, kept = -1, kx = -1;
-      if (pos0 > 0) {
-        for (int r = 0; r < kMaxTreeRank && kept < 0; ++r) {
-          int ch = -1;
-          for (int k = 0; k < p.tree_n; ++k)
-            if (p.tree_parent[k] == node && p.tree_rank[k] == r) ch = k;
-          if (ch < 0 || a + p.tree_depth[ch] > p.P) continue;
-          const int x = ci->tcand[p.tree_depth[ch] - 1][r];
-          const unsigned long long W = warp_weight(pr, x);
-          const uint32_t purpose = n_rej == 0 ? (uint32_t)PURPOSE_ACCEPT : kPurposeSibling + (uint32_t)n_rej;
-          const unsigned long long U = uniform_U(p.seed, sid, fid, round, s, purpose);
-          ++tests;
-          if (W > 0 && lt128(mul64(U, S_rem), shl53(W))) {
-            kept = ch;
-            kx = x;
-          } else {
-            rej[n_rej++] = x;
-            S_rem -= W;
-          }
-        }
-      }
-      if (kept >= 0) {
-        // rows are the first nodes in tree order: node i was fed at row i + 1 if it exists
-        const int kr = kept + 1 < n_rows ? kept + 1 : -1;
-        if (lane == 0) {
-          t_emit[n_emit] = kx;
-          t_path[plen] = kept;
-          t_path_row[plen] = kr;
-        }
-        ++n_emit;
-        ++plen;
-        if (s == p.P || kr < 0) break;                // the last position: nothing follows
-        node = kept;
-        row = kr;
-        continue;
-      }
-      if (s <= p.P) {
-        const int x = warp_draw_excluding(pr, rej, n_rej, S_rem, uniform_U(p.seed, sid, fid, round, s, PURPOSE_TARGET));
-        if (lane == 0) t_emit[n_emit] = x;
-        ++n_emit;
-      }
-      break;
-    }
-    if (lane == 0) {
-      t_res[0] = n_emit;
-      t_res[1] = plen;
-      t_res[2] = row;
-      t_res[3] = tests;
-    }
-  }
-  consumer_sync();
-  const int n_emit = t_res[0], plen = t_res[1], drow = t_res[2];
-  const int a_new = a + n_emit, n_next = min(p.tree_maxd, p.P - a_new);
-  // next candidates: warp j - 1 ranks the draft distribution of depth j of row drow (the
-  // record's ids with their fp32 logits; largest logit first, ties to the lower id)
-  for (int j = 1 + warp; j <= n_next; j += kConsumerWarps) {
-    const TopkRec* dr = cur + (size_t)drow * (kMaxDraft + 1) + j;
-    const float* lg = p.logits + ((size_t)drow * (kMaxDraft + 1) + j) * p.V;
-    unsigned long long key[kDrawPerLane];
-#pragma unroll
-    for (int e = 0; e < kDrawPerLane; ++e) {
-      const int i = lane * kDrawPerLane + e;
-      key[e] = 0ull;
-      if (i < dr->n) {
-        const int id = dr->ids[i];
-        key[e] = ((unsigned long long)f32_key(__ldcg(lg + id)) << 32) | (0xFFFFFFFFu - (uint32_t)id);
-      }
-    }
-    for (int r = 0; r < p.tree_m[j - 1]; ++r) {
-      unsigned long long best = 0ull;
-#pragma unroll
-      for (int e = 0; e < kDrawPerLane; ++e) best = key[e] > best ? key[e] : best;
-#pragma unroll
-      for (int off = 16; off; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-        best = o > best ? o : best;
-      }
-#pragma unroll
-      for (int e = 0; e < kDrawPerLane; ++e)
-        if (key[e] == best) key[e] = 0ull;
-      if (lane == 0) t_next[j - 1][r] = best ? (int)(0xFFFFFFFFu - (uint32_t)(best & 0xFFFFFFFFull)) : -1;
-    }
-  }
-  // the kept nodes' keys and values: slot kMaxPos + row -> position a + 2 + t
-  {
-    int n_mv = 0;
-    for (int t = 0; t < plen; ++t) n_mv += t_path_row[t] >= 0 ? 1 : 0;
-    const int D4 = p.D >> 2, per = p.L * p.NKV * n_mv * D4;
-    for (int i = threadIdx.x; i < 2 * per; i += kConsumerThreads) {
-      const bool isv = i >= per;
-      const int k = isv ? i - per : i;
-      const int d4 = k % D4, t = (k / D4) % n_mv, lg = k / (D4 * n_mv);   // lg = layer * NKV + kv head
-      float* base = (isv ? p.vcache : p.kcache) + (size_t)lg * p.kv_slots * p.D;
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(base + (size_t)(kMaxPos + t_path_row[t]) * p.D) + d4);
-      reinterpret_cast<float4*>(base + (size_t)(a + 2 + t) * p.D)[d4] = v;
-    }
-  }
-  consumer_sync();
-  // state of the next call
-  __shared__ int t_nvalid, t_maxd;
-  if (threadIdx.x == 0) {
-    int nv = 0, md = 0;
-    for (int i = 0; i < p.tree_n; ++i) {
-      const int d = p.tree_depth[i];
-      if (d <= n_next && a_new + d < p.P) {
-        ++nv;
-        md = max(md, d);
-      }
-    }
-    t_nvalid = nv;
-    t_maxd = md;
-    DevState* st = p.st;
-    int* codes_out = p.codes_out;
-    for (int t = 0; t < n_emit; ++t) {
-      st->codes[a + 1 + t] = t_emit[t];
-      if (codes_out) codes_out[a + t] = t_emit[t];
-      st->emitted_last[t] = t_emit[t];
-    }
-    const int calls = st0.calls + 1, heads = st0.heads_read + ci->phi[0] - ci->plo[0] + 1;   // + the last pass
-    const int kvr = st0.kv_rows + pos0 + n_rows, rf = st0.rows_fed + n_rows;
-    const int drafted = st0.drafted + t_res[3], accepted = st0.accepted + plen;
-    st->n_emit_last = n_emit;
-    st->n_acc_last = plen;
-    st->a = a_new;
-    st->n_d = n_next;
-    st->pos0 = a_new + 1;
-    st->n_rows = 1 + nv;
-    st->top_pos = a_new + 1 + md;
-    st->round = round + 1;
-    st->tpass = 0;
-    st->first_head_row = 0;
-    st->calls = calls;
-    st->heads_read = heads;
-    st->kv_rows = kvr;
-    st->rows_fed = rf;
-    st->drafted = drafted;
-    st->accepted = accepted;
-    st->call = call + 1;
-    st->done = a_new >= p.P ? 1 : 0;
-    if (a_new >= p.P && p.stats) {
-      mcd_frame_stats* fs = p.stats;
-      fs->calls = calls;
-      fs->codes = a_new;
-      fs->drafted = drafted;
-      fs->accepted = accepted;
-      fs->status = 0;
-      fs->heads_read = heads;
-      fs->kv_rows = kvr;
-      fs->rows_fed = rf;
-    }
-  }
-  for (int i = threadIdx.x; i < kMaxDraft * kMaxTreeRank; i += kConsumerThreads) {
-    const int d = i / kMaxTreeRank, r = i % kMaxTreeRank;
-    p.tree_cand[i] = (d < n_next && r < p.tree_m[d]) ? t_next[d][r] : -1;
-  }
-  consumer_sync();
-  // optional trace: the chain record, the draft row's logits and the tree record (every row's
-  // verify logits were copied by the top-k stage)
-  if (p.trace && round < kMaxCalls) {
-    uint8_t* tb = p.trace;
-    mcd_call_trace* tr = reinterpret_cast<mcd_call_trace*>(tb) + round;
-    float* dlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls) +
-                  (size_t)kMaxCalls * kMaxRows * p.V;
-    const size_t chain_bytes = sizeof(mcd_call_trace) * kMaxCalls + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4;
-    mcd_tree_trace* tt = reinterpret_cast<mcd_tree_trace*>(tb + chain_bytes) + round;
-    if (threadIdx.x == 0) {
-      tr->a = a;
-      tr->n_rows = n_rows;
-      tr->pos0 = pos0;
-      tr->n_drafts = t_res[3];
-      // code fed at call row n: the first call is one pass of plain rows; a tree call feeds
-      // c_a, then node n - 1's candidate
-      auto row_id = [&](int n) {
-        if (n >= n_rows) return -1;
-        if (pos0 == 0) return ci->r_id[n];
-        if (n == 0) return st0.codes[a];
-        return ci->tcand[p.tree_depth[n - 1] - 1][p.tree_rank[n - 1]];
-      };
-      for (int n = 0; n < kMaxRows; ++n) tr->input_ids[n] = row_id(n);
-      for (int i = 0; i < kMaxRows; ++i) tr->drafts[i] = -1;
-      tr->n_acc = plen;
-      tr->n_emit = n_emit;
-      for (int t = 0; t < kMaxRows; ++t) tr->emitted[t] = t < n_emit ? t_emit[t] : -1;
-      tr->n_next = n_next;
-      for (int j = 0; j < kMaxRows; ++j) tr->next_drafts[j] = j < n_next ? t_next[j][0] : -1;
-      tr->draft_row = drow;
-      tt->n_rows = n_rows;
-      for (int n = 0; n < kMaxTreeRows; ++n) {
-        tt->row_node[n] = n >= n_rows ? -1 : pos0 == 0 ? ci->r_node[n] : n - 1;
-        tt->row_id[n] = row_id(n);
-      }
-      tt->n_passes = (n_rows + kMaxCols - 1) / kMaxCols;
-      tt->path_len = plen;
-      for (int t = 0; t < kMaxDraft + 1; ++t) tt->path[t] = t < plen ? t_path[t] : -1;
-      tt->draft_row = drow;
-      tt->n_next = n_next;
-      for (int d = 0; d < kMaxDraft + 1; ++d)
-        for (int r = 0; r < kMaxTreeRank; ++r)
-          tt->next_cand[d][r] = (d < n_next && d < kMaxDraft && r < p.tree_m[d]) ? t_next[d][r] : -1;
-    }
-    for (int n = 0; n < n_next; ++n)
-      copy_logits(dlog + ((size_t)round * kMaxRows + n) * p.V, p.logits + ((size_t)drow * (kMaxDraft + 1) + n + 1) * p.V, p.V);
-  }
-  consumer_sync();
+  // LM heads of the call's last pass (the earlier ones are in the state)
+  const TreeCall t{&p.tree, &ci->st[0], ci->tcand, p.topk, p.logits, ci->phi[0] - ci->plo[0] + 1, p.stream_ids[0],
+                   p.frame_ids[0], p.codes_out, p.stats, p.trace};
+  accept_tree_call(p, t);
   if (threadIdx.x == 0) red_release_add(p.ctr + (size_t)(call + 1) * p.ctr_stride + ctr_ready(p.L), 1u);
 }
 
@@ -1579,7 +1360,7 @@ __device__ __forceinline__ bool read_call_state(Cons& c, int call, bool first) {
       // breadth-first node list (node i at row i + 1); pass t feeds rows 32 t .. 32 t + 31
       const DevState& st = sts[0];
       int R = 1;
-      while (R <= p.tree_n && p.tree_depth[R - 1] <= st.n_d && st.a + p.tree_depth[R - 1] < p.P) ++R;
+      while (R <= p.tree.n && p.tree.depth[R - 1] <= st.n_d && st.a + p.tree.depth[R - 1] < p.P) ++R;
       const int row0 = st.tpass * kMaxCols, Mp = max(0, min(R - row0, kMaxCols));
       if (R != st.n_rows || Mp == 0) atomicCAS(p.err, 0, (int)MCD_ERR_STATE);   // the acceptance step counted otherwise
       ci->row0 = row0;
@@ -1592,9 +1373,9 @@ __device__ __forceinline__ bool read_call_state(Cons& c, int call, bool first) {
           ci->r_id[n] = st.codes[st.a];
           ci->r_node[n] = -1;
         } else {
-          const int d = p.tree_depth[m - 1];
+          const int d = p.tree.depth[m - 1];
           ci->r_pos[n] = st.pos0 + d;
-          ci->r_id[n] = ci->tcand[d - 1][p.tree_rank[m - 1]];
+          ci->r_id[n] = ci->tcand[d - 1][p.tree.rank[m - 1]];
           ci->r_node[n] = (signed char)(m - 1);
         }
       }
@@ -1609,7 +1390,7 @@ __device__ __forceinline__ bool read_call_state(Cons& c, int call, bool first) {
         unsigned long long U = 0ull;
         while (r < Mp && r - start < G) {
           const int m = row0 + r;
-          const unsigned long long am = m > 0 ? p.tree_anc[m - 1] : 0ull;
+          const unsigned long long am = m > 0 ? p.tree.anc[m - 1] : 0ull;
           if (r > start && st.pos0 + 1 + __popcll(U | am) > kTreeKeys) break;
           U |= am;
           ++r;

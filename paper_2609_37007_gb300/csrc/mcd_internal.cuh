@@ -118,6 +118,14 @@ struct TopkRec {
   uint32_t W[kMaxTopK];
 };
 
+// Sparse tree of TREE mode: nodes in breadth-first order.
+struct TreeDef {
+  int n, maxd;
+  signed char parent[kMaxTree], rank[kMaxTree], depth[kMaxTree];
+  int m[kMaxDraft];                        // candidates needed per depth
+  unsigned long long anc[kMaxTree];        // node i: bit j set iff node j is i or an ancestor of i
+};
+
 struct FrameParams {
   // configuration
   int L, H, NH, NKV, D, F, P, V, C0V, K, top_k, qk_norm, wdtype, draft_mode;
@@ -180,11 +188,7 @@ struct FrameParams {
   int* n_emitted_out;
   unsigned long long* timeline;  // optional [kMaxCalls][32] %globaltimer stamps (CTA 0)
   int single_call;             // 1 = run exactly one call (stepwise API)
-  // sparse tree (TREE mode): nodes in breadth-first order
-  int tree_n, tree_maxd;
-  signed char tree_parent[kMaxTree], tree_rank[kMaxTree], tree_depth[kMaxTree];
-  int tree_m[kMaxDraft];       // candidates needed per depth
-  unsigned long long tree_anc[kMaxTree];   // node i: bit j set iff node j is i or an ancestor of i
+  TreeDef tree;                // TREE mode
   int* tree_cand;              // [kMaxDraft][kMaxTreeRank] candidates of the next call
   int n_cta;
   unsigned long long wait_ns;  // bound of every device-side wait

@@ -455,6 +455,29 @@ def test_tree_mode_trace_parity_tiny(name):
     env.dec.close()
 
 
+@pytest.mark.parametrize("nodes,depth", [(16, 3), (17, 3), (31, 3), (32, 3), (64, 3), (21, 7)])
+def test_tree_mode_trace_parity_batched(nodes, depth):
+    """Trees on the batched kernels (bf16 weights, from 17 nodes on; 16 stay on the frame kernel):
+    18 to 65 rows in one pass, depth 3 and, with three candidates below each kept node, depth 7.
+    Logits within 2e-2 as for every bf16 model; hi + lo operands make them about 1e-4 here."""
+    from oracle.tree import Tree, grow_tree
+    if depth == 7:
+        parent = [-1] * 3 + [3 * (d - 1) for d in range(1, 7) for _ in range(3)]
+        tree = Tree(parent=parent, rank=[0, 1, 2] * 7)
+    else:
+        tree = grow_tree([[0.6 / (r + 1) ** 0.5 for r in range(8)] for _ in range(3)], nodes)
+    assert tree.n == nodes
+    cfg = TINY_BF16.replace(draft_mode=3, draft_len=depth, n_pos=15 if depth == 7 else 8, vocab=256)
+    env = Env(cfg)
+    mcd.mcd_set_tree(env.dec.ctx, tree.parent, tree.rank)
+    for f in range(3):
+        fr = make_frame(cfg, f)
+        codes, st, tr = env.decode(fr, f, stream_id=1, trace=True)
+        assert st[4] == 0 and st[1] == cfg.n_pos, st
+        check_tree_trace_against_oracle(cfg, env.model, fr, 1, f, tr, codes, int(st[0]), tree, logit_tol=2e-2)
+    env.dec.close()
+
+
 def test_chain_tree_equals_greedy_drafts_on_gpu():
     cfg = TINY.replace(draft_len=3, n_pos=8)
     tree_env = Env(cfg.replace(draft_mode=3))

@@ -101,7 +101,9 @@ struct BatchBufs {
   int* head_list;         // [R * kRecSlots] grouped by head
   float* X;               // [R][H] residual stream
   float* ss;              // [2L + 1][R] per-row sums of squares of X after each residual write
-  float* qkv;             // [R][qkv_dim]
+  float* qkv;             // [R][qkv_dim]; tensor cores: qkv_nz partial sums, qkv_zs floats apart
+  int qkv_nz;
+  size_t qkv_zs;
   uint16_t* att;          // [R][NH * D] bf16 attention outputs
   uint16_t* act;          // [R][F] bf16 SwiGLU outputs
   float* logits;          // [R][kRecSlots][V]
@@ -114,7 +116,7 @@ struct BatchBufs {
   uint8_t* act_t;         // SwiGLU outputs
   uint8_t *att_lo, *act_lo;   // TREE mode: their low halves
   float* tree_q;          // TREE mode: [R][NH * D] normalised, rotated queries
-  float* part;            // [kTcSplit][Rtc][H] k-split partial sums of the residual products
+  float* part;            // [splits][Rtc][H] k-split partial sums of the residual products
   int Qcap;               // LM-head operand rows: every (row, j) pair, groups padded per head
   uint8_t* hq_hi;         // LM-head operand (normalised rows of the pairs, grouped by head)
   uint8_t* hq_lo;
@@ -716,10 +718,12 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
   {
     const int e_q = nq << lg4, e_k = e_q + (nk << lg4), e_v = e_k + (nk << lg4);
     const int e_cs = e_v + (nr << lg4), e_g = e_cs + (p.qk_norm ? 2 << lg4 : 0);
+    const int nz = b.qkv_nz;
     for (int i = tid; i < e_g; i += 256) {
       const int ch = i & (D4 - 1);
       const float* src;
       float* dst;
+      bool sum = nz > 1 && i < e_q;              // a row of the QKV product: its partial sums added
       if (i < e_q) {
         const int qi = i >> lg4;
         src = b.qkv + (size_t)(base + q_row[qi]) * p.qkv_dim + q_head[qi] * D;
@@ -731,6 +735,7 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
           src = (isv ? p.vcache : p.kcache) + cache_off + (size_t)j * D;
         else
           src = b.qkv + (size_t)(base + j - pos0) * p.qkv_dim + p.NH * D + (isv ? p.NKV * D : 0) + g * D;
+        sum = nz > 1 && j >= pos0;
         dst = isv ? vs[j] : ks[j];
       } else if (i < e_cs) {
         const int n = (i - e_v) >> lg4;
@@ -741,7 +746,19 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
         src = (w == 0 ? p.q_norm : p.k_norm) + (size_t)layer * D;
         dst = w == 0 ? gq : gk;
       }
-      cpa16(dst + 4 * ch, src + 4 * ch);
+      if (sum) {
+        float4 v = __ldcg(reinterpret_cast<const float4*>(src) + ch);
+        for (int z = 1; z < nz; ++z) {
+          const float4 w = __ldcg(reinterpret_cast<const float4*>(src + z * b.qkv_zs) + ch);
+          v.x += w.x;
+          v.y += w.y;
+          v.z += w.z;
+          v.w += w.w;
+        }
+        reinterpret_cast<float4*>(dst)[ch] = v;
+      } else {
+        cpa16(dst + 4 * ch, src + 4 * ch);
+      }
     }
     cpa_wait_all();
   }
@@ -1127,8 +1144,7 @@ __global__ void __launch_bounds__(256) batch_tree_rope_kernel(FrameParams p, Bat
   const int kind = vi < NH ? 0 : (vi < NH + p.NKV ? 1 : 2), h = kind == 0 ? vi : (kind == 1 ? vi - NH : vi - NH - p.NKV);
   const float* src = b.qkv + (size_t)r * p.qkv_dim + vi * D;
   float x[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) x[i] = i < nd ? __ldcg(src + lane + 32 * i) : 0.f;
+  qkv_row(x, src, nd, lane, b.qkv_nz, b.qkv_zs);
   if (kind < 2) {
     if (p.qk_norm) {
       float ss = 0.f;
@@ -1359,15 +1375,17 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
   BATCH_ALLOC(b.head_list, sizeof(int) * R * kRecSlots);
   BATCH_ALLOC(b.X, sizeof(float) * R * p.H);
   BATCH_ALLOC(b.ss, sizeof(float) * (2 * p.L + 1) * R);
-  BATCH_ALLOC(b.qkv, sizeof(float) * R * p.qkv_dim);
   BATCH_ALLOC(b.att, sizeof(uint16_t) * R * p.NH * p.D);
   BATCH_ALLOC(b.act, sizeof(uint16_t) * R * p.F);
   BATCH_ALLOC(b.logits, sizeof(float) * R * kRecSlots * p.V);
   BATCH_ALLOC(b.recs, sizeof(TopkRec) * 2 * R * kRecSlots);
   bs->use_tc = tc_block_supported(p);
   if (bs->use_tc) {
-    const int Rtc = bs->tree ? tc_operand_rows(rows, p.qkv_dim, p.n_cta) : (R + 127) / 128 * 128;
+    const int Rtc = tc_operand_rows(rows, p.qkv_dim, p.n_cta);
     b.Rtc = Rtc;
+    b.qkv_nz = tc_qkv_splits(p.qkv_dim, Rtc, p.H, p.n_cta);
+    b.qkv_zs = (size_t)Rtc * p.qkv_dim;
+    BATCH_ALLOC(b.qkv, sizeof(float) * b.qkv_nz * b.qkv_zs);
     if (bs->tree) {
       BATCH_ALLOC(b.att_lo, (size_t)Rtc * p.NH * p.D * 2);
       BATCH_ALLOC(b.act_lo, (size_t)Rtc * p.F * 2);
@@ -1377,7 +1395,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
     BATCH_ALLOC(b.xn_lo, (size_t)Rtc * p.H * 2);
     BATCH_ALLOC(b.att_t, (size_t)Rtc * p.NH * p.D * 2);
     BATCH_ALLOC(b.act_t, (size_t)Rtc * p.F * 2);
-    BATCH_ALLOC(b.part, (size_t)kTcSplit * Rtc * p.H * 4);
+    BATCH_ALLOC(b.part, sizeof(float) * tc_part_floats(Rtc, p.H));
     if (p.V % tc::kBM == 0) {
       b.Qcap = (R * kRecSlots + p.P * (kTcBN - 1) + kTcBN - 1) / kTcBN * kTcBN;
       BATCH_ALLOC(b.hq_hi, (size_t)b.Qcap * p.H * 2);
@@ -1387,6 +1405,9 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
     TcWeights& tw = bs->tw;
     tw.off = tc_layer_offsets(p);
     BATCH_ALLOC(tw.arena, tw.off.layer * p.L);
+  } else {
+    b.qkv_nz = 1;
+    BATCH_ALLOC(b.qkv, sizeof(float) * R * p.qkv_dim);
   }
 #undef BATCH_ALLOC
   if (cudaMemset(b.info, 0, sizeof(BatchInfo)) != cudaSuccess) return fail(MCD_ERR_CUDA);
@@ -1477,15 +1498,15 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     tc::launch(false, batch_attn_kernel, dim3(bs->max_streams, p.NKV), blk, 0, s, p, b, l);      // -> att_t
     // Wo (k-split partials) -> residual, ss, the gate/up operand
     tc_launch_resid<false>(wl + bs->tw.off.o, b.att_t, nullptr, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
-                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, (uint8_t*)nullptr);
+    tc_launch_resid_norm(false, R, b.X, b.part, qd, Rtc, H, p.n_cta, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
+                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, (uint8_t*)nullptr, s);
     // gate/up -> SwiGLU (into the down product's operand)
     tc_launch_gu<false>(wl + bs->tw.off.gu, b.xn_hi, nullptr, b.act_t, nullptr, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     // down (k-split partials) -> residual, ss, the next layer's QKV operand
     tc_launch_resid<false>(wl + bs->tw.off.d, b.act_t, nullptr, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
     const bool last = l + 1 == L;
-    tc::launch(false, tc_resid_norm_kernel, dim3(R), dim3(128), 0, s, b.X, b.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
-                                           last ? (const float*)nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo);
+    tc_launch_resid_norm(false, R, b.X, b.part, p.F, Rtc, H, p.n_cta, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
+                                           last ? (const float*)nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo, s);
   }
   for (int l = 0; l < L && !bs->use_tc; ++l) {
     {   // RMSNorm -> QKV
@@ -1562,7 +1583,7 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
 // Every kernel of one tree call.
 static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs, const BatchLoop& loop, cudaStream_t s) {
   const BatchBufs& b = bs->b;
-  const int R = b.R, L = p.L, H = p.H, Rtc = b.Rtc, qd = p.NH * p.D, z = tc_resid_split(Rtc);
+  const int R = b.R, L = p.L, H = p.H, Rtc = b.Rtc, qd = p.NH * p.D;
   const dim3 blk(256);
   const bool pdl = loop.valid != 0;
   const int* M = &b.info->M;
@@ -1575,13 +1596,13 @@ static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs,
     batch_tree_rope_kernel<<<(kMaxTreeRows * (p.NH + 2 * p.NKV) + 7) / 8, blk, 0, s>>>(p, b, l);
     batch_tree_attn_kernel<<<(kMaxTreeRows * p.NH + 7) / 8, blk, 0, s>>>(p, b, l);
     tc_launch_resid<true>(wl + bs->tw.off.o, b.att_t, b.att_lo, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_resid_norm_kernel<<<kMaxTreeRows, 128, 0, s>>>(b.X, b.part, tc_splits(qd, z), Rtc, H, M, b.ss + (size_t)(2 * l + 1) * R,
-                                                      p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, b.xn_lo);
+    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, qd, Rtc, H, p.n_cta, M, b.ss + (size_t)(2 * l + 1) * R,
+                                                      p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, b.xn_lo, s);
     tc_launch_gu<true>(wl + bs->tw.off.gu, b.xn_hi, b.xn_lo, b.act_t, b.act_lo, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + bs->tw.off.d, b.act_t, b.act_lo, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_resid_norm_kernel<<<kMaxTreeRows, 128, 0, s>>>(b.X, b.part, tc_splits(p.F, z), Rtc, H, M, b.ss + (size_t)(2 * l + 2) * R,
+    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, b.ss + (size_t)(2 * l + 2) * R,
                                                       l + 1 == L ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi,
-                                                      b.xn_lo);
+                                                      b.xn_lo, s);
   }
   enqueue_heads(p, bs, s);
   batch_topk_kernel<<<kMaxTreeRows * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);

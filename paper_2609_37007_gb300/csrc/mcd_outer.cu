@@ -644,7 +644,8 @@ __global__ void __launch_bounds__(128) pf_embed_kernel(const int* __restrict__ i
 // QK-norm + RoPE (position = row index) of every prompt row's query and key heads; K and V
 // rounded to bf16 into layer l's cache ([NKV][cap][D]), the rotated queries (fp32) into q.
 // One warp per (row, vector), lane holding dims lane + 32 i.
-__global__ void __launch_bounds__(256) pf_rope_kv_kernel(const float* __restrict__ qkv, int qkv_dim, const int* nrows,
+__global__ void __launch_bounds__(256) pf_rope_kv_kernel(const float* __restrict__ qkv, int nz, size_t zs, int qkv_dim,
+                                                         const int* nrows,
                                                          int NH, int NKV, int D, int qk_norm, const float* qn,
                                                          const float* kn, float eps, const float2* __restrict__ rope,
                                                          uint16_t* kc, uint16_t* vc, int cap, float* q) {
@@ -657,8 +658,7 @@ __global__ void __launch_bounds__(256) pf_rope_kv_kernel(const float* __restrict
   const int nd = D >> 5, half = D >> 1;
   const float* src = qkv + (size_t)r * qkv_dim + (kind == 0 ? h * D : NH * D + (kind == 2 ? NKV * D : 0) + h * D);
   float x[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) x[i] = i < nd ? __ldcg(src + lane + 32 * i) : 0.f;
+  qkv_row(x, src, nd, lane, nz, zs);
   if (kind < 2) {
     if (qk_norm) {
       float ssq = 0.f;
@@ -1158,9 +1158,9 @@ mcd_status mcd_outer_create(const mcd_outer_config* cfg, mcd_ctx* inner, mcd_out
     OUTER_ALLOC(t.w, t.off.layer * p.L);
     OUTER_ALLOC(t.X, sizeof(float) * (size_t)Rtc * p.H);
     OUTER_ALLOC(t.ss, sizeof(float) * (size_t)Rtc);
-    OUTER_ALLOC(t.qkv, sizeof(float) * (size_t)Rtc * p.qkv_dim);
+    OUTER_ALLOC(t.qkv, sizeof(float) * (size_t)std::max(Rtc, kTcQkvSplit * std::min(Rtc, kTcSmallRows)) * p.qkv_dim);
     OUTER_ALLOC(t.q, sizeof(float) * (size_t)Rtc * p.NH * p.D);
-    OUTER_ALLOC(t.part, sizeof(float) * (size_t)kTcSplit * Rtc * p.H);
+    OUTER_ALLOC(t.part, sizeof(float) * tc_part_floats(Rtc, p.H));
     OUTER_ALLOC(t.xn_hi, (size_t)Rtc * p.H * 2);
     OUTER_ALLOC(t.xn_lo, (size_t)Rtc * p.H * 2);
     OUTER_ALLOC(t.att_t, (size_t)Rtc * p.NH * p.D * 2);
@@ -1307,18 +1307,19 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
     uint16_t* vc = reinterpret_cast<uint16_t*>(st.vcache) + (size_t)l * kvl;
     tc_launch_qkv(wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
     const int vecs = p.NH + 2 * p.NKV;
-    tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
+    tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, tc_qkv_splits(p.qkv_dim, Rtc, H, p.n_cta),
+               (size_t)Rtc * p.qkv_dim, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
                                                          p.q_norm + (size_t)l * p.D, p.k_norm + (size_t)l * p.D, p.eps,
                                                          st.rope, kc, vc, st.cap, t.q);
     launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, t.att_lo, s);
     tc_launch_resid<true>(wl + t.off.o, t.att_t, t.att_lo, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(qd, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
-                                           p.eps, t.xn_hi, t.xn_lo);
+    tc_launch_resid_norm(pdl, n, t.X, t.part, qd, Rtc, H, p.n_cta, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
+                                           p.eps, t.xn_hi, t.xn_lo, s);
     tc_launch_gu<true>(wl + t.off.gu, t.xn_hi, t.xn_lo, t.act_t, t.act_lo, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + t.off.d, t.act_t, t.act_lo, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc::launch(pdl, tc_resid_norm_kernel, dim3(n), dim3(128), 0, s, t.X, t.part, tc_splits(p.F, tc_resid_split(Rtc)), Rtc, H, t.rows, t.ss,
+    tc_launch_resid_norm(pdl, n, t.X, t.part, p.F, Rtc, H, p.n_cta, t.rows, t.ss,
                                            l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : (const float*)nullptr, p.eps, t.xn_hi,
-                                           t.xn_lo);
+                                           t.xn_lo, s);
   }
   MCD_CHECK(cudaGetLastError());
   return MCD_OK;

@@ -60,22 +60,65 @@ __global__ void tc_weight_tile_kernel(const uint16_t* __restrict__ src, int rows
 }
 
 constexpr int kTcBN = 128;        // packed rows per tile: QKV (hi + lo operand), Wo, down
-constexpr int kTcSplit = 6;       // k-splits of the residual products (at most)
-// Splits of the residual products at Rtc packed rows: four (128-column tiles, 128 CTAs at 512
-// rows) from 512 rows on, where more splits' partial sums cost more than they save; six below
-// (3 x 8 x 6 = 144 CTAs at 128 rows, where 128-column tiles would leave 32 CTAs).
-inline int tc_resid_split(int Rtc) { return Rtc >= 512 ? 4 : kTcSplit; }
+constexpr int kTcSplit = 16;      // k-splits of the residual products (at most)
+constexpr int kTcQkvSplit = 4;    // k-splits of the QKV product (at most)
+// A product's column tiles and k-splits at Rtc operand rows.  Up to 128 rows a product is its
+// weight stream, and a few column tiles of 128-row weight tiles would leave most SMs without a
+// share of it: tiles of up to 64 columns, and as many k-splits as fill the SMs (at most z_max).
+// Frames of 8 streams (32 rows): 1191 us with QKV, Wo and down on 32 / 48 / 48 CTAs, 1059 on 128
+// each; a 32-node tree (33 rows) 1422 and 1358.
+struct TcShape {
+  int pitch, z;
+};
+inline TcShape tc_small_shape(int M, int Rtc, int n_sm, int z_max) {
+  const int units = Rtc / 16, T = (Rtc + 63) / 64, z = n_sm / ((M / tc::kBM) * T);
+  return TcShape{(units + T - 1) / T * 16, z < 1 ? 1 : (z > z_max ? z_max : z)};
+}
+constexpr int kTcSmallRows = 128;
+// Residual products above kTcSmallRows: six splits below 512 rows, four (128-column tiles, 128 CTAs at
+// 512 rows) from there on, where more splits' partial sums cost more than they save.
+inline TcShape tc_resid_shape(int H, int Rtc, int n_sm) {
+  if (Rtc <= kTcSmallRows) return tc_small_shape(H, Rtc, n_sm, kTcSplit);
+  const int n_mt = H / tc::kBM, units = Rtc / 16, z = Rtc >= 512 ? 4 : 6;
+  int T = n_sm / (n_mt * z);
+  if (T < 1) T = 1;
+  if (T < (Rtc + 255) / 256) T = (Rtc + 255) / 256;
+  if (T > units) T = units;
+  return TcShape{(units + T - 1) / T * 16, z};
+}
+// Non-empty k-splits of a product over K in z splits (gemm_tile's split of the k-slices).
+inline int tc_splits(int K, int z) {
+  const int nk = K / tc::kBK, per = (nk + z - 1) / z;
+  return (nk + per - 1) / per;
+}
 
 // Shared memory for the ring of a tile of up to 128 columns: two CTAs of consecutive kernels fit
 // an SM together, so the next product's weights stream in while this one finishes.
 constexpr int kTcCompact = 100 * 1024;
 constexpr int kTcCompactRows = 384;
 
+// Elements lane + 32 i (i < nd) of a row of the QKV product: its nz <= kTcQkvSplit partial sums, zs
+// floats apart, added.
+__device__ __forceinline__ void qkv_row(float (&x)[4], const float* src, int nd, int lane, int nz, size_t zs) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = i < nd ? __ldcg(src + lane + 32 * i) : 0.f;
+  if (nz == 1) return;
+  float y[kTcQkvSplit - 1][4];
+#pragma unroll
+  for (int z = 1; z < kTcQkvSplit; ++z)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[z - 1][i] = i < nd && z < nz ? __ldcg(src + z * zs + lane + 32 * i) : 0.f;
+#pragma unroll
+  for (int z = 0; z < kTcQkvSplit - 1; ++z)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] += y[z][i];
+}
+
 // q, k, v = W (x . g / rms) with the hi + lo operand.
 __global__ void __launch_bounds__(tc::kPThreads, 1) tc_qkv_kernel(const tc::GemmArgs g, float* out, int ld) {
   tc::gemm_persistent<kTcBN, true>(g, 1, [&](int m, int n, int, float v) { out[(size_t)n * ld + m] = v; });
 }
-// The same product, one 128 x pitch tile per CTA.
+// The same product, one 128 x pitch tile per CTA; k-split z writes partial sums out[z][Rtc][ld].
 constexpr int kQkvThreads = 256;
 template <int BN, int kBudget>
 __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::GemmArgs g, float* out, int ld,
@@ -83,8 +126,9 @@ __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::G
   tc::TileRun t;
   if (!tc::gemm_tile_run<BN, true, kBudget, true>(g, t)) return;
   const int M = *nrows;
+  float* o = out + (size_t)blockIdx.z * g.N * ld;
   tc::gemm_tile_drain<BN>(t, [&](int m, int n, float v) {
-    if (n < M) out[(size_t)n * ld + m] = v;
+    if (n < M) o[(size_t)n * ld + m] = v;
   });
 }
 
@@ -149,7 +193,7 @@ __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs
 }
 
 // Residual products (Wo, down): one 128 x pitch tile per CTA over the k-slices of split
-// blockIdx.z of kTcSplit; split z writes its partial sums part[z][n][m] (plain stores);
+// blockIdx.z; split z writes its partial sums part[z][n][m] (plain stores);
 // tc_resid_norm_kernel adds them into the residual stream.
 constexpr int kResidThreads = 256;
 template <int BN, bool kHilo, int kBudget>
@@ -167,6 +211,7 @@ __global__ void __launch_bounds__(kResidThreads, 1) tc_resid_kernel(const tc::Ge
 // Per packed row (one CTA, thread t owns elements 8t..8t+7): X += the nz partial sums, the
 // row's sum of squares (the next RMSNorm), and with a gain the next product's normalised
 // operand (hi; with lo also the remainder) as SW128 tiles.
+template <int NZ>       // partial sums held in registers (nz <= NZ)
 __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const float* __restrict__ part, int nz, int Rtc,
                                                             int H, const int* nrows, float* ss_out,
                                                             const float* __restrict__ gain, float eps, uint8_t* hi,
@@ -183,10 +228,10 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
   if (live) {
     float4* xr = reinterpret_cast<float4*>(X + (size_t)r * H + 8 * t);
     float4 a = xr[0], b = xr[1];
-    // every partial's loads issued before the first add (nz <= kTcSplit), added in split order
-    float4 u[kTcSplit], w[kTcSplit];
+    // every partial's loads issued before the first add, added in split order
+    float4 u[NZ], w[NZ];
 #pragma unroll
-    for (int z = 0; z < kTcSplit; ++z) {
+    for (int z = 0; z < NZ; ++z) {
       if (z < nz) {
         const float4* pr = reinterpret_cast<const float4*>(part + ((size_t)z * Rtc + r) * H + 8 * t);
         u[z] = __ldcg(pr);
@@ -194,7 +239,7 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
       }
     }
 #pragma unroll
-    for (int z = 0; z < kTcSplit; ++z) {
+    for (int z = 0; z < NZ; ++z) {
       if (z < nz) {
         a.x += u[z].x; a.y += u[z].y; a.z += u[z].z; a.w += u[z].w;
         b.x += w[z].x; b.y += w[z].y; b.z += w[z].z; b.w += w[z].w;
@@ -229,14 +274,6 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
     if (lo) *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
   }
 }
-
-// Non-empty k-splits of a residual product over K in z splits (gemm_tile's split of the
-// k-slices).
-static int tc_splits(int K, int z) {
-  const int nk = K / tc::kBK, per = (nk + z - 1) / z;
-  return (nk + per - 1) / per;
-}
-
 
 // The transformer-block products can use the tensor-core GEMM (shape and dtype limits).
 bool tc_block_supported(const FrameParams& p) {
@@ -325,7 +362,16 @@ inline int tc_operand_rows(int n, int qkv_dim, int n_sm) {
   const int unit = tc_qkv_persistent(n, qkv_dim, n_sm) ? kTcBN : 16;
   return (n + unit - 1) / unit * unit;
 }
-// q, k, v of Rtc operand rows.  Below tc_qkv_persistent's line the pitch is at most kTcBN: nt
+// Column tiles and k-splits of the QKV product (tile form); tc_qkv_splits: partial sums it leaves.
+inline TcShape tc_qkv_shape(int qkv_dim, int Rtc, int n_sm) {
+  if (Rtc <= kTcSmallRows) return tc_small_shape(qkv_dim, Rtc, n_sm, kTcQkvSplit);
+  return TcShape{tc::tile_pitch(qkv_dim, Rtc, n_sm), 1};
+}
+inline int tc_qkv_splits(int qkv_dim, int Rtc, int H, int n_sm) {
+  return tc_qkv_persistent(Rtc, qkv_dim, n_sm) ? 1 : tc_splits(H, tc_qkv_shape(qkv_dim, Rtc, n_sm).z);
+}
+// q, k, v of Rtc operand rows, as tc_qkv_splits partial sums out[z][Rtc][qkv_dim].  Below
+// tc_qkv_persistent's line the pitch is at most kTcBN: nt
 // tiles of 128 columns over n_mt weight tiles with nt n_mt < 0.8 n_sm leave n_sm / n_mt >= nt.
 inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t* xn_lo, float* out, int qkv_dim, int Rtc,
                           int H, const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
@@ -335,8 +381,9 @@ inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t*
                    tc::PLayout<kTcBN, true>::kSmemBytes, s, g, out, qkv_dim);
     return;
   }
-  g.bn = tc::tile_pitch(qkv_dim, Rtc, n_sm);
-  const dim3 grid((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM);
+  const TcShape sh = tc_qkv_shape(qkv_dim, Rtc, n_sm);
+  g.bn = sh.pitch;
+  const dim3 grid((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM, sh.z);
   if (g.bn <= 64)
     tc::launch(pdl, tc_qkv_tile_kernel<64, kTcCompact>, grid, dim3(kQkvThreads), tc::Layout<64, true, kTcCompact>::kSmemBytes,
                    s, g, out, qkv_dim, nrows);
@@ -352,7 +399,7 @@ template <bool kHilo>
 inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, const uint8_t* xn_lo, uint8_t* act_t, uint8_t* act_lo, int Rtc,
                          const int* nrows, int F, int H, int* err, unsigned long long wait_ns, int n_sm, bool pdl,
                          cudaStream_t s) {
-  const int pitch = tc::tile_pitch(2 * F, Rtc, n_sm);
+  const int pitch = Rtc <= 64 ? Rtc : tc::tile_pitch(2 * F, Rtc, n_sm);
   const tc::GemmArgs g{gu, xn, xn_lo, 2 * F, Rtc, H, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, 2 * F / tc::kBM);
   tc_pick<kHilo>(pitch, Rtc, [&](auto bn, auto budget) {
@@ -362,26 +409,38 @@ inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, const uint8_t* xn
   });
 }
 
-// Wo or down (A = w: H rows of K, B = act: Rtc rows) -> tc_resid_split(Rtc) partial sums.
-// T column tiles x (H / 128) weight tiles x z splits fill the SMs with one tile per CTA
-// (H = 1024: T = 4 of 128 packed rows at 512 rows, 128 CTAs; T = 3 of 48 / 48 / 32 at 128
-// rows, 144 CTAs).
+// Wo or down (A = w: H rows of K, B = act: Rtc rows) -> the partial sums of tc_resid_shape's splits
+// (H = 1024: 16 splits of one column tile up to 64 rows, 128 CTAs; 9 of two up to 128, 144 CTAs;
+// 4 of four at 512, 128 CTAs).
 template <bool kHilo>
 inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, const uint8_t* act_lo, float* part, int H, int Rtc, int K,
                             const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
-  const int n_mt = H / tc::kBM, units = Rtc / 16, z = tc_resid_split(Rtc);
-  int T = n_sm / (n_mt * z);
-  if (T < 1) T = 1;
-  if (T < (Rtc + 255) / 256) T = (Rtc + 255) / 256;
-  if (T > units) T = units;
-  const int pitch = (units + T - 1) / T * 16;
+  const TcShape sh = tc_resid_shape(H, Rtc, n_sm);
+  const int pitch = sh.pitch;
   const tc::GemmArgs g{w, act, act_lo, H, Rtc, K, nrows, err, wait_ns, pdl, pitch};
-  const dim3 grid((Rtc + pitch - 1) / pitch, n_mt, z);
+  const dim3 grid((Rtc + pitch - 1) / pitch, H / tc::kBM, sh.z);
   tc_pick<kHilo>(pitch, Rtc, [&](auto bn, auto budget) {
     constexpr int BN = decltype(bn)::value, B = decltype(budget)::value;
     tc::launch(pdl, tc_resid_kernel<BN, kHilo, B>, grid, dim3(kResidThreads), tc::Layout<BN, kHilo, B>::kSmemBytes, s, g,
                part, H, Rtc, nrows);
   });
+}
+
+// The residual pass of a product over K (tc_resid_norm_kernel) on `rows` CTAs.
+inline void tc_launch_resid_norm(bool pdl, int rows, float* X, const float* part, int K, int Rtc, int H, int n_sm,
+                                 const int* nrows, float* ss_out, const float* gain, float eps, uint8_t* hi, uint8_t* lo,
+                                 cudaStream_t s) {
+  const int nz = tc_splits(K, tc_resid_shape(H, Rtc, n_sm).z);
+  if (nz <= 6)
+    tc::launch(pdl, tc_resid_norm_kernel<6>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, ss_out, gain, eps, hi, lo);
+  else
+    tc::launch(pdl, tc_resid_norm_kernel<kTcSplit>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, ss_out, gain, eps,
+               hi, lo);
+}
+// Floats of partial sums a residual product leaves at up to Rtc operand rows.
+inline size_t tc_part_floats(int Rtc, int H) {
+  const size_t small = (size_t)kTcSplit * (Rtc < kTcSmallRows ? Rtc : kTcSmallRows), large = (size_t)6 * Rtc;
+  return (small > large ? small : large) * H;
 }
 
 }  // namespace

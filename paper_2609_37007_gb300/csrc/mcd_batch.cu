@@ -99,6 +99,7 @@ struct BatchBufs {
   int* sbase;             // [kMaxBatchStreams] first packed row of each stream (-1: inactive)
   int* pairs;             // [R * kRecSlots] (row << 3) | j
   int* head_list;         // [R * kRecSlots] grouped by head
+  int* head_slot;         // [R * kRecSlots] LM-head operand row of (row, j), -1: none
   float* X;               // [R][H] residual stream
   float* ss;              // [2L + 1][R] per-row sums of squares of X after each residual write
   float* qkv;             // [R][qkv_dim]; tensor cores: qkv_nz partial sums, qkv_zs floats apart
@@ -159,16 +160,23 @@ __device__ __forceinline__ size_t tile_byte_offset(const MatGeom& g, int mt, int
 // pack: the call's rows, distributions and head groups from every stream's state
 // ------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBufs b) {
-  __shared__ int s_cnt[256], s_pc[256], s_head[16], s_hcur[16];
+  __shared__ int s_cnt[16], s_pc[16], s_head[16], s_hcur[16], s_shift[16];
   const BatchFrame* fa = b.frame;
   const int S = fa->S, tid = threadIdx.x;
-  const int L = p.L;
-  for (int i = tid; i < (2 * L + 1) * b.R; i += blockDim.x) b.ss[i] = 0.f;
   if (tid < 16) s_head[tid] = 0;
   int nr = 0, np = 0;
-  DevState st;
+  struct {
+    int done, n_rows, pos0, a, code;
+    const int* drafts;
+  } st;
   if (tid < S) {
-    st = p.st[tid];
+    const DevState* q = p.st + tid;
+    st.done = q->done;
+    st.n_rows = q->n_rows;
+    st.pos0 = q->pos0;
+    st.a = q->a;
+    st.drafts = q->drafts;
+    st.code = q->codes[st.a];          // the last code emitted (the first call: c0)
     if (!st.done) {
       nr = st.n_rows;
       for (int n = 0; n < nr; ++n) {
@@ -218,7 +226,7 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
   if (tid < S && nr > 0) {
     for (int n = 0; n < nr; ++n) {
       const int pos = st.pos0 + n, r = base + n;
-      int id = st.pos0 == 0 ? (n == 0 ? -1 : st.codes[0]) : (n == 0 ? st.codes[st.a] : st.drafts[n - 1]);
+      int id = st.pos0 == 0 ? (n == 0 ? -1 : st.code) : (n == 0 ? st.code : st.drafts[n - 1]);
       BatchRow row;
       row.s = tid;
       row.n = n;
@@ -246,12 +254,14 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
   if (tid < kMaxBatchStreams) b.sbase[tid] = (tid < S && nr > 0) ? base : -1;
   __syncthreads();
   if (tid == 0) {
-    int off = 0;
+    int off = 0, q = 0;
     for (int P = 0; P < 16; ++P) {
       b.info->head_rows[P] = s_head[P];
       b.info->head_off[P] = off;
       s_hcur[P] = off;
+      s_shift[P] = q - off;              // operand rows: groups padded to 16
       off += s_head[P];
+      q += (s_head[P] + 15) / 16 * 16;
     }
     b.info->M = s_cnt[8 + 7];
     b.info->n_pairs = s_pc[8 + 7];
@@ -264,20 +274,57 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
     int pi = pbase;
     for (int n = 0; n < nr; ++n) {
       const int pos = st.pos0 + n, r = base + n;
-      if (pos < 1) continue;
-      const int kn = min(p.K, p.P - pos);
-      for (int j = 0; j <= kn; ++j) {
-        b.pairs[pi++] = (r << 3) | j;
-        b.head_list[atomicAdd(&s_hcur[pos + j], 1)] = (r << 3) | j;
+      const int kn = pos < 1 ? -1 : min(p.K, p.P - pos);
+      for (int j = 0; j < kRecSlots; ++j) {
+        int slot = -1;
+        if (j <= kn) {
+          b.pairs[pi++] = (r << 3) | j;
+          const int at = atomicAdd(&s_hcur[pos + j], 1);
+          b.head_list[at] = (r << 3) | j;
+          slot = at + s_shift[pos + j];
+        }
+        b.head_slot[r * kRecSlots + j] = slot;
       }
     }
   }
 }
 
+// embed (tensor-core path): X[r] = the row's input vector, and layer 0's QKV operand.  Thread t
+// owns elements 8t..8t+7.
+__global__ void __launch_bounds__(128) batch_embed_tc_kernel(FrameParams p, BatchBufs b) {
+  const int r = blockIdx.x, t = threadIdx.x;
+  tc::pdl_trigger();
+  if (r >= b.info->M) return;
+  const BatchRow row = b.rows[r];
+  const bool live = t < p.H / 8;
+  float v[8];
+  float ss = 0.f;
+  if (live) {
+    if (row.f32) {
+      const float* src = reinterpret_cast<const float*>(row.src) + 8 * t;      // any 4-byte alignment
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = __ldg(src + i);
+    } else {
+      const uint4 w = __ldg(reinterpret_cast<const uint4*>(row.src) + t);
+      v[0] = bf16_lo_f32(w.x); v[1] = bf16_hi_f32(w.x); v[2] = bf16_lo_f32(w.y); v[3] = bf16_hi_f32(w.y);
+      v[4] = bf16_lo_f32(w.z); v[5] = bf16_hi_f32(w.z); v[6] = bf16_lo_f32(w.w); v[7] = bf16_hi_f32(w.w);
+    }
+    float4* xr = reinterpret_cast<float4*>(b.X + (size_t)r * p.H + 8 * t);
+    xr[0] = make_float4(v[0], v[1], v[2], v[3]);
+    xr[1] = make_float4(v[4], v[5], v[6], v[7]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ss += v[i] * v[i];
+  }
+  const float tot = block_sum128(ss);
+  if (!live) return;
+  const NormChunk c = norm_chunk(v, rsqrtf(tot / (float)p.H + p.eps), p.attn_norm, t);
+  const size_t off = tc::sw128_offset(b.Rtc, r, t >> 3, t & 7);
+  *reinterpret_cast<uint4*>(b.xn_hi + off) = c.hi;
+  *reinterpret_cast<uint4*>(b.xn_lo + off) = c.lo;
+}
+
 // embed: X[r] = the row's input vector; ss[0][r] = sum of squares.
 __global__ void __launch_bounds__(256) batch_embed_kernel(FrameParams p, BatchBufs b) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= b.info->M) return;
   const BatchRow row = b.rows[r];
@@ -551,11 +598,6 @@ __global__ void __launch_bounds__(256) batch_gemm_kernel(const __grid_constant__
 // are split into n_t = ceil(rows / kHeadTileMax) tiles of equal width (a multiple of 16), so
 // every tile of the product belongs to one head and is no wider than the group needs.
 constexpr int kHeadTileMax = 176;      // three 60 KB ring stages with the hi + lo operand
-__device__ __forceinline__ int tc_head_qoff(const BatchInfo* info, int P) {
-  int o = 0;
-  for (int i = 1; i < P; ++i) o += (info->head_rows[i] + 15) / 16 * 16;
-  return o;
-}
 __host__ __device__ __forceinline__ int tc_head_tiles(int rows) { return (rows + kHeadTileMax - 1) / kHeadTileMax; }
 __host__ __device__ __forceinline__ int tc_head_width(int rows) {
   const int nt = tc_head_tiles(rows);
@@ -563,47 +605,6 @@ __host__ __device__ __forceinline__ int tc_head_width(int rows) {
 }
 // Grid bound over the tiles of every group: at most (K + 1) pairs per packed row.
 inline int tc_head_grid_x(int R, int K, int n_pos) { return (R * (K + 1) + kHeadTileMax - 1) / kHeadTileMax + n_pos; }
-
-// The pairs' normalised rows (final RMSNorm, hi + lo) as SW128 tiles of Qcap rows.
-__global__ void __launch_bounds__(256) tc_heads_operand_kernel(const float* __restrict__ X, const float* __restrict__ gain,
-                                                               const float* __restrict__ ss, int H, float eps,
-                                                               const BatchInfo* info, const int* __restrict__ head_list,
-                                                               int n_pos, int Qcap, uint8_t* hi, uint8_t* lo) {
-  __shared__ int s_off[16], s_rows[16], s_q[16];
-  tc::pdl_wait();
-  tc::pdl_trigger();
-  if (threadIdx.x < 16) {
-    const int P = threadIdx.x;
-    s_off[P] = info->head_off[P];
-    s_rows[P] = P >= 1 && P <= n_pos ? info->head_rows[P] : 0;
-    s_q[P] = P >= 1 && P <= n_pos ? tc_head_qoff(info, P) : 0;
-  }
-  __syncthreads();
-  const int T = info->n_pairs, cpr = H / 8;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < T * cpr; i += gridDim.x * blockDim.x) {
-    const int gi = i / cpr, ch = i - gi * cpr, k = ch * 8;
-    int P = 1;
-    while (P < n_pos && !(gi >= s_off[P] && gi < s_off[P] + s_rows[P])) ++P;
-    const int q = s_q[P] + (gi - s_off[P]);
-    const int r = head_list[gi] >> 3;
-    const float s = rsqrtf(ss[r] / (float)H + eps);
-    const float4 x0 = __ldcg(reinterpret_cast<const float4*>(X + (size_t)r * H + k));
-    const float4 x1 = __ldcg(reinterpret_cast<const float4*>(X + (size_t)r * H + k + 4));
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gain + k));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gain + k + 4));
-    const float v[8] = {x0.x * g0.x * s, x0.y * g0.y * s, x0.z * g0.z * s, x0.w * g0.w * s,
-                        x1.x * g1.x * s, x1.y * g1.y * s, x1.z * g1.z * s, x1.w * g1.w * s};
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      h[t] = pack_bf16x2(v[2 * t], v[2 * t + 1]);
-      l[t] = pack_bf16x2(v[2 * t] - bf16_lo_f32(h[t]), v[2 * t + 1] - bf16_hi_f32(h[t]));
-    }
-    const size_t off = tc::sw128_offset(Qcap, q, ch >> 3, ch & 7);
-    *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
-  }
-}
 
 // Logits of every pair: tile blockIdx.x (counted over the groups in head order) of head P's
 // group times head P's weights (m-tile blockIdx.y), plus the draft-offset bias for j >= 1.
@@ -1062,7 +1063,7 @@ __device__ __forceinline__ int tree_row_slot(const DevState* st, int r) {
 
 // pack: one thread per row.
 __global__ void __launch_bounds__(128) batch_tree_pack_kernel(FrameParams p, BatchBufs b) {
-  __shared__ int s_head[16], s_hcur[16], s_rows, s_pairs;
+  __shared__ int s_head[16], s_hcur[16], s_shift[16], s_rows, s_pairs;
   const BatchFrame* fa = b.frame;
   const TreeDef& tree = fa->tree;
   const DevState* st = p.st;
@@ -1112,12 +1113,14 @@ __global__ void __launch_bounds__(128) batch_tree_pack_kernel(FrameParams p, Bat
   }
   __syncthreads();
   if (r == 0) {
-    int off = 0;
+    int off = 0, q = 0;
     for (int P = 0; P < 16; ++P) {
       b.info->head_rows[P] = s_head[P];
       b.info->head_off[P] = off;
       s_hcur[P] = off;
+      s_shift[P] = q - off;              // operand rows: groups padded to 16
       off += s_head[P];
+      q += (s_head[P] + 15) / 16 * 16;
     }
     b.info->M = s_rows;
     b.info->n_pairs = off;
@@ -1126,9 +1129,15 @@ __global__ void __launch_bounds__(128) batch_tree_pack_kernel(FrameParams p, Bat
     b.info->next_call = call + 1;
   }
   __syncthreads();
-  for (int j = 0; j <= kn; ++j) {
-    b.pairs[atomicAdd(&s_pairs, 1)] = (r << 3) | j;
-    b.head_list[atomicAdd(&s_hcur[pos + j], 1)] = (r << 3) | j;
+  for (int j = 0; j < kRecSlots && pos >= 0; ++j) {
+    int slot = -1;
+    if (j <= kn) {
+      b.pairs[atomicAdd(&s_pairs, 1)] = (r << 3) | j;
+      const int at = atomicAdd(&s_hcur[pos + j], 1);
+      b.head_list[at] = (r << 3) | j;
+      slot = at + s_shift[pos + j];
+    }
+    b.head_slot[r * kRecSlots + j] = slot;
   }
 }
 
@@ -1373,6 +1382,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
   BATCH_ALLOC(b.sbase, sizeof(int) * kMaxBatchStreams);
   BATCH_ALLOC(b.pairs, sizeof(int) * R * kRecSlots);
   BATCH_ALLOC(b.head_list, sizeof(int) * R * kRecSlots);
+  BATCH_ALLOC(b.head_slot, sizeof(int) * R * kRecSlots);
   BATCH_ALLOC(b.X, sizeof(float) * R * p.H);
   BATCH_ALLOC(b.ss, sizeof(float) * (2 * p.L + 1) * R);
   BATCH_ALLOC(b.att, sizeof(uint16_t) * R * p.NH * p.D);
@@ -1460,17 +1470,23 @@ static int split_k(dim3 grid, int K, int n_sm) {
   return z;
 }
 
-// Final RMSNorm -> LM heads on the tensor cores, tiles grouped by head.
+// LM heads on the tensor cores, tiles grouped by head (operand: the last residual pass).
 static void enqueue_heads(const FrameParams& p, const BatchState* bs, cudaStream_t s) {
   const BatchBufs& b = bs->b;
-  const int R = b.R, L = p.L, H = p.H;
-  const dim3 blk(256);
-  tc::launch(false, tc_heads_operand_kernel, dim3(512), blk, 0, s, b.X, p.final_norm, b.ss + (size_t)(2 * L) * R, H, p.eps, b.info,
-                                             b.head_list, p.P, b.Qcap, b.hq_hi, b.hq_lo);
+  const int R = b.R, H = p.H;
   const tc::GemmArgs g{nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns, false, 0};
   tc::launch(false, tc_heads_kernel, dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
                  tc::Layout<kHeadTileMax, true>::kSmemBytes, s, g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
                                                                     p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
+}
+
+// The operand a residual pass leaves: the next layer's QKV operand, or after the last layer the LM
+// heads' (where they run on the tensor cores).
+static NormOut after_layer(const FrameParams& p, const BatchState* bs, int l) {
+  const BatchBufs& b = bs->b;
+  if (l + 1 < p.L) return NormOut{p.attn_norm + (size_t)(l + 1) * p.H, b.xn_hi, b.xn_lo, nullptr, 0};
+  if (bs->tw.heads) return NormOut{p.final_norm, b.hq_hi, b.hq_lo, b.head_slot, b.Qcap};
+  return NormOut{nullptr, nullptr, nullptr, nullptr, 0};
 }
 
 // Every kernel of one call, in stream order on `s`.
@@ -1485,29 +1501,28 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
   // node the last bodies of a frame are empty: no prefetch there.
   const bool pdl = loop.valid != 0;
   batch_pack_kernel<<<1, 256, 0, s>>>(p, b);
-  tc::launch(false, batch_embed_kernel, dim3(R), blk, 0, s, p, b);
+  if (bs->use_tc) batch_embed_tc_kernel<<<R, 128, 0, s>>>(p, b);
+  else batch_embed_kernel<<<R, 256, 0, s>>>(p, b);
   for (int l = 0; l < L && bs->use_tc; ++l) {
     const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
     const int Rtc = b.Rtc, qd = p.NH * p.D;
-    // RMSNorm -> QKV (hi + lo operand; after layer 0 written by the previous layer's last
+    const int* M = &b.info->M;
+    // RMSNorm -> QKV (hi + lo operand, written by the embedding or the previous layer's last
     // residual pass)
-    if (l == 0)
-      tc::launch(false, tc_norm_operand_kernel, dim3(256), blk, 0, s, b.X, p.attn_norm, b.ss, H, p.eps, &b.info->M, Rtc, b.xn_hi,
-                     b.xn_lo);
-    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc::launch(false, batch_attn_kernel, dim3(bs->max_streams, p.NKV), blk, 0, s, p, b, l);      // -> att_t
-    // Wo (k-split partials) -> residual, ss, the gate/up operand
-    tc_launch_resid<false>(wl + bs->tw.off.o, b.att_t, nullptr, b.part, H, Rtc, qd, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, R, b.X, b.part, qd, Rtc, H, p.n_cta, &b.info->M, b.ss + (size_t)(2 * l + 1) * R,
-                                           p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, (uint8_t*)nullptr, s);
+    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
+    // Wo (k-split partials) -> residual, the gate/up operand
+    tc_launch_resid<false>(wl + bs->tw.off.o, b.att_t, nullptr, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid_norm(false, R, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, nullptr, nullptr, 0}, s);
     // gate/up -> SwiGLU (into the down product's operand)
-    tc_launch_gu<false>(wl + bs->tw.off.gu, b.xn_hi, nullptr, b.act_t, nullptr, Rtc, &b.info->M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
-    // down (k-split partials) -> residual, ss, the next layer's QKV operand
-    tc_launch_resid<false>(wl + bs->tw.off.d, b.act_t, nullptr, b.part, H, Rtc, p.F, &b.info->M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    const bool last = l + 1 == L;
-    tc_launch_resid_norm(false, R, b.X, b.part, p.F, Rtc, H, p.n_cta, &b.info->M, b.ss + (size_t)(2 * l + 2) * R,
-                                           last ? (const float*)nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi, b.xn_lo, s);
+    tc_launch_gu<false>(wl + bs->tw.off.gu, b.xn_hi, nullptr, b.act_t, nullptr, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
+    // down (k-split partials) -> residual, the next operand
+    tc_launch_resid<false>(wl + bs->tw.off.d, b.act_t, nullptr, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_resid_norm(false, R, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
   }
+  if (bs->use_tc && !bs->tw.heads)      // the general LM heads read the rows' sums of squares
+    batch_rowss_kernel<<<(R + 7) / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * L) * R, b.info);
   for (int l = 0; l < L && !bs->use_tc; ++l) {
     {   // RMSNorm -> QKV
       GemmArgs a = gemm_args(p, b);
@@ -1583,26 +1598,23 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
 // Every kernel of one tree call.
 static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs, const BatchLoop& loop, cudaStream_t s) {
   const BatchBufs& b = bs->b;
-  const int R = b.R, L = p.L, H = p.H, Rtc = b.Rtc, qd = p.NH * p.D;
+  const int L = p.L, H = p.H, Rtc = b.Rtc, qd = p.NH * p.D;
   const dim3 blk(256);
   const bool pdl = loop.valid != 0;
   const int* M = &b.info->M;
   batch_tree_pack_kernel<<<1, 128, 0, s>>>(p, b);
-  batch_embed_kernel<<<kMaxTreeRows, blk, 0, s>>>(p, b);
-  tc_norm_operand_kernel<<<64, blk, 0, s>>>(b.X, p.attn_norm, b.ss, H, p.eps, M, Rtc, b.xn_hi, b.xn_lo);
+  batch_embed_tc_kernel<<<kMaxTreeRows, 128, 0, s>>>(p, b);
   for (int l = 0; l < L; ++l) {
     const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
     tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
     batch_tree_rope_kernel<<<(kMaxTreeRows * (p.NH + 2 * p.NKV) + 7) / 8, blk, 0, s>>>(p, b, l);
     batch_tree_attn_kernel<<<(kMaxTreeRows * p.NH + 7) / 8, blk, 0, s>>>(p, b, l);
     tc_launch_resid<true>(wl + bs->tw.off.o, b.att_t, b.att_lo, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, qd, Rtc, H, p.n_cta, M, b.ss + (size_t)(2 * l + 1) * R,
-                                                      p.ffn_norm + (size_t)l * H, p.eps, b.xn_hi, b.xn_lo, s);
+    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, b.xn_lo, nullptr, 0}, s);
     tc_launch_gu<true>(wl + bs->tw.off.gu, b.xn_hi, b.xn_lo, b.act_t, b.act_lo, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + bs->tw.off.d, b.act_t, b.act_lo, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, b.ss + (size_t)(2 * l + 2) * R,
-                                                      l + 1 == L ? nullptr : p.attn_norm + (size_t)(l + 1) * H, p.eps, b.xn_hi,
-                                                      b.xn_lo, s);
+    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
   }
   enqueue_heads(p, bs, s);
   batch_topk_kernel<<<kMaxTreeRows * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);

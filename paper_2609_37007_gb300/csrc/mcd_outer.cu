@@ -597,7 +597,6 @@ struct OuterTc {
   uint8_t* w = nullptr;            // per layer: SW128 copies of the weights
   TcLayerOffsets off;
   float* X = nullptr;              // [Rtc][H] residual stream
-  float* ss = nullptr;             // [Rtc] sums of squares (the next RMSNorm)
   float* qkv = nullptr;            // [Rtc][qkv_dim]
   float* q = nullptr;              // [Rtc][NH * D] normalised, rotated queries
   float* part = nullptr;           // [kTcSplit][Rtc][H] partial sums of the residual products
@@ -607,38 +606,41 @@ struct OuterTc {
 
 __global__ void pf_set_rows_kernel(int* rows, int n) { *rows = n; }
 
-// Prompt rows: X = the rows' text embeddings (bf16 table), ss = their sums of squares.  One
-// CTA per row, thread t owns elements 8t..8t+7.
+// Prompt rows: X = the rows' text embeddings (bf16 table) and layer 0's QKV operand.  One CTA per
+// row, thread t owns elements 8t..8t+7.
 __global__ void __launch_bounds__(128) pf_embed_kernel(const int* __restrict__ ids, const int* nrows,
                                                        const uint8_t* __restrict__ table, int vocab, int H, float* X,
-                                                       float* ss, int* err) {
+                                                       const float* __restrict__ gain, float eps, int Rtc, uint8_t* hi,
+                                                       uint8_t* lo, int* err) {
   tc::pdl_wait();
   tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= *nrows) return;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int t = threadIdx.x;
   int id = ids[r];
   if (id < 0 || id >= vocab) {              // an id outside the text table fails the prefill
     if (t == 0) atomicCAS(err, 0, (int)MCD_ERR_INVALID_ARG);
     id = 0;
   }
-  __shared__ float red[4];
+  const bool live = t < H / 8;
+  float v[8];
   float s2 = 0.f;
-  if (t < H / 8) {
+  if (live) {
     const uint4 w = __ldg(reinterpret_cast<const uint4*>(table + ((size_t)id * H + 8 * t) * 2));
-    const float v[8] = {bf16_lo_f32(w.x), bf16_hi_f32(w.x), bf16_lo_f32(w.y), bf16_hi_f32(w.y),
-                        bf16_lo_f32(w.z), bf16_hi_f32(w.z), bf16_lo_f32(w.w), bf16_hi_f32(w.w)};
+    v[0] = bf16_lo_f32(w.x); v[1] = bf16_hi_f32(w.x); v[2] = bf16_lo_f32(w.y); v[3] = bf16_hi_f32(w.y);
+    v[4] = bf16_lo_f32(w.z); v[5] = bf16_hi_f32(w.z); v[6] = bf16_lo_f32(w.w); v[7] = bf16_hi_f32(w.w);
     float4* xr = reinterpret_cast<float4*>(X + (size_t)r * H + 8 * t);
     xr[0] = make_float4(v[0], v[1], v[2], v[3]);
     xr[1] = make_float4(v[4], v[5], v[6], v[7]);
 #pragma unroll
     for (int i = 0; i < 8; ++i) s2 += v[i] * v[i];
   }
-#pragma unroll
-  for (int off = 16; off; off >>= 1) s2 += __shfl_xor_sync(0xFFFFFFFFu, s2, off);
-  if (lane == 0) red[warp] = s2;
-  __syncthreads();
-  if (t == 0) ss[r] = red[0] + red[1] + red[2] + red[3];
+  const float tot = block_sum128(s2);
+  if (!live) return;
+  const NormChunk c = norm_chunk(v, rsqrtf(tot / (float)H + eps), gain, t);
+  const size_t off = tc::sw128_offset(Rtc, r, t >> 3, t & 7);
+  *reinterpret_cast<uint4*>(hi + off) = c.hi;
+  *reinterpret_cast<uint4*>(lo + off) = c.lo;
 }
 
 // QK-norm + RoPE (position = row index) of every prompt row's query and key heads; K and V
@@ -1157,7 +1159,6 @@ mcd_status mcd_outer_create(const mcd_outer_config* cfg, mcd_ctx* inner, mcd_out
     t.off = tc_layer_offsets(p);
     OUTER_ALLOC(t.w, t.off.layer * p.L);
     OUTER_ALLOC(t.X, sizeof(float) * (size_t)Rtc * p.H);
-    OUTER_ALLOC(t.ss, sizeof(float) * (size_t)Rtc);
     OUTER_ALLOC(t.qkv, sizeof(float) * (size_t)std::max(Rtc, kTcQkvSplit * std::min(Rtc, kTcSmallRows)) * p.qkv_dim);
     OUTER_ALLOC(t.q, sizeof(float) * (size_t)Rtc * p.NH * p.D);
     OUTER_ALLOC(t.part, sizeof(float) * tc_part_floats(Rtc, p.H));
@@ -1299,8 +1300,8 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
   // every kernel a dependent launch: 2333 us for a 256-token prompt, 2444 with the products alone
   const bool pdl = true;
   pf_set_rows_kernel<<<1, 1, 0, s>>>(t.rows, n);
-  tc::launch(pdl, pf_embed_kernel, dim3(n), dim3(128), 0, s, text_ids, t.rows, st.text_table, st.text_vocab, H, t.X, t.ss, p.err);
-  tc::launch(pdl, tc_norm_operand_kernel, dim3(256), dim3(256), 0, s, t.X, p.attn_norm, t.ss, H, p.eps, t.rows, Rtc, t.xn_hi, t.xn_lo);
+  tc::launch(pdl, pf_embed_kernel, dim3(n), dim3(128), 0, s, text_ids, t.rows, st.text_table, st.text_vocab, H, t.X,
+             p.attn_norm, p.eps, Rtc, t.xn_hi, t.xn_lo, p.err);
   for (int l = 0; l < L; ++l) {
     const uint8_t* wl = t.w + (size_t)l * t.off.layer;
     uint16_t* kc = reinterpret_cast<uint16_t*>(st.kcache) + (size_t)l * kvl;
@@ -1313,13 +1314,12 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
                                                          st.rope, kc, vc, st.cap, t.q);
     launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, t.att_lo, s);
     tc_launch_resid<true>(wl + t.off.o, t.att_t, t.att_lo, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(pdl, n, t.X, t.part, qd, Rtc, H, p.n_cta, t.rows, t.ss, p.ffn_norm + (size_t)l * H,
-                                           p.eps, t.xn_hi, t.xn_lo, s);
+    tc_launch_resid_norm(pdl, n, t.X, t.part, qd, Rtc, H, p.n_cta, t.rows, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, t.xn_hi, t.xn_lo, nullptr, 0}, s);
     tc_launch_gu<true>(wl + t.off.gu, t.xn_hi, t.xn_lo, t.act_t, t.act_lo, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + t.off.d, t.act_t, t.act_lo, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(pdl, n, t.X, t.part, p.F, Rtc, H, p.n_cta, t.rows, t.ss,
-                                           l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : (const float*)nullptr, p.eps, t.xn_hi,
-                                           t.xn_lo, s);
+    tc_launch_resid_norm(pdl, n, t.X, t.part, p.F, Rtc, H, p.n_cta, t.rows, p.eps,
+                         NormOut{l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : nullptr, t.xn_hi, t.xn_lo, nullptr, 0}, s);
   }
   MCD_CHECK(cudaGetLastError());
   return MCD_OK;

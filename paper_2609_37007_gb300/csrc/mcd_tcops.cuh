@@ -17,33 +17,32 @@ namespace mcd {
 namespace {
 
 
-// Normalised operand rows x * gain / rms(x) of the call's packed rows as SW128 tiles (hi; with
-// lo also the bf16 remainder), one 8-element chunk per thread.
-__global__ void __launch_bounds__(256) tc_norm_operand_kernel(const float* __restrict__ X, const float* __restrict__ gain,
-                                                              const float* __restrict__ ss, int H, float eps,
-                                                              const int* nrows, int Rtc, uint8_t* hi, uint8_t* lo) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
-  const int M = *nrows, cpr = H / 8;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M * cpr; i += gridDim.x * blockDim.x) {
-    const int r = i / cpr, ch = i - r * cpr, k = ch * 8;
-    const float s = rsqrtf(ss[r] / (float)H + eps);
-    const float4 x0 = __ldcg(reinterpret_cast<const float4*>(X + (size_t)r * H + k));
-    const float4 x1 = __ldcg(reinterpret_cast<const float4*>(X + (size_t)r * H + k + 4));
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gain + k));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gain + k + 4));
-    const float v[8] = {x0.x * g0.x * s, x0.y * g0.y * s, x0.z * g0.z * s, x0.w * g0.w * s,
-                        x1.x * g1.x * s, x1.y * g1.y * s, x1.z * g1.z * s, x1.w * g1.w * s};
-    uint32_t h[4], l[4];
+// Eight elements 8t.. of a row, times gain and 1/rms, as the hi (and with lo also the remainder)
+// halves of a product's operand.
+struct NormChunk {
+  uint4 hi, lo;
+};
+__device__ __forceinline__ NormChunk norm_chunk(const float (&x)[8], float inv_rms, const float* __restrict__ gain, int t) {
+  const float4 g0 = __ldg(reinterpret_cast<const float4*>(gain + 8 * t));
+  const float4 g1 = __ldg(reinterpret_cast<const float4*>(gain + 8 * t + 4));
+  const float v[8] = {x[0] * g0.x * inv_rms, x[1] * g0.y * inv_rms, x[2] * g0.z * inv_rms, x[3] * g0.w * inv_rms,
+                      x[4] * g1.x * inv_rms, x[5] * g1.y * inv_rms, x[6] * g1.z * inv_rms, x[7] * g1.w * inv_rms};
+  uint32_t h[4], l[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
-      l[q] = pack_bf16x2(v[2 * q] - bf16_lo_f32(h[q]), v[2 * q + 1] - bf16_hi_f32(h[q]));
-    }
-    const size_t off = tc::sw128_offset(Rtc, r, ch >> 3, ch & 7);
-    *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-    if (lo) *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+  for (int q = 0; q < 4; ++q) {
+    h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+    l[q] = pack_bf16x2(v[2 * q] - bf16_lo_f32(h[q]), v[2 * q + 1] - bf16_hi_f32(h[q]));
   }
+  return NormChunk{make_uint4(h[0], h[1], h[2], h[3]), make_uint4(l[0], l[1], l[2], l[3])};
+}
+// Sum of s over the CTA's 128 threads (one barrier).
+__device__ __forceinline__ float block_sum128(float s) {
+  __shared__ float red[4];
+#pragma unroll
+  for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  return red[0] + red[1] + red[2] + red[3];
 }
 
 // Row-major bf16 [rows][K] -> an SW128-tiled matrix of R rows (weight load): source row r
@@ -208,21 +207,27 @@ __global__ void __launch_bounds__(kResidThreads, 1) tc_resid_kernel(const tc::Ge
   });
 }
 
+// Where a residual pass writes the row's normalised operand: `hi` / `lo` of Rtc rows at the row
+// itself; after the last layer, with `slots` (eight per row, -1: none), at those rows of the LM
+// heads' operand of slot_rows rows instead.
+struct NormOut {
+  const float* gain;          // null: no operand
+  uint8_t *hi, *lo;
+  const int* slots;
+  int slot_rows;
+};
 // Per packed row (one CTA, thread t owns elements 8t..8t+7): X += the nz partial sums, the
-// row's sum of squares (the next RMSNorm), and with a gain the next product's normalised
-// operand (hi; with lo also the remainder) as SW128 tiles.
+// row's sum of squares (the next RMSNorm), and the next product's normalised operand as SW128
+// tiles.
 template <int NZ>       // partial sums held in registers (nz <= NZ)
 __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const float* __restrict__ part, int nz, int Rtc,
-                                                            int H, const int* nrows, float* ss_out,
-                                                            const float* __restrict__ gain, float eps, uint8_t* hi,
-                                                            uint8_t* lo) {
+                                                            int H, const int* nrows, float eps, const NormOut out) {
   tc::pdl_wait();
   tc::pdl_trigger();
   const int r = blockIdx.x;
   if (r >= *nrows) return;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int t = threadIdx.x;
   const bool live = t < H / 8;
-  __shared__ float red[4];
   float x[8];
   float ss = 0.f;
   if (live) {
@@ -251,27 +256,21 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
 #pragma unroll
     for (int i = 0; i < 8; ++i) ss += x[i] * x[i];
   }
-#pragma unroll
-  for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
-  if (lane == 0) red[warp] = ss;
-  __syncthreads();
-  const float tot = red[0] + red[1] + red[2] + red[3];
-  if (t == 0) ss_out[r] = tot;
-  if (gain && live) {
-    const float s = rsqrtf(tot / (float)H + eps);
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gain + 8 * t));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gain + 8 * t + 4));
-    const float v[8] = {x[0] * g0.x * s, x[1] * g0.y * s, x[2] * g0.z * s, x[3] * g0.w * s,
-                        x[4] * g1.x * s, x[5] * g1.y * s, x[6] * g1.z * s, x[7] * g1.w * s};
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
-      l[q] = pack_bf16x2(v[2 * q] - bf16_lo_f32(h[q]), v[2 * q + 1] - bf16_hi_f32(h[q]));
-    }
+  const float tot = block_sum128(ss);
+  if (!out.gain || !live) return;
+  const NormChunk c = norm_chunk(x, rsqrtf(tot / (float)H + eps), out.gain, t);
+  if (!out.slots) {
     const size_t off = tc::sw128_offset(Rtc, r, t >> 3, t & 7);
-    *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-    if (lo) *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+    *reinterpret_cast<uint4*>(out.hi + off) = c.hi;
+    if (out.lo) *reinterpret_cast<uint4*>(out.lo + off) = c.lo;
+  } else {
+    for (int j = 0; j < 8; ++j) {
+      const int q = out.slots[8 * r + j];
+      if (q < 0) continue;
+      const size_t off = tc::sw128_offset(out.slot_rows, q, t >> 3, t & 7);
+      *reinterpret_cast<uint4*>(out.hi + off) = c.hi;
+      *reinterpret_cast<uint4*>(out.lo + off) = c.lo;
+    }
   }
 }
 
@@ -428,14 +427,12 @@ inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, const uint8_t*
 
 // The residual pass of a product over K (tc_resid_norm_kernel) on `rows` CTAs.
 inline void tc_launch_resid_norm(bool pdl, int rows, float* X, const float* part, int K, int Rtc, int H, int n_sm,
-                                 const int* nrows, float* ss_out, const float* gain, float eps, uint8_t* hi, uint8_t* lo,
-                                 cudaStream_t s) {
+                                 const int* nrows, float eps, const NormOut& out, cudaStream_t s) {
   const int nz = tc_splits(K, tc_resid_shape(H, Rtc, n_sm).z);
   if (nz <= 6)
-    tc::launch(pdl, tc_resid_norm_kernel<6>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, ss_out, gain, eps, hi, lo);
+    tc::launch(pdl, tc_resid_norm_kernel<6>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, eps, out);
   else
-    tc::launch(pdl, tc_resid_norm_kernel<kTcSplit>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, ss_out, gain, eps,
-               hi, lo);
+    tc::launch(pdl, tc_resid_norm_kernel<kTcSplit>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, eps, out);
 }
 // Floats of partial sums a residual product leaves at up to Rtc operand rows.
 inline size_t tc_part_floats(int Rtc, int H) {

@@ -869,17 +869,23 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParam
   TopkScratch& ts = *reinterpret_cast<TopkScratch*>(smem_raw);
   tc::pdl_wait();
   tc::pdl_trigger();
+  const int call = b.info->call, n_pair_ctas = (int)gridDim.x - b.R;
+  if ((int)blockIdx.x >= n_pair_ctas) {     // packed row r's verify logits into an optional trace
+    const int r = (int)blockIdx.x - n_pair_ctas;
+    if (!b.frame->trace || call >= kMaxCalls || r >= b.info->M || b.head_slot[r * kRecSlots] < 0) return;
+    const BatchRow row = b.rows[r];
+    uint8_t* tb = b.frame->trace + (size_t)row.s * p.trace_stride + sizeof(mcd_call_trace) * kMaxCalls;
+    float* dst = reinterpret_cast<float*>(tb) + ((size_t)call * kMaxRows + row.n) * p.V;
+    if (p.draft_mode == MCD_DRAFT_TREE)
+      dst = reinterpret_cast<float*>(tb + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4 + sizeof(mcd_tree_trace) * kMaxCalls) +
+            ((size_t)call * kMaxTreeRows + row.n) * p.V;
+    copy_logits(dst, b.logits + (size_t)r * kRecSlots * p.V, p.V);
+    return;
+  }
   if ((int)blockIdx.x >= b.info->n_pairs) return;
   const int e = b.pairs[blockIdx.x], r = e >> 3, j = e & 7;
   const int greedy = (j > 0 && p.draft_mode == MCD_DRAFT_GREEDY) ? 1 : 0;
-  const int call = b.info->call;
   TopkRec* recs = b.recs + (size_t)(call & 1) * b.R * kRecSlots;
-  if (p.draft_mode == MCD_DRAFT_TREE && j == 0 && b.frame->trace && call < kMaxCalls) {
-    // a tree call's verify logits, one row per CTA (the chain's are copied by its acceptance)
-    uint8_t* tb = b.frame->trace + sizeof(mcd_call_trace) * kMaxCalls + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4 +
-                  sizeof(mcd_tree_trace) * kMaxCalls;
-    copy_logits(reinterpret_cast<float*>(tb) + ((size_t)call * kMaxTreeRows + r) * p.V, b.logits + (size_t)r * kRecSlots * p.V, p.V);
-  }
   block_topk(b.logits + ((size_t)r * kRecSlots + j) * p.V, p.V, p.top_k, p.T, greedy, ts,
              recs + (size_t)r * kRecSlots + j);
 }
@@ -911,7 +917,6 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FramePar
   __shared__ AcceptResult s_res;
   __shared__ int s_next[kMaxDraft], s_old[kMaxDraft + 1];
   const int a = st->a, n_d = st->n_d, pos0 = st->pos0, n_rows = st->n_rows, qrow = st->q_row;
-  const int fr = st->first_head_row;
   if (threadIdx.x <= kMaxDraft) s_old[threadIdx.x] = (int)threadIdx.x < n_d ? st->drafts[threadIdx.x] : -1;
   __syncthreads();
   const unsigned sid = fa->stream_ids[s], fid = fa->frame_ids[s];
@@ -1025,27 +1030,28 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FramePar
   if (fa->trace && call < kMaxCalls) {
     uint8_t* tb = fa->trace + (size_t)s * p.trace_stride;
     mcd_call_trace* tr = reinterpret_cast<mcd_call_trace*>(tb) + call;
-    if (threadIdx.x == 0) {
-      tr->a = a;
-      tr->n_rows = n_rows;
-      tr->pos0 = pos0;
-      tr->n_drafts = n_d;
-      for (int n = 0; n < kMaxRows; ++n) tr->input_ids[n] = n < n_rows ? b.rows[base + n].id : -1;
-      for (int i = 0; i < kMaxRows; ++i) tr->drafts[i] = i < n_d ? s_old[i] : -1;
-      tr->n_acc = n_acc;
-      tr->n_emit = n_emit;
-      for (int t = 0; t < kMaxRows; ++t) tr->emitted[t] = t < n_emit ? s_res.emitted[t] : -1;
-      tr->n_next = n_next;
-      for (int j = 0; j < kMaxRows; ++j) tr->next_drafts[j] = j < n_next ? s_next[j] : -1;
-      tr->draft_row = m;
+    if (threadIdx.x < kMaxRows) {
+      const int t = threadIdx.x;
+      tr->input_ids[t] = t < n_rows ? b.rows[base + t].id : -1;
+      tr->drafts[t] = t < n_d ? s_old[t] : -1;
+      tr->emitted[t] = t < n_emit ? s_res.emitted[t] : -1;
+      tr->next_drafts[t] = t < n_next ? s_next[t] : -1;
+      if (t == 0) {
+        tr->a = a;
+        tr->n_rows = n_rows;
+        tr->pos0 = pos0;
+        tr->n_drafts = n_d;
+        tr->n_acc = n_acc;
+        tr->n_emit = n_emit;
+        tr->n_next = n_next;
+        tr->draft_row = m;
+      }
     }
-    float* vlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls);
-    float* dlog = vlog + (size_t)kMaxCalls * kMaxRows * p.V;
-    for (int n = fr; n < n_rows; ++n)
-      copy_logits(vlog + ((size_t)call * kMaxRows + n) * p.V, b.logits + (size_t)(base + n) * kRecSlots * p.V, p.V);
-    for (int n = 0; n < n_next; ++n)
-      copy_logits(dlog + ((size_t)call * kMaxRows + n) * p.V,
-                  b.logits + ((size_t)(base + m) * kRecSlots + n + 1) * p.V, p.V);
+    // the draft logits (the verify logits were copied beside the distributions)
+    float* dlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls) + (size_t)kMaxCalls * kMaxRows * p.V +
+                  (size_t)call * kMaxRows * p.V;
+    const float* lg = b.logits + ((size_t)(base + m) * kRecSlots + 1) * p.V;
+    copy_logits(dlog, lg, n_next * p.V);               // consecutive rows on both sides
   }
   if (threadIdx.x == 0) batch_call_end(p, b, loop, call, a_new < p.P);
 }
@@ -1590,7 +1596,7 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>
         <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN, p.P), blk, kGemmSmemHilo, s>>>(a);
   }
-  tc::launch(false, batch_topk_kernel, dim3(R * (p.K + 1)), dim3(kConsumerThreads), 0, s, p, b);
+  tc::launch(false, batch_topk_kernel, dim3(R * (p.K + 1) + R), dim3(kConsumerThreads), 0, s, p, b);
   tc::launch(false, batch_accept_kernel, dim3(bs->max_streams), dim3(kConsumerThreads), 0, s, p, b, loop);
   return cudaGetLastError();
 }
@@ -1617,7 +1623,7 @@ static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs,
     tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
   }
   enqueue_heads(p, bs, s);
-  batch_topk_kernel<<<kMaxTreeRows * (p.K + 1), kConsumerThreads, 0, s>>>(p, b);
+  batch_topk_kernel<<<kMaxTreeRows * (p.K + 1) + b.R, kConsumerThreads, 0, s>>>(p, b);
   batch_tree_accept_kernel<<<1, kConsumerThreads, 0, s>>>(p, b, loop);
   return cudaGetLastError();
 }

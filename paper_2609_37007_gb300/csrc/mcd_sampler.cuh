@@ -14,6 +14,7 @@
 // same fp32 exp32 agrees bit for bit; sums are order-free and need no fp64 arithmetic.
 #pragma once
 #include <cstddef>
+#include <type_traits>
 
 #include "mcd_internal.cuh"
 
@@ -30,6 +31,9 @@ struct TopkScratch {
   unsigned long long wsum[kConsumerWarps];
   uint32_t kept_key[kMaxTopK];           // the set in id order: keys and ids
   int kept_id[kMaxTopK];
+  static constexpr int kCand = kConsumerThreads;
+  __align__(16) uint32_t ckey[kCand];    // candidates of the set in id order: keys and ids
+  int cid[kCand];
 };
 static_assert(sizeof(TopkScratch) <= kActBytes, "top-k scratch must fit the activation region");
 
@@ -128,7 +132,16 @@ __device__ __forceinline__ uint32_t block_exscan(uint32_t v, TopkScratch& s, int
 // Block-wide (256 consumer threads) top-k of one fp32 row (V % 16 == 0, V <= 4096) into `out`
 // (global or shared), listed in ascending id order.  Thread t holds the keys of the E = 4 nj
 // consecutive ids E t .. E t + E - 1 (nj = ceil(V / 1024)) in registers, so thread order is id
-// order.  Finding the k-th largest key Tk:
+// order.  The usual form: every thread's largest key enters a 256-bin histogram over the value range
+// (one shared-memory atomic per thread, not one per key); the highest bin B with at least k of these
+// keys in the bins from B on bounds the set from below, since k keys of the row lie there; the
+// row's keys from bin B on (for k of 256 threads about k to 1.4 k) are compacted in id order, one
+// per thread, which counts the keys that precede its own (larger, or equal with a lower id): the
+// set is the candidates that fewer than k precede.  A row of up to 128 keys is all candidates.
+// 2048 keys, k = 50: 3990 cycles, of which 990 load and bound the row; 5710 with every key in the
+// histogram and a division for its scale.  A chain of dependent steps bounds both.
+// With fewer than k threads that hold keys, more than 256 candidates or a non-finite range the general form finds
+// the k-th largest key Tk:
 //   (1) block maximum and minimum;
 //   (2) a 256-bin histogram over the value range [min, max] (bin = trunc((v - min) * 256 /
 //       (max - min)), a monotone function of the key, so every bin is an interval of keys);
@@ -156,17 +169,22 @@ static __device__ __noinline__ void block_topk_j(const float* __restrict__ logit
   const int E = 4 * nj;                            // ids per thread
   const int n_valid = max(0, min(E, V - E * tid)); // ids E*tid .. E*tid + n_valid - 1 exist
   uint32_t key[4 * kJ];
+  float val[4 * kJ];
 #pragma unroll
   for (int j = 0; j < kJ; ++j) {
     const bool ok = 4 * j < n_valid;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (ok) v = __ldcg(reinterpret_cast<const float4*>(logits) + (nj * tid + j));
+    val[4 * j + 0] = v.x;
+    val[4 * j + 1] = v.y;
+    val[4 * j + 2] = v.z;
+    val[4 * j + 3] = v.w;
     key[4 * j + 0] = ok ? f32_key(v.x) : 0u;
     key[4 * j + 1] = ok ? f32_key(v.y) : 0u;
     key[4 * j + 2] = ok ? f32_key(v.z) : 0u;
     key[4 * j + 3] = ok ? f32_key(v.w) : 0u;
   }
-  uint32_t kmax = 0, kmin = 0xFFFFFFFFu;
+  uint32_t kmax = 0, kmin = 0xFFFFFFFFu;         // the thread's, then the block's
 #pragma unroll
   for (int e = 0; e < 4 * kJ; ++e) {
     if (e < n_valid) {
@@ -174,6 +192,7 @@ static __device__ __noinline__ void block_topk_j(const float* __restrict__ logit
       kmin = min(kmin, key[e]);
     }
   }
+  const uint32_t tmax = kmax;
   kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
   kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
   if (lane == 0) {
@@ -213,19 +232,15 @@ static __device__ __noinline__ void block_topk_j(const float* __restrict__ logit
   // ---- the k-th largest key -----------------------------------------------------------------
   const float vmin = key_f32(kmin), vmax = key_f32(kmax);
   const float range = __fsub_rn(vmax, vmin);
-  const float scale = __fdiv_rn((float)kBins, range);
-  const bool binned = isfinite(vmin) && isfinite(vmax) && range > 0.f && isfinite(range) && isfinite(scale);
+  const float scale = __fdividef((float)kBins, range);      // any positive factor keeps the order
+  const bool binned = isfinite(vmin) && isfinite(vmax) && range > 0.f && isfinite(range) && scale > 0.f && isfinite(scale);
   auto bin_of = [&](uint32_t kk) {
     return min(kBins - 1, __float2int_rz(__fmul_rn(__fsub_rn(key_f32(kk), vmin), scale)));
   };
-  uint32_t Tk = 0;
-  bool found = false;
-  if (binned) {                                                     // block-uniform
-#pragma unroll
-    for (int e = 0; e < 4 * kJ; ++e)
-      if (e < n_valid) atomicAdd(&s.hist[bin_of(key[e])], 1u);
-    consumer_sync();
-    // lane L holds bins 8L .. 8L + 7; S(b) = #keys in bins >= b; B = the largest b with S(b) >= k
+  // B = the largest bin with S(B) >= k, S(b) = #keys in the histogram's bins >= b (S(0) >= k); with
+  // `count` also the keys of bin B and of the bins above it
+  auto select_bin = [&](auto count, uint32_t& cntB, uint32_t& aboveB) -> int {
+    // lane L holds bins 8L .. 8L + 7
     uint32_t c8[8];
     {
       const uint4 h0 = reinterpret_cast<const uint4*>(s.hist)[2 * lane];
@@ -233,9 +248,7 @@ static __device__ __noinline__ void block_topk_j(const float* __restrict__ logit
       c8[0] = h0.x; c8[1] = h0.y; c8[2] = h0.z; c8[3] = h0.w;
       c8[4] = h1.x; c8[5] = h1.y; c8[6] = h1.z; c8[7] = h1.w;
     }
-    uint32_t local = 0;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) local += c8[b];
+    const uint32_t local = ((c8[0] + c8[1]) + (c8[2] + c8[3])) + ((c8[4] + c8[5]) + (c8[6] + c8[7]));
     uint32_t suf = local;                                // keys in the bins of lanes >= L
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -255,9 +268,110 @@ static __device__ __noinline__ void block_topk_j(const float* __restrict__ logit
     }
     const unsigned has = __ballot_sync(0xFFFFFFFFu, b_sel >= 0);   // a prefix of the lanes
     const int src = 31 - __clz(has);
-    const int B = __shfl_sync(0xFFFFFFFFu, b_sel, src);
-    const uint32_t cntB = __shfl_sync(0xFFFFFFFFu, b_cnt, src);
-    const uint32_t aboveB = __shfl_sync(0xFFFFFFFFu, b_above, src);
+    if constexpr (decltype(count)::value) {
+      cntB = __shfl_sync(0xFFFFFFFFu, b_cnt, src);
+      aboveB = __shfl_sync(0xFFFFFFFFu, b_above, src);
+    }
+    return __shfl_sync(0xFFFFFFFFu, b_sel, src);
+  };
+  // ---- the usual form: candidates from the threads' largest keys ------------------------------
+  const bool all = V <= 128;
+  if (all || (binned && E * k <= V)) {                              // block-uniform
+    float edge = 0.f;                                               // candidates: keys of bins >= B
+    if (!all) {
+      if (n_valid > 0) atomicAdd(&s.hist[bin_of(tmax)], 1u);
+      consumer_sync();
+      uint32_t unused;
+      edge = (float)select_bin(std::false_type{}, unused, unused);  // V / E >= k threads hold keys
+    }
+    uint32_t in = 0;                                                // bit e: key e is a candidate
+#pragma unroll
+    for (int e = 0; e < 4 * kJ; ++e)
+      if (e < n_valid && (all || __fmul_rn(__fsub_rn(val[e], vmin), scale) >= edge)) in |= 1u << e;
+    MCD_TOPK_STAMP(2)
+    uint32_t n_cand;
+    uint32_t at = block_exscan(__popc(in), s, 0, &n_cand);
+    if (n_cand <= (uint32_t)TopkScratch::kCand) {                   // block-uniform
+#pragma unroll
+      for (int e = 0; e < 4 * kJ; ++e) {
+        if (in & (1u << e)) {
+          s.ckey[at] = key[e];
+          s.cid[at] = E * tid + e;
+          ++at;
+        }
+      }
+      if (tid >= (int)n_cand && tid < (int)((n_cand + 3) & ~3u)) s.ckey[tid] = 0u;    // precede nothing
+      consumer_sync();
+      MCD_TOPK_STAMP(3)
+      const bool mine = tid < (int)n_cand;
+      uint32_t w = 0, before = 0;
+      if (warp * 32 < (int)n_cand) {
+        const uint32_t ki = mine ? s.ckey[tid] : 0xFFFFFFFFu;
+        const float zmax = __fdiv_rn(key_f32(kmax), T);
+        const float z = __fdiv_rn(key_f32(mine ? ki : kmax), T);
+        w = weight24(exp32_cw(__fsub_rn(z, zmax)));
+        // candidates of earlier warps precede this warp's on equal keys, those of later warps do not
+        const int n4 = (int)(n_cand + 3) >> 2, q0 = 8 * warp, q1 = min(n4, q0 + 8);
+        const uint4* ck = reinterpret_cast<const uint4*>(s.ckey);
+#pragma unroll 4
+        for (int q = 0; q < q0; ++q) {
+          const uint4 c = ck[q];
+          before += (c.x >= ki ? 1u : 0u) + (c.y >= ki ? 1u : 0u) + (c.z >= ki ? 1u : 0u) + (c.w >= ki ? 1u : 0u);
+        }
+#pragma unroll 4
+        for (int q = q0; q < q1; ++q) {
+          const uint4 c = ck[q];
+          const int j = 4 * (q - q0);
+          before += c.x > ki || (c.x == ki && j < lane) ? 1u : 0u;
+          before += c.y > ki || (c.y == ki && j + 1 < lane) ? 1u : 0u;
+          before += c.z > ki || (c.z == ki && j + 2 < lane) ? 1u : 0u;
+          before += c.w > ki || (c.w == ki && j + 3 < lane) ? 1u : 0u;
+        }
+#pragma unroll 4
+        for (int q = q1; q < n4; ++q) {
+          const uint4 c = ck[q];
+          before += (c.x > ki ? 1u : 0u) + (c.y > ki ? 1u : 0u) + (c.z > ki ? 1u : 0u) + (c.w > ki ? 1u : 0u);
+        }
+      }
+      const bool keep = mine && before < (uint32_t)k;
+      const unsigned kept = __ballot_sync(0xFFFFFFFFu, keep);
+      const uint32_t ws = __reduce_add_sync(0xFFFFFFFFu, keep ? w : 0u);      // 32 weights <= 2^24
+      if (lane == 0) {
+        s.wred[1][warp] = __popc(kept);
+        s.wsum[warp] = ws;
+      }
+      consumer_sync();
+      MCD_TOPK_STAMP(4)
+      int pos = __popc(kept & ((1u << lane) - 1u));
+      unsigned long long S = 0;
+#pragma unroll
+      for (int v = 0; v < kConsumerWarps; ++v) {
+        pos += v < warp ? (int)s.wred[1][v] : 0;
+        S += s.wsum[v];
+      }
+      if (keep) {
+        out->ids[pos] = s.cid[tid];
+        out->W[pos] = w;
+      }
+      if (tid == 0) {
+        out->S = S;
+        out->n = k;
+      }
+      MCD_TOPK_STAMP(5)
+      return;
+    }
+    s.hist[tid] = 0u;
+    consumer_sync();
+  }
+  uint32_t Tk = 0;
+  bool found = false;
+  if (binned) {                                                     // block-uniform
+#pragma unroll
+    for (int e = 0; e < 4 * kJ; ++e)
+      if (e < n_valid) atomicAdd(&s.hist[bin_of(key[e])], 1u);
+    consumer_sync();
+    uint32_t cntB, aboveB;
+    const int B = select_bin(std::true_type{}, cntB, aboveB);       // V >= k keys
     if (cntB <= 32u) {                                               // block-uniform
 #pragma unroll
       for (int e = 0; e < 4 * kJ; ++e)

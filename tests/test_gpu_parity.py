@@ -121,6 +121,40 @@ def test_topk_softmax_matches_oracle(V, k, T, ties):
     dec.close()
 
 
+@pytest.mark.parametrize("V,k", [(16, 16), (128, 50), (128, 128), (144, 36), (144, 37), (1024, 128), (1040, 65), (2048, 1),
+                                 (2064, 128), (4080, 127), (4096, 128)])
+def test_topk_candidate_edges(V, k):
+    """The candidate form of the top-k at its limits: rows that are all candidates (V <= 128), k
+    around the number of threads that hold keys, sorted rows (more than 256 candidates), ties across
+    the threshold, masked (-inf) and lowest-value entries, one distinct value.  Exact."""
+    dec = mcd.Decoder(TINY.replace(vocab=V, top_k=k, temperature=0.9))
+    rng = np.random.default_rng(V * 131 + k)
+    rnd = lambda: rng.standard_normal(V).astype(np.float32) * np.float32(2)
+    rows = [rnd() for _ in range(4)] + [np.sort(rnd()), np.sort(rnd())[::-1].copy(), np.full(V, 0.25, np.float32),
+                                        np.round(rnd()), np.round(rnd() * 4) / 4]
+    two = np.zeros(V, np.float32)
+    two[rng.permutation(V)[: max(1, k // 2)]] = 1.0
+    masked, low = rnd(), rnd()
+    masked[rng.permutation(V)[: V - k]] = -np.inf
+    low[rng.permutation(V)[: V // 3]] = np.finfo(np.float32).min
+    one = np.full(V, -3.0, np.float32)
+    one[V - 1] = 5.0
+    logits = np.stack(rows + [two, masked, low, one])
+    n = len(logits)
+    ids = torch.zeros((n, k), dtype=torch.int32, device=DEV)
+    w = torch.zeros((n, k), dtype=torch.int32, device=DEV)
+    sums = torch.zeros(n, dtype=torch.int64, device=DEV)
+    mcd.mcd_topk_softmax(dec.ctx, n, t(logits), ids, w, sums)
+    mcd.mcd_sync(dec.ctx)
+    ids, w, sums = ids.cpu().numpy(), w.cpu().numpy().view(np.uint32), sums.cpu().numpy()
+    for r in range(n):
+        d = topk_dist(logits[r], k, 0.9)
+        assert ids[r].tolist() == d.ids, r
+        assert [int(v) for v in w[r]] == d.W, r
+        assert int(sums[r]) == d.S, r
+    dec.close()
+
+
 def _begin(dec, cfg, stream_id=0, frame_idx=0):
     fr = make_frame(cfg, 0)
     cond = t(fr.cond)

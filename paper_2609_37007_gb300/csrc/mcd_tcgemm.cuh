@@ -161,7 +161,8 @@ struct GemmArgs {
   const int* n_active;   // optional (device): columns n >= *n_active are not computed
   int* err;
   unsigned long long wait_ns;
-  bool ahead;            // kPdl: fetch weights before pdl_wait
+  int ahead;             // kPdl, before pdl_wait: 0 nothing, 1 the set-up and the first weights
+                         // (A is no earlier kernel's output), 2 the set-up alone
   int bn;                // gemm_tile: 0 = tiles of BN columns; else tile x covers columns
                          // x * bn .. min(N, (x + 1) * bn) - 1 (bn a multiple of 16, <= BN)
 };
@@ -262,7 +263,7 @@ __device__ __forceinline__ bool gemm_tile_run(const GemmArgs& g, TileRun& t, int
   const uint64_t pol_a = policy_evict_first(), pol_b = policy_evict_last();
   int a_issued = 0;                        // (producer) stages whose A copy is under way
   if constexpr (kPdl) {
-    if (g.ahead && producer && blockIdx.x == 0)   // the thread that initialised the barriers
+    if (g.ahead == 1 && producer && blockIdx.x == 0)   // the thread that initialised the barriers
       for (; a_issued < min(nk, S); ++a_issued) issue_a(a_issued, pol_a);
   }
   if (warp == 1) {

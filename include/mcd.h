@@ -315,7 +315,7 @@ typedef struct {
  * of more than 32 rows runs as passes of up to 32 rows through the whole model (rows
  * 32 t .. 32 t + 31 in pass t; later rows attend to earlier ones through the cache); the
  * acceptance step follows the last pass.  bf16 models whose widths suit the tensor-core
- * products run trees of 17 nodes or more in one pass on the batched kernels instead (one
+ * products run trees of 16 nodes or more in one pass on the batched kernels instead (one
  * CUDA graph launch per frame); n_passes and heads_read count passes of 32 rows either way.  Until
  * set, the tree is the chain of draft_len rank-0 nodes.  Errors: MCD_ERR_INVALID_ARG
  * (malformed tree), MCD_ERR_STATE (context not in TREE mode). */

@@ -66,7 +66,7 @@ constexpr int kBatchMinStreams = 5;
 // Launches of this many streams go to the batched path even when the frame kernel fits them.
 bool batch_prefers(const FrameParams& p, int n_streams);
 // TREE mode: the batched kernels can run the context's tree calls, and do from this many nodes on.
-constexpr int kBatchMinTreeNodes = 17;
+constexpr int kBatchMinTreeNodes = 16;
 bool batch_tree_supported(const FrameParams& p);
 bool batch_tree_prefers(int nodes);
 mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out);

@@ -295,6 +295,185 @@ __device__ void outer_attention(Cons& c, const OuterStep& o, int layer, int g, i
   consumer_sync();
 }
 
+// The same task for one row of the standard geometry (D = 128, two query heads per KV head, bf16
+// cache).  Everything that does not depend on the row's QKV product is under way before the grid
+// barrier in front of it: the block's cached K and V (cp.async, kept as bf16), the RoPE row and the
+// gains.  After it warps 0 and 1 take a query head each, warps 2 and 3 the new key and value where
+// the block holds the row's position; then four threads per (query, key) score, and each warp
+// takes the softmax statistics of its query (redundantly) and 32 of the output's dims.
+// A chain of L2 round trips and shuffles bounds it.  12 rows at 333 positions with their prompt:
+// 10253 us with the general task and merge (9.1 k and 4.0 k of 48 k cycles per layer, stamped),
+// 9015 with these.
+constexpr int kRowLd = 160;            // staged row (bf16): neighbouring keys 16 banks apart
+struct RowAttn {
+  uint16_t *kb, *vb;                   // [32][kRowLd]
+  float *qs, *sc;                      // queries [2][128], scores [2][32]
+  __device__ explicit RowAttn(float* act)
+      : kb(reinterpret_cast<uint16_t*>(act)), vb(kb + kKeyBlock * kRowLd),
+        qs(reinterpret_cast<float*>(vb + kKeyBlock * kRowLd)), sc(qs + 256) {}
+};
+static_assert(2 * kKeyBlock * kRowLd * 2 + (256 + 2 * kKeyBlock) * 4 <= kActBytes, "row attention scratch");
+struct RowAhead {
+  float gain[4];
+  float2 rope[2];
+};
+__device__ __noinline__ RowAhead row_attention_ahead(const FrameParams& p, const OuterStep& o, float* act, int layer, int g, int b) {
+  const RowAttn a(act);
+  RowAhead ra{};
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int j0 = b * kKeyBlock, n_old = min(kKeyBlock, o.pos0 - j0);
+  const size_t off = (((size_t)layer * p.NKV + g) * o.cap + j0) * 128;
+  const uint16_t* kc = reinterpret_cast<const uint16_t*>(o.kcache) + off;
+  const uint16_t* vc = reinterpret_cast<const uint16_t*>(o.vcache) + off;
+  for (int i = tid; i < n_old * 16; i += kConsumerThreads) {
+    const int jj = i >> 4, ch = 8 * (i & 15);
+    cpa16(a.kb + jj * kRowLd + ch, kc + jj * 128 + ch);
+    cpa16(a.vb + jj * kRowLd + ch, vc + jj * 128 + ch);
+  }
+  if (warp < 3) {
+    const float* gg = (warp < 2 ? p.q_norm : p.k_norm) + (size_t)layer * 128;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ra.gain[i] = p.qk_norm ? __ldg(gg + lane + 32 * i) : 1.f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) ra.rope[i] = __ldg(o.rope + (size_t)o.pos0 * 64 + lane + 32 * i);
+  }
+  return ra;
+}
+__device__ __noinline__ void row_attention(const FrameParams& p, const OuterStep& o, float* act, int layer, int g, int b,
+                                           RowAhead ra) {
+  const RowAttn a(act);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pos0 = o.pos0;
+  const int j0 = b * kKeyBlock, nk = min(kKeyBlock, pos0 + 1 - j0);
+  const bool has_new = pos0 - j0 < kKeyBlock;
+  if (warp < (has_new ? 4 : 2)) {
+    const int NH = p.NH, NKV = p.NKV;
+    const float* src = p.qkv + (warp < 2 ? 2 * g + warp : warp == 2 ? NH + g : NH + NKV + g) * 128;
+    float x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = __ldcg(src + lane + 32 * i);
+    if (warp < 3) {
+      if (p.qk_norm) {
+        float ss = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ss += x[i] * x[i];
+#pragma unroll
+        for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
+        const float scl = rsqrtf(ss / 128.f + p.eps);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = x[i] * scl * ra.gain[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float e = x[i], f = x[i + 2];
+        x[i] = e * ra.rope[i].x - f * ra.rope[i].y;
+        x[i + 2] = f * ra.rope[i].x + e * ra.rope[i].y;
+      }
+    }
+    if (warp < 2) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a.qs[warp * 128 + lane + 32 * i] = x[i];
+    } else {              // rounded to the cache's bf16: the value every later read sees, this one included
+      uint16_t* row = (warp == 2 ? a.kb : a.vb) + (pos0 - j0) * kRowLd;
+      uint16_t* dst = reinterpret_cast<uint16_t*>(warp == 2 ? o.kcache : o.vcache) +
+                      (((size_t)layer * NKV + g) * o.cap + pos0) * 128;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint16_t bits = (uint16_t)bf16_rn_bits(x[i]);
+        row[lane + 32 * i] = bits;
+        dst[lane + 32 * i] = bits;
+      }
+    }
+  }
+  cpa_wait_all();
+  consumer_sync();
+  {
+    const int qi = tid >> 7, kk = (tid >> 2) & 31, part = tid & 3;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    if (kk < nk) {
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        const int d = 8 * (part + 4 * ch);
+        const uint4 k = *reinterpret_cast<const uint4*>(a.kb + kk * kRowLd + d);
+        const float4 q0 = *reinterpret_cast<const float4*>(a.qs + qi * 128 + d);
+        const float4 q1 = *reinterpret_cast<const float4*>(a.qs + qi * 128 + d + 4);
+        s0 += q0.x * bf16_lo_f32(k.x);
+        s1 += q0.y * bf16_hi_f32(k.x);
+        s2 += q0.z * bf16_lo_f32(k.y);
+        s3 += q0.w * bf16_hi_f32(k.y);
+        s0 += q1.x * bf16_lo_f32(k.z);
+        s1 += q1.y * bf16_hi_f32(k.z);
+        s2 += q1.z * bf16_lo_f32(k.w);
+        s3 += q1.w * bf16_hi_f32(k.w);
+      }
+    }
+    float sc = (s0 + s1) + (s2 + s3);
+    sc += __shfl_xor_sync(0xFFFFFFFFu, sc, 1);
+    sc += __shfl_xor_sync(0xFFFFFFFFu, sc, 2);
+    if (part == 0) a.sc[qi * kKeyBlock + kk] = kk < nk ? sc * rsqrtf(128.f) : -INFINITY;
+  }
+  consumer_sync();
+  const int qi = warp >> 2, d = 32 * (warp & 3) + 2 * (lane & 15), kh = lane >> 4;
+  const float s = a.sc[qi * kKeyBlock + lane];
+  uint32_t v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    v[i] = 2 * i + kh < nk ? *reinterpret_cast<const uint32_t*>(a.vb + (2 * i + kh) * kRowLd + d) : 0u;
+  float m = s;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
+  const float e = lane < nk ? __expf(s - m) : 0.f;
+  float l = e;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, off);
+  float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float w = __shfl_sync(0xFFFFFFFFu, e, 2 * i + kh);
+    acc.x += w * bf16_lo_f32(v[i]);
+    acc.y += w * bf16_hi_f32(v[i]);
+  }
+  acc.x += __shfl_xor_sync(0xFFFFFFFFu, acc.x, 16);
+  acc.y += __shfl_xor_sync(0xFFFFFFFFu, acc.y, 16);
+  float* rec = o.part + ((size_t)b * p.NH + 2 * g + qi) * kPartLd;
+  if (kh == 0) *reinterpret_cast<float2*>(rec + d) = acc;
+  if ((warp & 3) == 0 && lane == 0) {
+    rec[128] = m;
+    rec[129] = l;
+  }
+}
+
+// The merge (below) for one row of 128 dims: each warp computes the blocks' weights for itself while
+// its loads of the partial sums are in flight; threads d and d + 128 take alternate blocks.
+__device__ __noinline__ void row_merge(const FrameParams& p, const OuterStep& o, int h, float* ao) {
+  const int tid = threadIdx.x, lane = tid & 31, d = tid & 127, half = tid >> 7;
+  const int nb = o.pos0 / kKeyBlock + 1;
+  const float* rec = o.part + (size_t)h * kPartLd;
+  const size_t ld = (size_t)p.NH * kPartLd;
+  float m = -INFINITY, l = 0.f, v[16];
+  if (lane < nb) {
+    m = __ldcg(rec + lane * ld + 128);
+    l = __ldcg(rec + lane * ld + 129);
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = half + 2 * i < nb ? __ldcg(rec + (half + 2 * i) * ld + d) : 0.f;
+  float M = m;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
+  const float w = lane < nb ? __expf(m - M) : 0.f;
+  float den = w * l;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, off);
+  const float wn = w / den;
+  float acc = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc += __shfl_sync(0xFFFFFFFFu, wn, half + 2 * i) * v[i];
+  if (half) ao[128 + d] = acc;
+  consumer_sync();
+  if (!half) ao[d] = acc + ao[128 + d];
+  consumer_sync();
+}
+static_assert(kConsumerThreads == 256 && kMaxOuterTokens <= 32 * kKeyBlock, "row attention: threads, key blocks");
+
 // Attention output of query head h for every row: the merge of the key blocks' partial sums
 // (each block rescaled by e^{m_b - M}), written to ao [nr][D] in shared memory.
 __device__ void outer_merge(Cons& c, const OuterStep& o, int h, float* ao) {
@@ -435,6 +614,7 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
   auto no_key = [](int) { return 0; };
   auto no_prep = [](int, int, int) {};
   const int n_blocks = (o.pos0 + nr + kKeyBlock - 1) / kKeyBlock;
+  const bool row = STD && nr == 1 && p.NH == 16 && p.NKV == 8;        // row_attention's heads
 
   // a unit's m-block and k-chunk (the standard shapes' m-block counts are powers of two)
   constexpr int lg_wo = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WO>::Mu)), lg_wd = ilog2_c(1024 / (16 * StdUnit<WT, MAT_WD>::Mu));
@@ -463,8 +643,26 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
     cons_signal(c, ctr + ctr_stage(l, 0), 0, 0);
 
     // ---- attention: (KV head, key block) tasks, then one grid barrier -------------------------
-    if (!cons_wait(c, ctr + ctr_stage(l, 0), N)) return;
-    for (int t = blockIdx.x; t < p.NKV * n_blocks; t += p.n_cta) outer_attention<WT>(c, o, l, t % p.NKV, t / p.NKV);
+    if (row) {
+      int t = blockIdx.x;
+      const int n_tasks = 8 * n_blocks;
+      RowAhead ra{};
+      if (t < n_tasks) ra = row_attention_ahead(p, o, sm.act, l, t & 7, t >> 3);
+      if (!cons_wait(c, ctr + ctr_stage(l, 0), N)) {
+        cpa_wait_all();
+        return;
+      }
+      while (t < n_tasks) {
+        row_attention(p, o, sm.act, l, t & 7, t >> 3, ra);
+        t += p.n_cta;
+        if (t >= n_tasks) break;
+        consumer_sync();                                   // the scratch is read to the end
+        ra = row_attention_ahead(p, o, sm.act, l, t & 7, t >> 3);
+      }
+    } else {
+      if (!cons_wait(c, ctr + ctr_stage(l, 0), N)) return;
+      for (int t = blockIdx.x; t < p.NKV * n_blocks; t += p.n_cta) outer_attention<WT>(c, o, l, t % p.NKV, t / p.NKV);
+    }
     cons_signal(c, ctr + ctr_att(L, l), 0, 0);
 
     // ---- Wo + residual: unit u multiplies the merged output of head wo_key(u) ----------------
@@ -472,7 +670,10 @@ __device__ void run_outer(Cons& c, const OuterStep& o) {
     if (!cons_wait(c, ctr + ctr_att(L, l), N)) return;
     float* ao = reinterpret_cast<float*>(sm.bfrag);
     keyed_product<WT, WIDE, STD, MAT_WO, false>(
-        c, 0, 4 * l + 1, sp_wo, nr, D, wo_key, [&](int u0) { outer_merge(c, o, wo_key(u0), ao); },
+        c, 0, 4 * l + 1, sp_wo, nr, D, wo_key, [&](int u0) {
+          if (row) row_merge(p, o, wo_key(u0), ao);
+          else outer_merge(c, o, wo_key(u0), ao);
+        },
         [&](int, int n, int k, auto w) { return ld_shared_v<decltype(w)::value>(ao + n * D + k); },
         reinterpret_cast<uint8_t*>(sm.act), [&](int u, int mi, int rr, int n, float v) {
           resid_epi((wo_mb(u) * (STD ? StdUnit<WT, MAT_WO>::Mu : p.g[MAT_WO].Mu) + mi) * 16 + rr, n, v);

@@ -492,7 +492,7 @@ def test_tree_mode_trace_parity_tiny(name):
 @pytest.mark.parametrize("nodes,depth", [(16, 3), (17, 3), (31, 3), (32, 3), (64, 3), (21, 7)])
 def test_tree_mode_trace_parity_batched(nodes, depth):
     """Trees on the batched kernels (bf16 weights, from 16 nodes on, 17 rows):
-    18 to 65 rows in one pass, depth 3 and, with three candidates below each kept node, depth 7.
+    17 to 65 rows in one pass, depth 3 and, with three candidates below each kept node, depth 7.
     Logits within 2e-2 as for every bf16 model; hi + lo operands make them about 1e-4 here."""
     from oracle.tree import Tree, grow_tree
     if depth == 7:

@@ -238,6 +238,16 @@ def test_full_size_pipeline_parity(full_pipe):
     assert err < 2e-2
 
 
+@pytest.mark.parametrize("tokens", [1, 31, 63, 608])
+def test_decode_rows_at_key_block_edges(full_pipe, tokens):
+    """One-row attention of the standard geometry where the new position opens, continues and fills
+    a 32-key block, alone in the cache, and with more (KV head, block) tasks than SMs."""
+    env = full_pipe
+    prompt = make_prompt(env.ocfg)[:tokens]
+    frames, otr = env.run(prompt, 4)
+    check_pipeline(env, prompt, frames, otr, 2e-2)
+
+
 @pytest.mark.parametrize("heads,dim", [((4, 2), 64), ((2, 2), 128)])
 @pytest.mark.parametrize("tokens", [2, 16, 17, 18, 32, 33, 34, 65, 129, 130, 161, 260])
 def test_prompt_attention_at_tile_edges(heads, dim, tokens):

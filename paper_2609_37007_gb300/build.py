@@ -18,7 +18,7 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-cudart", "sh
          "-I" + os.path.join(ROOT, "include")]
 
 
-FRAME_KERNEL_SOURCES = ["mcd_frame.cu", "mcd_stage.cuh", "mcd_internal.cuh", "mcd_sampler.cuh"]
+FRAME_KERNEL_SOURCES = ["mcd_frame.cu", "mcd_tree.cuh", "mcd_stage.cuh", "mcd_internal.cuh", "mcd_sampler.cuh"]
 
 
 def source_digest(files=FRAME_KERNEL_SOURCES) -> str:

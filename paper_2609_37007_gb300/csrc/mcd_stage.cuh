@@ -13,7 +13,8 @@
 // turn the activations into bf16 hi/lo mma operands in one pass from global memory and
 // multiply each unit with mma.m16n8k16 (weights as the 16-row A side, up to 8 activation
 // columns per n-tile as B).  RMSNorm is applied as a per-column scale in the epilogue:
-// W (x . g) / rms.  Every wait is bounded.
+// W (x . g) / rms.  With up to 8 rows of the standard widths (STD) the operand stays in registers:
+// each thread loads the values of its own fragments (run_narrow).  Every wait is bounded.
 #pragma once
 #include <type_traits>
 #include "mcd_internal.cuh"

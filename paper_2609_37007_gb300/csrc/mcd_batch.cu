@@ -102,7 +102,7 @@ struct BatchBufs {
   int* head_slot;         // [R * kRecSlots] LM-head operand row of (row, j), -1: none
   float* X;               // [R][H] residual stream
   float* ss;              // [2L + 1][R] per-row sums of squares of X after each residual write
-  float* qkv;             // [R][qkv_dim]; tensor cores: qkv_nz partial sums, qkv_zs floats apart
+  float* qkv;             // [R][qkv_dim]; trees: qkv_nz partial sums, qkv_zs floats apart
   int qkv_nz;
   size_t qkv_zs;
   uint16_t* att;          // [R][NH * D] bf16 attention outputs
@@ -289,34 +289,34 @@ __global__ void __launch_bounds__(256) batch_pack_kernel(FrameParams p, BatchBuf
   }
 }
 
-// embed (tensor-core path): X[r] = the row's input vector, and layer 0's QKV operand.  Thread t
-// owns elements 8t..8t+7.
-__global__ void __launch_bounds__(128) batch_embed_tc_kernel(FrameParams p, BatchBufs b) {
+// embed (tensor-core path): X[r] = the row's input vector, and layer 0's QKV operand.  The sum of
+// squares takes the elements in batch_embed_kernel's order; then thread t owns elements 8t..8t+7.
+__global__ void __launch_bounds__(256) batch_embed_tc_kernel(FrameParams p, BatchBufs b) {
+  __shared__ __align__(16) float row_s[1024];
+  __shared__ float sw[8];
   const int r = blockIdx.x, t = threadIdx.x;
   tc::pdl_trigger();
   if (r >= b.info->M) return;
   const BatchRow row = b.rows[r];
-  const bool live = t < p.H / 8;
-  float v[8];
-  float ss = 0.f;
-  if (live) {
-    if (row.f32) {
-      const float* src = reinterpret_cast<const float*>(row.src) + 8 * t;      // any 4-byte alignment
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = __ldg(src + i);
-    } else {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(row.src) + t);
-      v[0] = bf16_lo_f32(w.x); v[1] = bf16_hi_f32(w.x); v[2] = bf16_lo_f32(w.y); v[3] = bf16_hi_f32(w.y);
-      v[4] = bf16_lo_f32(w.z); v[5] = bf16_hi_f32(w.z); v[6] = bf16_lo_f32(w.w); v[7] = bf16_hi_f32(w.w);
-    }
-    float4* xr = reinterpret_cast<float4*>(b.X + (size_t)r * p.H + 8 * t);
-    xr[0] = make_float4(v[0], v[1], v[2], v[3]);
-    xr[1] = make_float4(v[4], v[5], v[6], v[7]);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) ss += v[i] * v[i];
+  float s = 0.f;
+  for (int k = t; k < p.H; k += 256) {
+    const float v = row.f32 ? __ldg(reinterpret_cast<const float*>(row.src) + k)
+                            : bf16_bits_to_f32(__ldg(reinterpret_cast<const uint16_t*>(row.src) + k));
+    b.X[(size_t)r * p.H + k] = v;
+    row_s[k] = v;
+    s += v * v;
   }
-  const float tot = block_sum128(ss);
-  if (!live) return;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if ((t & 31) == 0) sw[t >> 5] = s;
+  __syncthreads();
+  if (t >= p.H / 8) return;
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) tot += sw[w];
+  float v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = row_s[8 * t + i];
   const NormChunk c = norm_chunk(v, rsqrtf(tot / (float)p.H + p.eps), p.attn_norm, t);
   const size_t off = tc::sw128_offset(b.Rtc, r, t >> 3, t & 7);
   *reinterpret_cast<uint4*>(b.xn_hi + off) = c.hi;
@@ -719,12 +719,10 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
   {
     const int e_q = nq << lg4, e_k = e_q + (nk << lg4), e_v = e_k + (nk << lg4);
     const int e_cs = e_v + (nr << lg4), e_g = e_cs + (p.qk_norm ? 2 << lg4 : 0);
-    const int nz = b.qkv_nz;
     for (int i = tid; i < e_g; i += 256) {
       const int ch = i & (D4 - 1);
       const float* src;
       float* dst;
-      bool sum = nz > 1 && i < e_q;              // a row of the QKV product: its partial sums added
       if (i < e_q) {
         const int qi = i >> lg4;
         src = b.qkv + (size_t)(base + q_row[qi]) * p.qkv_dim + q_head[qi] * D;
@@ -736,7 +734,6 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
           src = (isv ? p.vcache : p.kcache) + cache_off + (size_t)j * D;
         else
           src = b.qkv + (size_t)(base + j - pos0) * p.qkv_dim + p.NH * D + (isv ? p.NKV * D : 0) + g * D;
-        sum = nz > 1 && j >= pos0;
         dst = isv ? vs[j] : ks[j];
       } else if (i < e_cs) {
         const int n = (i - e_v) >> lg4;
@@ -747,19 +744,7 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
         src = (w == 0 ? p.q_norm : p.k_norm) + (size_t)layer * D;
         dst = w == 0 ? gq : gk;
       }
-      if (sum) {
-        float4 v = __ldcg(reinterpret_cast<const float4*>(src) + ch);
-        for (int z = 1; z < nz; ++z) {
-          const float4 w = __ldcg(reinterpret_cast<const float4*>(src + z * b.qkv_zs) + ch);
-          v.x += w.x;
-          v.y += w.y;
-          v.z += w.z;
-          v.w += w.w;
-        }
-        reinterpret_cast<float4*>(dst)[ch] = v;
-      } else {
-        cpa16(dst + 4 * ch, src + 4 * ch);
-      }
+      cpa16(dst + 4 * ch, src + 4 * ch);
     }
     cpa_wait_all();
   }
@@ -1399,7 +1384,7 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
   if (bs->use_tc) {
     const int Rtc = tc_operand_rows(rows, p.qkv_dim, p.n_cta);
     b.Rtc = Rtc;
-    b.qkv_nz = tc_qkv_splits(p.qkv_dim, Rtc, p.H, p.n_cta);
+    b.qkv_nz = tc_qkv_splits(p.qkv_dim, Rtc, p.H, p.n_cta, bs->tree);
     b.qkv_zs = (size_t)Rtc * p.qkv_dim;
     BATCH_ALLOC(b.qkv, sizeof(float) * b.qkv_nz * b.qkv_zs);
     if (bs->tree) {
@@ -1487,12 +1472,12 @@ static void enqueue_heads(const FrameParams& p, const BatchState* bs, cudaStream
 }
 
 // The operand a residual pass leaves: the next layer's QKV operand, or after the last layer the LM
-// heads' (where they run on the tensor cores).
+// heads' (where they run on the tensor cores; the general heads read the rows' sums of squares).
 static NormOut after_layer(const FrameParams& p, const BatchState* bs, int l) {
   const BatchBufs& b = bs->b;
-  if (l + 1 < p.L) return NormOut{p.attn_norm + (size_t)(l + 1) * p.H, b.xn_hi, b.xn_lo, nullptr, 0};
-  if (bs->tw.heads) return NormOut{p.final_norm, b.hq_hi, b.hq_lo, b.head_slot, b.Qcap};
-  return NormOut{nullptr, nullptr, nullptr, nullptr, 0};
+  if (l + 1 < p.L) return NormOut{p.attn_norm + (size_t)(l + 1) * p.H, b.xn_hi, b.xn_lo, nullptr, 0, nullptr};
+  if (bs->tw.heads) return NormOut{p.final_norm, b.hq_hi, b.hq_lo, b.head_slot, b.Qcap, nullptr};
+  return NormOut{nullptr, nullptr, nullptr, nullptr, 0, b.ss + (size_t)(2 * p.L) * b.R};
 }
 
 // Every kernel of one call, in stream order on `s`.
@@ -1507,7 +1492,7 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
   // node the last bodies of a frame are empty: no prefetch there.
   const bool pdl = loop.valid != 0;
   batch_pack_kernel<<<1, 256, 0, s>>>(p, b);
-  if (bs->use_tc) batch_embed_tc_kernel<<<R, 128, 0, s>>>(p, b);
+  if (bs->use_tc) batch_embed_tc_kernel<<<R, 256, 0, s>>>(p, b);
   else batch_embed_kernel<<<R, 256, 0, s>>>(p, b);
   for (int l = 0; l < L && bs->use_tc; ++l) {
     const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
@@ -1515,20 +1500,18 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     const int* M = &b.info->M;
     // RMSNorm -> QKV (hi + lo operand, written by the embedding or the previous layer's last
     // residual pass)
-    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_qkv(false, wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
     batch_attn_kernel<<<dim3(bs->max_streams, p.NKV), blk, 0, s>>>(p, b, l);      // -> att_t
     // Wo (k-split partials) -> residual, the gate/up operand
     tc_launch_resid<false>(wl + bs->tw.off.o, b.att_t, nullptr, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, R, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
-                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, nullptr, nullptr, 0}, s);
+    tc_launch_resid_norm(false, false, R, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, nullptr, nullptr, 0, nullptr}, s);
     // gate/up -> SwiGLU (into the down product's operand)
     tc_launch_gu<false>(wl + bs->tw.off.gu, b.xn_hi, nullptr, b.act_t, nullptr, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     // down (k-split partials) -> residual, the next operand
     tc_launch_resid<false>(wl + bs->tw.off.d, b.act_t, nullptr, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, R, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
+    tc_launch_resid_norm(false, false, R, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
   }
-  if (bs->use_tc && !bs->tw.heads)      // the general LM heads read the rows' sums of squares
-    batch_rowss_kernel<<<(R + 7) / 8, blk, 0, s>>>(b.X, H, b.ss + (size_t)(2 * L) * R, b.info);
   for (int l = 0; l < L && !bs->use_tc; ++l) {
     {   // RMSNorm -> QKV
       GemmArgs a = gemm_args(p, b);
@@ -1609,18 +1592,18 @@ static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs,
   const bool pdl = loop.valid != 0;
   const int* M = &b.info->M;
   batch_tree_pack_kernel<<<1, 128, 0, s>>>(p, b);
-  batch_embed_tc_kernel<<<kMaxTreeRows, 128, 0, s>>>(p, b);
+  batch_embed_tc_kernel<<<kMaxTreeRows, 256, 0, s>>>(p, b);
   for (int l = 0; l < L; ++l) {
     const uint8_t* wl = bs->tw.arena + (size_t)l * bs->tw.off.layer;
-    tc_launch_qkv(wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_qkv(true, wl + bs->tw.off.qkv, b.xn_hi, b.xn_lo, b.qkv, p.qkv_dim, Rtc, H, M, p.err, p.wait_ns, p.n_cta, pdl, s);
     batch_tree_rope_kernel<<<(kMaxTreeRows * (p.NH + 2 * p.NKV) + 7) / 8, blk, 0, s>>>(p, b, l);
     batch_tree_attn_kernel<<<(kMaxTreeRows * p.NH + 7) / 8, blk, 0, s>>>(p, b, l);
     tc_launch_resid<true>(wl + bs->tw.off.o, b.att_t, b.att_lo, b.part, H, Rtc, qd, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
-                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, b.xn_lo, nullptr, 0}, s);
+    tc_launch_resid_norm(true, false, kMaxTreeRows, b.X, b.part, qd, Rtc, H, p.n_cta, M, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, b.xn_hi, b.xn_lo, nullptr, 0, nullptr}, s);
     tc_launch_gu<true>(wl + bs->tw.off.gu, b.xn_hi, b.xn_lo, b.act_t, b.act_lo, Rtc, M, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + bs->tw.off.d, b.act_t, b.act_lo, b.part, H, Rtc, p.F, M, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
+    tc_launch_resid_norm(true, false, kMaxTreeRows, b.X, b.part, p.F, Rtc, H, p.n_cta, M, p.eps, after_layer(p, bs, l), s);
   }
   enqueue_heads(p, bs, s);
   batch_topk_kernel<<<kMaxTreeRows * (p.K + 1) + b.R, kConsumerThreads, 0, s>>>(p, b);

@@ -1507,20 +1507,20 @@ static mcd_status outer_tc_prefill(mcd_outer* o, const int32_t* text_ids, int n)
     const uint8_t* wl = t.w + (size_t)l * t.off.layer;
     uint16_t* kc = reinterpret_cast<uint16_t*>(st.kcache) + (size_t)l * kvl;
     uint16_t* vc = reinterpret_cast<uint16_t*>(st.vcache) + (size_t)l * kvl;
-    tc_launch_qkv(wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
+    tc_launch_qkv(true, wl + t.off.qkv, t.xn_hi, t.xn_lo, t.qkv, p.qkv_dim, Rtc, H, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
     const int vecs = p.NH + 2 * p.NKV;
-    tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, tc_qkv_splits(p.qkv_dim, Rtc, H, p.n_cta),
+    tc::launch(pdl, pf_rope_kv_kernel, dim3((n * vecs + 7) / 8), dim3(256), 0, s, t.qkv, tc_qkv_splits(p.qkv_dim, Rtc, H, p.n_cta, true),
                (size_t)Rtc * p.qkv_dim, p.qkv_dim, t.rows, p.NH, p.NKV, p.D, p.qk_norm,
                                                          p.q_norm + (size_t)l * p.D, p.k_norm + (size_t)l * p.D, p.eps,
                                                          st.rope, kc, vc, st.cap, t.q);
     launch_pf_attn(t.q, t.rows, n, p.NH, p.NKV, p.D, kc, vc, st.cap, Rtc, t.att_t, t.att_lo, s);
     tc_launch_resid<true>(wl + t.off.o, t.att_t, t.att_lo, t.part, H, Rtc, qd, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(pdl, n, t.X, t.part, qd, Rtc, H, p.n_cta, t.rows, p.eps,
-                         NormOut{p.ffn_norm + (size_t)l * H, t.xn_hi, t.xn_lo, nullptr, 0}, s);
+    tc_launch_resid_norm(true, pdl, n, t.X, t.part, qd, Rtc, H, p.n_cta, t.rows, p.eps,
+                         NormOut{p.ffn_norm + (size_t)l * H, t.xn_hi, t.xn_lo, nullptr, 0, nullptr}, s);
     tc_launch_gu<true>(wl + t.off.gu, t.xn_hi, t.xn_lo, t.act_t, t.act_lo, Rtc, t.rows, p.F, H, p.err, p.wait_ns, p.n_cta, pdl, s);
     tc_launch_resid<true>(wl + t.off.d, t.act_t, t.act_lo, t.part, H, Rtc, p.F, t.rows, p.err, p.wait_ns, p.n_cta, pdl, s);
-    tc_launch_resid_norm(pdl, n, t.X, t.part, p.F, Rtc, H, p.n_cta, t.rows, p.eps,
-                         NormOut{l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : nullptr, t.xn_hi, t.xn_lo, nullptr, 0}, s);
+    tc_launch_resid_norm(true, pdl, n, t.X, t.part, p.F, Rtc, H, p.n_cta, t.rows, p.eps,
+                         NormOut{l + 1 < L ? p.attn_norm + (size_t)(l + 1) * H : nullptr, t.xn_hi, t.xn_lo, nullptr, 0, nullptr}, s);
   }
   MCD_CHECK(cudaGetLastError());
   return MCD_OK;

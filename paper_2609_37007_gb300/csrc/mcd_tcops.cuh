@@ -61,11 +61,18 @@ __global__ void tc_weight_tile_kernel(const uint16_t* __restrict__ src, int rows
 constexpr int kTcBN = 128;        // packed rows per tile: QKV (hi + lo operand), Wo, down
 constexpr int kTcSplit = 16;      // k-splits of the residual products (at most)
 constexpr int kTcQkvSplit = 4;    // k-splits of the QKV product (at most)
-// A product's column tiles and k-splits at Rtc operand rows.  Up to 128 rows a product is its
-// weight stream, and a few column tiles of 128-row weight tiles would leave most SMs without a
-// share of it: tiles of up to 64 columns, and as many k-splits as fill the SMs (at most z_max).
-// Frames of 8 streams (32 rows): 1191 us with QKV, Wo and down on 32 / 48 / 48 CTAs, 1059 on 128
-// each; a 32-node tree (33 rows) 1422 and 1358.
+// A product's column tiles and k-splits at Rtc operand rows.
+//
+// Trees and prompts (free_k): up to 128 rows a product is its weight stream, and a few column
+// tiles of 128-row weight tiles would leave most SMs without a share of it: tiles of up to 64
+// columns, and as many k-splits as fill the SMs (at most z_max).  A 32-node tree (33 rows): 1422 us
+// per frame with QKV, Wo and down on 32 / 48 / 48 CTAs, 1358 on 128 each.
+//
+// Chain streams: the k-splits do not depend on the row count below 385 rows (QKV unsplit, Wo and
+// down six), so a stream's logits are the same bits whatever context it is decoded in.  Its Wo,
+// gate/up and down operands are single bf16 values, which turn a sum's last bit into 3e-4 of the
+// logits.  Split freely as well, frames of 8 / 16 / 32 streams would take 1021 / 1100 / 1219 us
+// instead of 1131 / 1175 / 1278.
 struct TcShape {
   int pitch, z;
 };
@@ -74,11 +81,11 @@ inline TcShape tc_small_shape(int M, int Rtc, int n_sm, int z_max) {
   return TcShape{(units + T - 1) / T * 16, z < 1 ? 1 : (z > z_max ? z_max : z)};
 }
 constexpr int kTcSmallRows = 128;
-// Residual products above kTcSmallRows: six splits below 512 rows, four (128-column tiles, 128 CTAs at
-// 512 rows) from there on, where more splits' partial sums cost more than they save.
-inline TcShape tc_resid_shape(int H, int Rtc, int n_sm) {
-  if (Rtc <= kTcSmallRows) return tc_small_shape(H, Rtc, n_sm, kTcSplit);
-  const int n_mt = H / tc::kBM, units = Rtc / 16, z = Rtc >= 512 ? 4 : 6;
+// Residual products otherwise: six splits, four from 385 rows (512 operand rows: 128-column tiles, 128
+// CTAs) on, where more splits' partial sums cost more than they save.
+inline TcShape tc_resid_shape(int H, int Rtc, int n_sm, bool free_k) {
+  if (free_k && Rtc <= kTcSmallRows) return tc_small_shape(H, Rtc, n_sm, kTcSplit);
+  const int n_mt = H / tc::kBM, units = Rtc / 16, z = Rtc > 384 ? 4 : 6;
   int T = n_sm / (n_mt * z);
   if (T < 1) T = 1;
   if (T < (Rtc + 255) / 256) T = (Rtc + 255) / 256;
@@ -209,12 +216,13 @@ __global__ void __launch_bounds__(kResidThreads, 1) tc_resid_kernel(const tc::Ge
 
 // Where a residual pass writes the row's normalised operand: `hi` / `lo` of Rtc rows at the row
 // itself; after the last layer, with `slots` (eight per row, -1: none), at those rows of the LM
-// heads' operand of slot_rows rows instead.
+// heads' operand of slot_rows rows instead.  ss (may be null): the rows' sums of squares.
 struct NormOut {
   const float* gain;          // null: no operand
   uint8_t *hi, *lo;
   const int* slots;
   int slot_rows;
+  float* ss;
 };
 // Per packed row (one CTA, thread t owns elements 8t..8t+7): X += the nz partial sums, the
 // row's sum of squares (the next RMSNorm), and the next product's normalised operand as SW128
@@ -257,6 +265,7 @@ __global__ void __launch_bounds__(128) tc_resid_norm_kernel(float* X, const floa
     for (int i = 0; i < 8; ++i) ss += x[i] * x[i];
   }
   const float tot = block_sum128(ss);
+  if (out.ss && t == 0) out.ss[r] = tot;
   if (!out.gain || !live) return;
   const NormChunk c = norm_chunk(x, rsqrtf(tot / (float)H + eps), out.gain, t);
   if (!out.slots) {
@@ -362,17 +371,17 @@ inline int tc_operand_rows(int n, int qkv_dim, int n_sm) {
   return (n + unit - 1) / unit * unit;
 }
 // Column tiles and k-splits of the QKV product (tile form); tc_qkv_splits: partial sums it leaves.
-inline TcShape tc_qkv_shape(int qkv_dim, int Rtc, int n_sm) {
-  if (Rtc <= kTcSmallRows) return tc_small_shape(qkv_dim, Rtc, n_sm, kTcQkvSplit);
+inline TcShape tc_qkv_shape(int qkv_dim, int Rtc, int n_sm, bool free_k) {
+  if (free_k && Rtc <= kTcSmallRows) return tc_small_shape(qkv_dim, Rtc, n_sm, kTcQkvSplit);
   return TcShape{tc::tile_pitch(qkv_dim, Rtc, n_sm), 1};
 }
-inline int tc_qkv_splits(int qkv_dim, int Rtc, int H, int n_sm) {
-  return tc_qkv_persistent(Rtc, qkv_dim, n_sm) ? 1 : tc_splits(H, tc_qkv_shape(qkv_dim, Rtc, n_sm).z);
+inline int tc_qkv_splits(int qkv_dim, int Rtc, int H, int n_sm, bool free_k) {
+  return tc_qkv_persistent(Rtc, qkv_dim, n_sm) ? 1 : tc_splits(H, tc_qkv_shape(qkv_dim, Rtc, n_sm, free_k).z);
 }
 // q, k, v of Rtc operand rows, as tc_qkv_splits partial sums out[z][Rtc][qkv_dim].  Below
 // tc_qkv_persistent's line the pitch is at most kTcBN: nt
 // tiles of 128 columns over n_mt weight tiles with nt n_mt < 0.8 n_sm leave n_sm / n_mt >= nt.
-inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t* xn_lo, float* out, int qkv_dim, int Rtc,
+inline void tc_launch_qkv(bool free_k, const uint8_t* w, const uint8_t* xn_hi, const uint8_t* xn_lo, float* out, int qkv_dim, int Rtc,
                           int H, const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
   tc::GemmArgs g{w, xn_hi, xn_lo, qkv_dim, Rtc, H, nrows, err, wait_ns, pdl, 0};
   if (tc_qkv_persistent(Rtc, qkv_dim, n_sm)) {
@@ -380,7 +389,7 @@ inline void tc_launch_qkv(const uint8_t* w, const uint8_t* xn_hi, const uint8_t*
                    tc::PLayout<kTcBN, true>::kSmemBytes, s, g, out, qkv_dim);
     return;
   }
-  const TcShape sh = tc_qkv_shape(qkv_dim, Rtc, n_sm);
+  const TcShape sh = tc_qkv_shape(qkv_dim, Rtc, n_sm, free_k);
   g.bn = sh.pitch;
   const dim3 grid((Rtc + g.bn - 1) / g.bn, qkv_dim / tc::kBM, sh.z);
   if (g.bn <= 64)
@@ -409,12 +418,12 @@ inline void tc_launch_gu(const uint8_t* gu, const uint8_t* xn, const uint8_t* xn
 }
 
 // Wo or down (A = w: H rows of K, B = act: Rtc rows) -> the partial sums of tc_resid_shape's splits
-// (H = 1024: 16 splits of one column tile up to 64 rows, 128 CTAs; 9 of two up to 128, 144 CTAs;
-// 4 of four at 512, 128 CTAs).
+// (H = 1024: trees and prompts 16 splits of one column tile up to 64 rows, 128 CTAs, and 9 of two up to
+// 128, 144 CTAs; otherwise 6 of up to three, 144 CTAs; 4 of four at 512, 128 CTAs).
 template <bool kHilo>
 inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, const uint8_t* act_lo, float* part, int H, int Rtc, int K,
                             const int* nrows, int* err, unsigned long long wait_ns, int n_sm, bool pdl, cudaStream_t s) {
-  const TcShape sh = tc_resid_shape(H, Rtc, n_sm);
+  const TcShape sh = tc_resid_shape(H, Rtc, n_sm, kHilo);
   const int pitch = sh.pitch;
   const tc::GemmArgs g{w, act, act_lo, H, Rtc, K, nrows, err, wait_ns, pdl, pitch};
   const dim3 grid((Rtc + pitch - 1) / pitch, H / tc::kBM, sh.z);
@@ -426,9 +435,9 @@ inline void tc_launch_resid(const uint8_t* w, const uint8_t* act, const uint8_t*
 }
 
 // The residual pass of a product over K (tc_resid_norm_kernel) on `rows` CTAs.
-inline void tc_launch_resid_norm(bool pdl, int rows, float* X, const float* part, int K, int Rtc, int H, int n_sm,
+inline void tc_launch_resid_norm(bool free_k, bool pdl, int rows, float* X, const float* part, int K, int Rtc, int H, int n_sm,
                                  const int* nrows, float eps, const NormOut& out, cudaStream_t s) {
-  const int nz = tc_splits(K, tc_resid_shape(H, Rtc, n_sm).z);
+  const int nz = tc_splits(K, tc_resid_shape(H, Rtc, n_sm, free_k).z);
   if (nz <= 6)
     tc::launch(pdl, tc_resid_norm_kernel<6>, dim3(rows), dim3(128), 0, s, X, part, nz, Rtc, H, nrows, eps, out);
   else

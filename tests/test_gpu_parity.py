@@ -421,6 +421,22 @@ def test_gemm_path_full_size(n_streams, checked):
     env.dec.close()
 
 
+def test_gemm_path_logits_do_not_depend_on_the_context():
+    """A stream's logits are the same bits in contexts of 20 to 360 packed rows: the products of
+    chain streams split their sums the same way at every row count below 385."""
+    base = TINY_BF16.replace(draft_len=3, vocab=256)
+    frames, ids = [make_frame(base, f) for f in range(5)], list(range(5))
+    runs = []
+    for streams in (5, 32, 90):
+        env = Env(base.replace(max_streams=streams))
+        codes, st, trs = decode_many(env, frames, ids, ids)
+        assert (st[:, 4] == 0).all()
+        runs.append((codes, np.stack(trs)))
+        env.dec.close()
+    for codes, trs in runs[1:]:
+        assert (codes == runs[0][0]).all() and (trs == runs[0][1]).all()
+
+
 def test_gemm_path_inside_a_captured_graph():
     """A frame captured into the caller's own graph (there the calls are enqueued one after
     another; the context's own graph loops over them) gives the codes of a direct call."""

@@ -77,7 +77,7 @@ struct BatchLoop {
   int valid;
 };
 
-// Per-frame arguments, copied to the device before each graph launch.
+// Per-frame arguments, passed by value to batch_begin_kernel: a graph that the caller captures owns them.
 struct BatchFrame {
   int S;
   unsigned stream_ids[kMaxBatchStreams];
@@ -1279,12 +1279,16 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(Fra
   if (threadIdx.x == 0) batch_call_end(p, b, loop, call, !__ldcg(&p.st->done));
 }
 
-__global__ void batch_begin_kernel(FrameParams p, BatchBufs b) {
-  const BatchFrame* fa = b.frame;
-  for (int s = threadIdx.x; s < fa->S; s += blockDim.x) init_stream_state(p.st + s, p.C0V > 0 ? fa->c0[s] : -1);
+// Start of a frame: its arguments to *frame, every stream's state and the call counters reset.
+__global__ void __launch_bounds__(256) batch_begin_kernel(const __grid_constant__ BatchFrame f, BatchFrame* frame,
+                                                          BatchInfo* info, DevState* st, int c0_vocab) {
+  static_assert(sizeof(BatchFrame) % 4 == 0, "copied in words");
+  for (int i = threadIdx.x; i < (int)(sizeof(BatchFrame) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(frame)[i] = reinterpret_cast<const int*>(&f)[i];
+  for (int s = threadIdx.x; s < f.S; s += blockDim.x) init_stream_state(st + s, c0_vocab > 0 ? f.c0[s] : -1);
   if (threadIdx.x == 0) {
-    b.info->next_call = 0;
-    b.info->arrived = 0u;
+    info->next_call = 0;
+    info->arrived = 0u;
   }
 }
 
@@ -1297,7 +1301,6 @@ namespace mcd {
 
 struct BatchState {
   BatchBufs b;
-  BatchFrame host_frame;
   int max_streams = 0;
   bool use_tc = false;        // QKV, Wo, gate/up and down on the tcgen05 GEMM
   bool tree = false;          // TREE mode: one stream's tree calls
@@ -1611,27 +1614,12 @@ static cudaError_t enqueue_tree_call(const FrameParams& p, const BatchState* bs,
   return cudaGetLastError();
 }
 
-// The frame's graph: the state reset, then the while node over the calls.
+// The frame's graph: the while node over the calls.
 static cudaError_t build_graph(const FrameParams& p, BatchState* bs) {
   cudaStream_t s = bs->cap;
   cudaError_t e = cudaGraphCreate(&bs->graph, 0);
   if (e != cudaSuccess) return e;
-  auto capture = [&](cudaGraph_t g, auto enqueue) {
-    cudaError_t c = cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-    if (c != cudaSuccess) return c;
-    const cudaError_t q = enqueue();
-    cudaGraph_t out = nullptr;
-    c = cudaStreamEndCapture(s, &out);
-    return q != cudaSuccess ? q : c;
-  };
-  e = capture(bs->graph, [&] {
-    batch_begin_kernel<<<1, 256, 0, s>>>(p, bs->b);
-    return cudaGetLastError();
-  });
-  if (e != cudaSuccess) return e;
-  cudaGraphNode_t begin = nullptr, loop_node = nullptr;
-  size_t n_nodes = 1;
-  if ((e = cudaGraphGetNodes(bs->graph, &begin, &n_nodes)) != cudaSuccess) return e;
+  cudaGraphNode_t loop_node = nullptr;
   BatchLoop loop{0, 1};
   e = cudaGraphConditionalHandleCreate(&loop.handle, bs->graph, 1, cudaGraphCondAssignDefault);
   if (e != cudaSuccess) return e;
@@ -1640,9 +1628,13 @@ static cudaError_t build_graph(const FrameParams& p, BatchState* bs) {
   np.conditional.handle = loop.handle;
   np.conditional.type = cudaGraphCondTypeWhile;
   np.conditional.size = 1;
-  if ((e = cudaGraphAddNode(&loop_node, bs->graph, &begin, nullptr, 1, &np)) != cudaSuccess) return e;
-  e = capture(np.conditional.phGraph_out[0], [&] { return (bs->tree ? enqueue_tree_call : enqueue_call)(p, bs, loop, s); });
+  if ((e = cudaGraphAddNode(&loop_node, bs->graph, nullptr, nullptr, 0, &np)) != cudaSuccess) return e;
+  e = cudaStreamBeginCaptureToGraph(s, np.conditional.phGraph_out[0], nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
+  const cudaError_t q = (bs->tree ? enqueue_tree_call : enqueue_call)(p, bs, loop, s);
+  cudaGraph_t body = nullptr;
+  e = cudaStreamEndCapture(s, &body);
+  if (q != cudaSuccess || e != cudaSuccess) return q != cudaSuccess ? q : e;
   return cudaGraphInstantiate(&bs->exec, bs->graph, 0);
 }
 
@@ -1662,7 +1654,7 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
       return cuda_status(e);
     }
   }
-  BatchFrame& f = bs->host_frame;
+  BatchFrame f;
   memset(&f, 0, sizeof(f));
   f.S = n;
   for (int i = 0; i < n; ++i) {
@@ -1676,13 +1668,12 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
   f.stats = stats;
   f.trace = trace;
   f.tree = p.tree;
-  MCD_CHECK(cudaMemcpyAsync(bs->b.frame, &f, sizeof(f), cudaMemcpyHostToDevice, stream));
+  batch_begin_kernel<<<1, 256, 0, stream>>>(f, bs->b.frame, bs->b.info, p.st, p.C0V);
+  MCD_CHECK(cudaGetLastError());
   if (!unrolled) {
     MCD_CHECK(cudaGraphLaunch(bs->exec, stream));
     return MCD_OK;
   }
-  batch_begin_kernel<<<1, 256, 0, stream>>>(p, bs->b);
-  MCD_CHECK(cudaGetLastError());
   for (int call = 0; call < p.P; ++call) MCD_CHECK((bs->tree ? enqueue_tree_call : enqueue_call)(p, bs, BatchLoop{0, 0}, stream));
   return MCD_OK;
 }

@@ -461,6 +461,62 @@ def test_gemm_path_inside_a_captured_graph():
     dec.close()
 
 
+@pytest.mark.parametrize("nodes", [0, 32])
+def test_captured_batched_frames_own_their_arguments(nodes):
+    """Frames of 16 streams or of a 32-node tree, captured into the caller's graphs, keep their ids,
+    inputs, outputs and tree: with other frames captured and decoded in between, a replay gives
+    the codes of a direct call with the captured arguments and writes nowhere else."""
+    from oracle.tree import grow_tree
+    n = 1 if nodes else 16
+    cfg = TINY_BF16.replace(max_streams=n, draft_len=3, vocab=256, n_pos=8, draft_mode=3 if nodes else 0)
+    acc = [[0.6 / (r + 1) ** 0.5 for r in range(8)] for _ in range(3)]
+    stream = torch.cuda.Stream()
+    dec = mcd.Decoder(cfg, make_weights(cfg), stream=stream)
+
+    def args(i):              # frame i of the test: its own ids, inputs, outputs and (TREE mode) tree
+        frames = [make_frame(cfg, 20 * i + s) for s in range(n)]
+        return dict(sids=[3 + 50 * i + s for s in range(n)], fids=[7 * i + s for s in range(n)],
+                    cond=t(np.stack([f.cond for f in frames])), emb=t(np.stack([f.c0_emb for f in frames])),
+                    codes=torch.full((n, cfg.n_pos), -1, dtype=torch.int32, device=DEV),
+                    stats=torch.zeros((n, 8), dtype=torch.int32, device=DEV),
+                    tree=grow_tree(acc, nodes + 8 * i) if nodes else None)
+
+    def decode(a, codes, stats):
+        if nodes:
+            mcd.mcd_set_tree(dec.ctx, a["tree"].parent, a["tree"].rank)
+        mcd.mcd_decode_frames(dec.ctx, a["sids"], a["fids"], a["cond"], None, a["emb"], codes, stats)
+
+    runs = [args(i) for i in range(3)]
+    want = []
+    for a in runs:
+        decode(a, a["codes"], a["stats"])
+        mcd.mcd_sync(dec.ctx)
+        want.append((a["codes"].clone(), a["stats"].clone()))
+        a["codes"].fill_(-1)
+        a["stats"].zero_()
+    torch.cuda.synchronize()
+    graphs = []
+    for a in runs[:2]:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+            decode(a, a["codes"], a["stats"])
+        graphs.append(g)
+    decode(runs[2], runs[2]["codes"], runs[2]["stats"])
+    mcd.mcd_sync(dec.ctx)
+    with torch.cuda.stream(stream):
+        graphs[1].replay()
+    mcd.mcd_sync(dec.ctx)
+    assert (runs[0]["codes"] == -1).all()
+    with torch.cuda.stream(stream):
+        graphs[0].replay()
+    mcd.mcd_sync(dec.ctx)
+    for a, (codes, stats) in zip(runs, want):
+        assert (codes >= 0).all() and torch.equal(a["codes"], codes) and torch.equal(a["stats"], stats)
+    for g in graphs:
+        g.reset()
+    dec.close()
+
+
 # ------------------------------------------------- sparse tree verification (Fig. 2) ---
 def _trees():
     from oracle.tree import Tree, grow_tree

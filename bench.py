@@ -292,7 +292,7 @@ def run_tree_sweep(args, weights):
     """Sparse tree verification (Sec. 2.2, Fig. 4): acceptance statistics per (depth, rank)
     from traced frames of a probe tree, greedy trees of N = 1..64 nodes grown from them,
     then per N: accepted tokens per call, microseconds per verify call and tokens/s.  One
-    JSON line per N; a call of more than 32 rows runs in ceil(rows / 32) weight passes."""
+    JSON line per N, with the weight passes of its fullest call as traced."""
     import torch
     from paper_2609_37007_gb300 import build as _build
     from paper_2609_37007_gb300 import mcd
@@ -334,9 +334,13 @@ def run_tree_sweep(args, weights):
     for N in args.tree_sizes:
         parent, rank = trees.grow_tree(acc, N)
         mcd.mcd_set_tree(dec.ctx, parent, rank)
+        mcd.mcd_set_trace(dec.ctx, tr)
         for i in range(3):
             mcd.mcd_decode_frame(dec.ctx, 0, i, cond[i], c0[i:i + 1], None, codes[i], stats[i])
         mcd.mcd_sync(dec.ctx)
+        mcd.mcd_set_trace(dec.ctx, None)
+        trecs = mcd.parse_tree_trace(tr.cpu().numpy(), cfg.vocab)[0]
+        passes = max(int(r["n_passes"]) for r in trecs[:int(stats[2, 0])])
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         clocks.start()
         e0.record(stream)
@@ -351,7 +355,7 @@ def run_tree_sweep(args, weights):
         t_us = e0.elapsed_time(e1) * 1e3
         calls, toks = int(st[:, 0].sum()), int(st[:, 1].sum())
         rows = 1 + len(parent)
-        print(json.dumps({"tree_nodes": len(parent), "rows_per_call": rows, "passes_per_full_call": -(-rows // 32),
+        print(json.dumps({"tree_nodes": len(parent), "rows_per_call": rows, "passes_per_full_call": passes,
                           "tokens_per_call": toks / calls, "us_per_verify_call": t_us / calls,
                           "tokens_per_s": toks / t_us * 1e6, "frames": n, "parent": parent, "rank": rank,
                           "clocks": clk}), flush=True)

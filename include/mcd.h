@@ -104,7 +104,8 @@ typedef struct {
   int32_t drafted;   /* drafts tested                                           */
   int32_t accepted;  /* drafts kept                                             */
   int32_t status;    /* 0, or an mcd_status value set by a failed device wait   */
-  int32_t heads_read;/* LM heads streamed, summed over the calls (byte accounting) */
+  int32_t heads_read;/* LM heads read, summed over the calls (byte accounting); a tree
+                      * call's heads count once per 32 rows, whatever kernels ran it  */
   int32_t kv_rows;   /* sum over calls of (first row position + rows): KV touched   */
   int32_t rows_fed;  /* sum over calls of rows fed                                  */
 } mcd_frame_stats;
@@ -295,7 +296,8 @@ typedef struct {
   int32_t draft_row;      /* row whose draft logits gave the next call's candidates       */
   int32_t n_next;         /* candidate depths of the next call                            */
   int32_t next_cand[8][8];/* [depth - 1][rank] candidate ids of the next call             */
-  int32_t n_passes;       /* weight passes of the call: ceil(n_rows / 32)                 */
+  int32_t n_passes;       /* weight passes of the call: 1 on the batched kernels, else
+                           * ceil(n_rows / 32)                                            */
   int32_t reserved[17];
 } mcd_tree_trace;
 
@@ -316,7 +318,8 @@ typedef struct {
  * 32 t .. 32 t + 31 in pass t; later rows attend to earlier ones through the cache); the
  * acceptance step follows the last pass.  bf16 models whose widths suit the tensor-core
  * products run trees of 16 nodes or more in one pass on the batched kernels instead (one
- * CUDA graph launch per frame); n_passes and heads_read count passes of 32 rows either way.  Until
+ * CUDA graph launch per frame); then n_passes is 1 and each head is read once, though heads_read
+ * still counts a call of n rows as ceil(n / 32) passes.  Until
  * set, the tree is the chain of draft_len rank-0 nodes.  Errors: MCD_ERR_INVALID_ARG
  * (malformed tree), MCD_ERR_STATE (context not in TREE mode). */
 mcd_status mcd_set_tree(mcd_ctx* ctx, int32_t n_nodes, const int32_t* parent, const int32_t* rank);

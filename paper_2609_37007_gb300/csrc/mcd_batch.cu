@@ -1256,8 +1256,9 @@ __global__ void __launch_bounds__(256) batch_tree_attn_kernel(FrameParams p, Bat
   }
 }
 
-// Acceptance of a tree call (mcd_tree.cuh) and the while node's condition.  heads_read counts a
-// call of more than 32 rows as the passes of 32 rows the frame kernel runs it in.
+// Acceptance of a tree call (mcd_tree.cuh) and the while node's condition.  The call is one pass;
+// heads_read counts its heads once per 32 rows all the same, so that a frame's statistics do not
+// depend on which kernels ran it.
 __global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
   tc::pdl_wait();
   tc::pdl_trigger();
@@ -1272,7 +1273,7 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(Fra
   if (!st.done) {
     const BatchFrame* fa = b.frame;
     const int heads = (min(p.P, st.top_pos + p.K) - st.a) * ((st.n_rows + kMaxCols - 1) / kMaxCols);
-    const TreeCall t{&fa->tree, &st, cand, b.recs + (size_t)(call & 1) * b.R * kRecSlots, b.logits, heads,
+    const TreeCall t{&fa->tree, &st, cand, b.recs + (size_t)(call & 1) * b.R * kRecSlots, b.logits, heads, 1,
                      fa->stream_ids[0], fa->frame_ids[0], fa->codes_out, fa->stats, fa->trace};
     accept_tree_call(p, t);
   }

@@ -1240,8 +1240,8 @@ __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
   Smem sm = smem_layout(mcd_dyn_smem);
   const CallInfo* ci = sm.ci;
   // LM heads of the call's last pass (the earlier ones are in the state)
-  const TreeCall t{&p.tree, &ci->st[0], ci->tcand, p.topk, p.logits, ci->phi[0] - ci->plo[0] + 1, p.stream_ids[0],
-                   p.frame_ids[0], p.codes_out, p.stats, p.trace};
+  const TreeCall t{&p.tree, &ci->st[0], ci->tcand, p.topk, p.logits, ci->phi[0] - ci->plo[0] + 1,
+                   (ci->st[0].n_rows + kMaxCols - 1) / kMaxCols, p.stream_ids[0], p.frame_ids[0], p.codes_out, p.stats, p.trace};
   accept_tree_call(p, t);
   if (threadIdx.x == 0) red_release_add(p.ctr + (size_t)(call + 1) * p.ctr_stride + ctr_ready(p.L), 1u);
 }

@@ -13,6 +13,7 @@ struct TreeCall {
   const TopkRec* recs;                      // [row][1 + draft]
   const float* logits;                      // [row][kMaxDraft + 1][V]
   int heads;                                // LM heads to count
+  int passes;                               // weight passes of the call
   unsigned stream_id, frame_id;
   int* codes_out;
   mcd_frame_stats* stats;
@@ -234,7 +235,7 @@ static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, co
         tt->row_node[n] = n >= n_rows || pos0 == 0 ? -1 : n - 1;
         tt->row_id[n] = row_id(n);
       }
-      tt->n_passes = (n_rows + kMaxCols - 1) / kMaxCols;
+      tt->n_passes = in.passes;
       tt->path_len = plen;
       for (int t = 0; t < kMaxDraft + 1; ++t) tt->path[t] = t < plen ? t_path[t] : -1;
       tt->draft_row = drow;

@@ -581,6 +581,8 @@ def test_tree_mode_trace_parity_batched(nodes, depth):
         codes, st, tr = env.decode(fr, f, stream_id=1, trace=True)
         assert st[4] == 0 and st[1] == cfg.n_pos, st
         check_tree_trace_against_oracle(cfg, env.model, fr, 1, f, tr, codes, int(st[0]), tree, logit_tol=2e-2)
+        trecs = mcd.parse_tree_trace(np.asarray(tr, dtype=np.uint8), cfg.vocab)[0]
+        assert all(int(r["n_passes"]) == 1 for r in trecs[:int(st[0])])        # the batched kernels ran it
     env.dec.close()
 
 

@@ -1275,7 +1275,12 @@ __global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(Fra
     const int heads = (min(p.P, st.top_pos + p.K) - st.a) * ((st.n_rows + kMaxCols - 1) / kMaxCols);
     const TreeCall t{&fa->tree, &st, cand, b.recs + (size_t)(call & 1) * b.R * kRecSlots, b.logits, heads, 1,
                      fa->stream_ids[0], fa->frame_ids[0], fa->codes_out, fa->stats, fa->trace};
-    accept_tree_call(p, t);
+    const TreeDrafts d = accept_tree_call(p, t);
+    if (fa->trace && st.round < kMaxCalls) {           // consecutive rows on both sides
+      float* dlog = reinterpret_cast<float*>(fa->trace + sizeof(mcd_call_trace) * kMaxCalls) +
+                    ((size_t)kMaxCalls + st.round) * kMaxRows * p.V;
+      copy_logits(dlog, b.logits + ((size_t)d.row * (kMaxDraft + 1) + 1) * p.V, d.n * p.V);
+    }
   }
   if (threadIdx.x == 0) batch_call_end(p, b, loop, call, !__ldcg(&p.st->done));
 }

@@ -702,26 +702,53 @@ __device__ __noinline__ void attention_tree_task(const FrameParams& p, int layer
   consumer_sync();
 }
 
-// Trace of a verify call: the verify logits of each packed row, every row by another CTA (those
-// after the CTAs that built the call's distributions).  Runs once the CTA has signalled its
-// distributions; the logits stay until the next call's LM heads, which wait for every CTA.  (One
-// CTA copying every row before it released the next call cost 14 us per call at one row, 20 us
-// at four and 127 us at 33.)
-__device__ __noinline__ void trace_verify_rows(const FrameParams& p) {
-  const CallInfo* ci = smem_layout(mcd_dyn_smem).ci;
+// Logits that leave a call (trace, stepwise call), copied once the CTA has signalled its
+// distributions or released the next call; they stay until the next call's LM heads, which wait for
+// every CTA.  The verify logits of each packed row go by the CTAs after those that built the
+// call's distributions (one CTA copying every row before it released the next call cost 14 us per
+// call at one row, 20 us at four and 127 us at 33); the draft rows (flags[6] of them from
+// logits row flags[5]) and stepwise logits by the CTA that ran the acceptance.
+// A leaf with few registers: ptxas allocates them over a kernel's whole call graph, and a copy routine
+// called from here and from the acceptance steps lengthened every wide call (untraced frames of 3 / 4
+// streams 1125 -> 1147 and 1178 -> 1206 us; 1106 and 1165 in this form).
+__device__ __noinline__ void call_outputs(const FrameParams& p) {
+  Smem sm = smem_layout(mcd_dyn_smem);
+  const CallInfo* ci = sm.ci;
+  consumer_sync();                              // the acceptance step's flags
   const bool tree = p.draft_mode == MCD_DRAFT_TREE, noisy = p.draft_mode == MCD_DRAFT_NOISY_TARGET;
+  const int M = ci->M, sa = sm.flags[4], first = sm.flags[2] ? ci->st[sa].first_head_row : 0;
   int at = 0;                                   // distributions of the call
-  for (int r = 0; r < ci->M; ++r)
+  for (int r = 0; r < M; ++r)
     if (ci->r_pos[r] >= 1) at += 1 + (noisy ? 0 : min(p.K, p.P - ci->r_pos[r]));
-  for (int r = 0; r < ci->M; ++r) {
-    if (ci->r_pos[r] < 1 || (at + r) % p.n_cta != (int)blockIdx.x) continue;
-    const int s = ci->r_s[r], round = ci->st[s].round;
-    if (round >= kMaxCalls) continue;
-    uint8_t* tb = p.trace + (size_t)s * p.trace_stride + sizeof(mcd_call_trace) * kMaxCalls;
-    const size_t chain = (size_t)2 * kMaxCalls * kMaxRows * p.V * 4 + sizeof(mcd_tree_trace) * kMaxCalls;
-    float* dst = tree ? reinterpret_cast<float*>(tb + chain) + ((size_t)round * kMaxTreeRows + ci->row0 + r) * p.V
-                      : reinterpret_cast<float*>(tb) + ((size_t)round * kMaxRows + ci->r_n[r]) * p.V;
-    copy_logits(dst, p.logits + (size_t)(ci->row0 + r) * (kMaxDraft + 1) * p.V, p.V);
+  const int n_step = sm.flags[2] && p.single_call && p.logits_out ? ci->st[sa].n_rows - first : 0;
+  for (int job = 0; job <= M + n_step; ++job) {
+    float* dst;
+    const float* src;
+    int n = p.V;
+    if (job <= M) {
+      const bool verify = job < M;
+      if (!p.trace) continue;
+      if (verify ? ci->r_pos[job] < 1 || (at + job) % p.n_cta != (int)blockIdx.x : !sm.flags[2] || sm.flags[6] == 0) continue;
+      const int s = verify ? ci->r_s[job] : sa, round = ci->st[s].round;
+      if (round >= kMaxCalls) continue;
+      uint8_t* tb = p.trace + (size_t)s * p.trace_stride + sizeof(mcd_call_trace) * kMaxCalls;
+      const size_t rows = (size_t)kMaxCalls * kMaxRows, at_row = (size_t)round * kMaxRows;
+      if (!verify) {                            // consecutive rows on both sides
+        dst = reinterpret_cast<float*>(tb) + (rows + at_row) * p.V;
+        src = p.logits + ((size_t)sm.flags[5] * (kMaxDraft + 1) + 1) * p.V;
+        n *= sm.flags[6];
+      } else {
+        dst = tree ? reinterpret_cast<float*>(tb + 2 * rows * p.V * 4 + sizeof(mcd_tree_trace) * kMaxCalls) +
+                         ((size_t)round * kMaxTreeRows + ci->row0 + job) * p.V
+                   : reinterpret_cast<float*>(tb) + (at_row + ci->r_n[job]) * p.V;
+        src = p.logits + (size_t)(ci->row0 + job) * (kMaxDraft + 1) * p.V;
+      }
+    } else {
+      const int r = job - M - 1;
+      dst = p.logits_out + (size_t)r * p.V;
+      src = p.logits + (size_t)(ci->base[sa] + first + r) * (kMaxDraft + 1) * p.V;
+    }
+    copy_logits(dst, src, n);
   }
 }
 
@@ -1032,6 +1059,7 @@ __device__ __forceinline__ void run_call(Cons& c, int call) {
     }
     sm.flags[2] = mine >= 0 ? 1 : 0;
     sm.flags[4] = mine;
+    sm.flags[6] = 0;
   }
   consumer_sync();
   if (*(volatile int*)&sm.flags[1]) c.abort_ = true;
@@ -1177,6 +1205,8 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
     st->call = call + 1;
     st->done = a_new >= p.P ? 1 : 0;
     st->q_row = base + m;  // q of the next call's drafts: this call's records of packed row base + m
+    sm.flags[5] = base + m;
+    sm.flags[6] = noisy ? 0 : s_nnext;
     if (p.single_call) {
       if (p.emitted_out)
         for (int t = 0; t < s_nemit; ++t) p.emitted_out[t] = s_emit[t];
@@ -1195,8 +1225,7 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
     }
   }
   consumer_sync();
-  // optional outputs: trace and stepwise logits
-  const int fr = ci->st[s].first_head_row;
+  // optional trace record (the logits: call_outputs)
   if (p.trace && round < kMaxCalls) {
     uint8_t* tb = p.trace + (size_t)s * p.trace_stride;
     mcd_call_trace* tr = reinterpret_cast<mcd_call_trace*>(tb) + round;
@@ -1214,15 +1243,7 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
       for (int j = 0; j < kMaxRows; ++j) tr->next_drafts[j] = (j < s_nnext && !noisy) ? s_next[j] : -1;
       tr->draft_row = m;
     }
-    // the draft rows of row m (the verify rows were copied by the top-k stage)
-    float* dlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls) + (size_t)kMaxCalls * kMaxRows * p.V;
-    for (int n = 0; n < s_nnext && !noisy; ++n)
-      copy_logits(dlog + ((size_t)round * kMaxRows + n) * p.V, p.logits + ((size_t)(base + m) * (kMaxDraft + 1) + n + 1) * p.V,
-                  p.V);
   }
-  if (p.single_call && p.logits_out)
-    for (int n = fr; n < n_rows; ++n)
-      copy_logits(p.logits_out + (size_t)(n - fr) * p.V, p.logits + (size_t)(base + n) * (kMaxDraft + 1) * p.V, p.V);
   consumer_sync();
   if (s == 0) timeline_p(p, sm.ci, 7, true);
   if (threadIdx.x == 0) {
@@ -1235,15 +1256,19 @@ __device__ __noinline__ void accept_step(const FrameParams& p, int call, int s) 
 }
 
 // Acceptance step of a tree call (mcd_tree.cuh) by the CTA that finished top-k last, then the
-// release of the next call.
+// release of the next call (draft logits of a trace: call_outputs).
 __device__ __noinline__ void accept_tree(const FrameParams& p, int call) {
   Smem sm = smem_layout(mcd_dyn_smem);
   const CallInfo* ci = sm.ci;
   // LM heads of the call's last pass (the earlier ones are in the state)
   const TreeCall t{&p.tree, &ci->st[0], ci->tcand, p.topk, p.logits, ci->phi[0] - ci->plo[0] + 1,
                    (ci->st[0].n_rows + kMaxCols - 1) / kMaxCols, p.stream_ids[0], p.frame_ids[0], p.codes_out, p.stats, p.trace};
-  accept_tree_call(p, t);
-  if (threadIdx.x == 0) red_release_add(p.ctr + (size_t)(call + 1) * p.ctr_stride + ctr_ready(p.L), 1u);
+  const TreeDrafts d = accept_tree_call(p, t);
+  if (threadIdx.x == 0) {
+    sm.flags[5] = d.row;
+    sm.flags[6] = d.n;
+    red_release_add(p.ctr + (size_t)(call + 1) * p.ctr_stride + ctr_ready(p.L), 1u);
+  }
 }
 
 // End of a tree call's pass that another pass follows (run by the CTA that finished top-k
@@ -1483,7 +1508,7 @@ __global__ void __launch_bounds__(kThreads, 1) frame_kernel(const __grid_constan
         else
           accept_step(p, call, sm.flags[4]);
       }
-      if (p.trace && !sm.ci->emu) trace_verify_rows(p);
+      if ((p.trace || p.single_call) && !sm.ci->emu) call_outputs(p);
     }
     if (tid == 0) sm.flags[0] = 1;  // stop the producer
   }

@@ -398,9 +398,9 @@ __device__ inline __noinline__ double2 normal_pair(unsigned long long seed, uint
 // ---------------------------------------------------------------------------------------
 // Bounded waits: every spin gives up after wait_ns and records MCD_ERR_TIMEOUT.
 // ---------------------------------------------------------------------------------------
-// (The polling loops are out of line: a stage's code is short when nothing has to be waited for.)
-__device__ inline __noinline__ bool wait_counter_slow(const unsigned* p, unsigned target, int* err,
-                                                      unsigned long long wait_ns) {
+__device__ __forceinline__ bool wait_counter(const unsigned* p, unsigned target, int* err,
+                                             unsigned long long wait_ns) {
+  if (ld_acquire(p) >= target) return true;
   uint64_t t0 = globaltimer();
   uint32_t it = 0;
   while (ld_acquire(p) < target) {
@@ -414,14 +414,10 @@ __device__ inline __noinline__ bool wait_counter_slow(const unsigned* p, unsigne
   }
   return true;
 }
-__device__ __forceinline__ bool wait_counter(const unsigned* p, unsigned target, int* err,
-                                             unsigned long long wait_ns) {
-  if (ld_acquire(p) >= target) return true;
-  return wait_counter_slow(p, target, err, wait_ns);
-}
 
-__device__ inline __noinline__ bool wait_mbar_slow(uint64_t* bar, uint32_t parity, int* err, unsigned long long wait_ns,
-                                                   const volatile int* stop) {
+__device__ __forceinline__ bool wait_mbar(uint64_t* bar, uint32_t parity, int* err, unsigned long long wait_ns,
+                                          const volatile int* stop) {
+  if (mbar_try_wait(bar, parity)) return true;
   uint64_t t0 = globaltimer();
   uint32_t it = 0;
   while (!mbar_try_wait(bar, parity)) {
@@ -435,11 +431,6 @@ __device__ inline __noinline__ bool wait_mbar_slow(uint64_t* bar, uint32_t parit
     }
   }
   return true;
-}
-__device__ __forceinline__ bool wait_mbar(uint64_t* bar, uint32_t parity, int* err, unsigned long long wait_ns,
-                                          const volatile int* stop) {
-  if (mbar_try_wait(bar, parity)) return true;
-  return wait_mbar_slow(bar, parity, err, wait_ns, stop);
 }
 
 }  // namespace mcd

@@ -60,24 +60,18 @@ __device__ __forceinline__ float exp32_cw(float d) {
 
 __device__ __forceinline__ uint32_t weight24(float e) { return __float2uint_rd(__fmul_rn(e, 16777216.0f)); }
 
-// Copy of a logits row (src 16-byte aligned, V a multiple of 16) by threads 0..nt-1 of the CTA:
-// 16-byte pieces, four in flight per thread, where the destination is aligned, else words.
-__device__ inline __noinline__ void copy_logits(float* dst, const float* src, int V, int nt = kConsumerThreads) {
+// Copy of V logits (src 16-byte aligned, V a multiple of 16) by the CTA's consumer threads: 16-byte
+// pieces where the destination is aligned, else words.  One load in flight per thread: four took the
+// persistent kernels' untraced frames longer (registers are allocated over the whole call graph; three
+// streams of the small fp32 model 231 -> 238 us) and traced ones no shorter than 1 %.
+__device__ __forceinline__ void copy_logits(float* dst, const float* src, int V) {
   if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-    float4* d = reinterpret_cast<float4*>(dst);
-    const float4* q = reinterpret_cast<const float4*>(src);
-    const int n = V >> 2;
-    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * nt) {
-      float4 v[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (i0 + e * nt < n) v[e] = __ldcg(q + i0 + e * nt);
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (i0 + e * nt < n) d[i0 + e * nt] = v[e];
-    }
+#pragma unroll 1
+    for (int i = threadIdx.x; i < V >> 2; i += kConsumerThreads)
+      reinterpret_cast<float4*>(dst)[i] = __ldcg(reinterpret_cast<const float4*>(src) + i);
   } else {
-    for (int i = threadIdx.x; i < V; i += nt) dst[i] = __ldcg(src + i);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < V; i += kConsumerThreads) dst[i] = __ldcg(src + i);
   }
 }
 

@@ -63,7 +63,8 @@ struct Smem {
   float* part;     // [kConsumerWarps][kMaxCols] partial sums of squares
   uint64_t* full;
   uint64_t* empty;
-  int* flags;      // [0] stop, [1] abort, [2] last-arriver, [4] stream whose acceptance this CTA runs
+  int* flags;      // [0] stop, [1] abort, [2] last-arriver, [4] stream whose acceptance this CTA runs,
+                   // [5] logits row of the next drafts, [6] their number (call_outputs)
   float* inv_rms;  // [kMaxCols]
   CallInfo* ci;    // snapshot of the call's state
 };
@@ -612,10 +613,11 @@ __device__ __forceinline__ StagePlan plan_stage(const Cons& c, int si, int n_uni
     while (cnt < sp.cap && u0 + cnt * sp.ur.step < sp.ur.end && opkey(u0 + cnt * sp.ur.step) == key) ++cnt;
     sp.cnt0 = cnt;
   }
-  // wide calls: computed here and not behind the wait, where the compiler would move what only
-  // the stage uses (3 streams 1148 -> 1134 us, a 32-node tree 2145 -> 2118; the small fp32 model's
-  // frames, whose waits are short, took 134 -> 151)
-  if constexpr (WIDE)
+  // wide calls of 16- or 8-bit weights: computed here and not behind the wait, where the compiler
+  // would move what only the stage uses (3 streams 1152 -> 1126 us, int8 1305 -> 1252, a tree of 8
+  // nodes 1556 -> 1526).  The small fp32 model's waits are short: its frames took 134 -> 151 with
+  // one stream, 240 -> 258 with three
+  if constexpr (WIDE && WT != MCD_WEIGHT_F32)
     for (int* v : {&sp.ur.first, &sp.ur.end, &sp.ur.step, &sp.cnt0, &sp.cap, &sp.lg_unit, &sp.lgn, &sp.role.mi, &sp.role.kg,
                    &sp.role.gn, &sp.role.kts, &sp.role.Gk, &sp.role.Gn, &sp.role.ntpw, &sp.role.lg_ntpw})
       pin(*v);

@@ -20,6 +20,11 @@ struct TreeCall {
   uint8_t* trace;
 };
 
+// Call row whose draft logits gave the next candidates, and their depths.
+struct TreeDrafts {
+  int row, n;
+};
+
 // Acceptance step of a tree call (one stream, by the 256 consumer threads of one CTA).
 // One warp walks the tree from the first row: the children of the current node are tested
 // in rank order, test i keeping its candidate x iff U * S' < 2^53 * W_x, S' being the
@@ -28,7 +33,7 @@ struct TreeCall {
 // and the call ends.  Then: the next call's candidates (the top-m ids by logit of each
 // draft distribution of the last visited row), the kept nodes' K / V moved to their
 // positions, the state update and the trace.
-static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, const TreeCall& in) {
+static __device__ __forceinline__ TreeDrafts accept_tree_call(const FrameParams& p, const TreeCall& in) {
   const DevState& st0 = *in.st;
   const TreeDef& tree = *in.tree;
   const int a = st0.a, pos0 = st0.pos0, n_rows = st0.n_rows, round = st0.round;
@@ -143,7 +148,6 @@ static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, co
   }
   consumer_sync();
   // state of the next call
-  __shared__ int t_nvalid, t_maxd;
   if (threadIdx.x == 0) {
     int nv = 0, md = 0;
     for (int i = 0; i < tree.n; ++i) {
@@ -153,8 +157,6 @@ static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, co
         md = max(md, d);
       }
     }
-    t_nvalid = nv;
-    t_maxd = md;
     DevState* st = p.st;
     int* codes_out = in.codes_out;
     for (int t = 0; t < n_emit; ++t) {
@@ -200,13 +202,10 @@ static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, co
     p.tree_cand[i] = (d < n_next && r < tree.m[d]) ? t_next[d][r] : -1;
   }
   consumer_sync();
-  // optional trace: the chain record, the draft row's logits and the tree record (every row's
-  // verify logits were copied by the top-k stage)
+  // optional trace: the chain record and the tree record (the caller copies the logits)
   if (in.trace && round < kMaxCalls) {
     uint8_t* tb = in.trace;
     mcd_call_trace* tr = reinterpret_cast<mcd_call_trace*>(tb) + round;
-    float* dlog = reinterpret_cast<float*>(tb + sizeof(mcd_call_trace) * kMaxCalls) +
-                  (size_t)kMaxCalls * kMaxRows * p.V;
     const size_t chain_bytes = sizeof(mcd_call_trace) * kMaxCalls + (size_t)2 * kMaxCalls * kMaxRows * p.V * 4;
     mcd_tree_trace* tt = reinterpret_cast<mcd_tree_trace*>(tb + chain_bytes) + round;
     if (threadIdx.x == 0) {
@@ -244,10 +243,9 @@ static __device__ __forceinline__ void accept_tree_call(const FrameParams& p, co
         for (int r = 0; r < kMaxTreeRank; ++r)
           tt->next_cand[d][r] = (d < n_next && d < kMaxDraft && r < tree.m[d]) ? t_next[d][r] : -1;
     }
-    for (int n = 0; n < n_next; ++n)
-      copy_logits(dlog + ((size_t)round * kMaxRows + n) * p.V, in.logits + ((size_t)drow * (kMaxDraft + 1) + n + 1) * p.V, p.V);
   }
   consumer_sync();
+  return TreeDrafts{drow, n_next};
 }
 
 }  // namespace mcd

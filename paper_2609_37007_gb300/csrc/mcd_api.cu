@@ -746,14 +746,14 @@ mcd_status mcd_decode_frames(mcd_ctx* c, int32_t n_streams, const uint32_t* stre
     if (!cond || !stream_ids || !frame_idx) return MCD_ERR_INVALID_ARG;
     if (p.C0V > 0 && !c0) return MCD_ERR_INVALID_ARG;
     if (p.C0V == 0 && !c0_emb) return MCD_ERR_INVALID_ARG;
-    c->frame_begun = false;
-    if (tree_batch) {            // as begin_frame leaves a context: 16-byte rows, the frame's counters
-      if ((reinterpret_cast<uintptr_t>(cond) & 15u) || (reinterpret_cast<uintptr_t>(c0_emb) & 15u))
-        return MCD_ERR_INVALID_ARG;
+    // (16-byte rows: what a tree call asks for on either route)
+    if (tree_batch && ((reinterpret_cast<uintptr_t>(cond) & 15u) || (reinterpret_cast<uintptr_t>(c0_emb) & 15u)))
+      return MCD_ERR_INVALID_ARG;
+    c->frame_begun = tree_batch;
+    if (tree_batch) {            // as launch_begin leaves a context: the frame's counters
       c->fp.stream_ids[0] = stream_ids[0];
       c->fp.frame_ids[0] = frame_idx[0];
       c->fp.S = 1;
-      c->frame_begun = true;
     }
     return batch_decode(c->batch, p, c->stream, n_streams, stream_ids, frame_idx, cond, c0, c0_emb, codes_out, stats,
                         p.trace);

@@ -586,6 +586,31 @@ def test_tree_mode_trace_parity_batched(nodes, depth):
     env.dec.close()
 
 
+@pytest.mark.parametrize("nodes", [8, 32])
+def test_refused_tree_call_leaves_the_context_as_it_was(nodes):
+    """A tree call with a misaligned row is refused on either route, and what followed the frame
+    before it (here mcd_draft) still works."""
+    from oracle.tree import grow_tree
+    cfg = TINY_BF16.replace(draft_mode=3, draft_len=3, n_pos=8, vocab=256)
+    env = Env(cfg)
+    tree = grow_tree([[0.6 / (r + 1) ** 0.5 for r in range(8)] for _ in range(3)], nodes)
+    mcd.mcd_set_tree(env.dec.ctx, tree.parent, tree.rank)
+    fr = make_frame(cfg, 0)
+    want, _, _ = env.decode(fr, 0)
+    cond, c0, emb = env.frame_inputs(fr)
+    shifted = torch.zeros(cfg.hidden + 1, device=DEV)[1:]
+    codes = torch.full((cfg.n_pos,), -1, dtype=torch.int32, device=DEV)
+    for bad in ((shifted, emb), (cond, shifted), (None, emb)):
+        with pytest.raises(mcd.MCDError):
+            mcd.mcd_decode_frame(env.dec.ctx, 0, 0, bad[0], c0, bad[1], codes)
+    drafts = torch.full((3,), -1, dtype=torch.int32, device=DEV)
+    mcd.mcd_draft(env.dec.ctx, 1, 0, torch.ones(cfg.hidden, device=DEV), drafts)
+    mcd.mcd_sync(env.dec.ctx)
+    assert (drafts >= 0).all() and (codes == -1).all()
+    assert list(env.decode(fr, 0)[0]) == list(want)
+    env.dec.close()
+
+
 def test_chain_tree_equals_greedy_drafts_on_gpu():
     cfg = TINY.replace(draft_len=3, n_pos=8)
     tree_env = Env(cfg.replace(draft_mode=3))

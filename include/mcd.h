@@ -319,7 +319,10 @@ typedef struct {
  * acceptance step follows the last pass.  bf16 models whose widths suit the tensor-core
  * products run trees of 16 nodes or more in one pass on the batched kernels instead (one
  * CUDA graph launch per frame); then n_passes is 1 and each head is read once, though heads_read
- * still counts a call of n rows as ceil(n / 32) passes.  Until
+ * still counts a call of n rows as ceil(n / 32) passes.  A TREE context of such a model holds a
+ * second, tiled copy of its layers and LM heads from mcd_create on, whatever its trees (213 MB
+ * for the MultiCodeDecoder, and buffers for 65 rows); where that memory is not to be had, every
+ * tree runs in passes.  The first tree of 16 nodes or more also builds the graph here.  Until
  * set, the tree is the chain of draft_len rank-0 nodes.  Errors: MCD_ERR_INVALID_ARG
  * (malformed tree), MCD_ERR_STATE (context not in TREE mode). */
 mcd_status mcd_set_tree(mcd_ctx* ctx, int32_t n_nodes, const int32_t* parent, const int32_t* rank);

@@ -844,6 +844,13 @@ mcd_status mcd_set_tree(mcd_ctx* c, int32_t n_nodes, const int32_t* parent, cons
     p.tree.anc[i] = (parent[i] < 0 ? 0ull : p.tree.anc[parent[i]]) | (1ull << i);
   }
   for (int d = 0; d < kMaxDraft; ++d) p.tree.m[d] = m[d];
+  // the batched kernels' graph is built here, not in the first frame (a 32-node tree's took 200 to
+  // 500 us longer); where that cannot be done now, the first frame does it
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (c->batch && batch_tree_prefers(n_nodes) &&
+      (cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone ||
+       batch_prepare(c->batch, p, &c->stream) != MCD_OK))
+    (void)cudaGetLastError();
   return MCD_OK;
 }
 

@@ -1644,6 +1644,22 @@ static cudaError_t build_graph(const FrameParams& p, BatchState* bs) {
   return cudaGraphInstantiate(&bs->exec, bs->graph, 0);
 }
 
+mcd_status batch_prepare(BatchState* bs, const FrameParams& p, const cudaStream_t* upload) {
+  if (bs->exec) return MCD_OK;
+  // the caller may be capturing a stream of its own: nothing here touches it
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  MCD_CHECK(cudaThreadExchangeStreamCaptureMode(&mode));
+  const cudaError_t e = build_graph(p, bs);
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    if (bs->graph) cudaGraphDestroy(bs->graph);
+    bs->graph = nullptr;
+    return cuda_status(e);
+  }
+  if (upload) MCD_CHECK(cudaGraphUpload(bs->exec, *upload));
+  return MCD_OK;
+}
+
 mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t stream, int n, const uint32_t* stream_ids,
                         const uint32_t* frame_ids, const float* cond, const int32_t* c0, const float* c0_emb,
                         int32_t* codes_out, mcd_frame_stats* stats, uint8_t* trace) {
@@ -1652,13 +1668,9 @@ mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t strea
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   MCD_CHECK(cudaStreamIsCapturing(stream, &capturing));
   const bool unrolled = capturing == cudaStreamCaptureStatusActive;
-  if (!unrolled && !bs->exec) {
-    const cudaError_t e = build_graph(p, bs);
-    if (e != cudaSuccess) {
-      if (bs->graph) cudaGraphDestroy(bs->graph);
-      bs->graph = nullptr;
-      return cuda_status(e);
-    }
+  if (!unrolled) {
+    const mcd_status r = batch_prepare(bs, p);
+    if (r != MCD_OK) return r;
   }
   BatchFrame f;
   memset(&f, 0, sizeof(f));

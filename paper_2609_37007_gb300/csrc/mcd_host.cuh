@@ -74,6 +74,9 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
 mcd_status batch_load_layer(BatchState* bs, const FrameParams& p, cudaStream_t st, const LayerSrc& src, int l);
 mcd_status batch_load_head(BatchState* bs, const FrameParams& p, cudaStream_t st, const uint8_t* src, int P);
 void batch_destroy(BatchState* bs);
+// Builds the frame graph (once; batch_decode does it otherwise); with `upload`, also moves it to the
+// device on that stream.
+mcd_status batch_prepare(BatchState* bs, const FrameParams& p, const cudaStream_t* upload = nullptr);
 mcd_status batch_decode(BatchState* bs, const FrameParams& p, cudaStream_t stream, int n, const uint32_t* stream_ids,
                         const uint32_t* frame_ids, const float* cond, const int32_t* c0, const float* c0_emb,
                         int32_t* codes_out, mcd_frame_stats* stats, uint8_t* trace);

@@ -586,6 +586,38 @@ def test_tree_mode_trace_parity_batched(nodes, depth):
     env.dec.close()
 
 
+def test_first_frame_of_a_large_tree_builds_no_graph():
+    """mcd_set_tree prepares what the batched kernels need: the first frame of a 32-node tree takes
+    as long as the next ones (measured 1.01 to 1.02 times; 1.18 to 1.19 where it builds the graph)."""
+    import time
+    from oracle.tree import grow_tree
+    cfg = TINY_BF16.replace(draft_mode=3, draft_len=3, n_pos=8, vocab=256)
+    w = make_weights(cfg)
+    tree = grow_tree([[0.6 / (r + 1) ** 0.5 for r in range(8)] for _ in range(3)], 32)
+    fr = make_frame(cfg, 0)
+    ratios = []
+    for rep in range(6):
+        env = Env(cfg, w)
+        cond, c0, emb = env.frame_inputs(fr)
+        codes = torch.full((cfg.n_pos,), -1, dtype=torch.int32, device=DEV)
+
+        def frame():
+            t0 = time.perf_counter()
+            mcd.mcd_decode_frame(env.dec.ctx, 0, 0, cond, c0, emb, codes)
+            torch.cuda.synchronize()
+            return time.perf_counter() - t0
+
+        frame()                                    # the default chain, on the frame kernel
+        mcd.mcd_set_tree(env.dec.ctx, tree.parent, tree.rank)
+        torch.cuda.synchronize()
+        first = frame()
+        ratios.append(first / min(frame() for _ in range(10)))
+        mcd.mcd_sync(env.dec.ctx)
+        env.dec.close()
+    print("first frame / later frames:", [round(r, 2) for r in ratios])
+    assert min(ratios[1:]) < 1.1, ratios           # the first context also loads the kernels
+
+
 @pytest.mark.parametrize("nodes", [8, 32])
 def test_refused_tree_call_leaves_the_context_as_it_was(nodes):
     """A tree call with a misaligned row is refused on either route, and what followed the frame

@@ -564,10 +564,9 @@ mcd_status mcd_create(const mcd_config* cfg, void* cuda_stream, mcd_ctx** out) {
   } else if (batch_tree_supported(p)) {
     // larger trees run on the batched kernels; without memory for their buffers the frame
     // kernel takes every tree
-    if (batch_create(p, 1, &c->batch) != MCD_OK) {
-      c->batch = nullptr;
-      (void)cudaGetLastError();
-    }
+    const mcd_status bs = batch_create(p, 1, &c->batch);
+    if (bs == MCD_ERR_OOM) (void)cudaGetLastError();       // (batch_create left nothing behind)
+    else if (bs != MCD_OK) return fail(bs);
   }
   *out = c;
   return MCD_OK;

@@ -1420,8 +1420,8 @@ mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out)
     BATCH_ALLOC(b.qkv, sizeof(float) * R * p.qkv_dim);
   }
 #undef BATCH_ALLOC
-  if (cudaMemset(b.info, 0, sizeof(BatchInfo)) != cudaSuccess) return fail(MCD_ERR_CUDA);
-  if (cudaStreamCreateWithFlags(&bs->cap, cudaStreamNonBlocking) != cudaSuccess) return fail(MCD_ERR_CUDA);
+  if ((e = cudaMemset(b.info, 0, sizeof(BatchInfo))) != cudaSuccess) return fail(cuda_status(e));
+  if ((e = cudaStreamCreateWithFlags(&bs->cap, cudaStreamNonBlocking)) != cudaSuccess) return fail(cuda_status(e));
   void* gemms[] = {(void*)batch_gemm_kernel<BSRC_NORM_HILO, EPI_QKV>, (void*)batch_gemm_kernel<BSRC_BF16, EPI_RESID>,
                    (void*)batch_gemm_kernel<BSRC_NORM, EPI_SWIGLU>, (void*)batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>};
   for (void* fn : gemms)

@@ -5,6 +5,7 @@ import ctypes
 import os
 import re
 import subprocess
+import sys
 
 import pytest
 
@@ -100,3 +101,55 @@ def test_null_context_calls_return_errors(lib):
     assert lib.mcd_decode_frame(None, 0, 0, None, None, None, None, None) == 1
     assert lib.mcd_num_ctas(None) == 0
     lib.mcd_destroy(None)
+
+
+FAKE_RUNTIME = r"""
+#include <stdlib.h>
+static int n_malloc;
+int cudaMalloc(void** p, size_t n) {
+  (void)n;
+  if (++n_malloc == atoi(getenv("FAIL_AT"))) return atoi(getenv("FAIL_CODE"));
+  *p = calloc(1, 1024);
+  return 0;
+}
+int allocations(void) { return n_malloc; }
+int cudaFree(void* p) { free(p); return 0; }
+int cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; *p = calloc(1, n); return 0; }
+int cudaFreeHost(void* p) { free(p); return 0; }
+int cudaGetDeviceCount(int* n) { *n = 1; return 0; }
+int cudaGetDevice(int* d) { *d = 0; return 0; }
+int cudaDeviceGetAttribute(int* v, int a, int d) { (void)d; *v = a == 16 ? 152 : 1; return 0; }
+int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n) { *n = 1; return 0; }
+#define OK(name) int name() { return 0; }
+OK(cudaFuncSetAttribute) OK(cudaMemset) OK(cudaMemsetAsync) OK(cudaStreamSynchronize) OK(cudaGetLastError)
+OK(cudaStreamCreateWithFlags) OK(cudaStreamDestroy) OK(__cudaPushCallConfiguration) OK(__cudaPopCallConfiguration)
+OK(__cudaGetKernel) OK(__cudaLaunchKernel)
+"""
+
+
+def test_tree_contexts_do_without_the_batched_buffers_only_when_memory_is_short(tmp_path):
+    """mcd_create of a TREE context whose last allocation (one of the batched kernels' buffers) fails:
+    out of memory leaves it to the frame kernel, any other error fails the call.  The CUDA runtime is
+    a fake that fails the allocation."""
+    from paper_2609_37007_gb300 import build
+    build.build()
+    (tmp_path / "fake.c").write_text(FAKE_RUNTIME)
+    fake = str(tmp_path / "fake.so")
+    subprocess.run(["gcc", "-w", "-std=gnu11", "-shared", "-fPIC", "-o", fake, str(tmp_path / "fake.c")], check=True)
+    code = ("import ctypes, sys; sys.path.insert(0, %r)\n"
+            "from paper_2609_37007_gb300 import mcd\n"
+            "from paper_2609_37007_gb300.synth import MCD\n"
+            "c, out = mcd.config_struct(MCD.replace(draft_mode=3)), ctypes.c_void_p()\n"
+            "status = mcd.load_library().mcd_create(ctypes.byref(c), None, ctypes.byref(out))\n"
+            "print(status, ctypes.CDLL(%r).allocations())\n" % (ROOT, fake))
+
+    def create(fail_at, fail_code):
+        env = dict(os.environ, LD_PRELOAD=fake, FAIL_AT=str(fail_at), FAIL_CODE=str(fail_code))
+        r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env=env, check=True)
+        return [int(v) for v in r.stdout.split()]
+
+    status, last = create(0, 0)
+    assert status == 0 and last > 20
+    assert create(last, 2) == [0, last]              # cudaErrorMemoryAllocation
+    assert create(last, 46)[0] == 3                  # cudaErrorDevicesUnavailable: MCD_ERR_CUDA
+    assert create(1, 2)[0] == 4                      # the weight arena itself: MCD_ERR_OOM

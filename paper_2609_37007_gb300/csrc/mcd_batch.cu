@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(256) batch_embed_tc_kernel(FrameParams p, Batc
   __shared__ __align__(16) float row_s[1024];
   __shared__ float sw[8];
   const int r = blockIdx.x, t = threadIdx.x;
+  tc::pdl_wait();
   tc::pdl_trigger();
   if (r >= b.info->M) return;
   const BatchRow row = b.rows[r];

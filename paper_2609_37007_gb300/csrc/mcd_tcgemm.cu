@@ -17,6 +17,7 @@ namespace tc {
 template <class Index>
 __global__ void __launch_bounds__(256) sw128_tile_kernel(const uint16_t* __restrict__ src, Index total, int R, int K, int ld,
                                                          uint8_t* __restrict__ dst) {
+  pdl_wait();
   pdl_trigger();
   const Index cpr = (Index)(K / 8), step = (Index)gridDim.x * 256;
   for (Index i = (Index)blockIdx.x * 256 + threadIdx.x; i < total; i += step) {

@@ -153,3 +153,18 @@ def test_tree_contexts_do_without_the_batched_buffers_only_when_memory_is_short(
     assert create(last, 2) == [0, last]              # cudaErrorMemoryAllocation
     assert create(last, 46)[0] == 3                  # cudaErrorDevicesUnavailable: MCD_ERR_CUDA
     assert create(1, 2)[0] == 4                      # the weight arena itself: MCD_ERR_OOM
+
+
+def test_dependent_launch_triggers_follow_their_wait():
+    """Every kernel that lets the next one start early (pdl_trigger) has waited for the ones in front
+    of it (pdl_wait) on the line before: the order that keeps two kernels at most in flight and a
+    grid from completing before the grids in front of it, however it is launched."""
+    found = 0
+    for path in glob.glob(os.path.join(ROOT, "paper_2609_37007_gb300", "csrc", "*.cu*")):
+        lines = [re.sub(r"//.*", "", line).strip() for line in open(path)]
+        lines = [line for line in lines if line]
+        for prev, line in zip([""] + lines, lines):
+            if re.fullmatch(r"(tc::)?pdl_trigger\(\);", line):
+                found += 1
+                assert re.fullmatch(r"(tc::)?pdl_wait\(\);", prev), (path, prev)
+    assert found >= 8

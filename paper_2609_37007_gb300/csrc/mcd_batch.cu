@@ -614,8 +614,6 @@ __global__ void __launch_bounds__(kHeadsThreads, 1) tc_heads_kernel(const tc::Ge
                                                                     size_t head_bytes, float* logits,
                                                                     const float* head_bias, const BatchInfo* info,
                                                                     const int* head_list, int n_pos, int K, int V) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
   int P = 0, qoff = 0, c0 = 0, nw = 0, rows = 0;
   for (int i = 1, o = 0, t = blockIdx.x; i <= n_pos; ++i) {
     const int r = info->head_rows[i], nt = tc_head_tiles(r);
@@ -853,8 +851,6 @@ __global__ void __launch_bounds__(256, 7) batch_attn_kernel(FrameParams p, Batch
 __global__ void __launch_bounds__(kConsumerThreads) batch_topk_kernel(FrameParams p, BatchBufs b) {
   __shared__ __align__(16) uint8_t smem_raw[sizeof(TopkScratch)];
   TopkScratch& ts = *reinterpret_cast<TopkScratch*>(smem_raw);
-  tc::pdl_wait();
-  tc::pdl_trigger();
   const int call = b.info->call, n_pair_ctas = (int)gridDim.x - b.R;
   if ((int)blockIdx.x >= n_pair_ctas) {     // packed row r's verify logits into an optional trace
     const int r = (int)blockIdx.x - n_pair_ctas;
@@ -890,8 +886,6 @@ __device__ __forceinline__ void batch_call_end(const FrameParams& p, const Batch
 }
 
 __global__ void __launch_bounds__(kConsumerThreads) batch_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
   const int s = blockIdx.x, call = b.info->call;
   const BatchFrame* fa = b.frame;
   const int base = s < fa->S ? b.sbase[s] : -1;
@@ -1136,8 +1130,6 @@ __global__ void __launch_bounds__(128) batch_tree_pack_kernel(FrameParams p, Bat
 // QK-norm + RoPE of every row's query and key heads; K and V to the row's cache slot, the
 // queries to tree_q.  One warp per (row, vector), lane holding dims lane + 32 i.
 __global__ void __launch_bounds__(256) batch_tree_rope_kernel(FrameParams p, BatchBufs b, int layer) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
   const int vecs = p.NH + 2 * p.NKV, w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int r = w / vecs, vi = w - r * vecs;
   if (r >= b.info->M) return;
@@ -1261,8 +1253,6 @@ __global__ void __launch_bounds__(256) batch_tree_attn_kernel(FrameParams p, Bat
 // heads_read counts its heads once per 32 rows all the same, so that a frame's statistics do not
 // depend on which kernels ran it.
 __global__ void __launch_bounds__(kConsumerThreads) batch_tree_accept_kernel(FrameParams p, BatchBufs b, BatchLoop loop) {
-  tc::pdl_wait();
-  tc::pdl_trigger();
   __shared__ DevState st;
   __shared__ int cand[kMaxDraft][kMaxTreeRank];
   const int call = b.info->call;
@@ -1476,9 +1466,9 @@ static void enqueue_heads(const FrameParams& p, const BatchState* bs, cudaStream
   const BatchBufs& b = bs->b;
   const int R = b.R, H = p.H;
   const tc::GemmArgs g{nullptr, b.hq_hi, b.hq_lo, p.V, b.Qcap, H, nullptr, p.err, p.wait_ns, false, 0};
-  tc::launch(false, tc_heads_kernel, dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), dim3(kHeadsThreads),
-                 tc::Layout<kHeadTileMax, true>::kSmemBytes, s, g, bs->tw.heads, (size_t)p.V * H * 2, b.logits,
-                                                                    p.head_bias, b.info, b.head_list, p.P, p.K, p.V);
+  tc_heads_kernel<<<dim3(tc_head_grid_x(R, p.K, p.P), p.V / tc::kBM, 1), kHeadsThreads,
+                    tc::Layout<kHeadTileMax, true>::kSmemBytes, s>>>(g, bs->tw.heads, (size_t)p.V * H * 2, b.logits, p.head_bias,
+                                                                     b.info, b.head_list, p.P, p.K, p.V);
 }
 
 // The operand a residual pass leaves: the next layer's QKV operand, or after the last layer the LM
@@ -1589,8 +1579,8 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
     batch_gemm_kernel<BSRC_NORM_HILO, EPI_HEADS>
         <<<dim3(a.g.M / kGM + (a.g.M % kGM != 0), R / kGN, p.P), blk, kGemmSmemHilo, s>>>(a);
   }
-  tc::launch(false, batch_topk_kernel, dim3(R * (p.K + 1) + R), dim3(kConsumerThreads), 0, s, p, b);
-  tc::launch(false, batch_accept_kernel, dim3(bs->max_streams), dim3(kConsumerThreads), 0, s, p, b, loop);
+  batch_topk_kernel<<<R * (p.K + 1) + R, kConsumerThreads, 0, s>>>(p, b);
+  batch_accept_kernel<<<bs->max_streams, kConsumerThreads, 0, s>>>(p, b, loop);
   return cudaGetLastError();
 }
 

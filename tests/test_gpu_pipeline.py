@@ -252,14 +252,17 @@ def test_decode_rows_at_key_block_edges(full_pipe, tokens):
 @pytest.mark.parametrize("tokens", [2, 16, 17, 18, 32, 33, 34, 65, 129, 130, 161, 260])
 def test_prompt_attention_at_tile_edges(heads, dim, tokens):
     """The batched prompt rows around the attention kernel's tiles: 16 query rows, 32 keys, four
-    warps of key blocks.  Tolerance: the bf16 model's 2e-2 (K and V are cached as bf16 values,
-    2^-9 relative each)."""
+    warps of key blocks.  Tolerance: operands are hi + lo pairs (2^-17 relative), so what is left of
+    the bf16 model's 2e-2 are cached K and V values that round to the other neighbour (2^-8
+    relative): those within 2^-17 of a boundary, about 2^-7 of them, whose independent errors add up
+    to sqrt(2^-7) of 2e-2, 1.8e-3 rms; 3e-3 for the largest.  Measured 1.4e-3 at most, 5.6e-3 to
+    1.1e-2 without the low halves of the attention's and SwiGLU's outputs."""
     ocfg = OUTER_TINY.replace(weight_dtype=WEIGHT_BF16, n_q_heads=heads[0], n_kv_heads=heads[1], head_dim=dim,
                               prompt_len=tokens)
     env = PipeEnv(ocfg, TINY.replace(weight_dtype=WEIGHT_BF16))
     try:
         prompt = make_prompt(ocfg)
         frames, otr = env.run(prompt, 1)
-        check_pipeline(env, prompt, frames, otr, 2e-2)
+        check_pipeline(env, prompt, frames, otr, 3e-3)
     finally:
         env.pl.close()

@@ -161,7 +161,8 @@ mcd_status mcd_load_weights(mcd_ctx* ctx, int32_t n, const char* const* names,
  *          [0, c0_vocab) fails the frame with MCD_ERR_INVALID_ARG (reported by mcd_sync).
  *   c0_emb dev float [hidden], 16-byte aligned: c0 embedding (c0_vocab == 0), else NULL.
  *   stats  dev mcd_frame_stats, optional (NULL).
- * One cooperative persistent-kernel launch runs every call of the frame on device. */
+ * One cooperative persistent-kernel launch runs every call of the frame on device (larger trees: one
+ * CUDA graph, see mcd_set_tree). */
 mcd_status mcd_decode_frame(mcd_ctx* ctx, uint32_t stream_id, uint32_t frame_idx,
                             const float* cond, const int32_t* c0, const float* c0_emb,
                             int32_t* codes_out, mcd_frame_stats* stats);
@@ -322,7 +323,8 @@ typedef struct {
  * still counts a call of n rows as ceil(n / 32) passes.  A TREE context of such a model holds a
  * second, tiled copy of its layers and LM heads from mcd_create on, whatever its trees (213 MB
  * for the MultiCodeDecoder, and buffers for 65 rows); where that memory is not to be had, every
- * tree runs in passes.  The first tree of 16 nodes or more also builds the graph here.  Until
+ * tree runs in passes.  The first tree of 16 nodes or more also builds the graph here.  A frame
+ * captured into the caller's graph runs trees of up to 31 nodes in one pass of the frame kernel.  Until
  * set, the tree is the chain of draft_len rank-0 nodes.  Errors: MCD_ERR_INVALID_ARG
  * (malformed tree), MCD_ERR_STATE (context not in TREE mode). */
 mcd_status mcd_set_tree(mcd_ctx* ctx, int32_t n_nodes, const int32_t* parent, const int32_t* rank);

@@ -735,8 +735,13 @@ mcd_status mcd_decode_frames(mcd_ctx* c, int32_t n_streams, const uint32_t* stre
   if (!c || !codes_out) return MCD_ERR_INVALID_ARG;
   if (!c->weights_loaded) return MCD_ERR_STATE;
   // (a tree call's stage stamps come from the frame kernel)
-  const bool tree_batch = c->batch && n_streams == 1 && batch_tree_supported(c->fp) && batch_tree_prefers(c->fp.tree.n) &&
-                          !c->fp.timeline;
+  bool tree_batch = c->batch && n_streams == 1 && batch_tree_supported(c->fp) && batch_tree_prefers(c->fp.tree.n, false) &&
+                    !c->fp.timeline;
+  if (tree_batch && !batch_tree_prefers(c->fp.tree.n, true)) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    MCD_CHECK(cudaStreamIsCapturing(c->stream, &capturing));
+    tree_batch = capturing == cudaStreamCaptureStatusNone;
+  }
   if (n_streams > kMaxStreams || batch_rows(c->fp, n_streams) > kMaxCols ||
       (c->batch && batch_prefers(c->fp, n_streams)) || tree_batch) {
     // many streams: the batched GEMM path (one CUDA graph launch per frame)
@@ -846,7 +851,7 @@ mcd_status mcd_set_tree(mcd_ctx* c, int32_t n_nodes, const int32_t* parent, cons
   // the batched kernels' graph is built here, not in the first frame (a 32-node tree's took 200 to
   // 500 us longer); where that cannot be done now, the first frame does it
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (c->batch && batch_tree_prefers(n_nodes) &&
+  if (c->batch && batch_tree_prefers(n_nodes, false) &&
       (cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone ||
        batch_prepare(c->batch, p, &c->stream) != MCD_OK))
     (void)cudaGetLastError();

@@ -1342,11 +1342,16 @@ bool batch_prefers(const FrameParams& p, int n_streams) {
 // starts a new pass every 32.  Measured per call, frame kernel / batched (us): 15 nodes 247 / 255,
 // 16 nodes 280 / 255, 17 nodes 281 / 256, 31 nodes 330 / 262, 32 nodes 459 / 262, 64 nodes 737 / 273.
 // Every operand is hi + lo here, at any row count (the frame kernel's are single bf16 values above
-// 16 rows: 1.7e-3 off a 64-bit evaluation at 32 nodes against 3.6e-6).
+// 16 rows: 1.7e-3 off a 64-bit evaluation at 32 nodes against 3.6e-6).  A captured frame
+// enqueues the bodies of all 15 calls, of which 5 to 7 did something in these frames, frame kernel /
+// batched (us): 16 nodes 1848 / 2329, 24 nodes 1546 / 1942, 31 nodes 1627 / 1953, 32 nodes (two
+// passes) 2302 / 1954, 64 nodes 3661 / 2014.
 bool batch_tree_supported(const FrameParams& p) {
   return p.draft_mode == MCD_DRAFT_TREE && tc_block_supported(p) && p.V % tc::kBM == 0;
 }
-bool batch_tree_prefers(int nodes) { return nodes >= kBatchMinTreeNodes; }
+bool batch_tree_prefers(int nodes, bool captured) {
+  return nodes >= (captured ? kBatchMinCapturedTreeNodes : kBatchMinTreeNodes);
+}
 
 mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out) {
   *out = nullptr;

@@ -65,10 +65,11 @@ int batch_rows(const FrameParams& p, int max_streams);
 constexpr int kBatchMinStreams = 5;
 // Launches of this many streams go to the batched path even when the frame kernel fits them.
 bool batch_prefers(const FrameParams& p, int n_streams);
-// TREE mode: the batched kernels can run the context's tree calls, and do from this many nodes on.
-constexpr int kBatchMinTreeNodes = 16;
+// TREE mode: the batched kernels can run the context's tree calls, and do from this many nodes on;
+// in a frame that the caller captures, where every possible call is enqueued, from the second.
+constexpr int kBatchMinTreeNodes = 16, kBatchMinCapturedTreeNodes = 32;
 bool batch_tree_supported(const FrameParams& p);
-bool batch_tree_prefers(int nodes);
+bool batch_tree_prefers(int nodes, bool captured);
 mcd_status batch_create(const FrameParams& p, int max_streams, BatchState** out);
 // The batched path's copies of layer l's weights for its tensor-core GEMMs (no-op without).
 mcd_status batch_load_layer(BatchState* bs, const FrameParams& p, cudaStream_t st, const LayerSrc& src, int l);

@@ -588,6 +588,44 @@ def test_tree_mode_trace_parity_batched(nodes, depth):
     env.dec.close()
 
 
+@pytest.mark.parametrize("nodes,batched", [(31, False), (32, True)])
+def test_captured_tree_frames_choose_the_shorter_route(nodes, batched):
+    """A captured frame of a tree whose call fits one pass of the frame kernel is its two kernels; from
+    33 rows on it is the batched kernels of every possible call.  Either replays correctly."""
+    import ctypes
+    from oracle.tree import grow_tree
+    rt = ctypes.CDLL("libcudart.so.13")
+    cfg = TINY_BF16.replace(draft_mode=3, draft_len=3, n_pos=8, vocab=256)
+    stream = torch.cuda.Stream()
+    env = Env(cfg)
+    env.dec.close()
+    env.dec = mcd.Decoder(cfg, env.w, stream=stream)
+    tree = grow_tree([[0.6 / (r + 1) ** 0.5 for r in range(8)] for _ in range(3)], nodes)
+    mcd.mcd_set_tree(env.dec.ctx, tree.parent, tree.rank)
+    fr = make_frame(cfg, 2)
+    cond, c0, emb = env.frame_inputs(fr)
+    codes = torch.full((cfg.n_pos,), -1, dtype=torch.int32, device=DEV)
+    stats = torch.zeros(8, dtype=torch.int32, device=DEV)
+    tr = torch.zeros(mcd.mcd_trace_bytes(env.dec.ctx), dtype=torch.uint8, device=DEV)
+    mcd.mcd_set_trace(env.dec.ctx, tr)
+    torch.cuda.synchronize()
+    s, graph, exe, count = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_size_t()
+    assert rt.cudaStreamBeginCapture(s, 1) == 0                # thread-local mode
+    mcd.mcd_decode_frame(env.dec.ctx, 1, 2, cond, c0, emb, codes, stats)
+    assert rt.cudaStreamEndCapture(s, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+    assert (count.value > 100) if batched else (count.value == 2), count.value
+    assert rt.cudaGraphInstantiate(ctypes.byref(exe), graph, ctypes.c_ulonglong(0)) == 0
+    assert rt.cudaGraphLaunch(exe, s) == 0
+    mcd.mcd_sync(env.dec.ctx)
+    assert int(stats[4]) == 0 and int(stats[1]) == cfg.n_pos
+    check_tree_trace_against_oracle(cfg, env.model, fr, 1, 2, tr.cpu().numpy(), codes.cpu().numpy(), int(stats[0]), tree,
+                                    logit_tol=8e-5 if batched else 2e-2)
+    rt.cudaGraphExecDestroy(exe)
+    rt.cudaGraphDestroy(graph)
+    env.dec.close()
+
+
 def test_first_frame_of_a_large_tree_builds_no_graph():
     """mcd_set_tree prepares what the batched kernels need: the first frame of a 32-node tree takes
     as long as the next ones (measured 1.01 to 1.02 times; 1.18 to 1.19 where it builds the graph)."""

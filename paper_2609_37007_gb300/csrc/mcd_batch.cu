@@ -1,6 +1,7 @@
 // Batched decoding of many independent streams (up to 128 streams, 512 packed rows per
-// call), and of one stream's larger sparse trees: the per-frame draft-and-verify loop of arXiv 2609.37007 (Sec. 2.2, Fig. 3) for
-// every stream at once, with the rows of all unfinished streams re-packed every call.
+// call), and of one stream's larger sparse trees: the per-frame draft-and-verify loop of
+// arXiv 2609.37007 (Sec. 2.2, Fig. 3) for every stream at once, with the rows of all unfinished
+// streams re-packed every call.
 //
 // With hundreds of rows per call the weight matrices are multiplied as real GEMMs, so this
 // path is a sequence of grid-wide kernels per call instead of the persistent frame kernel:
@@ -10,10 +11,11 @@
 //
 // captured once per context as a CUDA graph: a while node whose body is one call, repeated
 // until every stream's frame is complete (a call never emits fewer than one code, so n_pos
-// calls always finish a frame).  Where the caller itself captures a graph, which cannot embed
+// calls always finish a frame).  A small kernel in front of the graph takes the frame's arguments by
+// value.  Where the caller itself captures a graph, which cannot embed
 // one that holds a conditional node, the n_pos bodies are enqueued one after another; bodies
 // after the last active call find no rows and return at once.  Measured with frames of 5 calls of
-// 15: 1792 us per frame of 8 streams and 2486 of 128 with the bodies enqueued, 1327 and 1955
+// 15: 1725 us per frame of 8 streams and 2400 of 128 with the bodies enqueued, 1116 and 1758
 // with the while node.  RMSNorm never gets its own pass.  With bf16
 // weights whose widths are multiples of 128 (the MultiCodeDecoder's) every product runs on
 // the tcgen05 GEMM (mcd_tcgemm.cuh, block kernels in mcd_tcops.cuh): weights and operand
@@ -109,7 +111,7 @@ struct BatchBufs {
   uint16_t* act;          // [R][F] bf16 SwiGLU outputs
   float* logits;          // [R][kRecSlots][V]
   TopkRec* recs;          // [2][R][kRecSlots]
-  // tensor-core GEMM operands (SW128 tiles of Rtc rows, Rtc = R rounded up to 128)
+  // tensor-core GEMM operands (SW128 tiles of Rtc rows: tc_operand_rows)
   int Rtc;
   uint8_t* xn_hi;         // normalised rows, bf16 (and the low halves for the QKV product)
   uint8_t* xn_lo;
@@ -1492,8 +1494,8 @@ static cudaError_t enqueue_call(const FrameParams& p, const BatchState* bs, cons
   const dim3 blk(256);
   // The products are dependent launches (their weights stream in while the kernel before them
   // runs); the small kernels between them start the ordinary way.  Frames of 5 calls, 8 / 128
-  // streams: 1235 / 1868 us with ordinary launches, 1169 / 1805 with dependent products, 1208 /
-  // 1810 with every kernel dependent, 1275 / 1901 with only the small ones.  Outside the while
+  // streams, when this was introduced: 1235 / 1868 us with ordinary launches, 1169 / 1805 with
+  // dependent products, 1208 / 1810 with every kernel dependent, 1275 / 1901 with only the small ones.  Outside the while
   // node the last bodies of a frame are empty: no prefetch there.
   const bool pdl = loop.valid != 0;
   batch_pack_kernel<<<1, 256, 0, s>>>(p, b);

@@ -186,7 +186,7 @@ struct FrameParams {
   float* logits_out;           // stepwise: verify logits of the single call
   int* emitted_out;
   int* n_emitted_out;
-  unsigned long long* timeline;  // optional [kMaxCalls][32] %globaltimer stamps (CTA 0)
+  unsigned long long* timeline;  // optional [kMaxCalls][kTimelineSlots] %globaltimer stamps
   int single_call;             // 1 = run exactly one call (stepwise API)
   TreeDef tree;                // TREE mode
   int* tree_cand;              // [kMaxDraft][kMaxTreeRank] candidates of the next call

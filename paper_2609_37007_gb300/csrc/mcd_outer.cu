@@ -302,8 +302,8 @@ __device__ void outer_attention(Cons& c, const OuterStep& o, int layer, int g, i
 // the block holds the row's position; then four threads per (query, key) score, and each warp
 // takes the softmax statistics of its query (redundantly) and 32 of the output's dims.
 // A chain of L2 round trips and shuffles bounds it.  12 rows at 333 positions with their prompt:
-// 10253 us with the general task and merge (9.1 k and 4.0 k of 48 k cycles per layer, stamped),
-// 9015 with these.
+// 10253 us with the general task and merge (9.1 k and 4.0 k of 48 k cycles per layer, stamped in an
+// instrumented copy), 9016 with these; 8850 with the waits of every stage inline.
 constexpr int kRowLd = 160;            // staged row (bf16): neighbouring keys 16 banks apart
 struct RowAttn {
   uint16_t *kb, *vb;                   // [32][kRowLd]
@@ -790,17 +790,17 @@ using namespace mcd;
 // layers as one batch (tcgen05 products with hi + lo operands, causal attention, K / V written
 // to the cache); outer_kernel then runs the c0 head on the last row's residual and samples c0.
 // With single bf16 operands outside QKV the last row had to run through outer_kernel's layers
-// again: 2.30 ms for 256 tokens, 0.61 of them in that row, against 1.66 ms; and the prompt's
-// outputs were 8.6e-5 off a 64-bit evaluation against 2.1e-5.
+// again: 2.30 ms for 256 tokens, 0.61 of them in that row, against 1.69 ms; and the prompt's
+// outputs were 8.6e-5 off a 64-bit evaluation against 2.2e-5.
 struct OuterTc {
   bool on = false;
   int Rtc = 0;                     // capacity in operand rows
   uint8_t* w = nullptr;            // per layer: SW128 copies of the weights
   TcLayerOffsets off;
   float* X = nullptr;              // [Rtc][H] residual stream
-  float* qkv = nullptr;            // [Rtc][qkv_dim]
+  float* qkv = nullptr;            // [Rtc][qkv_dim], up to kTcSmallRows rows kTcQkvSplit partial sums
   float* q = nullptr;              // [Rtc][NH * D] normalised, rotated queries
-  float* part = nullptr;           // [kTcSplit][Rtc][H] partial sums of the residual products
+  float* part = nullptr;           // k-split partial sums of the residual products (tc_part_floats)
   uint8_t *xn_hi = nullptr, *xn_lo = nullptr, *att_t = nullptr, *att_lo = nullptr, *act_t = nullptr, *act_lo = nullptr;   // operands
   int* rows = nullptr;             // device: live rows
 };
@@ -908,8 +908,9 @@ __global__ void __launch_bounds__(256) pf_rope_kv_kernel(const float* __restrict
 //
 // Measured on a 256-token prompt (28 layers, 16 / 8 heads x 128): 5.45 ms with one warp per
 // (row, head) and scalar products, where every warp read all its K and V for a single row (126
-// us per layer under the profiler); 2.86 ms with this kernel.  Error of the prompt's outputs
-// against a 64-bit evaluation: 8.1e-5 before, 8.2e-5 now (bf16 cache and operands set it).
+// us per layer under the profiler); 2.86 ms with this kernel at the time, 1.69 ms now.  It left the
+// prompt's error against a 64-bit evaluation where it was (8.1e-5, then 8.2e-5): the products' single
+// bf16 operands set that, and with hi + lo operands it is 2.2e-5.
 constexpr int kPfRows = 16, kPfKeys = 32, kPfWarps = 4;
 template <int D>
 struct PfAttn {

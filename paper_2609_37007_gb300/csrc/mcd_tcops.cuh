@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kQkvThreads, 1) tc_qkv_tile_kernel(const tc::G
 // the gate and up values of eight consecutive features of one packed row; it writes
 // silu(gate) * up as one 16-byte bf16 chunk of the down product's SW128 operand (k-slice b,
 // element (row n, feature m)).  Packed rows at or past *nrows are not written.
-// kHilo (the prompt): the operand and the result are hi + lo pairs of bf16 (about 16 mantissa bits).
+// kHilo (trees and prompts): the operand and the result are hi + lo pairs of bf16 (about 16 mantissa bits).
 constexpr int kGuThreads = 256;
 template <int BN, bool kHilo, int kBudget>
 __global__ void __launch_bounds__(kGuThreads, 1) tc_gu_kernel(const tc::GemmArgs g, uint8_t* act_t, uint8_t* act_lo, int Rtc,

@@ -1341,7 +1341,8 @@ bool batch_prefers(const FrameParams& p, int n_streams) {
 }
 
 // A tree call of 1 + nodes rows is one pass here; the persistent frame kernel pays for every row and
-// starts a new pass every 32.  Measured per call, frame kernel / batched (us): 15 nodes 247 / 255,
+// starts a new pass every 32.  Measured per call when the line was drawn, frame kernel / batched
+// (us): 15 nodes 247 / 255,
 // 16 nodes 280 / 255, 17 nodes 281 / 256, 31 nodes 330 / 262, 32 nodes 459 / 262, 64 nodes 737 / 273.
 // Every operand is hi + lo here, at any row count (the frame kernel's are single bf16 values above
 // 16 rows: 1.7e-3 off a 64-bit evaluation at 32 nodes against 3.6e-6).  A captured frame
